@@ -472,6 +472,7 @@ bgrpo_status bgrpo_tree_fuse_advantage(bgrpo_tree* t, const float* leaf_rewards_
     p.status = t->status;
     p.node_scratch = t->node_scratch;
     p.lv = t->lv;
+    p.runs = runs_of(t->lv, t->desc.T);
     p.n_trees = t->desc.n_trees;
     p.nodes_cap = t->desc.nodes_cap;
     p.T = t->desc.T;
@@ -494,6 +495,7 @@ bgrpo_status bgrpo_tree_fusion_ess(bgrpo_tree* t, float beta, float logp_scale, 
     p.node_scratch = t->node_scratch;
     p.status = t->status;
     p.lv = t->lv;
+    p.runs = runs_of(t->lv, t->desc.T);
     p.n_trees = t->desc.n_trees;
     p.nodes_cap = t->desc.nodes_cap;
     p.T = t->desc.T;
@@ -518,10 +520,10 @@ bgrpo_status bgrpo_tree_prune(bgrpo_tree* t, int32_t width_mode, int32_t k_or_b,
         p.pruned_bits |= 1ull << pruned_steps_host[q];
     }
     p.rbar = t->buf.rbar;
-    p.table = t->buf.node_table;
     p.mask = t->buf.mask;
     p.status = t->status;
     p.lv = t->lv;
+    p.runs = runs_of(t->lv, t->desc.T);
     p.n_trees = t->desc.n_trees;
     p.nodes_cap = t->desc.nodes_cap;
     p.T = t->desc.T;

@@ -88,6 +88,25 @@ struct LevelInfo {                       // layout of the tree grown so far
     int32_t fanout[BGRPO_MAX_T];         // children per node produced by step i (K or 1)
 };
 
+// Runs of a finished tree: maximal stretches of depths without a fork in between.  Run r covers the depths
+// first[r] .. first[r+1]-1, which all have the same width; an only child has its parent's leaves below it, hence its fused
+// value, its place among the siblings at every split and its kept leaves, so the reductions do their work per run and only
+// loads and stores are per depth.
+struct RunInfo {
+    int32_t n;
+    int32_t first[BGRPO_MAX_T + 2];      // first[n] = T + 1
+};
+
+inline RunInfo runs_of(const LevelInfo& lv, int T) {
+    RunInfo r;
+    r.n = 0;
+    r.first[r.n++] = 0;
+    for (int i = 0; i < T; ++i)
+        if (lv.fanout[i] > 1) r.first[r.n++] = i + 1;
+    r.first[r.n] = T + 1;
+    return r;
+}
+
 }  // namespace bgrpo
 
 struct bgrpo_tree {
@@ -110,7 +129,7 @@ struct bgrpo_tree {
     int32_t* status;
     unsigned int* counters;              // one ticket counter per (tree, node row)
     double* partials;                    // [n_trees*nodes_cap][nchunks][3]   (reward reductions)
-    double* node_scratch;                // [n_trees][2][nodes_cap]: per-node state of the tree reductions when a tree
+    double* node_scratch;                // [n_trees][2][nodes_cap]: per-chain state of the tree reductions when a tree
                                          // is too large for one CTA's shared memory
     float* partialsf;                    // [n_trees*nodes_cap][partials_per_row] (log-prob sums of the rollout kernels)
     unsigned int* mlp_tickets;           // 64-channel trees only: scratch of the MLP stage's split over the hidden dimension
@@ -210,23 +229,23 @@ struct FusedLaunch {
 cudaError_t launch_rollout_fused(const FusedLaunch& p, int32_t nodes, cudaStream_t s);
 
 // ---- tree reductions (tree_reduce.cu) -------------------------------------------------------------------------
-constexpr size_t kTreeSmemLimit = 200 * 1024;   // per-node doubles beyond this live in node_scratch instead of shared memory
+constexpr size_t kTreeSmemLimit = 200 * 1024;   // per-chain state beyond this lives in node_scratch instead of shared memory
 struct FuseLaunch {
     const float* leaf_r; const float* logp; float* rbar; float* adv; int32_t* status;
-    double* node_scratch;      // [n_trees][2][nodes_cap], used when three doubles per node exceed kTreeSmemLimit (trees of more than 8 533 nodes)
-    LevelInfo lv; int32_t n_trees, nodes_cap, T, nodes; double beta_scaled; float eps, clip;
+    double* node_scratch;      // [n_trees][2][nodes_cap], used when two doubles per chain exceed kTreeSmemLimit (trees of more than 12 800 chains)
+    LevelInfo lv; RunInfo runs; int32_t n_trees, nodes_cap, T, nodes; double beta_scaled; float eps, clip;
 };
 cudaError_t launch_fuse_advantage(const FuseLaunch& p, cudaStream_t s);
 
 struct EssLaunch {
     const float* logp; float* ess; double* node_scratch; int32_t* status;
-    LevelInfo lv; int32_t n_trees, nodes_cap, T, nodes; double beta_scaled;
+    LevelInfo lv; RunInfo runs; int32_t n_trees, nodes_cap, T, nodes; double beta_scaled;
 };
 cudaError_t launch_fusion_ess(const EssLaunch& p, cudaStream_t s);
 
 struct PruneLaunch {
-    const float* rbar; const int32_t* table; uint8_t* mask; int32_t* status;
-    LevelInfo lv; int32_t n_trees, nodes_cap, T, nodes, mode, k, last_split, ignore_last, values_in_smem; uint64_t pruned_bits;
+    const float* rbar; uint8_t* mask; int32_t* status;
+    LevelInfo lv; RunInfo runs; int32_t n_trees, nodes_cap, T, nodes, mode, k, last_split, ignore_last; uint64_t pruned_bits;
 };
 cudaError_t launch_prune(const PruneLaunch& p, cudaStream_t s);
 

@@ -761,3 +761,37 @@ def test_prune_has_no_node_limit(B):
         torch.cuda.synchronize()
         ref = credit.gradient_mask(topo, rbar[0], mode, k, (4,), False)
         assert np.array_equal(s.mask.cpu().numpy()[0], ref), mode
+
+
+@pytest.mark.parametrize("T,K,splits", [(1, 2, ()), (1, 3, (0,)), (9, 2, tuple(range(9))), (12, 2, (0, 1, 2, 3, 4, 5, 6, 8, 9, 10)), (8, 1, (2, 5)),
+                                        (7, 4, (0, 1, 3, 4, 5))])
+def test_reductions_where_their_branches_change(B, T, K, splits):
+    """Trees at the edges of the reductions' branches: one run only, forks at every step, long chains, K = 1 "forks", and
+    Extreme-b on 512 leaves (ranked by counting) and 1024 (radix selection), with exact ties.  Masks are whole numbers;
+    fused values, advantages and effective sample sizes within the bounds of the tests above."""
+    w, s, topo = _grown_session(B, T, K, splits)
+    rng = np.random.default_rng(100 * T + K)
+    r = np.round(rng.standard_normal((2, topo.leaves)), 1).astype(np.float32)
+    lp = (-0.9 + 0.3 * rng.standard_normal((2, topo.nodes))).astype(np.float32)
+    lp[:, 0] = 0
+    s.logp.copy_(torch.from_numpy(lp))
+    ess = torch.empty_like(s.logp)
+    for beta in (0.0, 1.0):
+        B.tree_fuse_advantage(s.tree, torch.from_numpy(r).cuda(), beta, 1.0, 1e-6, 5.0)
+        B.tree_fusion_ess(s.tree, beta, 1.0, ess)
+        torch.cuda.synchronize()
+        for t in range(2):
+            rbar = credit.fuse_rewards(topo, r[t], lp[t].astype(np.float64), beta, 1.0)
+            ref_ess = credit.fusion_ess(topo, lp[t].astype(np.float64), beta, 1.0)
+            assert np.abs(s.rbar.cpu().numpy()[t] - rbar).max() <= 1e-6 * max(1.0, np.abs(rbar).max())
+            assert adv_close(s.adv.cpu().numpy()[t], credit.depth_advantages(topo, rbar, f32(1e-6), 5.0))
+            assert np.all(np.abs(ess.cpu().numpy()[t, :topo.nodes] - ref_ess) <= 1e-5 * ref_ess)
+    coarse = np.round(rng.standard_normal((2, topo.nodes)), 1).astype(np.float32)
+    s.rbar.copy_(torch.from_numpy(coarse))
+    for mode, k in ((B.WIDTH_EXTREME_B, 1), (B.WIDTH_EXTREME_B, 100), (B.WIDTH_PER_SPLIT_TOPK, 1), (B.WIDTH_LAST_SPLIT_TOPK, 2)):
+        s.mask.fill_(9)
+        B.tree_prune(s.tree, mode, k, (T - 1,), False)
+        torch.cuda.synchronize()
+        for t in range(2):
+            assert np.array_equal(s.mask.cpu().numpy()[t], credit.gradient_mask(topo, coarse[t], mode, k, (T - 1,), False)), (mode, k, t)
+    B.tree_sync_status(s.tree)
