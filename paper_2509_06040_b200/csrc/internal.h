@@ -95,6 +95,8 @@ struct LevelInfo {                       // layout of the tree grown so far
 struct RunInfo {
     int32_t n;
     int32_t first[BGRPO_MAX_T + 2];      // first[n] = T + 1
+    int32_t chain0[BGRPO_MAX_T + 2];     // index of the run's first chain (a node and the only children below it); chain0[n] = number of chains
+    int32_t of_depth[BGRPO_MAX_T + 1];
 };
 
 inline RunInfo runs_of(const LevelInfo& lv, int T) {
@@ -104,6 +106,11 @@ inline RunInfo runs_of(const LevelInfo& lv, int T) {
     for (int i = 0; i < T; ++i)
         if (lv.fanout[i] > 1) r.first[r.n++] = i + 1;
     r.first[r.n] = T + 1;
+    r.chain0[0] = 0;
+    for (int q = 0; q < r.n; ++q) {
+        r.chain0[q + 1] = r.chain0[q] + lv.width[r.first[q]];
+        for (int d = r.first[q]; d < r.first[q + 1]; ++d) r.of_depth[d] = q;
+    }
     return r;
 }
 

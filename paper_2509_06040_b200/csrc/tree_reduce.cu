@@ -33,13 +33,8 @@ struct Layout {
     int chain0[BGRPO_MAX_T + 2];        // chain0[runs.n] = number of chains
     __device__ void fill(const LevelInfo& lv, const RunInfo& runs, int T) {
         for (int d = threadIdx.x; d <= T + 1; d += kTreeThreads) off[d] = lv.offset[d];
-        for (int r = threadIdx.x; r <= runs.n; r += kTreeThreads) {
-            int c = 0;
-            for (int q = 0; q < r; ++q) c += lv.width[runs.first[q]];
-            chain0[r] = c;
-            if (r < runs.n)
-                for (int d = runs.first[r]; d < runs.first[r + 1]; ++d) run[d] = r;
-        }
+        for (int d = threadIdx.x; d <= T; d += kTreeThreads) run[d] = runs.of_depth[d];
+        for (int r = threadIdx.x; r <= runs.n; r += kTreeThreads) chain0[r] = runs.chain0[r];
     }
 };
 
@@ -51,7 +46,7 @@ __device__ __forceinline__ void chain_sums(double* out, const float* logp, const
         while (m >= lay.chain0[r + 1]) ++r;
         const int j = m - lay.chain0[r];
         double c = 0.0;
-#pragma unroll 4
+#pragma unroll 8
         for (int d = runs.first[r + 1] - 1; d >= runs.first[r]; --d) c += beta * static_cast<double>(logp[lay.off[d] + j]);
         out[m] = c;
     }
@@ -69,7 +64,7 @@ fuse_advantage_kernel(const __grid_constant__ FuseLaunch p) {
     lay.fill(p.lv, p.runs, T);
     if (threadIdx.x == 0) bad = 0;
     __syncthreads();
-    const int chains = lay.chain0[R];
+    const int chains = p.runs.chain0[R];
     const bool in_smem = static_cast<size_t>(chains) * 2 * sizeof(double) <= kTreeSmemLimit;
     double* rb = in_smem ? sm : p.node_scratch + static_cast<int64_t>(tree) * 2 * p.nodes_cap;   // fused value per chain
     double* ls = rb + (in_smem ? chains : p.nodes_cap);      // log S of the chain's last node + beta * logp along the chain
@@ -167,7 +162,7 @@ fusion_ess_kernel(const __grid_constant__ EssLaunch p) {
     const int T = p.T, R = p.runs.n;
     lay.fill(p.lv, p.runs, T);
     __syncthreads();
-    const int chains = lay.chain0[R];
+    const int chains = p.runs.chain0[R];
     const bool in_smem = static_cast<size_t>(chains) * 2 * sizeof(double) <= kTreeSmemLimit;
     double* ls = in_smem ? sm : p.node_scratch + static_cast<int64_t>(tree) * 2 * p.nodes_cap;
     double* lq = ls + (in_smem ? chains : p.nodes_cap);
@@ -294,7 +289,7 @@ prune_kernel(const __grid_constant__ PruneLaunch p) {
     uint8_t* mask = p.mask + row0;
     lay.fill(p.lv, p.runs, T);
     __syncthreads();
-    const int chains = lay.chain0[R];
+    const int chains = p.runs.chain0[R];
     const bool in_smem = static_cast<size_t>(chains) <= kTreeSmemLimit;
     if (!BGRPO_IN_BOUNDS(p.status, chains <= p.nodes && p.nodes <= p.nodes_cap && tree < p.n_trees)) return;
     auto depth_ok = [&](int d) { return d > 0 && !((p.pruned_bits >> (d - 1)) & 1ull) && !(p.ignore_last && d == T); };
@@ -447,14 +442,8 @@ cudaError_t launch_objective(const ObjectiveLaunch& p, cudaStream_t s) {
     return launch_overlapped(objective_kernel, p.n_trees, kTreeThreads, 0, s, p);
 }
 
-static int chains_of(const LevelInfo& lv, const RunInfo& runs) {
-    int64_t c = 0;
-    for (int r = 0; r < runs.n; ++r) c += lv.width[runs.first[r]];
-    return static_cast<int>(c);
-}
-
 cudaError_t launch_fusion_ess(const EssLaunch& p, cudaStream_t s) {
-    size_t smem = static_cast<size_t>(chains_of(p.lv, p.runs)) * 2 * sizeof(double);
+    size_t smem = static_cast<size_t>(p.runs.chain0[p.runs.n]) * 2 * sizeof(double);
     if (smem > kTreeSmemLimit) smem = 0;          // per-chain state in the caller's scratch
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(fusion_ess_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
@@ -464,7 +453,7 @@ cudaError_t launch_fusion_ess(const EssLaunch& p, cudaStream_t s) {
 }
 
 cudaError_t launch_fuse_advantage(const FuseLaunch& p, cudaStream_t s) {
-    size_t smem = static_cast<size_t>(chains_of(p.lv, p.runs)) * 2 * sizeof(double);
+    size_t smem = static_cast<size_t>(p.runs.chain0[p.runs.n]) * 2 * sizeof(double);
     if (smem > kTreeSmemLimit) smem = 0;          // per-chain state in the caller's scratch
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(fuse_advantage_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
@@ -474,7 +463,7 @@ cudaError_t launch_fuse_advantage(const FuseLaunch& p, cudaStream_t s) {
 }
 
 cudaError_t launch_prune(const PruneLaunch& p, cudaStream_t s) {
-    size_t smem = static_cast<size_t>(chains_of(p.lv, p.runs));
+    size_t smem = static_cast<size_t>(p.runs.chain0[p.runs.n]);
     if (smem > kTreeSmemLimit) smem = 0;          // the paths are walked node by node, Extreme-b flags live in the mask
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(prune_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
