@@ -16,6 +16,7 @@ from dataclasses import dataclass
 from typing import Optional, Sequence
 
 import numpy as np
+import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 # BGRPO_DEBUG_BOUNDS=1 selects the build whose kernels check every index they derive (python -m ...build --debug-bounds)
@@ -116,7 +117,10 @@ def _ptr(t) -> Optional[int]:
 
 def _stream(stream) -> Optional[int]:
     if stream is None:
-        import torch
+        # The raw handle of the current stream, without the Stream object and the device probing around it (0.3 us instead
+        # of 4.3 us: as much as a kernel launch, on every call of a launch-bound program).
+        if torch.cuda.is_initialized():
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()) or None
         if not torch.cuda.is_available():
             return None
         return torch.cuda.current_stream().cuda_stream or None

@@ -46,6 +46,7 @@ class TreeSession:
         self.tree = None
         self.mu = self.target = self.packed = self.v = self.reward_draws = None
         self.pruned_steps = ()
+        self._beta, self._eps, self._adv_clip = (float(np.float32(x)) for x in (w.beta, w.eps, w.adv_clip))
         self._split_flags = np.ascontiguousarray([1 if i in w.splits else 0 for i in range(w.T)], dtype=np.uint8)
 
     # -- inputs ---------------------------------------------------------------------------------------------------
@@ -115,9 +116,7 @@ class TreeSession:
             raise ValueError(w.reward)
 
     def fuse_advantage(self):
-        w = self.w
-        B.tree_fuse_advantage(self.tree, self.leaf_r, float(np.float32(w.beta)), 1.0, float(np.float32(w.eps)),
-                              float(np.float32(w.adv_clip)))
+        B.tree_fuse_advantage(self.tree, self.leaf_r, self._beta, 1.0, self._eps, self._adv_clip)
 
     def prune(self):
         w = self.w
