@@ -21,7 +21,7 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libbgrpo.so")
 LIB_DEBUG = os.path.join(HERE, "libbgrpo_debug.so")
-SOURCES = ["api.cu", "tree_step.cu", "tree_reward.cu", "tree_fused.cu", "tree_reduce.cu", "mlp_velocity.cu", "static_scratch.cu"]
+SOURCES = ["api.cu", "tree_step.cu", "tree_logprob.cu", "tree_reward.cu", "tree_fused.cu", "tree_reduce.cu", "mlp_velocity.cu", "static_scratch.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-Xptxas", "-v"]
 

@@ -401,27 +401,61 @@ bgrpo_status bgrpo_tree_logprob(bgrpo_tree* t, int32_t step, const float* v_dev,
     if (step == -1 && v_dev) return fail(BGRPO_ERR_INVALID_ARG, "step -1 works with the bound linear velocity only");
     if (!v_dev && !t->mu) return fail(BGRPO_ERR_STATE, "no velocity: pass v_dev or bind a linear velocity");
     if (v_dev && !aligned(v_dev, 16)) return fail(BGRPO_ERR_INVALID_ARG, "v misaligned");
-    const int first = step < 0 ? 0 : step, last = step < 0 ? t->depth - 1 : step;
     {   // a step's own sums may still be pending and could live in the rows this call is about to rewrite
         const cudaError_t e0 = flush_pending(t, as_stream(stream));
         if (e0 != cudaSuccess) return cuda_fail(e0, "log-prob flush kernel");
     }
-    for (int i = first; i <= last; ++i) {
-        StepLaunch p;
-        fill_step_launch(t, i, v_dev, &p);
-        p.W_in = t->lv.width[i];
-        p.off_in = t->lv.offset[i];
-        p.off_out = t->lv.offset[i + 1];
-        p.fan = t->lv.fanout[i];
-        p.is_split = 0;
-        p.shared_noise = 0;
-        p.write_children = 0;
+    if (step < 0) {
+        LogprobLaunch p;
+        p.latents = t->buf.latents;
+        p.mu = t->mu;
         p.logp_out = logp_out_dev;
-        cudaError_t e = launch_step(p, as_stream(stream));
-        if (e != cudaSuccess) return cuda_fail(e, "logprob kernel");
-        t->pending = FinalizeDesc{logp_out_dev, t->lv.width[i + 1], t->lv.offset[i + 1], p.g, p.inv_2g2, p.logp_const};
+        p.partials = reinterpret_cast<double*>(t->partialsf);
+        p.status = t->status;
+        p.D = t->D;
+        p.n_trees = t->desc.n_trees;
+        p.nodes_cap = t->desc.nodes_cap;
+        p.nchunks = static_cast<int32_t>((t->D / 4 + kLogprobChunkVec - 1) / kLogprobChunkVec);
+        p.per_row = static_cast<int32_t>(partials_per_row(t->D));
+        p.depth = t->depth;
+        for (int d = 0; d <= t->depth + 1; ++d) p.off[d] = t->lv.offset[d];
+        for (int i = 0; i < t->depth; ++i) {
+            const StepCoef& k = t->coef[i];
+            p.ca[i] = k.lin_a;
+            p.cb[i] = k.lin_b;
+            p.g[i] = k.g;
+            p.inv_2g2[i] = k.inv_2g2;
+            p.logp_const[i] = k.logp_const;
+        }
+        // a fork and the chains below it; run 0 is the chain below the root
+        const RunInfo runs = runs_of(t->lv, t->depth);
+        p.n_runs = runs.n;
+        p.families = 0;
+        for (int r = 0; r < runs.n; ++r) {
+            const int d0 = r == 0 ? 0 : runs.first[r] - 1;
+            p.run_d0[r] = d0;
+            p.run_fan[r] = r == 0 ? 1 : t->lv.fanout[d0];
+            p.run_len[r] = runs.first[r + 1] - (d0 + 1);
+            p.run_families[r] = p.run_len[r] > 0 ? t->lv.width[d0] : 0;
+            p.families += p.run_families[r];
+        }
+        const cudaError_t e = launch_logprob_tree(p, as_stream(stream));
+        return e == cudaSuccess ? BGRPO_OK : cuda_fail(e, "logprob kernel");
     }
-    const cudaError_t e = flush_pending(t, as_stream(stream));
+    StepLaunch p;
+    fill_step_launch(t, step, v_dev, &p);
+    p.W_in = t->lv.width[step];
+    p.off_in = t->lv.offset[step];
+    p.off_out = t->lv.offset[step + 1];
+    p.fan = t->lv.fanout[step];
+    p.is_split = 0;
+    p.shared_noise = 0;
+    p.write_children = 0;
+    p.logp_out = logp_out_dev;
+    cudaError_t e = launch_step(p, as_stream(stream));
+    if (e != cudaSuccess) return cuda_fail(e, "logprob kernel");
+    t->pending = FinalizeDesc{logp_out_dev, t->lv.width[step + 1], t->lv.offset[step + 1], p.g, p.inv_2g2, p.logp_const};
+    e = flush_pending(t, as_stream(stream));
     if (e != cudaSuccess) return cuda_fail(e, "log-prob flush kernel");
     return BGRPO_OK;
 }

@@ -206,6 +206,24 @@ cudaError_t launch_root(const bgrpo_tree* t, cudaStream_t s);
 cudaError_t launch_step(const StepLaunch& p, cudaStream_t s);
 cudaError_t launch_finalize(const bgrpo_tree* t, const FinalizeDesc& f, cudaStream_t s);
 
+// ---- log-probs of all stored edges (tree_logprob.cu) ---------------------------------------------------------------
+constexpr int kLogprobChunkVec = 512;      // float4 of a row per CTA; one double per (row, chunk) fits the step kernel's partials
+static_assert(kLogprobChunkVec == kStepChunkVec && kStepWarps == 2, "the partials of both kernels share their place");
+struct LogprobLaunch {
+    const float* latents;
+    const float* mu;           // [n_trees][D]
+    float* logp_out;
+    double* partials;          // [rows][nchunks]
+    int32_t* status;
+    int64_t D;
+    int32_t n_trees, nodes_cap, nchunks, per_row, depth;
+    int32_t families, n_runs;                          // families per tree, in all runs
+    int32_t run_families[BGRPO_MAX_T + 1], run_d0[BGRPO_MAX_T + 1], run_fan[BGRPO_MAX_T + 1], run_len[BGRPO_MAX_T + 1];
+    int32_t off[BGRPO_MAX_T + 2];
+    float ca[BGRPO_MAX_T], cb[BGRPO_MAX_T], g[BGRPO_MAX_T], inv_2g2[BGRPO_MAX_T], logp_const[BGRPO_MAX_T];   // by step
+};
+cudaError_t launch_logprob_tree(const LogprobLaunch& p, cudaStream_t s);
+
 struct RewardLaunch {
     const float* latents; const float* target; float* r; double* partials; unsigned int* counters; int32_t* status;
     int64_t D; int32_t n_trees, nodes_cap, nchunks, nchunks_cap, leaves, off_leaf; float scale; int32_t mode;  // 0 mse, 1 cos; nchunks_cap: partial slots reserved per row

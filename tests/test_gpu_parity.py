@@ -795,3 +795,51 @@ def test_reductions_where_their_branches_change(B, T, K, splits):
         for t in range(2):
             assert np.array_equal(s.mask.cpu().numpy()[t], credit.gradient_mask(topo, coarse[t], mode, k, (T - 1,), False)), (mode, k, t)
     B.tree_sync_status(s.tree)
+
+
+@pytest.mark.parametrize("tokens,channels,n_trees,T,K,splits,grown", [
+    (1, 4, 1, 3, 2, (1,), 3),                 # one float4 a row
+    (512, 4, 2, 5, 3, (0, 3), 5),             # exactly one chunk a row
+    (513, 4, 1, 6, 4, (2,), 4),               # one float4 more; a partly grown tree that ends in a chain
+    (1021, 16, 2, 4, 2, (0, 1, 2, 3), 4),     # ragged last chunk, no chains
+    (300, 64, 3, 7, 2, (), 7),                # no fork at all
+])
+def test_logprob_families_at_their_edges(B, tokens, channels, n_trees, T, K, splits, grown):
+    """Stored edges scored per step and all at once (families walked down the chains), closed form and supplied velocity,
+    against the float64 formula on the stored latents; each call twice."""
+    w = Workload(name="families", n_trees=n_trees, tokens=tokens, channels=channels, T=T, K=K, splits=splits, sigma=0.3,
+                 velocity="linear", reward="neg_mse_mu")
+    s = _session(w)
+    s.upload_inputs(make_inputs(w))
+    s.init()
+    for i in range(grown):
+        s.step(i)
+    widths, offs = B.tree_levels(s.tree)
+    g = torch.Generator(device="cuda").manual_seed(tokens)
+    lat, mu, grid, sig, s0 = s.latents.double(), s.mu.double(), w.t_grid().astype(np.float64), f32(w.sigma), f32(w.s0)
+    every = torch.full_like(s.logp, 7.0)
+    B.tree_logprob(s.tree, -1, None, every)
+    for i in range(grown):
+        W, F = widths[i], widths[i + 1] // widths[i]
+        t, h = grid[i], grid[i] - grid[i + 1]
+        z = lat[:, offs[i]:offs[i] + W]
+        child = lat[:, offs[i + 1]:offs[i + 1] + W * F].view(n_trees, W, F, w.D)
+        k = (t - (1 - t) * s0 * s0) / ((1 - t) ** 2 * s0 * s0 + t * t)
+        v_lin = -mu[:, None] + k * (z - (1 - t) * mu[:, None])
+        v_given = torch.randn(n_trees, W, w.D, device="cuda", generator=g)
+        for v, given in ((v_lin, None), (v_given.double(), v_given)):
+            mean = z - h * v - sig * sig * h / (2 * t) * (z + (1 - t) * v)
+            ref = -((child - mean[:, :, None]) ** 2).mean(-1) / (2 * sig * sig * h) - math.log(sig * math.sqrt(h)) - 0.5 * math.log(2 * math.pi)
+            ref = ref.view(n_trees, W * F)
+            bound = 1e-5 * ref.abs().clamp(min=1.0)
+            got = torch.full_like(s.logp, 7.0)
+            for _ in range(2):
+                B.tree_logprob(s.tree, i, given, got)
+            rows = slice(offs[i + 1], offs[i + 1] + W * F)
+            assert bool(((got[:, rows].double() - ref).abs() <= bound).all()), i
+            if given is None:
+                assert bool(((every[:, rows].double() - ref).abs() <= bound).all()), i
+            got[:, rows] = 7.0
+            assert bool((got == 7.0).all())                 # only the addressed edges were written
+    assert bool((every[:, 0] == 7.0).all())
+    B.tree_sync_status(s.tree)
