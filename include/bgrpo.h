@@ -145,10 +145,10 @@ bgrpo_status bgrpo_velocity_linear_bind(bgrpo_tree* tree, const float* mu_dev, f
 bgrpo_status bgrpo_tree_step(bgrpo_tree* tree, int32_t split_flag, const float* v_dev, void* stream);
 
 /* tree_rollout: the remaining steps of the tree, depth .. T-1, in one host call (Algorithm 1, "Build rollout tree": for
- * every step, the velocity of every live node, then the step that forks or advances it).  The same kernels in the same
- * order as calling bgrpo_velocity_mlp (when packed_dev is given) and bgrpo_tree_step step by step, so every output is
- * identical bit for bit; what it saves is the caller's per-call overhead, which on single-tree workloads (launches of
- * 5-40 us) is comparable to the launches themselves.
+ * every step, the velocity of every live node, then the step that forks or advances it).  With packed_dev the same kernels
+ * in the same order as calling bgrpo_velocity_mlp and bgrpo_tree_step step by step; a whole tree under the bound linear
+ * velocity takes the one launch of bgrpo_tree_rollout_fused where that covers it.  Every output is identical bit for bit to
+ * the step-by-step calls either way (log-probs because the sums of squares are added as integers).
  *   split_flags_host  host array of T flags (indexed by step), non-zero = fork every node into K children
  *   packed_dev        device, packed MLP weights (bgrpo_velocity_mlp_pack), or NULL for the bound linear velocity
  *   v_dev             device [n_trees][W_max][D] float32 scratch for the velocities of the widest frontier (NULL allowed
@@ -163,8 +163,7 @@ bgrpo_status bgrpo_tree_rollout(bgrpo_tree* tree, const uint8_t* split_flags_hos
  * element by itself, so one thread can carry its elements from the root to every leaf, depth first, and write each
  * node once: nothing is read back between depths.  Call it on a freshly initialised or reset tree.  split_flags_host:
  * host array of T flags, non-zero = step i forks every node into K children.  Latents, node table and log-probs are the
- * ones T calls of tree_step give (latents and table bit for bit; log-probs up to the order of a float32 partial sum),
- * and buffers.logp is final when the call's kernels have run.  At most 6 split steps.
+ * ones T calls of tree_step give, and buffers.logp is final when the call's kernels have run.  At most 6 split steps.
  * Errors: STATE (tree not at depth 0, no bound linear velocity), CAPACITY (tree exceeds nodes_cap), UNSUPPORTED (more
  * than 6 split steps: use tree_step), INVALID_ARG (a split on an ODE step of the hybrid schedule), CUDA. */
 bgrpo_status bgrpo_tree_rollout_fused(bgrpo_tree* tree, const uint8_t* split_flags_host, void* stream);

@@ -108,11 +108,11 @@ void bind_buffers(bgrpo_tree* t, const bgrpo_buffers* b) {
     t->counters = reinterpret_cast<unsigned int*>(sc + kScratchHeader);
     t->partials = reinterpret_cast<double*>(sc + kScratchHeader + ((rows * sizeof(unsigned int) + 255) / 256) * 256);
     t->node_scratch = t->partials + rows * static_cast<size_t>(t->nchunks) * 3;
-    t->partialsf = reinterpret_cast<float*>(t->node_scratch + rows * 2);
+    t->partials_logp = t->node_scratch + rows * 2;
     t->mlp_tickets = nullptr;
     t->mlp_partials = nullptr;
     if (desc->channels == BGRPO_MLP_CHANNELS) {
-        const size_t used = reinterpret_cast<char*>(t->partialsf + rows * static_cast<size_t>(partials_per_row(t->D))) - sc;
+        const size_t used = static_cast<size_t>(static_cast<char*>(t->partials_logp) - sc) + rows * static_cast<size_t>(partials_per_row(t->D)) * sizeof(uint32_t);
         t->mlp_tickets = reinterpret_cast<unsigned int*>(sc + ((used + 255) / 256) * 256);
         t->mlp_partials = reinterpret_cast<float*>(reinterpret_cast<char*>(t->mlp_tickets) + kMlpTicketBytes);
     }
@@ -255,7 +255,7 @@ static void fill_step_launch(const bgrpo_tree* t, int step, const float* v_dev, 
     p->mu = v_dev ? nullptr : t->mu;
     p->logp = t->buf.logp;
     p->table = t->buf.node_table;
-    p->partialsf = t->partialsf;
+    p->partials = t->partials_u64();
     p->status = t->status;
     p->per_row = static_cast<int32_t>(partials_per_row(t->D));
     p->prev = t->pending;
@@ -269,8 +269,6 @@ static void fill_step_launch(const bgrpo_tree* t, int step, const float* v_dev, 
     p->ca = v_dev ? k.a : k.lin_a;
     p->cb = v_dev ? k.b : k.lin_b;
     p->g = k.g;
-    p->inv_2g2 = k.inv_2g2;
-    p->logp_const = k.logp_const;
     p->mix_shared = t->mix_shared;
     p->mix_innov = t->mix_innov;
 }
@@ -295,13 +293,11 @@ bgrpo_status bgrpo_tree_step(bgrpo_tree* t, int32_t split_flag, const float* v_d
     p.fan = fan;
     p.is_split = split_flag ? 1 : 0;
     p.shared_noise = (split_flag && !t->independent && t->coef[i].g > 0.0f) ? 1 : 0;
-    p.write_children = 1;
-    p.logp_out = t->buf.logp;
     cudaError_t e = launch_step(p, as_stream(stream));
     if (e != cudaSuccess) return cuda_fail(e, "step kernel");
     // this launch summed the previous level's log-probs in its prologue; its own are pending until the next
     // launch, or until the flush below when the tree is complete
-    t->pending = FinalizeDesc{t->buf.logp, static_cast<int32_t>(W_out), static_cast<int32_t>(off_out), p.g, p.inv_2g2, p.logp_const};
+    t->pending = FinalizeDesc{t->buf.logp, static_cast<int32_t>(W_out), static_cast<int32_t>(off_out), t->coef[i].g, t->coef[i].logp_const};
     if (i + 1 == t->desc.T) {
         e = flush_pending(t, as_stream(stream));
         if (e != cudaSuccess) return cuda_fail(e, "log-prob flush kernel");
@@ -318,6 +314,23 @@ bgrpo_status bgrpo_tree_rollout(bgrpo_tree* t, const uint8_t* split_flags_host, 
     if (!t || !split_flags_host) return fail(BGRPO_ERR_INVALID_ARG, "tree or split_flags is NULL");
     if (packed_dev && !v_dev) return fail(BGRPO_ERR_INVALID_ARG, "the MLP velocity needs a velocity buffer");
     if (!packed_dev && !t->mu) return fail(BGRPO_ERR_STATE, "no velocity: pass the packed MLP weights or bind a linear velocity");
+    if (!packed_dev && t->depth == 0) {
+        // A whole tree under the closed form: one launch gives the same bits (latents, table and, the sums of squares being
+        // exact, log-probs).  What that kernel does not cover, and every error, is left to the steps.
+        int64_t width = 1, nodes = 1;
+        int n_splits = 0;
+        bool covered = true;
+        for (int i = 0; i < t->desc.T && covered; ++i) {
+            if (split_flags_host[i]) {
+                ++n_splits;
+                width *= t->desc.K;
+                covered = n_splits <= kFusedMaxSplits && !(((t->ode_bits >> i) & 1ull) && t->desc.sigma > 0.0f);
+            }
+            nodes += width;
+            covered = covered && nodes <= t->desc.nodes_cap;
+        }
+        if (covered) return bgrpo_tree_rollout_fused(t, split_flags_host, stream);
+    }
     for (int i = t->depth; i < t->desc.T; ++i) {
         if (packed_dev) {
             const bgrpo_status st = bgrpo_velocity_mlp(t, packed_dev, hidden, v_dev, stream);
@@ -338,40 +351,34 @@ bgrpo_status bgrpo_tree_rollout_fused(bgrpo_tree* t, const uint8_t* split_flags_
     std::memset(&p, 0, sizeof(p));
     int n_splits = 0;
     int64_t width = 1, off = 1;
-    p.off[0] = 0;
-    p.off[1] = 1;
     for (int i = 0; i < T; ++i) {
         const bool split = split_flags_host[i] != 0;
         if (split) {
             if (((t->ode_bits >> i) & 1ull) && t->desc.sigma > 0.0f)
                 return fail(BGRPO_ERR_INVALID_ARG, "a split step must be an SDE step of the hybrid schedule");
             ++n_splits;
-            p.split_bits |= 1ull << i;
             width *= t->desc.K;
         }
+        const StepCoef& k = t->coef[i];
+        p.step[i].ca = k.lin_a;
+        p.step[i].cb = k.lin_b;
+        p.step[i].g = k.g;
+        p.step[i].child0 = static_cast<uint32_t>(off) | (split ? kForks : 0u);
+        p.step[i].logp_const = k.logp_const;
         off += width;
         if (off > t->desc.nodes_cap) return fail(BGRPO_ERR_CAPACITY, "children exceed nodes_cap");
-        p.off[i + 2] = static_cast<int32_t>(off);
-        const StepCoef& k = t->coef[i];
-        p.ca[i] = k.lin_a;
-        p.cb[i] = k.lin_b;
-        p.g[i] = k.g;
-        p.inv_2g2[i] = k.inv_2g2;
-        p.logp_const[i] = k.logp_const;
     }
     if (n_splits > kFusedMaxSplits) return fail(BGRPO_ERR_UNSUPPORTED, "more split steps than the whole-tree kernel walks; use tree_step");
     p.latents = t->buf.latents;
     p.mu = t->mu;
     p.logp = t->buf.logp;
     p.table = t->buf.node_table;
-    p.partialsf = t->partialsf;
+    p.partials = static_cast<uint32_t*>(t->partials_logp);
     p.status = t->status;
     p.per_row_cap = static_cast<int32_t>(partials_per_row(t->D));
     p.D = t->D;
     p.n_trees = t->desc.n_trees;
     p.nodes_cap = t->desc.nodes_cap;
-    p.nchunks = static_cast<int32_t>((t->D / 4 + kFusedChunkVec - 1) / kFusedChunkVec);
-    p.per_row = static_cast<int32_t>(fused_partials_per_row(t->D));
     p.T = T;
     p.K = t->desc.K;
     p.shared_noise = t->independent ? 0 : 1;
@@ -384,11 +391,11 @@ bgrpo_status bgrpo_tree_rollout_fused(bgrpo_tree* t, const uint8_t* split_flags_
     // host mirror of the finished tree
     int32_t w = 1;
     for (int i = 0; i < T; ++i) {
-        const int fan = ((p.split_bits >> i) & 1ull) ? t->desc.K : 1;
+        const int fan = (p.step[i].child0 & kForks) ? t->desc.K : 1;
         t->lv.fanout[i] = fan;
         w *= fan;
         t->lv.width[i + 1] = w;
-        t->lv.offset[i + 2] = p.off[i + 2];
+        t->lv.offset[i + 2] = t->lv.offset[i + 1] + w;
     }
     t->pending.logp_out = nullptr;
     t->depth = T;
@@ -405,28 +412,31 @@ bgrpo_status bgrpo_tree_logprob(bgrpo_tree* t, int32_t step, const float* v_dev,
         const cudaError_t e0 = flush_pending(t, as_stream(stream));
         if (e0 != cudaSuccess) return cuda_fail(e0, "log-prob flush kernel");
     }
+    LogprobLaunch p;
+    p.latents = t->buf.latents;
+    p.mu = t->mu;
+    p.v = v_dev;
+    p.logp_out = logp_out_dev;
+    p.partials = static_cast<double*>(t->partials_logp);
+    p.status = t->status;
+    p.D = t->D;
+    p.n_trees = t->desc.n_trees;
+    p.nodes_cap = t->desc.nodes_cap;
+    p.nchunks = static_cast<int32_t>((t->D / 4 + kLogprobChunkVec - 1) / kLogprobChunkVec);
+    p.per_row = static_cast<int32_t>(partials_per_row(t->D));
+    p.first_step = step < 0 ? 0 : step;
+    p.depth = step < 0 ? t->depth : step + 1;
+    for (int d = 0; d <= p.depth + 1; ++d) p.off[d] = t->lv.offset[d];
+    for (int i = p.first_step; i < p.depth; ++i) {
+        const StepCoef& k = t->coef[i];
+        p.ca[i] = v_dev ? k.a : k.lin_a;
+        p.cb[i] = v_dev ? k.b : k.lin_b;
+        p.g[i] = k.g;
+        p.inv_2g2[i] = k.inv_2g2;
+        p.logp_const[i] = k.logp_const;
+    }
+    cudaError_t e;
     if (step < 0) {
-        LogprobLaunch p;
-        p.latents = t->buf.latents;
-        p.mu = t->mu;
-        p.logp_out = logp_out_dev;
-        p.partials = reinterpret_cast<double*>(t->partialsf);
-        p.status = t->status;
-        p.D = t->D;
-        p.n_trees = t->desc.n_trees;
-        p.nodes_cap = t->desc.nodes_cap;
-        p.nchunks = static_cast<int32_t>((t->D / 4 + kLogprobChunkVec - 1) / kLogprobChunkVec);
-        p.per_row = static_cast<int32_t>(partials_per_row(t->D));
-        p.depth = t->depth;
-        for (int d = 0; d <= t->depth + 1; ++d) p.off[d] = t->lv.offset[d];
-        for (int i = 0; i < t->depth; ++i) {
-            const StepCoef& k = t->coef[i];
-            p.ca[i] = k.lin_a;
-            p.cb[i] = k.lin_b;
-            p.g[i] = k.g;
-            p.inv_2g2[i] = k.inv_2g2;
-            p.logp_const[i] = k.logp_const;
-        }
         // a fork and the chains below it; run 0 is the chain below the root
         const RunInfo runs = runs_of(t->lv, t->depth);
         p.n_runs = runs.n;
@@ -439,25 +449,13 @@ bgrpo_status bgrpo_tree_logprob(bgrpo_tree* t, int32_t step, const float* v_dev,
             p.run_families[r] = p.run_len[r] > 0 ? t->lv.width[d0] : 0;
             p.families += p.run_families[r];
         }
-        const cudaError_t e = launch_logprob_tree(p, as_stream(stream));
-        return e == cudaSuccess ? BGRPO_OK : cuda_fail(e, "logprob kernel");
+        e = launch_logprob_tree(p, as_stream(stream));
+    } else {
+        p.families = t->lv.width[step];
+        p.run_fan[0] = t->lv.fanout[step];
+        e = launch_logprob_step(p, as_stream(stream));
     }
-    StepLaunch p;
-    fill_step_launch(t, step, v_dev, &p);
-    p.W_in = t->lv.width[step];
-    p.off_in = t->lv.offset[step];
-    p.off_out = t->lv.offset[step + 1];
-    p.fan = t->lv.fanout[step];
-    p.is_split = 0;
-    p.shared_noise = 0;
-    p.write_children = 0;
-    p.logp_out = logp_out_dev;
-    cudaError_t e = launch_step(p, as_stream(stream));
-    if (e != cudaSuccess) return cuda_fail(e, "logprob kernel");
-    t->pending = FinalizeDesc{logp_out_dev, t->lv.width[step + 1], t->lv.offset[step + 1], p.g, p.inv_2g2, p.logp_const};
-    e = flush_pending(t, as_stream(stream));
-    if (e != cudaSuccess) return cuda_fail(e, "log-prob flush kernel");
-    return BGRPO_OK;
+    return e == cudaSuccess ? BGRPO_OK : cuda_fail(e, "logprob kernel");
 }
 
 static bgrpo_status reward_common(bgrpo_tree* t, const float* target, float scale, float* r, int mode, void* stream) {

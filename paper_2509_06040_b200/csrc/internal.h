@@ -22,19 +22,21 @@ constexpr int kStepVec = 8;
 constexpr int kStepChunkVec = kStepThreads * kStepVec;   // 512 float4 = 8 KiB per operand tile
 constexpr int kStepWarps = kStepThreads / 32;            // log-prob partials per (row, chunk)
 constexpr int kStepCtasPerSm = 8;
-// Whole-tree rollout kernel: 128-thread CTAs, 2 float4 per thread (measured on B200 against 64/256 threads and 1/2/4
-// float4: within 6 % of one another), one log-prob partial per node row and warp; at most kFusedMaxSplits split steps
-// (one register-resident parent mean per split level on the depth-first walk).
+// Whole-tree rollout kernel: 128-thread CTAs, 4 float4 per thread (1 and 2 measured 37 and 16 % slower on the video tree), four
+// CTAs per SM (5 and 6: equal and 6 % slower there, 16 and 40 % slower on a single image tree), one log-prob partial per
+// node row and warp; at most kFusedMaxSplits split steps (the means of the open forks wait in shared memory).
 constexpr int kFusedThreads = 128;
-constexpr int kFusedVec = 2;
+constexpr int kFusedVec = 4;
+constexpr int kFusedCtasPerSm = 4;
 constexpr int kFusedChunkVec = kFusedThreads * kFusedVec;   // float4 of a row per CTA
 constexpr int kFusedMaxSplits = 6;
-// log-prob partials of the whole-tree kernel per node row: one float per warp of every CTA that covers the row
+// log-prob partials of the whole-tree kernel per node row: one 32-bit word per warp of every CTA that covers the row
 inline int64_t fused_partials_per_row(int64_t D) { return ((D / 4 + kFusedChunkVec - 1) / kFusedChunkVec) * (kFusedThreads / 32); }
-// floats of log-prob partials reserved per node row: the larger of the two rollout kernels' layouts
+// 32-bit words of log-prob partials reserved per node row: the larger of the rollout kernels' layouts (64 bits per chunk and
+// warp in the step kernel); an even number, so that every row starts on 8 bytes
 inline int64_t partials_per_row(int64_t D) {
     const int64_t D4 = D / 4;
-    const int64_t step = ((D4 + kStepChunkVec - 1) / kStepChunkVec) * kStepWarps;
+    const int64_t step = ((D4 + kStepChunkVec - 1) / kStepChunkVec) * kStepWarps * 2;
     const int64_t fused = fused_partials_per_row(D);
     return step > fused ? step : fused;
 }
@@ -79,7 +81,7 @@ struct StepCoef {
 struct FinalizeDesc {
     float* logp_out;       // nullptr: nothing pending
     int32_t W, off;        // rows off .. off+W-1 of every tree
-    float g, inv_2g2, logp_const;
+    float g, logp_const;
 };
 
 struct LevelInfo {                       // layout of the tree grown so far
@@ -138,7 +140,8 @@ struct bgrpo_tree {
     double* partials;                    // [n_trees*nodes_cap][nchunks][3]   (reward reductions)
     double* node_scratch;                // [n_trees][2][nodes_cap]: per-chain state of the tree reductions when a tree
                                          // is too large for one CTA's shared memory
-    float* partialsf;                    // [n_trees*nodes_cap][partials_per_row] (log-prob sums of the rollout kernels)
+    void* partials_logp;                 // [n_trees*nodes_cap][partials_per_row] 32-bit words: log-prob sums, each kernel's own layout
+    unsigned long long* partials_u64() const { return static_cast<unsigned long long*>(partials_logp); }
     unsigned int* mlp_tickets;           // 64-channel trees only: scratch of the MLP stage's split over the hidden dimension
     float* mlp_partials;
     bgrpo::FinalizeDesc pending;         // level whose log-probs still have to be summed
@@ -192,14 +195,12 @@ struct StepLaunch {
     uint32_t node_id_base;     // tree_id_base * nodes_cap
     PhiloxKeys keys;
     float ca, cb;              // mean = ca*z + cb*x, x = v or mu
-    float g, inv_2g2, logp_const;
+    float g;
     float mix_shared, mix_innov;
     int32_t shared_noise;      // 1: finite s at a split step
-    int32_t write_children;    // 1: tree_step; 0: tree_logprob (children are read, nothing but logp is written)
-    float* logp_out;           // destination of the log-probs (== logp for tree_step)
     int32_t* status;           // the tree's status word
-    int32_t per_row;           // floats reserved per node row in partialsf
-    float* partialsf;          // [rows][nchunks][kStepWarps] warp sums of (z' - mean)^2
+    int32_t per_row;           // 32-bit words reserved per node row in the partials
+    unsigned long long* partials;   // [rows][nchunks][kStepWarps] warp sums of quantized squares (philox.cuh)
     FinalizeDesc prev;         // level to finalize in this launch's prologue (logp_out == nullptr: none)
 };
 cudaError_t launch_root(const bgrpo_tree* t, cudaStream_t s);
@@ -208,21 +209,24 @@ cudaError_t launch_finalize(const bgrpo_tree* t, const FinalizeDesc& f, cudaStre
 
 // ---- log-probs of all stored edges (tree_logprob.cu) ---------------------------------------------------------------
 constexpr int kLogprobChunkVec = 512;      // float4 of a row per CTA; one double per (row, chunk) fits the step kernel's partials
-static_assert(kLogprobChunkVec == kStepChunkVec && kStepWarps == 2, "the partials of both kernels share their place");
+static_assert(kLogprobChunkVec == kStepChunkVec, "one double per (row, chunk) fits what the step kernel needs");
 struct LogprobLaunch {
     const float* latents;
     const float* mu;           // [n_trees][D]
     float* logp_out;
+    const float* v;            // one step's edges: [n_trees][W][D], or nullptr: closed-form velocity
     double* partials;          // [rows][nchunks]
     int32_t* status;
     int64_t D;
     int32_t n_trees, nodes_cap, nchunks, per_row, depth;
+    int32_t first_step;        // log-probs are written from this step's edges on
     int32_t families, n_runs;                          // families per tree, in all runs
     int32_t run_families[BGRPO_MAX_T + 1], run_d0[BGRPO_MAX_T + 1], run_fan[BGRPO_MAX_T + 1], run_len[BGRPO_MAX_T + 1];
     int32_t off[BGRPO_MAX_T + 2];
     float ca[BGRPO_MAX_T], cb[BGRPO_MAX_T], g[BGRPO_MAX_T], inv_2g2[BGRPO_MAX_T], logp_const[BGRPO_MAX_T];   // by step
 };
-cudaError_t launch_logprob_tree(const LogprobLaunch& p, cudaStream_t s);
+cudaError_t launch_logprob_tree(const LogprobLaunch& p, cudaStream_t s);      // all edges, closed form
+cudaError_t launch_logprob_step(const LogprobLaunch& p, cudaStream_t s);      // the edges of step depth - 1 = first_step
 
 struct RewardLaunch {
     const float* latents; const float* target; float* r; double* partials; unsigned int* counters; int32_t* status;
@@ -234,23 +238,32 @@ cudaError_t launch_philox_words(uint64_t seed, uint32_t node, uint32_t step, uin
 cudaError_t launch_philox_normals(uint64_t seed, uint32_t node, uint32_t step, uint32_t tag, float* out, int64_t n, cudaStream_t s);
 
 // ---- whole-tree rollout (tree_fused.cu) -------------------------------------------------------------------------
+struct alignas(16) FusedStep {
+    float ca, cb, g;
+    uint32_t child0;           // offset of the depth the step makes, bit 31: the step forks
+    uint32_t px, ph;           // what the noise counters of all nodes of the step share (noise_step in philox.cuh)
+    float logp_const;
+    uint32_t pad;
+};
 struct FusedLaunch {
     float* latents;
     const float* mu;           // [n_trees][D]
     float* logp;
     int32_t* table;
-    float* partialsf;          // [rows][per_row]: one float per warp of the CTAs that cover a row
+    uint32_t* partials;        // [rows][per_row]: one word per warp of the CTAs that cover a row
     int32_t* status;           // the tree's status word
-    int32_t per_row_cap;       // floats reserved per node row in partialsf
+    int32_t per_row_cap;       // words reserved per node row
     int64_t D;
-    int32_t n_trees, nodes_cap, nchunks, per_row, T, K, shared_noise;   // nchunks: CTAs per tree
+    int32_t n_trees, nodes_cap, T, K, shared_noise;
+    int32_t nchunks, per_row;  // CTAs that cover a row; set by launch_rollout_fused, like the next four
+    int32_t par, subtrees, levels;                     // forks dealt out to the grid, K^par, forks walked
+    int32_t split_step[kFusedMaxSplits];
     uint32_t node_id_base;
-    uint64_t split_bits;       // bit i: step i forks every node into K children
     PhiloxKeys keys;
     float mix_shared, mix_innov;
-    int32_t off[BGRPO_MAX_T + 2];                      // first local index of every depth
-    float ca[BGRPO_MAX_T], cb[BGRPO_MAX_T], g[BGRPO_MAX_T], inv_2g2[BGRPO_MAX_T], logp_const[BGRPO_MAX_T];
+    FusedStep step[BGRPO_MAX_T];                       // set by the caller but for px, ph
 };
+constexpr uint32_t kForks = 0x80000000u;
 cudaError_t launch_rollout_fused(const FusedLaunch& p, int32_t nodes, cudaStream_t s);
 
 // ---- tree reductions (tree_reduce.cu) -------------------------------------------------------------------------

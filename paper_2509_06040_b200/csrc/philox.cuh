@@ -28,12 +28,6 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, const PhiloxKeys& keys) 
     return c;
 }
 
-// u = ((x >> 9) + 0.5) * 2^-23, built without an integer-to-float conversion: the 23 kept bits become the
-// mantissa of a float in [1, 2), and subtracting 1 - 2^-24 is exact.
-__device__ __forceinline__ float uniform_open(uint32_t x) {
-    return __uint_as_float((x >> 9) | 0x3f800000u) - 0.99999994f;
-}
-
 // Hardware special-function approximations (flush-to-zero forms: one MUFU each, no denormal fix-up code).
 __device__ __forceinline__ float fast_sqrt(float x) {
     float y;
@@ -56,7 +50,33 @@ __device__ __forceinline__ float fast_cos(float x) {
     return y;
 }
 
-// One Box-Muller pair from two words: (r cos 2 pi u_b, r sin 2 pi u_b), r = sqrt(-2 ln u_a).
+// Two float32 operations in one instruction (the same rounding as the two single ones).
+__device__ __forceinline__ float2 mul2(float a, float2 b) {
+    float2 d;
+    asm("{\n\t.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %2};\n\tmov.b64 y, {%3, %4};\n\tmul.rn.f32x2 z, x, y;\n\tmov.b64 {%0, %1}, z;\n\t}"
+        : "=f"(d.x), "=f"(d.y) : "f"(a), "f"(b.x), "f"(b.y));
+    return d;
+}
+__device__ __forceinline__ float2 fma2(float a, float2 b, float2 c) {
+    float2 d;
+    asm("{\n\t.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %2};\n\tmov.b64 y, {%3, %4};\n\tmov.b64 z, {%5, %6};\n\tfma.rn.f32x2 z, x, y, z;\n\tmov.b64 {%0, %1}, z;\n\t}"
+        : "=f"(d.x), "=f"(d.y) : "f"(a), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return d;
+}
+__device__ __forceinline__ float4 mul4(float a, const float4& b) {
+    const float2 lo = mul2(a, make_float2(b.x, b.y)), hi = mul2(a, make_float2(b.z, b.w));
+    return make_float4(lo.x, lo.y, hi.x, hi.y);
+}
+__device__ __forceinline__ float4 fma4(float a, const float4& b, const float4& c) {
+    const float2 lo = fma2(a, make_float2(b.x, b.y), make_float2(c.x, c.y)), hi = fma2(a, make_float2(b.z, b.w), make_float2(c.z, c.w));
+    return make_float4(lo.x, lo.y, hi.x, hi.y);
+}
+
+// The float in [1, 2) whose mantissa is the word's top 23 bits: one funnel shift, (0x7f : x) >> 9 = 0x3f800000 | x >> 9.
+__device__ __forceinline__ float one_to_two(uint32_t x) { return __uint_as_float(__funnelshift_r(x, 0x7fu, 9)); }
+
+// One Box-Muller pair from two words: (r cos 2 pi u_b, r sin 2 pi u_b), r = sqrt(-2 ln u_a).  r2 receives r^2, the pair's
+// sum of squares.
 //
 // Accuracy (the result must stay within ~1e-4 of the exact value so that g * xi, g ~ 0.1, moves a
 // latent by well under 1e-5):
@@ -66,28 +86,91 @@ __device__ __forceinline__ float fast_cos(float x) {
 //    -2 ln(1 - w) = 2w + w^2 + ... (truncation below 1.3e-6 relative) replaces the log.
 //  * the angle is folded to (-pi, pi), where the hardware sine/cosine are good to about 4e-7 absolute,
 //    and the sign change is absorbed into r.
-__device__ __forceinline__ float2 box_muller(uint32_t wa, uint32_t wb) {
-    const float ua = uniform_open(wa);
+__device__ __forceinline__ float2 box_muller(uint32_t wa, uint32_t wb, float& r2) {
+    const float ua = one_to_two(wa) - 0.99999994f;             // ((x >> 9) + 0.5) * 2^-23, exact
     const float w = 1.0f - ua;
     const float series = fmaf(w, w, w + w);
     const float viaLog = -1.3862944f * fast_log2(ua);          // -2 ln 2 * log2(u)
-    const float r2 = (w < 0.001953125f) ? series : viaLog;
+    r2 = (w < 0.001953125f) ? series : viaLog;
     const float nr = -fast_sqrt(r2);
     // 2 pi u_b - pi with u_b = m - (1 - 2^-24), m in [1, 2) the float built from the word's top 23 bits: the constant
     // term takes the subtraction in (its float32 rounding moves the angle by < 5e-7, i.e. xi by < 3e-6)
-    const float th = fmaf(__uint_as_float((wb >> 9) | 0x3f800000u), 6.2831855f, -9.4247776f);
-    return make_float2(nr * fast_cos(th), nr * fast_sin(th));
+    const float th = fmaf(one_to_two(wb), 6.2831855f, -9.4247776f);
+    return mul2(nr, make_float2(fast_cos(th), fast_sin(th)));
 }
 
-__device__ __forceinline__ float4 normal4(uint4 w) {
-    const float2 a = box_muller(w.x, w.y);
-    const float2 b = box_muller(w.z, w.w);
+// Four normals and their sum of squares.
+__device__ __forceinline__ float4 normal4(uint4 w, float& squares) {
+    float ra, rb;
+    const float2 a = box_muller(w.x, w.y, ra);
+    const float2 b = box_muller(w.z, w.w, rb);
+    squares = ra + rb;
     return make_float4(a.x, a.y, b.x, b.y);
+}
+
+// The first two Philox rounds split into what depends on (element block, tag) only and on (node, step) only: the first
+// part is kept by a thread that draws the same elements for many nodes, the second is the same for a whole warp (uniform
+// registers).  philox_from() goes on with round 3; the words are those of philox4x32_10.
+struct NoiseElement { uint32_t x, y, z; };
+struct NoiseNode { uint32_t x, z, w; };
+__device__ __forceinline__ NoiseElement noise_element(uint32_t block, uint32_t tag, const PhiloxKeys& keys) {
+    uint32_t hi0, lo0, hi1, lo1;
+    mulhilo(kPhiloxM0, block, hi0, lo0);
+    mulhilo(kPhiloxM1, hi0 ^ tag ^ keys.k[0][1], hi1, lo1);
+    return {hi1, lo1, lo0};
+}
+__device__ __forceinline__ NoiseNode noise_node(uint32_t node, uint32_t step, const PhiloxKeys& keys) {
+    uint32_t hi1, lo1, hi0, lo0;
+    mulhilo(kPhiloxM1, step, hi1, lo1);
+    mulhilo(kPhiloxM0, hi1 ^ node ^ keys.k[0][0], hi0, lo0);
+    return {lo1 ^ keys.k[1][0], hi0 ^ keys.k[1][1], lo0};
+}
+// The part of a NoiseNode that all nodes of a step share, for the host to tabulate: px = lo(M1 step) ^ k[1][0],
+// ph = hi(M1 step) ^ k[0][0].
+inline void noise_step(uint32_t step, const PhiloxKeys& keys, uint32_t& px, uint32_t& ph) {
+    const uint64_t prod = static_cast<uint64_t>(kPhiloxM1) * step;
+    px = static_cast<uint32_t>(prod) ^ keys.k[1][0];
+    ph = static_cast<uint32_t>(prod >> 32) ^ keys.k[0][0];
+}
+__device__ __forceinline__ NoiseNode noise_node_of(uint32_t node, uint32_t px, uint32_t ph, const PhiloxKeys& keys) {
+    uint32_t hi0, lo0;
+    mulhilo(kPhiloxM0, ph ^ node, hi0, lo0);
+    return {px, hi0 ^ keys.k[1][1], lo0};
+}
+__device__ __forceinline__ uint4 philox_from(const NoiseElement& e, const NoiseNode& n, const PhiloxKeys& keys) {
+    uint4 c = make_uint4(e.x ^ n.x, e.y, e.z ^ n.z, n.w);
+#pragma unroll
+    for (int r = 2; r < 10; ++r) {
+        uint32_t hi0, lo0, hi1, lo1;
+        mulhilo(kPhiloxM0, c.x, hi0, lo0);
+        mulhilo(kPhiloxM1, c.z, hi1, lo1);
+        c = make_uint4(hi1 ^ c.y ^ keys.k[r][0], lo1, hi0 ^ c.w ^ keys.k[r][1], lo0);
+    }
+    return c;
+}
+
+// Log-prob sums of the rollout kernels.  The squares of four normals (at most 2 * 33.3 with independent noise, twice that
+// with a shared part) are rounded to a multiple of 2^-18 - 2e-6 of their mean, the rounding of a float32 log-prob of four
+// elements - and added as integers: sums are exact from there on, so they do not depend on how a kernel cuts the row, and
+// the level-by-level and the whole-tree kernel agree bit for bit.  One thread may add up to eight (2^31), one warp's sum of
+// at most two per lane fits 32 bits.
+constexpr float kSquareScale = 262144.0f;
+__device__ __forceinline__ uint32_t quantized_squares(float squares) { return __float2uint_rn(squares * kSquareScale); }
+__device__ __forceinline__ float squares_of(const float4& x) { return fmaf(x.x, x.x, fmaf(x.y, x.y, fmaf(x.z, x.z, x.w * x.w))); }
+// the log-prob of an edge from its row's sum: -(1/D) sum (z' - mean)^2 / (2 g^2) + const with (z' - mean)^2 = g^2 xi^2
+__device__ __forceinline__ float logp_from_squares(unsigned long long sum, int64_t D, float g, float logp_const) {
+    return g == 0.0f ? 0.0f : static_cast<float>(static_cast<double>(logp_const) - static_cast<double>(sum) * (0.5 / static_cast<double>(kSquareScale)) / static_cast<double>(D));
+}
+__device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long x) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+    return x;
 }
 
 __device__ __forceinline__ float4 noise4(uint32_t block, uint32_t node, uint32_t step, uint32_t tag,
                                          const PhiloxKeys& keys) {
-    return normal4(philox4x32_10(make_uint4(block, node, step, tag), keys));
+    float squares;
+    return normal4(philox4x32_10(make_uint4(block, node, step, tag), keys), squares);
 }
 
 }  // namespace bgrpo

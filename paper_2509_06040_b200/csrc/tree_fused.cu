@@ -6,197 +6,243 @@
 // from shared prefixes is taken literally: a prefix is computed once and never re-read.
 //
 // Every node gets exactly the value the level-by-level path gives it: the same Philox counters (element block, global
-// node id, step, tag), the same float32 expressions (mean = ca z + cb mu, child = g xi + mean, Eq. 2 noise mixing).
-// Log-prob sums use their own partial layout (one float per node row and warp of the CTAs that cover the row) and are
-// completed by finalize_tree_kernel in a fixed order, in double.
+// node id, step, tag), the same float32 expressions (mean = ca z + cb mu, child = g xi + mean, Eq. 2 noise mixing), the same
+// integer sums of squares for the log-probs (philox.cuh).
+//
+// Bound: the noise, that is the FMA pipe: one of Philox' wide multiplies takes it four cycles, Box-Muller's and the update's
+// float32 operations one each, and they do not overlap; a register-only loop draws 1.18 T normals a second.  So everything
+// around the noise is kept small.  The walk is one loop with one copy of the noise code, not a recursion over split levels
+// (which took 113-168 registers, spilled, and did not fit the instruction cache): a node's local index, written in base K,
+// is the path that leads to it, and the means of the open forks wait in shared memory.  A thread takes four float4 (one: 42
+// instructions per element instead of 24, nearly twice the time), the first two Philox rounds are split into a part per element
+// and a part per node.  Video tree (110 edges x 2.1 M elements): 379 -> 249 us, 0.93 T normals/s; four trees of 129 600
+// elements: 162 -> 102 us; one: 103 -> 40 us.
+//
+// A tree of few elements gives too few CTAs, so the first forks can be dealt out to the grid as well: a CTA then walks the
+// subtree of one assignment of the first p.par forks, recomputing the prefix that leads to it; of the CTAs that share a
+// prefix node, the one whose remaining assignments are all zero writes it.
 #include "internal.h"
 #include "philox.cuh"
 
 namespace bgrpo {
 namespace {
 
-struct Ctx {
-    uint32_t e[kFusedVec];        // float4 index of each of this thread's pieces
-    bool live[kFusedVec];         // inside the row
-    float4 mu[kFusedVec];
-    float4* tree_base;            // latents of this tree, as float4
-    int64_t tree_row0;            // first row of this tree in the per-node buffers
-    uint32_t gid0;                // global node id of the tree's local node 0
-    int chunk, warp, lane;
-    bool writes_table;            // one thread per tree appends the node-table rows
-};
+template <bool SHARED>
+__global__ void __launch_bounds__(kFusedThreads, kFusedCtasPerSm)
+rollout_fused_kernel(const __grid_constant__ FusedLaunch p) {
+    constexpr int VEC = kFusedVec;
+    extern __shared__ float4 s_stack[];             // [open fork][VEC] means, SHARED: and as many xi_0
+    pdl_release();
+    const int chunk = blockIdx.x % p.nchunks;
+    const int group = blockIdx.x / p.nchunks;       // (tree, assignment of the first forks)
+    const int tree = group / p.subtrees;
+    int sub = group - tree * p.subtrees;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t row0 = static_cast<int64_t>(tree) * p.nodes_cap;
+    const uint32_t gid0 = p.node_id_base + static_cast<uint32_t>(row0);
+    const uint32_t D4 = static_cast<uint32_t>(p.D >> 2);
+    float4* const tree_base = reinterpret_cast<float4*>(p.latents + row0 * p.D);
+    const float4* __restrict__ mu_row = reinterpret_cast<const float4*>(p.mu + static_cast<int64_t>(tree) * p.D);
+    const bool writes_table = chunk == 0 && threadIdx.x == 0;
+    // nodes below this many forks are this CTA's to write
+    int emit_from = p.par;
+    for (int s = sub; emit_from > 0 && s % p.K == 0; s /= p.K) --emit_from;
 
-__device__ __forceinline__ float4 fma4(float a, const float4& x, const float4& y) {
-    return make_float4(fmaf(a, x.x, y.x), fmaf(a, x.y, y.y), fmaf(a, x.z, y.z), fmaf(a, x.w, y.w));
-}
-
-// One child: z' = mean + g xi, its latent row, its squared residual partial, its node-table row.
-__device__ __forceinline__ void emit_child(const FusedLaunch& p, const Ctx& cx, int step, int parent_local, int child_local,
-                                           int split_step, int branch_id, float g, const float4 (&m)[kFusedVec],
-                                           const float4 (&xi0)[kFusedVec], bool shared, float4 (&c)[kFusedVec]) {
-    const uint32_t gid = cx.gid0 + static_cast<uint32_t>(child_local);
-    if (!BGRPO_IN_BOUNDS(p.status, child_local > 0 && child_local < p.nodes_cap && parent_local >= 0 && parent_local < child_local &&
-                                       (cx.chunk + 1) * (kFusedThreads / 32) <= p.per_row_cap)) return;
-    float acc = 0.0f;
-    float4* row = cx.tree_base + static_cast<size_t>(child_local) * static_cast<size_t>(p.D >> 2);
+    uint32_t e[VEC];
+    bool live[VEC];
+    NoiseElement el[VEC];
 #pragma unroll
-    for (int k = 0; k < kFusedVec; ++k) {
-        if (cx.live[k]) {
-            float4 xi = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (g != 0.0f) {
-                xi = noise4(cx.e[k], gid, static_cast<uint32_t>(step), BGRPO_TAG_INNOV, p.keys);
-                if (shared) {
-                    xi.x = fmaf(p.mix_innov, xi.x, p.mix_shared * xi0[k].x);
-                    xi.y = fmaf(p.mix_innov, xi.y, p.mix_shared * xi0[k].y);
-                    xi.z = fmaf(p.mix_innov, xi.z, p.mix_shared * xi0[k].z);
-                    xi.w = fmaf(p.mix_innov, xi.w, p.mix_shared * xi0[k].w);
-                }
+    for (int k = 0; k < VEC; ++k) {
+        e[k] = (static_cast<uint32_t>(chunk) * VEC + k) * kFusedThreads + threadIdx.x;
+        live[k] = e[k] < D4;
+        el[k] = noise_element(e[k], BGRPO_TAG_INNOV, p.keys);
+    }
+    if (!BGRPO_IN_BOUNDS(p.status, tree < p.n_trees && static_cast<uint32_t>(chunk) * VEC * kFusedThreads < D4 && (chunk + 1) * (kFusedThreads / 32) <= p.per_row &&
+                                       p.per_row <= p.per_row_cap)) return;
+    uint32_t* const partials = p.partials + row0 * p.per_row + chunk * (kFusedThreads / 32) + warp;
+    pdl_wait();
+    float4 mu[VEC], m[VEC], xi0[VEC];               // m: the mean of the next child, xi0: mix_shared times the shared noise of its fork
+    FusedStep st = p.step[0];
+#pragma unroll
+    for (int k = 0; k < VEC; ++k) {
+        mu[k] = live[k] ? __ldg(mu_row + e[k]) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 z = live[k] ? __ldcs(tree_base + e[k]) : make_float4(0.f, 0.f, 0.f, 0.f);       // root latent (row 0 of the tree)
+        m[k] = fma4(st.ca, z, mul4(st.cb, mu[k]));
+        xi0[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    int i = 0;                                      // the node about to be made: child of step i (st),
+    uint32_t j = 0, parent = 0;                     // with index j in its depth, below the local node parent
+    int forks = 0;                                  // forks on its path, the one of step i included
+    // Step i forks: chooses the first child to make below index j and keeps what its siblings need.
+    auto open_fork = [&]() {
+        if (SHARED && st.g != 0.0f) {
+            const NoiseNode node = noise_node_of(gid0 + parent, st.px, st.ph, p.keys);
+#pragma unroll
+            for (int k = 0; k < VEC; ++k) {
+                float squares;
+                xi0[k] = mul4(p.mix_shared, normal4(philox_from(noise_element(e[k], BGRPO_TAG_SHARED, p.keys), node, p.keys), squares));
             }
-            c[k] = fma4(g, xi, m[k]);
-            __stcs(row + cx.e[k], c[k]);
-            // z' - mean is g xi up to the rounding of z': sum xi^2, times g^2 once per warp
-            acc = fmaf(xi.x, xi.x, acc);
-            acc = fmaf(xi.y, xi.y, acc);
-            acc = fmaf(xi.z, xi.z, acc);
-            acc = fmaf(xi.w, xi.w, acc);
         }
-    }
+        j *= p.K;
+        if (forks < p.par) {
+            int div = 1;
+            for (int q = forks + 1; q < p.par; ++q) div *= p.K;
+            j += (sub / div) % p.K;
+        } else {
+            const int level = forks - p.par;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    acc *= g * g;
-    const int64_t r = cx.tree_row0 + child_local;
-    if (cx.lane == 0) p.partialsf[r * p.per_row + cx.chunk * (kFusedThreads / 32) + cx.warp] = acc;
-    if (cx.writes_table) {
-        const int64_t rows = static_cast<int64_t>(p.n_trees) * p.nodes_cap;
-        p.table[r] = parent_local;
-        p.table[rows + r] = step + 1;
-        p.table[2 * rows + r] = split_step;
-        p.table[3 * rows + r] = branch_id;
-    }
-}
-
-// Walks the subtree below local node j of depth i, whose latent pieces are in z.  S counts the splits on the path so
-// far: each split level keeps its parent's mean in registers while the children's subtrees are walked one by one.
-// MAXS bounds the number of split levels the instantiation walks, SHARED says whether split steps mix in a per-parent
-// xi_0 (finite s): the common case (few splits, independent children) then carries neither the deeper levels' code nor
-// registers for xi_0.
-template <int S, int MAXS, bool SHARED>
-__device__ __forceinline__ void walk(const FusedLaunch& p, const Ctx& cx, int i, int j, int split_step, int branch_id,
-                                     float4 (&z)[kFusedVec]) {
-    const float4 zero[kFusedVec] = {};
-    for (; i < p.T; ++i) {
-        const float ca = p.ca[i], cb = p.cb[i], g = p.g[i];
-        float4 m[kFusedVec];
+            for (int k = 0; k < VEC; ++k) {
+                s_stack[(level * VEC + k) * kFusedThreads + threadIdx.x] = m[k];
+                if (SHARED) s_stack[((p.levels + level) * VEC + k) * kFusedThreads + threadIdx.x] = xi0[k];
+            }
+        }
+        ++forks;
+    };
+    if (st.child0 & kForks) open_fork();
+    while (true) {
+        const uint32_t child = (st.child0 & ~kForks) + j;
+        if (!BGRPO_IN_BOUNDS(p.status, child > 0 && child < static_cast<uint32_t>(p.nodes_cap))) return;
+        const bool emit = forks >= emit_from;
+        uint32_t acc = 0u;
+        float4 z[VEC];
+        if (st.g != 0.0f) {
+            const NoiseNode node = noise_node_of(gid0 + child, st.px, st.ph, p.keys);
 #pragma unroll
-        for (int k = 0; k < kFusedVec; ++k)
-            m[k] = make_float4(fmaf(ca, z[k].x, cb * cx.mu[k].x), fmaf(ca, z[k].y, cb * cx.mu[k].y),
-                               fmaf(ca, z[k].z, cb * cx.mu[k].z), fmaf(ca, z[k].w, cb * cx.mu[k].w));
-        const int parent_local = p.off[i] + j;
-        if (!((p.split_bits >> i) & 1ull)) {
-            emit_child(p, cx, i, parent_local, p.off[i + 1] + j, split_step, branch_id, g, m, zero, false, z);
+            for (int k = 0; k < VEC; ++k) {
+                float squares;
+                float4 xi = normal4(philox_from(el[k], node, p.keys), squares);
+                if (SHARED && (st.child0 & kForks)) {
+                    xi = fma4(p.mix_innov, xi, xi0[k]);
+                    squares = squares_of(xi);
+                }
+                z[k] = fma4(st.g, xi, m[k]);
+                acc += live[k] ? quantized_squares(squares) : 0u;
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < VEC; ++k) z[k] = m[k];
+        }
+        if (emit) {
+            float4* row = tree_base + static_cast<uint64_t>(child) * D4;
+#pragma unroll
+            for (int k = 0; k < VEC; ++k)
+                if (live[k]) __stcs(row + e[k], z[k]);
+            acc = __reduce_add_sync(0xffffffffu, acc);
+            if (lane == 0) partials[static_cast<uint64_t>(child) * static_cast<uint32_t>(p.per_row)] = acc;
+            if (writes_table) {
+                const int64_t rows = static_cast<int64_t>(p.n_trees) * p.nodes_cap, r = row0 + child;
+                p.table[r] = static_cast<int32_t>(parent);
+                p.table[rows + r] = i + 1;
+                p.table[2 * rows + r] = forks > 0 ? p.split_step[forks - 1] : -1;
+                p.table[3 * rows + r] = forks > 0 ? static_cast<int32_t>(j % p.K) : 0;
+            }
+        }
+        parent = child;
+        if (++i < p.T) {                            // go down
+            st = p.step[i];
+#pragma unroll
+            for (int k = 0; k < VEC; ++k) m[k] = fma4(st.ca, z[k], mul4(st.cb, mu[k]));
+            if (st.child0 & kForks) open_fork();
             continue;
         }
-        if constexpr (S < MAXS) {
-            const bool shared = SHARED && g != 0.0f;
-            float4 xi0[kFusedVec] = {};
-            if (shared) {
+        const uint32_t K = p.K;
+        while (forks > p.par && j % K == K - 1) { j /= K; --forks; }       // back to the deepest fork with a child left
+        if (forks == p.par) return;
+        ++j;
+        i = p.split_step[forks - 1];
+        st = p.step[i];
+        parent = (i > 0 ? p.step[i - 1].child0 & ~kForks : 0u) + j / K;
+        const int level = forks - 1 - p.par;
 #pragma unroll
-                for (int k = 0; k < kFusedVec; ++k)
-                    if (cx.live[k])
-                        xi0[k] = noise4(cx.e[k], cx.gid0 + static_cast<uint32_t>(parent_local), static_cast<uint32_t>(i), BGRPO_TAG_SHARED, p.keys);
-            }
-            for (int b = 0; b < p.K; ++b) {
-                float4 c[kFusedVec];
-                const int child = j * p.K + b;
-                emit_child(p, cx, i, parent_local, p.off[i + 1] + child, i, b, g, m, xi0, shared, c);
-                walk<S + 1, MAXS, SHARED>(p, cx, i + 1, child, i, b, c);
-            }
+        for (int k = 0; k < VEC; ++k) {
+            m[k] = s_stack[(level * VEC + k) * kFusedThreads + threadIdx.x];
+            if (SHARED) xi0[k] = s_stack[((p.levels + level) * VEC + k) * kFusedThreads + threadIdx.x];
         }
-        return;
     }
 }
 
-template <int MAXS, bool SHARED>
-__global__ void __launch_bounds__(kFusedThreads)
-rollout_fused_kernel(const __grid_constant__ FusedLaunch p) {
-    pdl_release();
-    pdl_wait();
-    Ctx cx;
-    cx.chunk = blockIdx.x % p.nchunks;
-    const int tree = blockIdx.x / p.nchunks;
-    cx.warp = threadIdx.x >> 5;
-    cx.lane = threadIdx.x & 31;
-    cx.tree_row0 = static_cast<int64_t>(tree) * p.nodes_cap;
-    cx.gid0 = p.node_id_base + static_cast<uint32_t>(cx.tree_row0);
-    cx.tree_base = reinterpret_cast<float4*>(p.latents + cx.tree_row0 * p.D);
-    cx.writes_table = (cx.chunk == 0 && threadIdx.x == 0);
-    const uint32_t D4 = static_cast<uint32_t>(p.D >> 2);
-    const float4* __restrict__ mu = reinterpret_cast<const float4*>(p.mu + static_cast<int64_t>(tree) * p.D);
-    float4 z[kFusedVec];
-#pragma unroll
-    for (int k = 0; k < kFusedVec; ++k) {
-        cx.e[k] = static_cast<uint32_t>(cx.chunk) * kFusedChunkVec + k * kFusedThreads + threadIdx.x;
-        cx.live[k] = cx.e[k] < D4;
-        cx.mu[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-        z[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (cx.live[k]) {
-            cx.mu[k] = __ldg(mu + cx.e[k]);
-            z[k] = __ldcs(cx.tree_base + cx.e[k]);          // root latent (row 0 of the tree)
-        }
-    }
-    walk<0, MAXS, SHARED>(p, cx, 0, 0, -1, 0, z);
-}
-
-// Completes the log-probs of every non-root node of every tree from the fused kernel's partial sums: one warp per node
-// row, lanes stride over the row's per_row floats in index order, then a fixed shuffle tree; double
-// throughout.
+// Completes the log-probs of every non-root node: THREADS threads per node row add up its words.
+template <int THREADS>
 __global__ void __launch_bounds__(256)
 finalize_tree_kernel(const __grid_constant__ FusedLaunch p, int32_t nodes) {
     pdl_release();
     pdl_wait();
-    const int lane = threadIdx.x & 31;
-    const int64_t w = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    constexpr int kRows = 256 / THREADS;
+    const int64_t w = static_cast<int64_t>(blockIdx.x) * kRows + threadIdx.x / THREADS;
     const int64_t total = static_cast<int64_t>(p.n_trees) * (nodes - 1);
     if (w >= total) return;
     const int tree = static_cast<int>(w / (nodes - 1));
     const int local = 1 + static_cast<int>(w - static_cast<int64_t>(tree) * (nodes - 1));
     int step = 0;                                       // the node's depth is step + 1
-    while (step + 1 < p.T && local >= p.off[step + 2]) ++step;
+    while (step + 1 < p.T && static_cast<uint32_t>(local) >= (p.step[step + 1].child0 & ~kForks)) ++step;
     const int64_t row = static_cast<int64_t>(tree) * p.nodes_cap + local;
-    const int per_row = p.per_row;
-    if (!BGRPO_IN_BOUNDS(p.status, local < p.nodes_cap && per_row <= p.per_row_cap)) return;
-    const float* q = p.partialsf + row * per_row;
-    double s = 0.0;
-    for (int c = lane; c < per_row; c += 32) s += static_cast<double>(__ldcg(q + c));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) {
-        const float g = p.g[step];
-        p.logp[row] = (g == 0.0f) ? 0.0f
-                                   : static_cast<float>(-(s / static_cast<double>(p.D)) * static_cast<double>(p.inv_2g2[step]) +
-                                                        static_cast<double>(p.logp_const[step]));
+    if (!BGRPO_IN_BOUNDS(p.status, local < p.nodes_cap && p.per_row <= p.per_row_cap)) return;
+    const uint32_t* q = p.partials + row * p.per_row;
+    unsigned long long s = 0;
+#pragma unroll 8
+    for (int c = threadIdx.x % THREADS; c < p.per_row; c += THREADS) s += __ldcg(q + c);
+    s = warp_sum_u64(s);
+    if (THREADS > 32) {
+        __shared__ unsigned long long s_sum[8];
+        if ((threadIdx.x & 31) == 0) s_sum[threadIdx.x >> 5] = s;
+        __syncthreads();
+        if (threadIdx.x == 0)
+            for (int i = 1; i < 8; ++i) s += s_sum[i];
     }
+    if (threadIdx.x % THREADS == 0) p.logp[row] = logp_from_squares(s, p.D, p.step[step].g, p.step[step].logp_const);
 }
 
 }  // namespace
 
-cudaError_t launch_rollout_fused(const FusedLaunch& p, int32_t nodes, cudaStream_t s) {
-    const int64_t items = static_cast<int64_t>(p.n_trees) * p.nchunks;
+cudaError_t launch_rollout_fused(const FusedLaunch& p0, int32_t nodes, cudaStream_t s) {
+    FusedLaunch p = p0;
+    int n_splits = 0;
+    for (int i = 0; i < p.T; ++i) {
+        noise_step(static_cast<uint32_t>(i), p.keys, p.step[i].px, p.step[i].ph);
+        if (!(p.step[i].child0 & kForks)) continue;
+        if (n_splits == kFusedMaxSplits) return cudaErrorInvalidValue;
+        p.split_step[n_splits++] = i;
+    }
+    const int64_t D4 = p.D / 4;
+    p.nchunks = static_cast<int32_t>((D4 + kFusedChunkVec - 1) / kFusedChunkVec);
+    p.per_row = static_cast<int32_t>(fused_partials_per_row(p.D));
+    // Dealing out a fork more makes K times as many CTAs that walk a shorter subtree but compute the prefix again.  An SM works
+    // at the same rate from about three CTAs on, so the time goes with the CTAs of the busiest SM (at least three) times the
+    // nodes a CTA walks.  Measured, us a rollout, forks dealt out 0 / 1 / 2 / 3 (the rule's choice in brackets): four trees of
+    // 129 600 elements 213 / - / [102] / 111, one video tree 255 / [249] / 268 / -; one tree of 129 600 elements 54 with none, 40
+    // with four and with the rule's three.
+    int64_t best = -1;
+    int32_t subtrees = 1;
+    for (int par = 0; par <= n_splits; ++par, subtrees *= p.K) {
+        int64_t walk = 0, width = 1;
+        for (int i = 0, forks = 0; i < p.T; ++i) {
+            if ((p.step[i].child0 & kForks) && forks++ >= par) width *= p.K;
+            walk += width;
+        }
+        const int64_t ctas = (static_cast<int64_t>(p.n_trees) * p.nchunks * subtrees + 147) / 148;
+        const int64_t cost = (ctas < 3 ? 3 : ctas) * walk;
+        if (best < 0 || cost <= best) {
+            best = cost;
+            p.par = par;
+            p.subtrees = subtrees;
+        }
+    }
+    p.levels = n_splits - p.par;
+    const int64_t items = static_cast<int64_t>(p.n_trees) * p.nchunks * p.subtrees;
     if (items <= 0 || items > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     const unsigned int grid = static_cast<unsigned int>(items);
-    const int n_splits = __builtin_popcountll(p.split_bits);
-    if (n_splits > kFusedMaxSplits) return cudaErrorInvalidValue;
-    cudaError_t e;
-    if (p.shared_noise) {
-        if (n_splits <= 3) e = launch_overlapped(rollout_fused_kernel<3, true>, grid, kFusedThreads, 0, s, p);
-        else e = launch_overlapped(rollout_fused_kernel<kFusedMaxSplits, true>, grid, kFusedThreads, 0, s, p);
-    } else {
-        if (n_splits <= 3) e = launch_overlapped(rollout_fused_kernel<3, false>, grid, kFusedThreads, 0, s, p);
-        else e = launch_overlapped(rollout_fused_kernel<kFusedMaxSplits, false>, grid, kFusedThreads, 0, s, p);
-    }
+    const size_t smem = static_cast<size_t>(p.levels) * kFusedChunkVec * sizeof(float4) * (p.shared_noise ? 2 : 1);
+    cudaError_t e = cudaSuccess;
+    if (smem > 48 * 1024)
+        e = p.shared_noise ? cudaFuncSetAttribute(rollout_fused_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem))
+                           : cudaFuncSetAttribute(rollout_fused_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (e == cudaSuccess)
+        e = p.shared_noise ? launch_overlapped(rollout_fused_kernel<true>, grid, kFusedThreads, smem, s, p)
+                           : launch_overlapped(rollout_fused_kernel<false>, grid, kFusedThreads, smem, s, p);
     if (e != cudaSuccess || nodes < 2) return e;
-    const int64_t warps = static_cast<int64_t>(p.n_trees) * (nodes - 1);
-    return launch_overlapped(finalize_tree_kernel, static_cast<unsigned int>((warps + 7) / 8), 256, 0, s, p, nodes);
+    const int64_t rows = static_cast<int64_t>(p.n_trees) * (nodes - 1);
+    if (p.per_row >= 512) return launch_overlapped(finalize_tree_kernel<256>, static_cast<unsigned int>(rows), 256, 0, s, p, nodes);
+    return launch_overlapped(finalize_tree_kernel<32>, static_cast<unsigned int>((rows + 7) / 8), 256, 0, s, p, nodes);
 }
 
 }  // namespace bgrpo

@@ -1,12 +1,14 @@
-// Log-probs of all stored edges under the closed-form velocity (the numerator of rho_e in Eq. 5): per edge the mean squared
-// distance of the stored child from the Euler-Maruyama mean of its parent.  HBM-bound: every latent is read once, 4 bytes
-// per element and edge.
+// Log-probs of stored edges under a given velocity (the numerator of rho_e in Eq. 5): per edge the mean squared distance of
+// the stored child from the Euler-Maruyama mean of its parent.  HBM-bound.
 //
-// A CTA takes one chunk of the row for one *family*: a node, its F children and the only children below each of them down
+// All edges under the closed-form velocity: every latent is read once, 4 bytes per element and edge.  A CTA takes one chunk of the row for one *family*: a node, its F children and the only children below each of them down
 // to the next fork.  It keeps the parent's piece in registers and walks down, so a node is read once although it is child
 // of one edge and parent of the next; the next node's loads are issued before the current one is used.  A small kernel with
 // one warp per row adds the chunks up.  On a video tree of 111 nodes x 2.1 M elements: 155 us (6.06 TB/s) for the whole
 // tree, where one launch per level, each reading parents and children, took 290 us.
+//
+// One step's edges under a given velocity (12 bytes per element and edge without a fork): one CTA per parent and chunk, all
+// its loads issued before the first is used.
 //
 // The sums of squares are float32 inside a warp's 512 elements, double from there on, one double per (row, chunk), added in
 // chunk order.
@@ -101,17 +103,87 @@ logprob_tree_kernel(const __grid_constant__ LogprobLaunch p) {
     }
 }
 
-// One warp per non-root row: the row's chunk partials in index order within each lane, then a fixed shuffle tree.
+// One step's edges: parent, velocity and first child of a chunk are loaded together, further children one after the other.
+constexpr int kEdgeThreads = 64, kEdgeVec = kLogprobChunkVec / kEdgeThreads, kEdgeWarps = kEdgeThreads / 32;
+
+template <bool FULL>
+__device__ __forceinline__ void score_chunk(const float4* __restrict__ zp, const float4* __restrict__ xp, const float4* __restrict__ cp, size_t D4,
+                                            uint32_t vecs, int fan, float ca, float cb, float (*acc_out)[kEdgeWarps]) {
+    float4 m[kEdgeVec], x[kEdgeVec], c[kEdgeVec];
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < kEdgeVec; ++k) {
+        const uint32_t t = threadIdx.x + k * kEdgeThreads;
+        const bool in = FULL || t < vecs;
+        m[k] = in ? __ldcs(zp + t) : zero;
+        x[k] = in ? __ldcs(xp + t) : zero;
+        c[k] = in ? __ldcs(cp + t) : zero;
+    }
+#pragma unroll
+    for (int k = 0; k < kEdgeVec; ++k)
+        m[k] = make_float4(fmaf(ca, m[k].x, cb * x[k].x), fmaf(ca, m[k].y, cb * x[k].y), fmaf(ca, m[k].z, cb * x[k].z), fmaf(ca, m[k].w, cb * x[k].w));
+    for (int b = 0; b < fan; ++b) {
+        if (b > 0) {
+#pragma unroll
+            for (int k = 0; k < kEdgeVec; ++k) {
+                const uint32_t t = threadIdx.x + k * kEdgeThreads;
+                c[k] = (FULL || t < vecs) ? __ldcs(cp + b * D4 + t) : zero;
+            }
+        }
+        float acc = 0.0f;
+#pragma unroll
+        for (int k = 0; k < kEdgeVec; ++k) {
+            const float dx = c[k].x - m[k].x, dy = c[k].y - m[k].y, dz = c[k].z - m[k].z, dw = c[k].w - m[k].w;
+            acc = fmaf(dx, dx, acc);
+            acc = fmaf(dy, dy, acc);
+            acc = fmaf(dz, dz, acc);
+            acc = fmaf(dw, dw, acc);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+        if ((threadIdx.x & 31) == 0) acc_out[b][threadIdx.x >> 5] = acc;
+    }
+}
+
+__global__ void __launch_bounds__(kEdgeThreads, 8)
+logprob_step_kernel(const __grid_constant__ LogprobLaunch p) {
+    __shared__ float s_acc[BGRPO_MAX_K][kEdgeWarps];
+    pdl_release();
+    pdl_wait();
+    const int chunk = blockIdx.x % p.nchunks;
+    const int row = blockIdx.x / p.nchunks;                 // tree * families + f
+    const int tree = row / p.families, f = row - tree * p.families;
+    const int d0 = p.first_step, fan = p.run_fan[0];
+    const uint32_t D4 = static_cast<uint32_t>(p.D >> 2), e = static_cast<uint32_t>(chunk) * kLogprobChunkVec;
+    const int64_t row0 = static_cast<int64_t>(tree) * p.nodes_cap, child = row0 + p.off[d0 + 1] + f * fan;
+    if (!BGRPO_IN_BOUNDS(p.status, tree < p.n_trees && e < D4 && p.off[d0] + f < p.off[d0 + 1] && p.off[d0 + 1] + (f + 1) * fan <= p.nodes_cap &&
+                                       p.nchunks * 2 <= p.per_row)) return;
+    const float4* zp = reinterpret_cast<const float4*>(p.latents + (row0 + p.off[d0] + f) * p.D) + e;
+    const float4* cp = reinterpret_cast<const float4*>(p.latents + child * p.D) + e;
+    const float4* xp = (p.v != nullptr ? reinterpret_cast<const float4*>(p.v + static_cast<int64_t>(row) * p.D)
+                                       : reinterpret_cast<const float4*>(p.mu + static_cast<int64_t>(tree) * p.D)) + e;
+    if (D4 - e >= kLogprobChunkVec) score_chunk<true>(zp, xp, cp, D4, kLogprobChunkVec, fan, p.ca[d0], p.cb[d0], s_acc);
+    else score_chunk<false>(zp, xp, cp, D4, D4 - e, fan, p.ca[d0], p.cb[d0], s_acc);
+    __syncthreads();
+    if (threadIdx.x < fan) {
+        double s = 0.0;
+#pragma unroll
+        for (int w = 0; w < kEdgeWarps; ++w) s += static_cast<double>(s_acc[threadIdx.x][w]);
+        p.partials[(child + threadIdx.x) * p.nchunks + chunk] = s;
+    }
+}
+
+// One warp per row: the row's chunk partials in index order within each lane, then a fixed shuffle tree.
 __global__ void __launch_bounds__(256)
 logprob_finish_kernel(const __grid_constant__ LogprobLaunch p) {
     pdl_release();
     pdl_wait();
-    const int edges = p.off[p.depth + 1] - 1;
+    const int first = p.off[p.first_step + 1], edges = p.off[p.depth + 1] - first;
     const int64_t w = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (w >= static_cast<int64_t>(p.n_trees) * edges) return;
     const int tree = static_cast<int>(w / edges);
-    const int local = 1 + static_cast<int>(w - static_cast<int64_t>(tree) * edges);
-    int step = 0;                                           // the node's depth is step + 1
+    const int local = first + static_cast<int>(w - static_cast<int64_t>(tree) * edges);
+    int step = p.first_step;                                // the node's depth is step + 1
     while (step + 1 < p.depth && local >= p.off[step + 2]) ++step;
     const int64_t row = static_cast<int64_t>(tree) * p.nodes_cap + local;
     if (!BGRPO_IN_BOUNDS(p.status, local < p.nodes_cap && p.nchunks * 2 <= p.per_row)) return;
@@ -127,6 +199,11 @@ logprob_finish_kernel(const __grid_constant__ LogprobLaunch p) {
                                                                    static_cast<double>(p.logp_const[step]));
 }
 
+cudaError_t launch_finish(const LogprobLaunch& p, cudaStream_t s) {
+    const int64_t rows = static_cast<int64_t>(p.n_trees) * (p.off[p.depth + 1] - p.off[p.first_step + 1]);
+    return launch_overlapped(logprob_finish_kernel, static_cast<unsigned int>((rows + 7) / 8), 256, 0, s, p);
+}
+
 }  // namespace
 
 cudaError_t launch_logprob_tree(const LogprobLaunch& p, cudaStream_t s) {
@@ -135,8 +212,14 @@ cudaError_t launch_logprob_tree(const LogprobLaunch& p, cudaStream_t s) {
     if (items < 0 || items > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     const cudaError_t e = launch_overlapped(logprob_tree_kernel, static_cast<unsigned int>(items), kThreads, 0, s, p);
     if (e != cudaSuccess) return e;
-    const int64_t rows = static_cast<int64_t>(p.n_trees) * (p.off[p.depth + 1] - 1);
-    return launch_overlapped(logprob_finish_kernel, static_cast<unsigned int>((rows + 7) / 8), 256, 0, s, p);
+    return launch_finish(p, s);
+}
+
+cudaError_t launch_logprob_step(const LogprobLaunch& p, cudaStream_t s) {
+    const int64_t items = static_cast<int64_t>(p.n_trees) * p.families * p.nchunks;
+    if (items <= 0 || items > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+    const cudaError_t e = launch_overlapped(logprob_step_kernel, static_cast<unsigned int>(items), kEdgeThreads, 0, s, p);
+    return e != cudaSuccess ? e : launch_finish(p, s);
 }
 
 }  // namespace bgrpo

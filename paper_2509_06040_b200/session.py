@@ -24,7 +24,7 @@ class TreeSession:
     def __init__(self, w, n_trees: Optional[int] = None, tree_id_base: int = 0, device="cuda:0", nodes_cap=None,
                  fused_rollout: bool = False):
         self.w = w
-        # one launch for all T steps (closed-form velocity only) instead of one tree_step per depth
+        # all T steps in one launch, asked for by name (closed-form velocity only)
         self.fused_rollout = fused_rollout and w.velocity == "linear"
         self.n_trees = w.n_trees if n_trees is None else n_trees
         self.device = torch.device(device)
@@ -131,7 +131,7 @@ class TreeSession:
 
     def kernel_launches_per_pass(self) -> int:
         w = self.w
-        if self.fused_rollout:
+        if w.velocity == "linear" and len(w.splits) <= 6:
             n = 1 + 2                                              # root + whole-tree rollout + its log-prob sums
         else:
             n = 1 + w.T * (2 if w.velocity == "mlp" else 1) + 1   # root + (mlp +) step per depth + log-prob flush
