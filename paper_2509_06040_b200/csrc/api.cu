@@ -412,31 +412,30 @@ bgrpo_status bgrpo_tree_logprob(bgrpo_tree* t, int32_t step, const float* v_dev,
         const cudaError_t e0 = flush_pending(t, as_stream(stream));
         if (e0 != cudaSuccess) return cuda_fail(e0, "log-prob flush kernel");
     }
-    LogprobLaunch p;
-    p.latents = t->buf.latents;
-    p.mu = t->mu;
-    p.v = v_dev;
-    p.logp_out = logp_out_dev;
-    p.partials = static_cast<double*>(t->partials_logp);
-    p.status = t->status;
-    p.D = t->D;
-    p.n_trees = t->desc.n_trees;
-    p.nodes_cap = t->desc.nodes_cap;
-    p.nchunks = static_cast<int32_t>((t->D / 4 + kLogprobChunkVec - 1) / kLogprobChunkVec);
-    p.per_row = static_cast<int32_t>(partials_per_row(t->D));
-    p.first_step = step < 0 ? 0 : step;
-    p.depth = step < 0 ? t->depth : step + 1;
-    for (int d = 0; d <= p.depth + 1; ++d) p.off[d] = t->lv.offset[d];
-    for (int i = p.first_step; i < p.depth; ++i) {
-        const StepCoef& k = t->coef[i];
-        p.ca[i] = v_dev ? k.a : k.lin_a;
-        p.cb[i] = v_dev ? k.b : k.lin_b;
-        p.g[i] = k.g;
-        p.inv_2g2[i] = k.inv_2g2;
-        p.logp_const[i] = k.logp_const;
-    }
     cudaError_t e;
+    const int32_t nchunks = static_cast<int32_t>((t->D / 4 + kLogprobChunkVec - 1) / kLogprobChunkVec);
     if (step < 0) {
+        LogprobLaunch p;
+        p.latents = t->buf.latents;
+        p.mu = t->mu;
+        p.logp_out = logp_out_dev;
+        p.partials = static_cast<double*>(t->partials_logp);
+        p.status = t->status;
+        p.D = t->D;
+        p.n_trees = t->desc.n_trees;
+        p.nodes_cap = t->desc.nodes_cap;
+        p.nchunks = nchunks;
+        p.per_row = static_cast<int32_t>(partials_per_row(t->D));
+        p.depth = t->depth;
+        for (int d = 0; d <= t->depth + 1; ++d) p.off[d] = t->lv.offset[d];
+        for (int i = 0; i < t->depth; ++i) {
+            const StepCoef& k = t->coef[i];
+            p.ca[i] = k.lin_a;
+            p.cb[i] = k.lin_b;
+            p.g[i] = k.g;
+            p.inv_2g2[i] = k.inv_2g2;
+            p.logp_const[i] = k.logp_const;
+        }
         // a fork and the chains below it; run 0 is the chain below the root
         const RunInfo runs = runs_of(t->lv, t->depth);
         p.n_runs = runs.n;
@@ -451,8 +450,28 @@ bgrpo_status bgrpo_tree_logprob(bgrpo_tree* t, int32_t step, const float* v_dev,
         }
         e = launch_logprob_tree(p, as_stream(stream));
     } else {
-        p.families = t->lv.width[step];
-        p.run_fan[0] = t->lv.fanout[step];
+        const StepCoef& k = t->coef[step];
+        LogprobStepLaunch p;
+        p.latents = t->buf.latents;
+        p.v = v_dev;
+        p.mu = v_dev ? nullptr : t->mu;
+        p.logp_out = logp_out_dev;
+        p.partials = static_cast<double*>(t->partials_logp);
+        p.status = t->status;
+        p.D = t->D;
+        p.n_trees = t->desc.n_trees;
+        p.nodes_cap = t->desc.nodes_cap;
+        p.nchunks = nchunks;
+        p.per_row = static_cast<int32_t>(partials_per_row(t->D));
+        p.W = t->lv.width[step];
+        p.off = t->lv.offset[step];
+        p.off_child = t->lv.offset[step + 1];
+        p.fan = t->lv.fanout[step];
+        p.ca = v_dev ? k.a : k.lin_a;
+        p.cb = v_dev ? k.b : k.lin_b;
+        p.g = k.g;
+        p.inv_2g2 = k.inv_2g2;
+        p.logp_const = k.logp_const;
         e = launch_logprob_step(p, as_stream(stream));
     }
     return e == cudaSuccess ? BGRPO_OK : cuda_fail(e, "logprob kernel");

@@ -209,24 +209,36 @@ cudaError_t launch_finalize(const bgrpo_tree* t, const FinalizeDesc& f, cudaStre
 
 // ---- log-probs of all stored edges (tree_logprob.cu) ---------------------------------------------------------------
 constexpr int kLogprobChunkVec = 512;      // float4 of a row per CTA; one double per (row, chunk) fits the step kernel's partials
-static_assert(kLogprobChunkVec == kStepChunkVec, "one double per (row, chunk) fits what the step kernel needs");
+static_assert(kLogprobChunkVec == kStepChunkVec, "two doubles per (row, chunk) take what the step kernel needs");
 struct LogprobLaunch {
     const float* latents;
     const float* mu;           // [n_trees][D]
     float* logp_out;
-    const float* v;            // one step's edges: [n_trees][W][D], or nullptr: closed-form velocity
     double* partials;          // [rows][nchunks]
     int32_t* status;
     int64_t D;
     int32_t n_trees, nodes_cap, nchunks, per_row, depth;
-    int32_t first_step;        // log-probs are written from this step's edges on
     int32_t families, n_runs;                          // families per tree, in all runs
     int32_t run_families[BGRPO_MAX_T + 1], run_d0[BGRPO_MAX_T + 1], run_fan[BGRPO_MAX_T + 1], run_len[BGRPO_MAX_T + 1];
     int32_t off[BGRPO_MAX_T + 2];
     float ca[BGRPO_MAX_T], cb[BGRPO_MAX_T], g[BGRPO_MAX_T], inv_2g2[BGRPO_MAX_T], logp_const[BGRPO_MAX_T];   // by step
 };
 cudaError_t launch_logprob_tree(const LogprobLaunch& p, cudaStream_t s);      // all edges, closed form
-cudaError_t launch_logprob_step(const LogprobLaunch& p, cudaStream_t s);      // the edges of step depth - 1 = first_step
+// One step's edges.  A small parameter block of its own: with the other one's 2.4 KB the sixteen calls that score an image
+// tree took 5 us longer.
+struct LogprobStepLaunch {
+    const float* latents;
+    const float* v;            // [n_trees][W][D], or nullptr: closed-form velocity
+    const float* mu;           // [n_trees][D]
+    float* logp_out;
+    double* partials;          // [rows][2 nchunks]: one per chunk and warp
+    int32_t* status;
+    int64_t D;
+    int32_t n_trees, nodes_cap, nchunks, per_row;
+    int32_t W, off, off_child, fan;
+    float ca, cb, g, inv_2g2, logp_const;
+};
+cudaError_t launch_logprob_step(const LogprobStepLaunch& p, cudaStream_t s);
 
 struct RewardLaunch {
     const float* latents; const float* target; float* r; double* partials; unsigned int* counters; int32_t* status;

@@ -10,8 +10,8 @@
 // One step's edges under a given velocity (12 bytes per element and edge without a fork): one CTA per parent and chunk, all
 // its loads issued before the first is used.
 //
-// The sums of squares are float32 inside a warp's 512 elements, double from there on, one double per (row, chunk), added in
-// chunk order.
+// The sums of squares are float32 inside a warp's elements of a chunk (512, or 1024 for one step's edges), double from there
+// on, added in chunk order.
 #include "internal.h"
 
 namespace bgrpo {
@@ -108,7 +108,7 @@ constexpr int kEdgeThreads = 64, kEdgeVec = kLogprobChunkVec / kEdgeThreads, kEd
 
 template <bool FULL>
 __device__ __forceinline__ void score_chunk(const float4* __restrict__ zp, const float4* __restrict__ xp, const float4* __restrict__ cp, size_t D4,
-                                            uint32_t vecs, int fan, float ca, float cb, float (*acc_out)[kEdgeWarps]) {
+                                            uint32_t vecs, int fan, float ca, float cb, double* out, int parts) {
     float4 m[kEdgeVec], x[kEdgeVec], c[kEdgeVec];
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
@@ -141,67 +141,69 @@ __device__ __forceinline__ void score_chunk(const float4* __restrict__ zp, const
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-        if ((threadIdx.x & 31) == 0) acc_out[b][threadIdx.x >> 5] = acc;
+        if ((threadIdx.x & 31) == 0) out[static_cast<int64_t>(b) * parts] = static_cast<double>(acc);
     }
 }
 
 __global__ void __launch_bounds__(kEdgeThreads, 8)
-logprob_step_kernel(const __grid_constant__ LogprobLaunch p) {
-    __shared__ float s_acc[BGRPO_MAX_K][kEdgeWarps];
+logprob_step_kernel(const __grid_constant__ LogprobStepLaunch p) {
     pdl_release();
     pdl_wait();
     const int chunk = blockIdx.x % p.nchunks;
-    const int row = blockIdx.x / p.nchunks;                 // tree * families + f
-    const int tree = row / p.families, f = row - tree * p.families;
-    const int d0 = p.first_step, fan = p.run_fan[0];
+    const int row = blockIdx.x / p.nchunks;                 // tree * W + j
+    const int tree = row / p.W, j = row - tree * p.W;
     const uint32_t D4 = static_cast<uint32_t>(p.D >> 2), e = static_cast<uint32_t>(chunk) * kLogprobChunkVec;
-    const int64_t row0 = static_cast<int64_t>(tree) * p.nodes_cap, child = row0 + p.off[d0 + 1] + f * fan;
-    if (!BGRPO_IN_BOUNDS(p.status, tree < p.n_trees && e < D4 && p.off[d0] + f < p.off[d0 + 1] && p.off[d0 + 1] + (f + 1) * fan <= p.nodes_cap &&
-                                       p.nchunks * 2 <= p.per_row)) return;
-    const float4* zp = reinterpret_cast<const float4*>(p.latents + (row0 + p.off[d0] + f) * p.D) + e;
+    const int64_t row0 = static_cast<int64_t>(tree) * p.nodes_cap, child = row0 + p.off_child + j * p.fan;
+    const int parts = p.nchunks * kEdgeWarps;
+    if (!BGRPO_IN_BOUNDS(p.status, tree < p.n_trees && e < D4 && p.off + j < p.off_child && p.off_child + (j + 1) * p.fan <= p.nodes_cap &&
+                                       parts * 2 <= p.per_row)) return;
+    const float4* zp = reinterpret_cast<const float4*>(p.latents + (row0 + p.off + j) * p.D) + e;
     const float4* cp = reinterpret_cast<const float4*>(p.latents + child * p.D) + e;
     const float4* xp = (p.v != nullptr ? reinterpret_cast<const float4*>(p.v + static_cast<int64_t>(row) * p.D)
                                        : reinterpret_cast<const float4*>(p.mu + static_cast<int64_t>(tree) * p.D)) + e;
-    if (D4 - e >= kLogprobChunkVec) score_chunk<true>(zp, xp, cp, D4, kLogprobChunkVec, fan, p.ca[d0], p.cb[d0], s_acc);
-    else score_chunk<false>(zp, xp, cp, D4, D4 - e, fan, p.ca[d0], p.cb[d0], s_acc);
-    __syncthreads();
-    if (threadIdx.x < fan) {
-        double s = 0.0;
-#pragma unroll
-        for (int w = 0; w < kEdgeWarps; ++w) s += static_cast<double>(s_acc[threadIdx.x][w]);
-        p.partials[(child + threadIdx.x) * p.nchunks + chunk] = s;
-    }
+    double* out = p.partials + child * parts + chunk * kEdgeWarps + (threadIdx.x >> 5);
+    if (D4 - e >= kLogprobChunkVec) score_chunk<true>(zp, xp, cp, D4, kLogprobChunkVec, p.fan, p.ca, p.cb, out, parts);
+    else score_chunk<false>(zp, xp, cp, D4, D4 - e, p.fan, p.ca, p.cb, out, parts);
 }
 
-// One warp per row: the row's chunk partials in index order within each lane, then a fixed shuffle tree.
-__global__ void __launch_bounds__(256)
-logprob_finish_kernel(const __grid_constant__ LogprobLaunch p) {
-    pdl_release();
-    pdl_wait();
-    const int first = p.off[p.first_step + 1], edges = p.off[p.depth + 1] - first;
-    const int64_t w = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (w >= static_cast<int64_t>(p.n_trees) * edges) return;
-    const int tree = static_cast<int>(w / edges);
-    const int local = first + static_cast<int>(w - static_cast<int64_t>(tree) * edges);
-    int step = p.first_step;                                // the node's depth is step + 1
-    while (step + 1 < p.depth && local >= p.off[step + 2]) ++step;
-    const int64_t row = static_cast<int64_t>(tree) * p.nodes_cap + local;
-    if (!BGRPO_IN_BOUNDS(p.status, local < p.nodes_cap && p.nchunks * 2 <= p.per_row)) return;
-    const double* q = p.partials + row * p.nchunks;
+// One warp: a row's partials in index order within each lane, then a fixed shuffle tree; lane 0 writes the log-prob.
+__device__ __forceinline__ void finish_row(const double* q, int n, int64_t D, float g, float inv_2g2, float logp_const, float* out) {
     double s = 0.0;
 #pragma unroll 8
-    for (int c = threadIdx.x & 31; c < p.nchunks; c += 32) s += __ldcg(q + c);
+    for (int c = threadIdx.x & 31; c < n; c += 32) s += __ldcg(q + c);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
     if ((threadIdx.x & 31) == 0)
-        p.logp_out[row] = (p.g[step] == 0.0f) ? 0.0f
-                                              : static_cast<float>(-(s / static_cast<double>(p.D)) * static_cast<double>(p.inv_2g2[step]) +
-                                                                   static_cast<double>(p.logp_const[step]));
+        *out = (g == 0.0f) ? 0.0f : static_cast<float>(-(s / static_cast<double>(D)) * static_cast<double>(inv_2g2) + static_cast<double>(logp_const));
 }
 
-cudaError_t launch_finish(const LogprobLaunch& p, cudaStream_t s) {
-    const int64_t rows = static_cast<int64_t>(p.n_trees) * (p.off[p.depth + 1] - p.off[p.first_step + 1]);
-    return launch_overlapped(logprob_finish_kernel, static_cast<unsigned int>((rows + 7) / 8), 256, 0, s, p);
+__global__ void __launch_bounds__(256)
+logprob_step_finish_kernel(const __grid_constant__ LogprobStepLaunch p) {
+    pdl_release();
+    pdl_wait();
+    const int w = blockIdx.x * 8 + (threadIdx.x >> 5), W = p.W * p.fan;
+    if (w >= p.n_trees * W) return;
+    const int tree = w / W, parts = p.nchunks * kEdgeWarps;
+    const int64_t row = static_cast<int64_t>(tree) * p.nodes_cap + p.off_child + (w - tree * W);
+    if (!BGRPO_IN_BOUNDS(p.status, p.off_child + W <= p.nodes_cap && parts * 2 <= p.per_row)) return;
+    finish_row(p.partials + row * parts, parts, p.D, p.g, p.inv_2g2, p.logp_const, p.logp_out + row);
+}
+
+// All edges: one warp per non-root row.
+__global__ void __launch_bounds__(256)
+logprob_tree_finish_kernel(const __grid_constant__ LogprobLaunch p) {
+    pdl_release();
+    pdl_wait();
+    const int edges = p.off[p.depth + 1] - 1;
+    const int64_t w = static_cast<int64_t>(blockIdx.x) * 8 + (threadIdx.x >> 5);
+    if (w >= static_cast<int64_t>(p.n_trees) * edges) return;
+    const int tree = static_cast<int>(w / edges);
+    const int local = 1 + static_cast<int>(w - static_cast<int64_t>(tree) * edges);
+    int step = 0;                                           // the node's depth is step + 1
+    while (step + 1 < p.depth && local >= p.off[step + 2]) ++step;
+    const int64_t row = static_cast<int64_t>(tree) * p.nodes_cap + local;
+    if (!BGRPO_IN_BOUNDS(p.status, local < p.nodes_cap && p.nchunks * 2 <= p.per_row)) return;
+    finish_row(p.partials + row * p.nchunks, p.nchunks, p.D, p.g[step], p.inv_2g2[step], p.logp_const[step], p.logp_out + row);
 }
 
 }  // namespace
@@ -212,14 +214,17 @@ cudaError_t launch_logprob_tree(const LogprobLaunch& p, cudaStream_t s) {
     if (items < 0 || items > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     const cudaError_t e = launch_overlapped(logprob_tree_kernel, static_cast<unsigned int>(items), kThreads, 0, s, p);
     if (e != cudaSuccess) return e;
-    return launch_finish(p, s);
+    const int64_t rows = static_cast<int64_t>(p.n_trees) * (p.off[p.depth + 1] - 1);
+    return launch_overlapped(logprob_tree_finish_kernel, static_cast<unsigned int>((rows + 7) / 8), 256, 0, s, p);
 }
 
-cudaError_t launch_logprob_step(const LogprobLaunch& p, cudaStream_t s) {
-    const int64_t items = static_cast<int64_t>(p.n_trees) * p.families * p.nchunks;
+cudaError_t launch_logprob_step(const LogprobStepLaunch& p, cudaStream_t s) {
+    const int64_t items = static_cast<int64_t>(p.n_trees) * p.W * p.nchunks;
     if (items <= 0 || items > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     const cudaError_t e = launch_overlapped(logprob_step_kernel, static_cast<unsigned int>(items), kEdgeThreads, 0, s, p);
-    return e != cudaSuccess ? e : launch_finish(p, s);
+    if (e != cudaSuccess) return e;
+    const int64_t rows = static_cast<int64_t>(p.n_trees) * p.W * p.fan;
+    return launch_overlapped(logprob_step_finish_kernel, static_cast<unsigned int>((rows + 7) / 8), 256, 0, s, p);
 }
 
 }  // namespace bgrpo
