@@ -297,7 +297,8 @@ bgrpo_status bgrpo_tree_step(bgrpo_tree* t, int32_t split_flag, const float* v_d
     if (e != cudaSuccess) return cuda_fail(e, "step kernel");
     // this launch summed the previous level's log-probs in its prologue; its own are pending until the next
     // launch, or until the flush below when the tree is complete
-    t->pending = FinalizeDesc{t->buf.logp, static_cast<int32_t>(W_out), static_cast<int32_t>(off_out), t->coef[i].g, t->coef[i].logp_const};
+    const int warps = step_threads(static_cast<int64_t>(p.n_trees) * p.W_in * p.nchunks) / 32;
+    t->pending = FinalizeDesc{t->buf.logp, static_cast<int32_t>(W_out), static_cast<int32_t>(off_out), p.nchunks * warps, t->coef[i].g, t->coef[i].logp_const};
     if (i + 1 == t->desc.T) {
         e = flush_pending(t, as_stream(stream));
         if (e != cudaSuccess) return cuda_fail(e, "log-prob flush kernel");

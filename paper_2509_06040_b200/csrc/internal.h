@@ -17,11 +17,14 @@ constexpr int kRewardChunkVec = kStreamThreads * kRewardVec;   // float4 per (ro
 // thread, persistent grids and a shared-memory ring fed by bulk asynchronous copies: the kernel is bound by
 // instruction issue (Philox + Box-Muller), and eight independent noise chains per thread with many small CTAs
 // per SM gave the best rate on both the 8 B/element and the 12 B/element workloads.
-constexpr int kStepThreads = 64;
+// A launch of less than four such CTAs per SM has no throughput to lose: it takes as long as one thread's work, so the same
+// chunk goes to 256 threads of 2 float4.
+constexpr int kStepThreads = 64, kStepThreadsSmall = 256;
 constexpr int kStepVec = 8;
 constexpr int kStepChunkVec = kStepThreads * kStepVec;   // 512 float4 = 8 KiB per operand tile
-constexpr int kStepWarps = kStepThreads / 32;            // log-prob partials per (row, chunk)
-constexpr int kStepCtasPerSm = 8;
+constexpr int kStepCtasPerSm = 8, kStepCtasPerSmSmall = 4;
+constexpr int64_t kStepSmallGrid = 148 * 4;
+inline int step_threads(int64_t items) { return items < kStepSmallGrid ? kStepThreadsSmall : kStepThreads; }
 // Whole-tree rollout kernel: 128-thread CTAs, 4 float4 per thread (1 and 2 measured 37 and 16 % slower on the video tree), four
 // CTAs per SM (5 and 6: equal and 6 % slower there, 16 and 40 % slower on a single image tree), one log-prob partial per
 // node row and warp; at most kFusedMaxSplits split steps (the means of the open forks wait in shared memory).
@@ -36,7 +39,7 @@ inline int64_t fused_partials_per_row(int64_t D) { return ((D / 4 + kFusedChunkV
 // warp in the step kernel); an even number, so that every row starts on 8 bytes
 inline int64_t partials_per_row(int64_t D) {
     const int64_t D4 = D / 4;
-    const int64_t step = ((D4 + kStepChunkVec - 1) / kStepChunkVec) * kStepWarps * 2;
+    const int64_t step = ((D4 + kStepChunkVec - 1) / kStepChunkVec) * (kStepThreadsSmall / 32) * 2;
     const int64_t fused = fused_partials_per_row(D);
     return step > fused ? step : fused;
 }
@@ -81,6 +84,7 @@ struct StepCoef {
 struct FinalizeDesc {
     float* logp_out;       // nullptr: nothing pending
     int32_t W, off;        // rows off .. off+W-1 of every tree
+    int32_t per_row;       // partials per row
     float g, logp_const;
 };
 
@@ -200,7 +204,7 @@ struct StepLaunch {
     int32_t shared_noise;      // 1: finite s at a split step
     int32_t* status;           // the tree's status word
     int32_t per_row;           // 32-bit words reserved per node row in the partials
-    unsigned long long* partials;   // [rows][nchunks][kStepWarps] warp sums of quantized squares (philox.cuh)
+    unsigned long long* partials;   // [rows][nchunks][warps of a CTA] sums of quantized squares (philox.cuh)
     FinalizeDesc prev;         // level to finalize in this launch's prologue (logp_out == nullptr: none)
 };
 cudaError_t launch_root(const bgrpo_tree* t, cudaStream_t s);

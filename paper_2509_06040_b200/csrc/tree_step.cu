@@ -63,10 +63,10 @@ root_kernel(float* latents, int32_t* table, float* logp, unsigned int* counters,
 
 // Adds up the pending level's partial sums: one warp per row.
 __device__ __forceinline__ void finalize_rows(const FinalizeDesc& f, const unsigned long long* partials, int32_t n_trees, int32_t nodes_cap,
-                                              int32_t nchunks, int64_t D, int warp_global, int warps_total, int32_t* status, int32_t per_row_cap) {
+                                              int64_t D, int warp_global, int warps_total, int32_t* status, int32_t per_row_cap) {
     const int lane = threadIdx.x & 31;
     const int n_rows = n_trees * f.W;
-    const int per_row = nchunks * kStepWarps;
+    const int per_row = f.per_row;
     for (int idx = warp_global; idx < n_rows; idx += warps_total) {
         const int tree = idx / f.W;
         const int64_t row = static_cast<int64_t>(tree) * nodes_cap + f.off + (idx - tree * f.W);
@@ -80,12 +80,12 @@ __device__ __forceinline__ void finalize_rows(const FinalizeDesc& f, const unsig
     }
 }
 
-template <bool FULL>
+template <int THREADS, bool FULL>
 __device__ __forceinline__ void load_tile(const float4* __restrict__ zp, const float4* __restrict__ xop, bool streamed,
-                                          uint32_t vecs, float4 (&z)[kStepVec], float4 (&x)[kStepVec]) {
+                                          uint32_t vecs, float4 (&z)[kStepChunkVec / THREADS], float4 (&x)[kStepChunkVec / THREADS]) {
 #pragma unroll
-    for (int k = 0; k < kStepVec; ++k) {
-        const uint32_t t = threadIdx.x + k * kStepThreads;
+    for (int k = 0; k < kStepChunkVec / THREADS; ++k) {
+        const uint32_t t = threadIdx.x + k * THREADS;
         if (FULL || t < vecs) {
             z[k] = __ldcs(zp + t);                                   // read once: evict first
             x[k] = streamed ? __ldcs(xop + t) : __ldg(xop + t);      // the target mean is shared by the whole level
@@ -93,8 +93,8 @@ __device__ __forceinline__ void load_tile(const float4* __restrict__ zp, const f
     }
 }
 
-template <int FAN, bool SHARED, bool FULL, bool NOISY>
-__device__ __forceinline__ void compute_tile(const StepLaunch& p, const float4 (&z)[kStepVec], const float4 (&x)[kStepVec],
+template <int FAN, bool SHARED, int THREADS, bool FULL, bool NOISY>
+__device__ __forceinline__ void compute_tile(const StepLaunch& p, const float4 (&z)[kStepChunkVec / THREADS], const float4 (&x)[kStepChunkVec / THREADS],
                                              uint32_t vecs, uint32_t e_base, uint32_t D4, float4* zc, uint32_t gid_parent,
                                              uint32_t gid_child0, uint32_t (&acc)[FAN]) {
     NoiseNode shared_node, node[FAN];
@@ -102,8 +102,8 @@ __device__ __forceinline__ void compute_tile(const StepLaunch& p, const float4 (
 #pragma unroll
     for (int b = 0; b < FAN; ++b) node[b] = noise_node(gid_child0 + b, p.step, p.keys);
 #pragma unroll
-    for (int k = 0; k < kStepVec; ++k) {
-        const uint32_t t = threadIdx.x + k * kStepThreads;
+    for (int k = 0; k < kStepChunkVec / THREADS; ++k) {
+        const uint32_t t = threadIdx.x + k * THREADS;
         if (FULL || t < vecs) {
             const uint32_t e = e_base + t;
             float4 xi[FAN];
@@ -132,15 +132,16 @@ __device__ __forceinline__ void compute_tile(const StepLaunch& p, const float4 (
     }
 }
 
-template <int FAN, bool SHARED, bool NOISY = true>
-__global__ void __launch_bounds__(kStepThreads, kStepCtasPerSm)
+template <int FAN, bool SHARED, bool NOISY, int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS == kStepThreads ? kStepCtasPerSm : kStepCtasPerSmSmall)
 step_kernel(const __grid_constant__ StepLaunch p) {
+    constexpr int kWarps = THREADS / 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     pdl_release();
     pdl_wait();           // the parents, the velocity and the pending partial sums come from earlier kernels
     // the previous level's log-probs (a handful of rows): summed by this launch
     if (p.prev.logp_out != nullptr)
-        finalize_rows(p.prev, p.partials, p.n_trees, p.nodes_cap, p.nchunks, p.D, blockIdx.x * kStepWarps + warp, gridDim.x * kStepWarps, p.status, p.per_row);
+        finalize_rows(p.prev, p.partials, p.n_trees, p.nodes_cap, p.D, blockIdx.x * kWarps + warp, gridDim.x * kWarps, p.status, p.per_row);
 
     const int chunk = blockIdx.x % p.nchunks;
     const int row = blockIdx.x / p.nchunks;             // tree * W_in + j
@@ -154,7 +155,7 @@ step_kernel(const __grid_constant__ StepLaunch p) {
     const int child0 = p.off_out + j * FAN;
     const bool streamed = (p.v != nullptr);
     if (!BGRPO_IN_BOUNDS(p.status, tree < p.n_trees && parent < p.nodes_cap && child0 + FAN <= p.nodes_cap && e_base < D4 &&
-                                       2 * (chunk + 1) * kStepWarps <= p.per_row)) return;
+                                       2 * (chunk + 1) * kWarps <= p.per_row)) return;
     const float4* __restrict__ zp = reinterpret_cast<const float4*>(p.latents + (tree_row0 + parent) * p.D) + e_base;
     const float4* __restrict__ xop = (streamed ? reinterpret_cast<const float4*>(p.v + static_cast<int64_t>(row) * p.D)
                                                : reinterpret_cast<const float4*>(p.mu + static_cast<int64_t>(tree) * p.D)) + e_base;
@@ -165,20 +166,20 @@ step_kernel(const __grid_constant__ StepLaunch p) {
     uint32_t acc[FAN];
 #pragma unroll
     for (int b = 0; b < FAN; ++b) acc[b] = 0u;
-    float4 z[kStepVec], x[kStepVec];
+    float4 z[kStepChunkVec / THREADS], x[kStepChunkVec / THREADS];
     if (vecs == kStepChunkVec) {
-        load_tile<true>(zp, xop, streamed, vecs, z, x);
-        compute_tile<FAN, SHARED, true, NOISY>(p, z, x, vecs, e_base, D4, zc, gid_parent, gid_child0, acc);
+        load_tile<THREADS, true>(zp, xop, streamed, vecs, z, x);
+        compute_tile<FAN, SHARED, THREADS, true, NOISY>(p, z, x, vecs, e_base, D4, zc, gid_parent, gid_child0, acc);
     } else {
-        load_tile<false>(zp, xop, streamed, vecs, z, x);
-        compute_tile<FAN, SHARED, false, NOISY>(p, z, x, vecs, e_base, D4, zc, gid_parent, gid_child0, acc);
+        load_tile<THREADS, false>(zp, xop, streamed, vecs, z, x);
+        compute_tile<FAN, SHARED, THREADS, false, NOISY>(p, z, x, vecs, e_base, D4, zc, gid_parent, gid_child0, acc);
     }
     // one number per (child row, chunk, warp): a lane's sum takes up to 31 bits, so its halves are added apart
 #pragma unroll
     for (int b = 0; b < FAN; ++b) {
         const uint32_t lo = __reduce_add_sync(0xffffffffu, acc[b] & 0xffffu), hi = __reduce_add_sync(0xffffffffu, acc[b] >> 16);
         if (lane == 0)
-            p.partials[((tree_row0 + child0 + b) * p.nchunks + chunk) * kStepWarps + warp] = (static_cast<unsigned long long>(hi) << 16) + lo;
+            p.partials[((tree_row0 + child0 + b) * p.nchunks + chunk) * kWarps + warp] = (static_cast<unsigned long long>(hi) << 16) + lo;
     }
     if (chunk == 0 && threadIdx.x < FAN) {      // node-table rows of the new children
         const int b = threadIdx.x;
@@ -193,11 +194,11 @@ step_kernel(const __grid_constant__ StepLaunch p) {
 
 // Flush: adds up a pending level outside a step launch (the tree is complete, or tree_logprob is done).
 __global__ void __launch_bounds__(kStreamThreads)
-finalize_kernel(const FinalizeDesc f, const unsigned long long* partials, int32_t n_trees, int32_t nodes_cap, int32_t nchunks, int64_t D,
+finalize_kernel(const FinalizeDesc f, const unsigned long long* partials, int32_t n_trees, int32_t nodes_cap, int64_t D,
                 int32_t* status, int32_t per_row_cap) {
     pdl_release();
     pdl_wait();
-    finalize_rows(f, partials, n_trees, nodes_cap, nchunks, D, blockIdx.x * (kStreamThreads / 32) + (threadIdx.x >> 5),
+    finalize_rows(f, partials, n_trees, nodes_cap, D, blockIdx.x * (kStreamThreads / 32) + (threadIdx.x >> 5),
                   gridDim.x * (kStreamThreads / 32), status, per_row_cap);
 }
 
@@ -214,11 +215,21 @@ __global__ void debug_trip_kernel(int32_t* status) {
     if (!BGRPO_IN_BOUNDS(status, threadIdx.x > 0)) return;      // thread 0 fails the test; nothing is accessed
 }
 
-template <int FAN>
+template <int FAN, int THREADS>
 cudaError_t launch_step_fan(const StepLaunch& p, unsigned int grid, cudaStream_t s) {
-    if (p.g == 0.0f) return launch_overlapped(step_kernel<FAN, false, false>, grid, kStepThreads, 0, s, p);     // ODE step
-    if (p.shared_noise) return launch_overlapped(step_kernel<FAN, true>, grid, kStepThreads, 0, s, p);
-    return launch_overlapped(step_kernel<FAN, false>, grid, kStepThreads, 0, s, p);
+    if (p.g == 0.0f) return launch_overlapped(step_kernel<FAN, false, false, THREADS>, grid, THREADS, 0, s, p);     // ODE step
+    if (p.shared_noise) return launch_overlapped(step_kernel<FAN, true, true, THREADS>, grid, THREADS, 0, s, p);
+    return launch_overlapped(step_kernel<FAN, false, true, THREADS>, grid, THREADS, 0, s, p);
+}
+template <int THREADS>
+cudaError_t launch_step_threads(const StepLaunch& p, unsigned int grid, cudaStream_t s) {
+    switch (p.fan) {
+        case 1: return launch_step_fan<1, THREADS>(p, grid, s);
+        case 2: return launch_step_fan<2, THREADS>(p, grid, s);
+        case 3: return launch_step_fan<3, THREADS>(p, grid, s);
+        case 4: return launch_step_fan<4, THREADS>(p, grid, s);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 }  // namespace
@@ -239,20 +250,14 @@ cudaError_t launch_step(const StepLaunch& p, cudaStream_t s) {
     const int64_t items = static_cast<int64_t>(p.n_trees) * p.W_in * p.nchunks;
     if (items <= 0 || items > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     const unsigned int grid = static_cast<unsigned int>(items);
-    switch (p.fan) {
-        case 1: return launch_step_fan<1>(p, grid, s);
-        case 2: return launch_step_fan<2>(p, grid, s);
-        case 3: return launch_step_fan<3>(p, grid, s);
-        case 4: return launch_step_fan<4>(p, grid, s);
-        default: return cudaErrorInvalidValue;
-    }
+    return step_threads(items) == kStepThreads ? launch_step_threads<kStepThreads>(p, grid, s) : launch_step_threads<kStepThreadsSmall>(p, grid, s);
 }
 
 cudaError_t launch_finalize(const bgrpo_tree* t, const FinalizeDesc& f, cudaStream_t s) {
     const int rows = t->desc.n_trees * f.W;
     const int grid = (rows + (kStreamThreads / 32) - 1) / (kStreamThreads / 32);
     return launch_overlapped(finalize_kernel, grid < 1 ? 1 : grid, kStreamThreads, 0, s, f, static_cast<const unsigned long long*>(t->partials_u64()),
-                             t->desc.n_trees, t->desc.nodes_cap, t->nchunks_step, t->D, t->status,
+                             t->desc.n_trees, t->desc.nodes_cap, t->D, t->status,
                              static_cast<int32_t>(partials_per_row(t->D)));
 }
 
