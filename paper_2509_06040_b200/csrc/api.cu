@@ -434,7 +434,7 @@ bgrpo_status bgrpo_tree_logprob(bgrpo_tree* t, int32_t step, const float* v_dev,
             p.ca[i] = k.lin_a;
             p.cb[i] = k.lin_b;
             p.g[i] = k.g;
-            p.inv_2g2[i] = k.inv_2g2;
+            p.scale[i] = static_cast<double>(k.inv_2g2) / static_cast<double>(t->D);
             p.logp_const[i] = k.logp_const;
         }
         // a fork and the chains below it; run 0 is the chain below the root
@@ -471,7 +471,7 @@ bgrpo_status bgrpo_tree_logprob(bgrpo_tree* t, int32_t step, const float* v_dev,
         p.ca = v_dev ? k.a : k.lin_a;
         p.cb = v_dev ? k.b : k.lin_b;
         p.g = k.g;
-        p.inv_2g2 = k.inv_2g2;
+        p.scale = static_cast<double>(k.inv_2g2) / static_cast<double>(t->D);
         p.logp_const = k.logp_const;
         e = launch_logprob_step(p, as_stream(stream));
     }

@@ -198,6 +198,7 @@ struct StepLaunch {
     int32_t W_in, off_in, off_out, fan, step, is_split;
     uint32_t node_id_base;     // tree_id_base * nodes_cap
     PhiloxKeys keys;
+    double half_per;           // logp_half_per(D), set by launch_step
     float ca, cb;              // mean = ca*z + cb*x, x = v or mu
     float g;
     float mix_shared, mix_innov;
@@ -225,7 +226,8 @@ struct LogprobLaunch {
     int32_t families, n_runs;                          // families per tree, in all runs
     int32_t run_families[BGRPO_MAX_T + 1], run_d0[BGRPO_MAX_T + 1], run_fan[BGRPO_MAX_T + 1], run_len[BGRPO_MAX_T + 1];
     int32_t off[BGRPO_MAX_T + 2];
-    float ca[BGRPO_MAX_T], cb[BGRPO_MAX_T], g[BGRPO_MAX_T], inv_2g2[BGRPO_MAX_T], logp_const[BGRPO_MAX_T];   // by step
+    float ca[BGRPO_MAX_T], cb[BGRPO_MAX_T], g[BGRPO_MAX_T], logp_const[BGRPO_MAX_T];   // by step
+    double scale[BGRPO_MAX_T];
 };
 cudaError_t launch_logprob_tree(const LogprobLaunch& p, cudaStream_t s);      // all edges, closed form
 // One step's edges.  A small parameter block of its own: with the other one's 2.4 KB the sixteen calls that score an image
@@ -240,7 +242,8 @@ struct LogprobStepLaunch {
     int64_t D;
     int32_t n_trees, nodes_cap, nchunks, per_row;
     int32_t W, off, off_child, fan;
-    float ca, cb, g, inv_2g2, logp_const;
+    float ca, cb, g, logp_const;
+    double scale;              // 1 / (2 g^2 D), from the host: a double division takes longer than the rest of the sum
 };
 cudaError_t launch_logprob_step(const LogprobStepLaunch& p, cudaStream_t s);
 
@@ -276,6 +279,7 @@ struct FusedLaunch {
     int32_t split_step[kFusedMaxSplits];
     uint32_t node_id_base;
     PhiloxKeys keys;
+    double half_per;           // logp_half_per(D), set by launch_rollout_fused
     float mix_shared, mix_innov;
     FusedStep step[BGRPO_MAX_T];                       // set by the caller but for px, ph
 };

@@ -158,8 +158,10 @@ constexpr float kSquareScale = 262144.0f;
 __device__ __forceinline__ uint32_t quantized_squares(float squares) { return __float2uint_rn(squares * kSquareScale); }
 __device__ __forceinline__ float squares_of(const float4& x) { return fmaf(x.x, x.x, fmaf(x.y, x.y, fmaf(x.z, x.z, x.w * x.w))); }
 // the log-prob of an edge from its row's sum: -(1/D) sum (z' - mean)^2 / (2 g^2) + const with (z' - mean)^2 = g^2 xi^2
-__device__ __forceinline__ float logp_from_squares(unsigned long long sum, int64_t D, float g, float logp_const) {
-    return g == 0.0f ? 0.0f : static_cast<float>(static_cast<double>(logp_const) - static_cast<double>(sum) * (0.5 / static_cast<double>(kSquareScale)) / static_cast<double>(D));
+// (half_per: 0.5 / (kSquareScale D), from the host: a double division takes longer than the rest of the sum)
+inline double logp_half_per(int64_t D) { return 0.5 / static_cast<double>(kSquareScale) / static_cast<double>(D); }
+__device__ __forceinline__ float logp_from_squares(unsigned long long sum, double half_per, float g, float logp_const) {
+    return g == 0.0f ? 0.0f : static_cast<float>(static_cast<double>(logp_const) - static_cast<double>(sum) * half_per);
 }
 __device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long x) {
 #pragma unroll

@@ -179,7 +179,7 @@ finalize_tree_kernel(const __grid_constant__ FusedLaunch p, int32_t nodes) {
     if (!BGRPO_IN_BOUNDS(p.status, local < p.nodes_cap && p.per_row <= p.per_row_cap)) return;
     const uint32_t* q = p.partials + row * p.per_row;
     unsigned long long s = 0;
-#pragma unroll 8
+#pragma unroll 4
     for (int c = threadIdx.x % THREADS; c < p.per_row; c += THREADS) s += __ldcg(q + c);
     s = warp_sum_u64(s);
     if (THREADS > 32) {
@@ -189,13 +189,14 @@ finalize_tree_kernel(const __grid_constant__ FusedLaunch p, int32_t nodes) {
         if (threadIdx.x == 0)
             for (int i = 1; i < 8; ++i) s += s_sum[i];
     }
-    if (threadIdx.x % THREADS == 0) p.logp[row] = logp_from_squares(s, p.D, p.step[step].g, p.step[step].logp_const);
+    if (threadIdx.x % THREADS == 0) p.logp[row] = logp_from_squares(s, p.half_per, p.step[step].g, p.step[step].logp_const);
 }
 
 }  // namespace
 
 cudaError_t launch_rollout_fused(const FusedLaunch& p0, int32_t nodes, cudaStream_t s) {
     FusedLaunch p = p0;
+    p.half_per = logp_half_per(p.D);
     int n_splits = 0;
     for (int i = 0; i < p.T; ++i) {
         noise_step(static_cast<uint32_t>(i), p.keys, p.step[i].px, p.step[i].ph);

@@ -167,14 +167,14 @@ logprob_step_kernel(const __grid_constant__ LogprobStepLaunch p) {
 }
 
 // One warp: a row's partials in index order within each lane, then a fixed shuffle tree; lane 0 writes the log-prob.
-__device__ __forceinline__ void finish_row(const double* q, int n, int64_t D, float g, float inv_2g2, float logp_const, float* out) {
+__device__ __forceinline__ void finish_row(const double* q, int n, float g, double scale, float logp_const, float* out) {
     double s = 0.0;
-#pragma unroll 8
+#pragma unroll 4
     for (int c = threadIdx.x & 31; c < n; c += 32) s += __ldcg(q + c);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
     if ((threadIdx.x & 31) == 0)
-        *out = (g == 0.0f) ? 0.0f : static_cast<float>(-(s / static_cast<double>(D)) * static_cast<double>(inv_2g2) + static_cast<double>(logp_const));
+        *out = (g == 0.0f) ? 0.0f : static_cast<float>(static_cast<double>(logp_const) - s * scale);
 }
 
 __global__ void __launch_bounds__(256)
@@ -186,7 +186,7 @@ logprob_step_finish_kernel(const __grid_constant__ LogprobStepLaunch p) {
     const int tree = w / W, parts = p.nchunks * kEdgeWarps;
     const int64_t row = static_cast<int64_t>(tree) * p.nodes_cap + p.off_child + (w - tree * W);
     if (!BGRPO_IN_BOUNDS(p.status, p.off_child + W <= p.nodes_cap && parts * 2 <= p.per_row)) return;
-    finish_row(p.partials + row * parts, parts, p.D, p.g, p.inv_2g2, p.logp_const, p.logp_out + row);
+    finish_row(p.partials + row * parts, parts, p.g, p.scale, p.logp_const, p.logp_out + row);
 }
 
 // All edges: one warp per non-root row.
@@ -203,7 +203,7 @@ logprob_tree_finish_kernel(const __grid_constant__ LogprobLaunch p) {
     while (step + 1 < p.depth && local >= p.off[step + 2]) ++step;
     const int64_t row = static_cast<int64_t>(tree) * p.nodes_cap + local;
     if (!BGRPO_IN_BOUNDS(p.status, local < p.nodes_cap && p.nchunks * 2 <= p.per_row)) return;
-    finish_row(p.partials + row * p.nchunks, p.nchunks, p.D, p.g[step], p.inv_2g2[step], p.logp_const[step], p.logp_out + row);
+    finish_row(p.partials + row * p.nchunks, p.nchunks, p.g[step], p.scale[step], p.logp_const[step], p.logp_out + row);
 }
 
 }  // namespace

@@ -63,7 +63,7 @@ root_kernel(float* latents, int32_t* table, float* logp, unsigned int* counters,
 
 // Adds up the pending level's partial sums: one warp per row.
 __device__ __forceinline__ void finalize_rows(const FinalizeDesc& f, const unsigned long long* partials, int32_t n_trees, int32_t nodes_cap,
-                                              int64_t D, int warp_global, int warps_total, int32_t* status, int32_t per_row_cap) {
+                                              double half_per, int warp_global, int warps_total, int32_t* status, int32_t per_row_cap) {
     const int lane = threadIdx.x & 31;
     const int n_rows = n_trees * f.W;
     const int per_row = f.per_row;
@@ -73,10 +73,10 @@ __device__ __forceinline__ void finalize_rows(const FinalizeDesc& f, const unsig
         if (!BGRPO_IN_BOUNDS(status, f.off + f.W <= nodes_cap && 2 * per_row <= per_row_cap)) continue;
         const unsigned long long* q = partials + row * per_row;
         unsigned long long s = 0;
-#pragma unroll 8
+#pragma unroll 4
         for (int c = lane; c < per_row; c += 32) s += __ldcg(q + c);
         s = warp_sum_u64(s);
-        if (lane == 0) f.logp_out[row] = logp_from_squares(s, D, f.g, f.logp_const);
+        if (lane == 0) f.logp_out[row] = logp_from_squares(s, half_per, f.g, f.logp_const);
     }
 }
 
@@ -141,7 +141,7 @@ step_kernel(const __grid_constant__ StepLaunch p) {
     pdl_wait();           // the parents, the velocity and the pending partial sums come from earlier kernels
     // the previous level's log-probs (a handful of rows): summed by this launch
     if (p.prev.logp_out != nullptr)
-        finalize_rows(p.prev, p.partials, p.n_trees, p.nodes_cap, p.D, blockIdx.x * kWarps + warp, gridDim.x * kWarps, p.status, p.per_row);
+        finalize_rows(p.prev, p.partials, p.n_trees, p.nodes_cap, p.half_per, blockIdx.x * kWarps + warp, gridDim.x * kWarps, p.status, p.per_row);
 
     const int chunk = blockIdx.x % p.nchunks;
     const int row = blockIdx.x / p.nchunks;             // tree * W_in + j
@@ -194,11 +194,11 @@ step_kernel(const __grid_constant__ StepLaunch p) {
 
 // Flush: adds up a pending level outside a step launch (the tree is complete, or tree_logprob is done).
 __global__ void __launch_bounds__(kStreamThreads)
-finalize_kernel(const FinalizeDesc f, const unsigned long long* partials, int32_t n_trees, int32_t nodes_cap, int64_t D,
+finalize_kernel(const FinalizeDesc f, const unsigned long long* partials, int32_t n_trees, int32_t nodes_cap, double half_per,
                 int32_t* status, int32_t per_row_cap) {
     pdl_release();
     pdl_wait();
-    finalize_rows(f, partials, n_trees, nodes_cap, D, blockIdx.x * (kStreamThreads / 32) + (threadIdx.x >> 5),
+    finalize_rows(f, partials, n_trees, nodes_cap, half_per, blockIdx.x * (kStreamThreads / 32) + (threadIdx.x >> 5),
                   gridDim.x * (kStreamThreads / 32), status, per_row_cap);
 }
 
@@ -246,7 +246,9 @@ cudaError_t launch_root(const bgrpo_tree* t, cudaStream_t s) {
                              static_cast<uint32_t>(t->desc.tree_id_base * t->desc.nodes_cap), make_philox_keys(t->desc.seed));
 }
 
-cudaError_t launch_step(const StepLaunch& p, cudaStream_t s) {
+cudaError_t launch_step(const StepLaunch& p0, cudaStream_t s) {
+    StepLaunch p = p0;
+    p.half_per = logp_half_per(p.D);
     const int64_t items = static_cast<int64_t>(p.n_trees) * p.W_in * p.nchunks;
     if (items <= 0 || items > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     const unsigned int grid = static_cast<unsigned int>(items);
@@ -257,7 +259,7 @@ cudaError_t launch_finalize(const bgrpo_tree* t, const FinalizeDesc& f, cudaStre
     const int rows = t->desc.n_trees * f.W;
     const int grid = (rows + (kStreamThreads / 32) - 1) / (kStreamThreads / 32);
     return launch_overlapped(finalize_kernel, grid < 1 ? 1 : grid, kStreamThreads, 0, s, f, static_cast<const unsigned long long*>(t->partials_u64()),
-                             t->desc.n_trees, t->desc.nodes_cap, t->D, t->status,
+                             t->desc.n_trees, t->desc.nodes_cap, logp_half_per(t->D), t->status,
                              static_cast<int32_t>(partials_per_row(t->D)));
 }
 
