@@ -302,9 +302,9 @@ bgrpo_status bgrpo_philox_normal_fill(uint64_t seed, uint32_t node_id, uint32_t 
  * over several calls, one after the other).  D must be a positive multiple of 4 (INVALID_ARG otherwise).
  * The call allocates and frees nothing.  The first call on each device looks up the array's device address (a host
  * symbol lookup, done once per device with that device current); make that first call outside any stream capture.
- * All calls on a device share the one array and it keeps the previous call's contents: the call clears the counters
- * it needs on `stream` before its kernel, but two calls that can overlap on the GPU (different streams without an
- * ordering between them) race on it and give wrong results - keep calls stream-ordered. */
+ * All calls on a device share the one array and its counters return to zero with every call, but two calls that can
+ * overlap on the GPU (different streams without an ordering between them) race on it and give wrong results - keep calls
+ * stream-ordered. */
 #define BGRPO_STATIC_SCRATCH_BYTES (512 * 1024)
 #define BGRPO_STATIC_MAX_ROWS 1024
 bgrpo_status bgrpo_reward_mse_static(const float* rows_dev, const float* target_dev, int32_t n_rows, int64_t D,

@@ -497,6 +497,7 @@ static bgrpo_status reward_common(bgrpo_tree* t, const float* target, float scal
     p.leaves = t->lv.width[t->desc.T];
     p.off_leaf = t->lv.offset[t->desc.T];
     p.scale = scale;
+    p.inv_D = 1.0 / static_cast<double>(t->D);
     p.mode = mode;
     cudaError_t e = launch_reward(p, as_stream(stream));
     if (e != cudaSuccess) return cuda_fail(e, "reward kernel");

@@ -103,6 +103,7 @@ struct RunInfo {
     int32_t first[BGRPO_MAX_T + 2];      // first[n] = T + 1
     int32_t chain0[BGRPO_MAX_T + 2];     // index of the run's first chain (a node and the only children below it); chain0[n] = number of chains
     int32_t of_depth[BGRPO_MAX_T + 1];
+    double inv_width[BGRPO_MAX_T + 1], inv_fan;      // per run; reciprocals from the host: a double division is a few hundred cycles
 };
 
 inline RunInfo runs_of(const LevelInfo& lv, int T) {
@@ -113,8 +114,11 @@ inline RunInfo runs_of(const LevelInfo& lv, int T) {
         if (lv.fanout[i] > 1) r.first[r.n++] = i + 1;
     r.first[r.n] = T + 1;
     r.chain0[0] = 0;
+    r.inv_fan = 1.0;
     for (int q = 0; q < r.n; ++q) {
         r.chain0[q + 1] = r.chain0[q] + lv.width[r.first[q]];
+        r.inv_width[q] = 1.0 / lv.width[r.first[q]];
+        if (q > 0) r.inv_fan = 1.0 / lv.fanout[r.first[q] - 1];      // the same at every fork
         for (int d = r.first[q]; d < r.first[q + 1]; ++d) r.of_depth[d] = q;
     }
     return r;
@@ -249,7 +253,7 @@ cudaError_t launch_logprob_step(const LogprobStepLaunch& p, cudaStream_t s);
 
 struct RewardLaunch {
     const float* latents; const float* target; float* r; double* partials; unsigned int* counters; int32_t* status;
-    int64_t D; int32_t n_trees, nodes_cap, nchunks, nchunks_cap, leaves, off_leaf; float scale; int32_t mode;  // 0 mse, 1 cos; nchunks_cap: partial slots reserved per row
+    int64_t D; int32_t n_trees, nodes_cap, nchunks, nchunks_cap, leaves, off_leaf; float scale; double inv_D; int32_t mode;  // 0 mse, 1 cos; nchunks_cap: partial slots reserved per row
 };
 cudaError_t launch_reward(const RewardLaunch& p, cudaStream_t s);
 
@@ -274,8 +278,9 @@ struct FusedLaunch {
     int32_t per_row_cap;       // words reserved per node row
     int64_t D;
     int32_t n_trees, nodes_cap, T, K, shared_noise;
-    int32_t nchunks, per_row;  // CTAs that cover a row; set by launch_rollout_fused, like the next four
-    int32_t par, subtrees, levels;                     // forks dealt out to the grid, K^par, forks walked
+    int32_t nchunks, per_row;  // CTAs that cover a row; set by launch_rollout_fused, like the next six
+    int32_t par, subtrees, levels, nodes;              // forks dealt out to the grid, K^par, forks walked, nodes of a tree
+    int32_t sums_at;           // 0, or 1 + where in shared memory (float4) the sums of a row of one CTA are
     int32_t split_step[kFusedMaxSplits];
     uint32_t node_id_base;
     PhiloxKeys keys;

@@ -27,11 +27,13 @@
 namespace bgrpo {
 namespace {
 
+constexpr uint32_t kNotMine = 0xffffffffu;          // no warp's sum: that is at most 128 squares of 133 * 2^18
+
 template <bool SHARED>
 __global__ void __launch_bounds__(kFusedThreads, kFusedCtasPerSm)
 rollout_fused_kernel(const __grid_constant__ FusedLaunch p) {
     constexpr int VEC = kFusedVec;
-    extern __shared__ float4 s_stack[];             // [open fork][VEC] means, SHARED: and as many xi_0
+    extern __shared__ float4 s_stack[];             // [open fork][VEC] means, SHARED: and as many xi_0; rows of one CTA: the sums of all nodes
     pdl_release();
     const int chunk = blockIdx.x % p.nchunks;
     const int group = blockIdx.x / p.nchunks;       // (tree, assignment of the first forks)
@@ -60,6 +62,12 @@ rollout_fused_kernel(const __grid_constant__ FusedLaunch p) {
     if (!BGRPO_IN_BOUNDS(p.status, tree < p.n_trees && static_cast<uint32_t>(chunk) * VEC * kFusedThreads < D4 && (chunk + 1) * (kFusedThreads / 32) <= p.per_row &&
                                        p.per_row <= p.per_row_cap)) return;
     uint32_t* const partials = p.partials + row0 * p.per_row + chunk * (kFusedThreads / 32) + warp;
+    // a row that is one CTA's alone: its sums stay here and the CTA writes the log-probs of the nodes it makes
+    uint32_t (*const s_sums)[kFusedThreads / 32] = p.sums_at > 0 ? reinterpret_cast<uint32_t (*)[kFusedThreads / 32]>(s_stack + p.sums_at - 1) : nullptr;
+    if (s_sums) {
+        for (int n = threadIdx.x; n < p.nodes; n += kFusedThreads) s_sums[n][0] = kNotMine;
+        __syncthreads();
+    }
     pdl_wait();
     float4 mu[VEC], m[VEC], xi0[VEC];               // m: the mean of the next child, xi0: mix_shared times the shared noise of its fork
     FusedStep st = p.step[0];
@@ -128,7 +136,10 @@ rollout_fused_kernel(const __grid_constant__ FusedLaunch p) {
             for (int k = 0; k < VEC; ++k)
                 if (live[k]) __stcs(row + e[k], z[k]);
             acc = __reduce_add_sync(0xffffffffu, acc);
-            if (lane == 0) partials[static_cast<uint64_t>(child) * static_cast<uint32_t>(p.per_row)] = acc;
+            if (lane == 0) {
+                if (s_sums) s_sums[child][warp] = acc;
+                else partials[static_cast<uint64_t>(child) * static_cast<uint32_t>(p.per_row)] = acc;
+            }
             if (writes_table) {
                 const int64_t rows = static_cast<int64_t>(p.n_trees) * p.nodes_cap, r = row0 + child;
                 p.table[r] = static_cast<int32_t>(parent);
@@ -147,7 +158,7 @@ rollout_fused_kernel(const __grid_constant__ FusedLaunch p) {
         }
         const uint32_t K = p.K;
         while (forks > p.par && j % K == K - 1) { j /= K; --forks; }       // back to the deepest fork with a child left
-        if (forks == p.par) return;
+        if (forks == p.par) break;
         ++j;
         i = p.split_step[forks - 1];
         st = p.step[i];
@@ -158,6 +169,17 @@ rollout_fused_kernel(const __grid_constant__ FusedLaunch p) {
             m[k] = s_stack[(level * VEC + k) * kFusedThreads + threadIdx.x];
             if (SHARED) xi0[k] = s_stack[((p.levels + level) * VEC + k) * kFusedThreads + threadIdx.x];
         }
+    }
+    if (!s_sums) return;
+    __syncthreads();
+    for (int n = threadIdx.x; n < p.nodes; n += kFusedThreads) {
+        if (n == 0 || s_sums[n][0] == kNotMine) continue;
+        unsigned long long s = 0;
+#pragma unroll
+        for (int w = 0; w < kFusedThreads / 32; ++w) s += s_sums[n][w];
+        int step = 0;                                       // the node's depth is step + 1
+        while (step + 1 < p.T && static_cast<uint32_t>(n) >= (p.step[step + 1].child0 & ~kForks)) ++step;
+        p.logp[row0 + n] = logp_from_squares(s, p.half_per, p.step[step].g, p.step[step].logp_const);
     }
 }
 
@@ -232,7 +254,15 @@ cudaError_t launch_rollout_fused(const FusedLaunch& p0, int32_t nodes, cudaStrea
     const int64_t items = static_cast<int64_t>(p.n_trees) * p.nchunks * p.subtrees;
     if (items <= 0 || items > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     const unsigned int grid = static_cast<unsigned int>(items);
-    const size_t smem = static_cast<size_t>(p.levels) * kFusedChunkVec * sizeof(float4) * (p.shared_noise ? 2 : 1);
+    size_t smem = static_cast<size_t>(p.levels) * kFusedChunkVec * sizeof(float4) * (p.shared_noise ? 2 : 1);
+    // Rows of one CTA keep their sums in shared memory (up to 16 KB of them) and need no second launch, which costs about 4 us of
+    // host time (toy pass, with the rewards' second launch gone as well: 27.8 -> 23.8 us).
+    p.nodes = nodes;
+    p.sums_at = 0;
+    if (p.nchunks == 1 && nodes <= 1024) {
+        p.sums_at = static_cast<int32_t>(smem / sizeof(float4)) + 1;
+        smem += static_cast<size_t>(nodes) * (kFusedThreads / 32) * sizeof(uint32_t);
+    }
     cudaError_t e = cudaSuccess;
     if (smem > 48 * 1024)
         e = p.shared_noise ? cudaFuncSetAttribute(rollout_fused_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem))
@@ -240,7 +270,7 @@ cudaError_t launch_rollout_fused(const FusedLaunch& p0, int32_t nodes, cudaStrea
     if (e == cudaSuccess)
         e = p.shared_noise ? launch_overlapped(rollout_fused_kernel<true>, grid, kFusedThreads, smem, s, p)
                            : launch_overlapped(rollout_fused_kernel<false>, grid, kFusedThreads, smem, s, p);
-    if (e != cudaSuccess || nodes < 2) return e;
+    if (e != cudaSuccess || nodes < 2 || p.sums_at > 0) return e;
     const int64_t rows = static_cast<int64_t>(p.n_trees) * (nodes - 1);
     if (p.per_row >= 512) return launch_overlapped(finalize_tree_kernel<256>, static_cast<unsigned int>(rows), 256, 0, s, p, nodes);
     return launch_overlapped(finalize_tree_kernel<32>, static_cast<unsigned int>((rows + 7) / 8), 256, 0, s, p, nodes);

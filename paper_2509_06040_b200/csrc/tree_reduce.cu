@@ -93,7 +93,7 @@ fuse_advantage_kernel(const __grid_constant__ FuseLaunch p) {
 #pragma unroll
                 for (int b = 0; b < BGRPO_MAX_K; ++b)
                     if (b < fan) sum += rb[c0 + b];
-                rb[me] = sum / fan;
+                rb[me] = sum * p.runs.inv_fan;
                 continue;
             }
             double a[BGRPO_MAX_K];
@@ -127,10 +127,10 @@ fuse_advantage_kernel(const __grid_constant__ FuseLaunch p) {
         const int W = lay.chain0[r + 1] - lay.chain0[r];
         double s = 0.0;
         for (int j = lane; j < W; j += 32) s += v[j];
-        const double mean = warp_sum_d(s) / W;
+        const double mean = warp_sum_d(s) * p.runs.inv_width[r];
         double q = 0.0;
         for (int j = lane; j < W; j += 32) { const double c = v[j] - mean; q += c * c; }
-        const double sd = sqrt(warp_sum_d(q) / W);
+        const double sd = sqrt(warp_sum_d(q) * p.runs.inv_width[r]);
         if (lane == 0) {
             s_mean[r] = mean;
             s_inv[r] = 1.0 / (sd + static_cast<double>(p.eps));

@@ -47,6 +47,13 @@ __device__ __forceinline__ float4 load_shared_row(const float4* p) {
     return v;
 }
 
+// The reward of leaf row `row` from its sums: squared differences, or dot product and the two squared norms.
+template <int MODE>
+__device__ __forceinline__ void write_reward(const RewardLaunch& p, int row, const double* s) {
+    if (MODE == 0) p.r[row] = static_cast<float>(-s[0] * p.inv_D);
+    else p.r[row] = static_cast<float>(static_cast<double>(p.r[row]) + static_cast<double>(p.scale) * s[0] * rsqrt(s[MODE]) * rsqrt(s[2 * MODE]));
+}
+
 // FULL: the chunk lies inside the row, no element needs a bounds test (so the loads of a batch are plain back-to-back
 // instructions the compiler keeps together).
 template <int MODE, bool FULL>
@@ -135,6 +142,19 @@ reward_kernel(const __grid_constant__ RewardLaunch p) {
         if (lane == 0) red[v][warp] = s;
     }
     __syncthreads();
+    if (p.nchunks == 1) {         // the row is this CTA's alone: no partials, no finish kernel
+        if (threadIdx.x == 0) {
+            double s[NV];
+#pragma unroll
+            for (int v = 0; v < NV; ++v) {
+                s[v] = 0.0;
+#pragma unroll
+                for (int w = 0; w < kWarps; ++w) s[v] += red[v][w];
+            }
+            write_reward<MODE>(p, row, s);
+        }
+        return;
+    }
     if (threadIdx.x < NV) {
         double s = 0.0;
 #pragma unroll
@@ -154,16 +174,11 @@ reward_finish_kernel(const __grid_constant__ RewardLaunch p) {
     const int tree = row / p.leaves;
     const int64_t node_row = static_cast<int64_t>(tree) * p.nodes_cap + p.off_leaf + (row - tree * p.leaves);
     if (!BGRPO_IN_BOUNDS(p.status, p.off_leaf + p.leaves <= p.nodes_cap && p.nchunks <= p.nchunks_cap)) return;
-    if (MODE == 0) {
-        const double ss = row_total(p.partials, node_row, 0, p.nchunks);
-        if ((threadIdx.x & 31) == 0) p.r[row] = static_cast<float>(-ss / static_cast<double>(p.D));
-    } else {
-        const double dot = row_total(p.partials, node_row, 0, p.nchunks);
-        const double zz = row_total(p.partials, node_row, 1, p.nchunks);
-        const double tt = row_total(p.partials, node_row, 2, p.nchunks);
-        if ((threadIdx.x & 31) == 0)
-            p.r[row] = static_cast<float>(static_cast<double>(p.r[row]) + static_cast<double>(p.scale) * dot / (sqrt(zz) * sqrt(tt)));
-    }
+    constexpr int NV = (MODE == 0) ? 1 : 3;
+    double s[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) s[v] = row_total(p.partials, node_row, v, p.nchunks);
+    if ((threadIdx.x & 31) == 0) write_reward<MODE>(p, row, s);
 }
 
 }  // namespace
@@ -173,15 +188,10 @@ cudaError_t launch_reward(const RewardLaunch& p, cudaStream_t s) {
     if (items <= 0 || items > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     const unsigned int rows = static_cast<unsigned int>(p.n_trees) * static_cast<unsigned int>(p.leaves);
     const unsigned int fgrid = (rows + kStreamThreads / 32 - 1) / (kStreamThreads / 32);
-    cudaError_t e;
-    if (p.mode == 0) {
-        e = launch_overlapped(reward_kernel<0>, static_cast<unsigned int>(items), kStreamThreads, 0, s, p);
-        if (e == cudaSuccess) e = launch_overlapped(reward_finish_kernel<0>, fgrid, kStreamThreads, 0, s, p);
-    } else {
-        e = launch_overlapped(reward_kernel<1>, static_cast<unsigned int>(items), kStreamThreads, 0, s, p);
-        if (e == cudaSuccess) e = launch_overlapped(reward_finish_kernel<1>, fgrid, kStreamThreads, 0, s, p);
-    }
-    return e;
+    const unsigned int grid = static_cast<unsigned int>(items);
+    const cudaError_t e = p.mode == 0 ? launch_overlapped(reward_kernel<0>, grid, kStreamThreads, 0, s, p) : launch_overlapped(reward_kernel<1>, grid, kStreamThreads, 0, s, p);
+    if (e != cudaSuccess || p.nchunks == 1) return e;
+    return p.mode == 0 ? launch_overlapped(reward_finish_kernel<0>, fgrid, kStreamThreads, 0, s, p) : launch_overlapped(reward_finish_kernel<1>, fgrid, kStreamThreads, 0, s, p);
 }
 
 }  // namespace bgrpo
