@@ -4,11 +4,11 @@
 // K children of a parent share the result (the saving the rollout tree exists for).
 //
 // One persistent CTA per SM walks 128-token tiles.  For each tile the hidden dimension is cut into chunks of 128:
-//     GEMM1(c): D1[128 tok][128 hid]  = A[128 tok][64]      * W1_c        (4 MMAs of K = 16, accumulator in TMEM)
-//     GELU     : H_c = bf16(2 GELU(D1))  TMEM -> registers -> TMEM: the hidden activation never leaves tensor memory
+//     GEMM1(c): D1[128 tok][128 hid]  = A[128 tok][64]      * 2 W1_c      (4 MMAs of K = 16, accumulator in TMEM)
+//     GELU     : H_c = bf16(4 GELU(D1 / 2))  TMEM -> registers -> TMEM: the hidden activation never leaves tensor memory
 //     GEMM2(c): D2[128 tok][64]      += H_c[128 tok][128]   * W2_c        (8 MMAs of K = 16, A operand read from TMEM)
-// and the output tile is v = 0.5 D2 (the factor 1/2 of GELU is a power of two: taking it out of the 3072 activations
-// of a token and applying it to the 64 outputs changes no rounding).
+// and the output tile is v = D2 / 4 (the factors are powers of two: taking them out of the 3072 activations of a token and
+// applying them to the 64 outputs changes no rounding).
 // Tensor memory (512 columns): three chunk buffers of 128 columns and two output accumulators of 64.  A chunk buffer
 // holds D1 of its chunk and then, in place, the packed activations: a warp reads its 64 accumulator columns into
 // registers and later writes its 32 packed columns over the first half of exactly those columns, so no warp ever writes
@@ -37,6 +37,8 @@
 //
 // Every wait is bounded (about 2 s of SM clock): on a timeout the thread raises the abort flag, all roles drain, tensor memory is
 // released and bit 2 of the status word is set.
+#include <cuda_bf16.h>
+
 #include "internal.h"
 
 namespace bgrpo {
@@ -209,16 +211,19 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
     return r;
 }
-// Twice the GELU in its tanh form on the hardware tanh: x (1 + tanh(sqrt(2/pi) (x + 0.044715 x^3))).  The tanh form
-// differs from the erf form by < 5e-4 absolute, below the bf16 rounding of the activation that follows; bf16(2a) is
-// exactly 2 bf16(a), and the output tile takes the factor back.  One special-function instruction per activation: this
-// is the slow, range-free form, used only where the packed polynomial below does not apply.
-__device__ __forceinline__ float gelu_x2(float x) {
-    const float x2 = x * x;
+// The packed W1 is 2 W1, so the accumulator of GEMM1 is y = 2x, and the activation handed to GEMM2 is 4 GELU(x); the
+// output tile takes the factor back.  All of it is powers of two: no rounding changes.
+//
+// 4 GELU(y / 2) in the tanh form on the hardware tanh: 2x (1 + tanh(sqrt(2/pi) (x + 0.044715 x^3))).  The tanh form
+// differs from the erf form by < 5e-4 absolute, below the bf16 rounding of the activation that follows.  One
+// special-function instruction per activation: this is the slow, range-free form, used only where the packed polynomial
+// below does not apply.
+__device__ __forceinline__ float gelu_x4(float y) {
+    const float x = 0.5f * y, x2 = x * x;
     const float u = x * fmaf(x2, 0.0356774081f, 0.7978845608f);
     float th;
     asm("tanh.approx.f32 %0, %1;" : "=f"(th) : "f"(u));
-    return fmaf(x, th, x);
+    return fmaf(y, th, y);
 }
 // Packed bf16 arithmetic on two activations at a time (one FMA-pipe instruction for both halves).
 __device__ __forceinline__ uint32_t bf2_mul(uint32_t a, uint32_t b) {
@@ -231,28 +236,27 @@ __device__ __forceinline__ uint32_t bf2_fma(uint32_t a, uint32_t b, uint32_t c) 
     asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
     return d;
 }
-// Twice the erf-form GELU for |x| < 1 without a special-function instruction:
+// The erf-form GELU for |x| < 1 without a special-function instruction:
 //     2 GELU(x) = x + x erf(x / sqrt 2) = x + s Q(s),   s = x^2,
 // with Q a quadratic in s fitted to erf(x / sqrt 2) / x on [0, 1] (minimax in s Q(s), the coefficients rounded to bf16
 // one after the other and the rest refitted by csrc/gelu_poly_fit.py; the polynomial is within 8e-5 of the function).
+// In y = 2x it is 4 GELU(x) = y + t R(t) with t = y^2 and R's coefficients Q0 / 2, Q1 / 8, Q2 / 32, exact in bf16 too.
 // Evaluated on a packed pair in bf16: one multiply and three fused multiply-adds on the FMA pipe, where one hardware
 // tanh per activation (sixteen per clock and SM) bounds the whole stage at twice the tensor-core time.  The last
-// operation, fma(t, s, x), adds the small even part to x and rounds once, so for the usual |x| << 1 the result differs
-// from the correctly rounded activation by the rounding of x to bf16 and little else.
-constexpr uint32_t kGeluQ0 = 0x3f4c3f4cu;   //  0.796875
-constexpr uint32_t kGeluQ1 = 0xbe04be04u;   // -0.12890625
-constexpr uint32_t kGeluQ2 = 0x3c723c72u;   //  0.0147705078125
-constexpr uint32_t kGeluRangeBf16 = 0x3f80u;   // bf16 bits of 1.0: the polynomial's range
-__device__ __forceinline__ uint32_t gelu_x2_poly(uint32_t xb) {
-    const uint32_t s = bf2_mul(xb, xb);
-    uint32_t t = bf2_fma(kGeluQ2, s, kGeluQ1);
-    t = bf2_fma(t, s, kGeluQ0);
-    return bf2_fma(t, s, xb);
-}
-// Running maximum of magnitudes over packed pairs (the sign bits of the result carry no meaning).
-__device__ __forceinline__ uint32_t bf2_absmax(uint32_t m, uint32_t x) {
-    asm("max.xorsign.abs.bf16x2 %0, %0, %1;" : "+r"(m) : "r"(x));
-    return m;
+// operation adds the small even part to y and rounds once, so for the usual |x| << 1 the result differs from the
+// correctly rounded activation by the rounding of x to bf16 and little else.
+constexpr uint32_t kGeluR0 = 0x3ecc3eccu;   //  0.796875 / 2
+constexpr uint32_t kGeluR1 = 0xbc84bc84u;   // -0.12890625 / 8
+constexpr uint32_t kGeluR2 = 0x39f239f2u;   //  0.0147705078125 / 32
+// The polynomial's range |x| < 1 is |y| < 2: the top exponent bit of both bf16 halves clear.  One bit to look at is why y
+// is doubled: the check of 32 packed pairs is 16 three-operand ORs where a running maximum of magnitudes took 32
+// operations (1 036 800 tokens, hidden 3072: 733 -> 719 us).  NaN and infinity have the bit set.
+constexpr uint32_t kGeluOutside = 0x40004000u;
+__device__ __forceinline__ uint32_t gelu_x4_poly(uint32_t y) {
+    const uint32_t s = bf2_mul(y, y);
+    uint32_t t = bf2_fma(kGeluR2, s, kGeluR1);
+    t = bf2_fma(t, s, kGeluR0);
+    return bf2_fma(t, s, y);
 }
 // byte offset of the 16-byte piece `c16` of row r inside a 128-byte-swizzled tile of 128-byte rows
 __device__ __forceinline__ uint32_t sw128(uint32_t r, uint32_t c16) { return r * 128u + ((c16 ^ (r & 7u)) << 4); }
@@ -294,7 +298,9 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     // the swizzled operand tiles need 1024-byte alignment; the launch reserves 1 KiB of slack for this round-up
     MlpSmem& sm = *reinterpret_cast<MlpSmem*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // The shuffle tells the compiler that the warp index is the same in all lanes: roles, ring positions and tensor-memory
+    // addresses then live in uniform registers (1 036 800 tokens, hidden 3072: 775 -> 744 us; 7 200 tokens: 30.9 -> 29.3 us).
+    const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     volatile int* abort_flag = &sm.abort_flag;
 
     if (threadIdx.x == 0) {
@@ -511,7 +517,7 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p) {
             }
         }
 
-        // v = 0.5 D2 of tile t (this warp's 32 rows x 16 channels)
+        // v = D2 / 4 of tile t (this warp's 32 rows x 16 channels)
         auto output_tile = [&](int t) -> bool {
             const int b = t & 1;
             if (!__all_sync(0xffffffffu, mbar_wait(&sm.d2_full[b], static_cast<uint32_t>(t >> 1) & 1u, abort_flag) ? 1 : 0)) return false;
@@ -527,8 +533,8 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p) {
             float4 val[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j)
-                val[j] = make_float4(0.5f * __uint_as_float(out[4 * j]), 0.5f * __uint_as_float(out[4 * j + 1]),
-                                     0.5f * __uint_as_float(out[4 * j + 2]), 0.5f * __uint_as_float(out[4 * j + 3]));
+                val[j] = make_float4(0.25f * __uint_as_float(out[4 * j]), 0.25f * __uint_as_float(out[4 * j + 1]),
+                                     0.25f * __uint_as_float(out[4 * j + 2]), 0.25f * __uint_as_float(out[4 * j + 3]));
             if (S > 1) {
                 // This CTA holds the sum over its share of the hidden dimension only.  Every part stores its tile; the
                 // part that draws the last ticket adds them up in part order (the host gives such a CTA one tile).
@@ -595,25 +601,24 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p) {
         // 32 accumulator columns -> 16 registers of packed bf16 activation pairs
         // One chunk of this warp: 64 accumulator columns arrive as float32, are rounded to packed bf16 pairs at once (32
         // registers) and D1 is handed back before any arithmetic, so GEMM1 of chunk g + 2 runs under the activation of
-        // chunk g.  The packed polynomial covers |x| < 1; a running maximum of magnitudes shows whether any of this
-        // thread's 64 values lies outside (or is not finite), and only then the thread takes the hardware-tanh form
-        // for its values.  With weights and latents of the usual scale (pre-activations of standard deviation ~0.2) that
+        // chunk g.  The packed polynomial covers |x| < 1; one bit of the packed pairs shows whether any of this thread's
+        // 64 values lies outside (or is not finite), and only then the thread takes the hardware-tanh form for its values.  With weights and latents of the usual scale (pre-activations of standard deviation ~0.2) that
         // never happens.
         auto pack16 = [&](const uint32_t (&acc)[32], uint32_t* xb) {
 #pragma unroll
             for (int m = 0; m < 16; ++m) xb[m] = pack_bf16(__uint_as_float(acc[2 * m]), __uint_as_float(acc[2 * m + 1]));
         };
         auto activate = [&](uint32_t (&xb)[32]) {
-            uint32_t big = 0u;
+            uint32_t bits = 0u;
 #pragma unroll
-            for (int m = 0; m < 32; ++m) big = bf2_absmax(big, xb[m]);
-            if ((big & 0x7fffu) < kGeluRangeBf16 && ((big >> 16) & 0x7fffu) < kGeluRangeBf16) {
+            for (int m = 0; m < 32; m += 2) bits |= xb[m] | xb[m + 1];
+            if ((bits & kGeluOutside) == 0u) {
 #pragma unroll
-                for (int m = 0; m < 32; ++m) xb[m] = gelu_x2_poly(xb[m]);
+                for (int m = 0; m < 32; ++m) xb[m] = gelu_x4_poly(xb[m]);
             } else {
 #pragma unroll
                 for (int m = 0; m < 32; ++m)
-                    xb[m] = pack_bf16(gelu_x2(__uint_as_float(xb[m] << 16)), gelu_x2(__uint_as_float(xb[m] & 0xffff0000u)));
+                    xb[m] = pack_bf16(gelu_x4(__uint_as_float(xb[m] << 16)), gelu_x4(__uint_as_float(xb[m] & 0xffff0000u)));
             }
         };
         const uint32_t my_cols = tmem + lane_addr + (sub & 1u) * 64u;     // this warp's 64 columns inside a chunk buffer
@@ -661,7 +666,7 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p) {
 }
 
 // Reorders W1 [64][H] and W2 [H][64] (bf16 bits) into per-chunk shared-memory images: for chunk c,
-//   bytes [0, 16 KiB):      W1_c as [128 n = hidden][64 k = channel], 128-byte rows, 128-byte swizzle
+//   bytes [0, 16 KiB):      2 W1_c as [128 n = hidden][64 k = channel], 128-byte rows, 128-byte swizzle
 //   bytes [16 KiB, 32 KiB): W2_c as two tiles [64 n = channel][64 k = hidden], one per half of the chunk's hidden range
 __global__ void mlp_pack_kernel(const uint16_t* __restrict__ W1, const uint16_t* __restrict__ W2, int hidden, unsigned char* __restrict__ packed) {
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;      // one bf16 element of W1 and one of W2 per thread
@@ -670,7 +675,8 @@ __global__ void mlp_pack_kernel(const uint16_t* __restrict__ W1, const uint16_t*
         const int k = idx / hidden, j = idx - k * hidden;
         const int c = j / kHc, n = j - c * kHc;
         const uint32_t off = static_cast<uint32_t>(n) * 128u + (((static_cast<uint32_t>(k) >> 3) ^ (static_cast<uint32_t>(n) & 7u)) << 4) + (static_cast<uint32_t>(k) & 7u) * 2u;
-        *reinterpret_cast<uint16_t*>(packed + static_cast<size_t>(c) * kChunkBytes + off) = W1[idx];
+        *reinterpret_cast<uint16_t*>(packed + static_cast<size_t>(c) * kChunkBytes + off) =
+            __bfloat16_as_ushort(__float2bfloat16(2.f * __bfloat162float(__ushort_as_bfloat16(W1[idx]))));
     }
     {   // W2[j][n]
         const int j = idx / kCh, n = idx - j * kCh;
