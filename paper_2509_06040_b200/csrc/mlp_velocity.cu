@@ -262,9 +262,14 @@ __device__ __forceinline__ uint32_t gelu_x4_poly(uint32_t y) {
 __device__ __forceinline__ uint32_t sw128(uint32_t r, uint32_t c16) { return r * 128u + ((c16 ^ (r & 7u)) << 4); }
 
 // Converts rows [r_begin, r_end) of the float32 staging tile to the bf16 K-major swizzled A tile; one warp, two rows per
-// step (16 lanes x 16 bytes cover a row).
-__device__ __forceinline__ void convert_rows(const float* stage, unsigned char* atile, int r_begin, int r_end, int lane) {
+// step (16 lanes x 16 bytes cover a row).  Rows from `valid` on lie past the last token and are made zero first: left to
+// what the staging buffer held before, a few NaNs sent the rows of a ragged last tile through the slow activation, and
+// with one tile per CTA that CTA took twice as long as all others (16 200 tokens, hidden 3072: 31 us in place of 16).
+__device__ __forceinline__ void convert_rows(float* stage, unsigned char* atile, int r_begin, int r_end, int valid, int lane) {
     const uint32_t c4 = static_cast<uint32_t>(lane & 15);
+    if (valid < r_end)        // at most once in a launch
+        for (int r = r_begin + (lane >> 4); r < r_end; r += 2)
+            if (r >= valid) *reinterpret_cast<float4*>(stage + r * kCh + c4 * 4u) = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 8
     for (int r0 = r_begin; r0 < r_end; r0 += 2) {
         const uint32_t r = static_cast<uint32_t>(r0 + (lane >> 4));
@@ -348,6 +353,11 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p) {
     const int n_my_tiles = (p.n_tiles > cta) ? (p.n_tiles - 1 - cta) / n_ctas + 1 : 0;
     const int NC = p.n_chunks / S;            // chunks this CTA adds up per tile: part * NC .. part * NC + NC - 1
     const int n_my_chunks = n_my_tiles * NC;
+
+    auto tile_rows = [&](int it) -> int {     // tokens of this CTA's tile number `it`
+        const int64_t left = p.n_tokens - (static_cast<int64_t>(cta) + static_cast<int64_t>(it) * n_ctas) * kTok;
+        return left < kTok ? static_cast<int>(left) : kTok;
+    };
 
     if (warp == 0) {
         // ---------------------------------------------------------------- weight producers (lane 0: W1, lane 1: W2)
@@ -451,12 +461,10 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p) {
     } else if (warp == kLoaderWarp) {
         // ---------------------------------------------------------------- latent tile -> staging -> bf16, K-major swizzled
         // Tokens of the frontier are numbered tree by tree; the rows of one tree are contiguous in the pool, so a tile is
-        // one copy per tree it touches.  Rows past the last token keep whatever the staging buffer held: a row of A
-        // only feeds the same row of the output, which is not written.
+        // one copy per tree it touches.
         auto issue_tile_copy = [&](int it) {       // one lane
             const int64_t tok0 = (static_cast<int64_t>(cta) + static_cast<int64_t>(it) * n_ctas) * kTok;
-            int64_t remaining = p.n_tokens - tok0;
-            if (remaining > kTok) remaining = kTok;
+            int64_t remaining = tile_rows(it);
             mbar_expect_tx(&sm.stage_full, static_cast<uint32_t>(remaining) * (kCh * 4u));
             int64_t q = tok0;
             float* dst = sm.stage;
@@ -488,7 +496,7 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p) {
                 if (ok && it >= 2) ok = mbar_wait(&sm.a_empty[ab], static_cast<uint32_t>((it >> 1) - 1) & 1u, abort_flag);
                 ok = __all_sync(0xffffffffu, ok ? 1 : 0) != 0;
                 if (!ok) break;
-                convert_rows(sm.stage, sm.a[ab], 0, kTok, lane);
+                convert_rows(sm.stage, sm.a[ab], 0, kTok, tile_rows(it), lane);
                 proxy_fence();
             }
             __syncwarp();
@@ -510,7 +518,7 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p) {
         if (n_my_tiles > 0) {         // this warp's eight rows of the first A tile (see the loader warp)
             ok = __all_sync(0xffffffffu, mbar_wait(&sm.stage_full, 0u, abort_flag) ? 1 : 0) != 0;
             if (ok) {
-                convert_rows(sm.stage, sm.a[0], ew * (kTok / kEpiWarps), (ew + 1) * (kTok / kEpiWarps), lane);
+                convert_rows(sm.stage, sm.a[0], ew * (kTok / kEpiWarps), (ew + 1) * (kTok / kEpiWarps), tile_rows(0), lane);
                 proxy_fence();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&sm.first_a);
