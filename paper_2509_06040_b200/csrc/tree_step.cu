@@ -16,17 +16,21 @@ __global__ void __launch_bounds__(kStreamThreads)
 root_kernel(float* latents, int32_t* table, float* logp, unsigned int* counters, int32_t* status, int64_t D,
             int32_t n_trees, int32_t nodes_cap, int32_t nchunks, uint32_t node_id_base, const __grid_constant__ PhiloxKeys keys) {
     pdl_release();
-    pdl_wait();           // the buffers may still be read by the kernels of the previous pass
     const int chunk = blockIdx.x % nchunks;
     const int tree = blockIdx.x / nchunks;
     const int64_t D4 = D >> 2;
     if (!BGRPO_IN_BOUNDS(status, tree < n_trees && static_cast<int64_t>(chunk) * kChunkVec < D4)) return;
     float4* z = reinterpret_cast<float4*>(latents + static_cast<int64_t>(tree) * nodes_cap * D);
     const uint32_t gid = node_id_base + static_cast<uint32_t>(tree) * nodes_cap;
+    float4 noise[kVecPerThread];
+#pragma unroll
+    for (int k = 0; k < kVecPerThread; ++k)
+        noise[k] = noise4(static_cast<uint32_t>(chunk) * kChunkVec + k * kStreamThreads + threadIdx.x, gid, 0u, BGRPO_TAG_ROOT, keys);
+    pdl_wait();           // the buffers may still be read by the kernels of the previous pass
 #pragma unroll
     for (int k = 0; k < kVecPerThread; ++k) {
         const int64_t e = static_cast<int64_t>(chunk) * kChunkVec + k * kStreamThreads + threadIdx.x;
-        if (e < D4) z[e] = noise4(static_cast<uint32_t>(e), gid, 0u, BGRPO_TAG_ROOT, keys);
+        if (e < D4) z[e] = noise[k];
     }
     const int64_t rows = static_cast<int64_t>(n_trees) * nodes_cap;
     if (chunk == 0) {
@@ -44,7 +48,8 @@ root_kernel(float* latents, int32_t* table, float* logp, unsigned int* counters,
 }
 
 // ---------------------------------------------------------------------------------------------------------------
-// Fused step.  One CTA of kStepThreads threads per work item (tree, parent, chunk of kStepChunkVec float4).
+// Fused step.  One CTA per work item (tree, parent, chunk of kStepChunkVec float4): kStepThreads threads of kStepVec float4,
+// or kStepThreadsSmall threads of a quarter of that where the launch is less than one wave (step_threads()).
 //
 // A thread issues the 128-bit loads of its kStepVec float4 of the parent tile and of the operand tile (velocity or
 // target mean) first, then generates the noise of all its elements - Philox and Box-Muller depend on indices only,
@@ -93,41 +98,53 @@ __device__ __forceinline__ void load_tile(const float4* __restrict__ zp, const f
     }
 }
 
+// The noise of a parent's children for one float4 of elements; adds its squares.
+template <int FAN, bool SHARED>
+struct StepNoise {
+    NoiseNode shared_node, node[FAN];
+    __device__ __forceinline__ StepNoise(const StepLaunch& p, uint32_t gid_parent, uint32_t gid_child0) {
+        if (SHARED) shared_node = noise_node(gid_parent, p.step, p.keys);
+#pragma unroll
+        for (int b = 0; b < FAN; ++b) node[b] = noise_node(gid_child0 + b, p.step, p.keys);
+    }
+    __device__ __forceinline__ void draw(const StepLaunch& p, uint32_t e, float4 (&xi)[FAN], uint32_t (&acc)[FAN]) const {
+        float squares;
+        float4 xi0;
+        if (SHARED) xi0 = mul4(p.mix_shared, normal4(philox_from(noise_element(e, BGRPO_TAG_SHARED, p.keys), shared_node, p.keys), squares));
+        const NoiseElement el = noise_element(e, BGRPO_TAG_INNOV, p.keys);
+#pragma unroll
+        for (int b = 0; b < FAN; ++b) {
+            xi[b] = normal4(philox_from(el, node[b], p.keys), squares);
+            if (SHARED) {
+                xi[b] = fma4(p.mix_innov, xi[b], xi0);
+                squares = squares_of(xi[b]);
+            }
+            // z' - mean is g xi up to the rounding of z' (relative 6e-8 of |z'|, far below the 1e-5 the log-prob
+            // is good to)
+            acc[b] += quantized_squares(squares);
+        }
+    }
+};
+
+template <int FAN, bool NOISY>
+__device__ __forceinline__ void store_children(const StepLaunch& p, float4 z, float4 x, const float4 (&xi)[FAN], float4* zc, uint32_t D4) {
+    const float4 m = fma4(p.ca, z, mul4(p.cb, x));
+#pragma unroll
+    for (int b = 0; b < FAN; ++b)       // deterministic step: the child is the mean
+        zc[static_cast<size_t>(b) * D4] = NOISY ? fma4(p.g, xi[b], m) : m;
+}
+
 template <int FAN, bool SHARED, int THREADS, bool FULL, bool NOISY>
 __device__ __forceinline__ void compute_tile(const StepLaunch& p, const float4 (&z)[kStepChunkVec / THREADS], const float4 (&x)[kStepChunkVec / THREADS],
-                                             uint32_t vecs, uint32_t e_base, uint32_t D4, float4* zc, uint32_t gid_parent,
-                                             uint32_t gid_child0, uint32_t (&acc)[FAN]) {
-    NoiseNode shared_node, node[FAN];
-    if (SHARED) shared_node = noise_node(gid_parent, p.step, p.keys);
-#pragma unroll
-    for (int b = 0; b < FAN; ++b) node[b] = noise_node(gid_child0 + b, p.step, p.keys);
+                                             uint32_t vecs, uint32_t e_base, uint32_t D4, float4* zc, const StepNoise<FAN, SHARED>& noise,
+                                             uint32_t (&acc)[FAN]) {
 #pragma unroll
     for (int k = 0; k < kStepChunkVec / THREADS; ++k) {
         const uint32_t t = threadIdx.x + k * THREADS;
         if (FULL || t < vecs) {
-            const uint32_t e = e_base + t;
             float4 xi[FAN];
-            if (NOISY) {
-                float squares;
-                float4 xi0;
-                if (SHARED) xi0 = mul4(p.mix_shared, normal4(philox_from(noise_element(e, BGRPO_TAG_SHARED, p.keys), shared_node, p.keys), squares));
-                const NoiseElement el = noise_element(e, BGRPO_TAG_INNOV, p.keys);
-#pragma unroll
-                for (int b = 0; b < FAN; ++b) {
-                    xi[b] = normal4(philox_from(el, node[b], p.keys), squares);
-                    if (SHARED) {
-                        xi[b] = fma4(p.mix_innov, xi[b], xi0);
-                        squares = squares_of(xi[b]);
-                    }
-                    // z' - mean is g xi up to the rounding of z' (relative 6e-8 of |z'|, far below the 1e-5 the log-prob
-                    // is good to)
-                    acc[b] += quantized_squares(squares);
-                }
-            }
-            const float4 m = fma4(p.ca, z[k], mul4(p.cb, x[k]));
-#pragma unroll
-            for (int b = 0; b < FAN; ++b)       // deterministic step: the child is the mean
-                zc[static_cast<size_t>(b) * D4 + e] = NOISY ? fma4(p.g, xi[b], m) : m;
+            if (NOISY) noise.draw(p, e_base + t, xi, acc);
+            store_children<FAN, NOISY>(p, z[k], x[k], xi, zc + e_base + t, D4);
         }
     }
 }
@@ -138,10 +155,17 @@ step_kernel(const __grid_constant__ StepLaunch p) {
     constexpr int kWarps = THREADS / 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     pdl_release();
-    pdl_wait();           // the parents, the velocity and the pending partial sums come from earlier kernels
-    // the previous level's log-probs (a handful of rows): summed by this launch
-    if (p.prev.logp_out != nullptr)
-        finalize_rows(p.prev, p.partials, p.n_trees, p.nodes_cap, p.half_per, blockIdx.x * kWarps + warp, gridDim.x * kWarps, p.status, p.per_row);
+    // the previous level's log-probs (a handful of rows) are summed by this launch
+    auto finalize_previous = [&] {
+        if (p.prev.logp_out != nullptr)
+            finalize_rows(p.prev, p.partials, p.n_trees, p.nodes_cap, p.half_per, blockIdx.x * kWarps + warp, gridDim.x * kWarps, p.status, p.per_row);
+    };
+    // The parents, the velocity and the pending partial sums come from earlier kernels.  A launch of many waves waits for
+    // them here: its loads travel while the noise is generated.
+    if (THREADS == kStepThreads) {
+        pdl_wait();
+        finalize_previous();
+    }
 
     const int chunk = blockIdx.x % p.nchunks;
     const int row = blockIdx.x / p.nchunks;             // tree * W_in + j
@@ -167,12 +191,31 @@ step_kernel(const __grid_constant__ StepLaunch p) {
 #pragma unroll
     for (int b = 0; b < FAN; ++b) acc[b] = 0u;
     float4 z[kStepChunkVec / THREADS], x[kStepChunkVec / THREADS];
-    if (vecs == kStepChunkVec) {
+    const StepNoise<FAN, SHARED> noise(p, gid_parent, gid_child0);
+    if (THREADS == kStepThreadsSmall) {
+        // A launch of less than a wave sits through the end of the kernel before it: the noise, which needs nothing but
+        // indices, is drawn before the wait, and what is left behind it is a load, a few FMAs and a store (16 steps of one
+        // tree of 256 tokens, each after the MLP stage: 249 -> 235 us for the pass).
+        float4 xi[kStepChunkVec / THREADS][FAN];
+        if (NOISY) {
+#pragma unroll
+            for (int k = 0; k < kStepChunkVec / THREADS; ++k)
+                if (threadIdx.x + k * THREADS < vecs) noise.draw(p, e_base + threadIdx.x + k * THREADS, xi[k], acc);
+        }
+        pdl_wait();
+        load_tile<THREADS, false>(zp, xop, streamed, vecs, z, x);
+        finalize_previous();
+#pragma unroll
+        for (int k = 0; k < kStepChunkVec / THREADS; ++k) {
+            const uint32_t t = threadIdx.x + k * THREADS;
+            if (t < vecs) store_children<FAN, NOISY>(p, z[k], x[k], xi[k], zc + e_base + t, D4);
+        }
+    } else if (vecs == kStepChunkVec) {
         load_tile<THREADS, true>(zp, xop, streamed, vecs, z, x);
-        compute_tile<FAN, SHARED, THREADS, true, NOISY>(p, z, x, vecs, e_base, D4, zc, gid_parent, gid_child0, acc);
+        compute_tile<FAN, SHARED, THREADS, true, NOISY>(p, z, x, vecs, e_base, D4, zc, noise, acc);
     } else {
         load_tile<THREADS, false>(zp, xop, streamed, vecs, z, x);
-        compute_tile<FAN, SHARED, THREADS, false, NOISY>(p, z, x, vecs, e_base, D4, zc, gid_parent, gid_child0, acc);
+        compute_tile<FAN, SHARED, THREADS, false, NOISY>(p, z, x, vecs, e_base, D4, zc, noise, acc);
     }
     // one number per (child row, chunk, warp): a lane's sum takes up to 31 bits, so its halves are added apart
 #pragma unroll

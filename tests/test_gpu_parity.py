@@ -843,3 +843,62 @@ def test_logprob_families_at_their_edges(B, tokens, channels, n_trees, T, K, spl
             assert bool((got == 7.0).all())                 # only the addressed edges were written
     assert bool((every[:, 0] == 7.0).all())
     B.tree_sync_status(s.tree)
+
+
+@pytest.mark.parametrize("tokens,channels,n_trees,T,K,splits,s", [
+    (9, 4, 591, 2, 1, (), math.inf),              # step launches of 591, 592, 593 CTAs: the wide ones and the narrow ones
+    (9, 4, 592, 2, 1, (), math.inf),
+    (9, 4, 593, 2, 1, (), math.inf),
+    (513, 4, 295, 2, 1, (), math.inf),            # the same with a second chunk of one float4 (two-CTA rows in the whole-tree launch)
+    (513, 4, 296, 2, 1, (), math.inf),
+    (512, 4, 147, 3, 4, (0,), 2.0),               # a full chunk, four children, shared noise; 588 and 592 CTAs in the steps after the fork
+    (512, 4, 148, 3, 4, (0,), 2.0),
+    (1, 4, 3, 4, 3, (0, 2), 1.0),                 # one float4 a row; every fork dealt out to the grid
+    (9, 4, 1, 20, 2, (0, 1, 2, 3, 4, 5), math.inf),   # 1023 nodes: the rows' sums stay in shared memory
+    (9, 4, 1, 21, 2, (0, 1, 2, 3, 4, 5), math.inf),   # 1087 nodes: they do not
+    (9, 4, 450, 6, 2, (0, 1, 2, 3, 4, 5), 2.0),   # no fork dealt out: six open forks with their shared noise in shared memory
+])
+def test_step_and_whole_tree_launches_agree_where_their_shapes_change(B, tokens, channels, n_trees, T, K, splits, s):
+    """The two rollouts share the noise stream, the float32 expressions and the integer sums, and nothing of their launch
+    shapes: latents, log-probs and tables are bit-equal.  (Both are compared with the oracle above.)"""
+    w = Workload(name="shapes", n_trees=n_trees, tokens=tokens, channels=channels, T=T, K=K, splits=splits, sigma=0.3,
+                 velocity="linear", reward="neg_mse_mu", branch_corr_s=s)
+    inp = make_inputs(w)
+    runs = []
+    for fused in (False, True):
+        r = _session(w, fused_rollout=fused)
+        r.upload_inputs(inp)
+        r.logp.fill_(7.0)
+        if fused:
+            r.rollout()
+        else:
+            r.init()
+            for i in range(T):
+                r.step(i)
+        B.tree_sync_status(r.tree)
+        runs.append(r)
+    step, whole = runs
+    assert torch.equal(step.latents, whole.latents)
+    assert torch.equal(step.logp, whole.logp)
+    assert torch.equal(step.node_table, whole.node_table)
+
+
+@pytest.mark.parametrize("tokens,channels", [(1, 4), (4096, 4), (4097, 4), (8193, 4)])      # rows of one, one, two and three chunks
+def test_leaf_rewards_where_a_row_outgrows_its_cta(B, tokens, channels):
+    w = Workload(name="rw", n_trees=2, tokens=tokens, channels=channels, T=2, K=2, splits=(0,), sigma=0.3,
+                 velocity="linear", reward="normal_plus_cos")
+    inp = make_inputs(w)
+    s = _session(w)
+    s.upload_inputs(inp)
+    s.rollout()
+    leaf = s.latents[:, -w.leaves:].double()
+    target = s.target.double().view(2, 1, w.D)
+    cos = (leaf * target).sum(-1) / (leaf.norm(dim=-1) * target.norm(dim=-1))
+    refs = (torch.from_numpy(inp.reward_draws).cuda().double() + 0.1 * cos, -((leaf - target) ** 2).mean(-1))
+    for _ in range(2):
+        s.rewards()
+        got = [s.leaf_r.clone()]
+        B.leaf_reward_mse(s.tree, s.target, s.leaf_r)
+        got.append(s.leaf_r.clone())
+        for g, ref in zip(got, refs):         # sums in float64, one rounding to float32
+            assert bool(((g.double() - ref).abs() <= 1e-6 * ref.abs().clamp(min=1.0)).all())
