@@ -150,8 +150,6 @@ struct bgrpo_tree {
                                          // is too large for one CTA's shared memory
     void* partials_logp;                 // [n_trees*nodes_cap][partials_per_row] 32-bit words: log-prob sums, each kernel's own layout
     unsigned long long* partials_u64() const { return static_cast<unsigned long long*>(partials_logp); }
-    unsigned int* mlp_tickets;           // 64-channel trees only: scratch of the MLP stage's split over the hidden dimension
-    float* mlp_partials;
     bgrpo::FinalizeDesc pending;         // level whose log-probs still have to be summed
 };
 
@@ -175,18 +173,25 @@ namespace bgrpo {
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <typename... Params, typename... Args>
-cudaError_t launch_overlapped(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args&&... args) {
+cudaError_t launch_overlapped_clusters(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, int cluster, Args&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = static_cast<unsigned int>(cluster);
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+template <typename... Params, typename... Args>
+cudaError_t launch_overlapped(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args&&... args) {
+    return launch_overlapped_clusters(kernel, grid, block, smem, s, 1, std::forward<Args>(args)...);
 }
 #endif
 
@@ -319,16 +324,10 @@ struct ObjectiveLaunch {
 cudaError_t launch_objective(const ObjectiveLaunch& p, cudaStream_t s);
 
 // ---- MLP velocity (mlp_velocity.cu) -----------------------------------------------------------------------------
-// Frontiers of fewer tiles than SMs are also cut along the hidden dimension; the partial output tiles (128 tokens x 64
-// channels, float) of at most this many CTAs and one ticket counter per tile live in the tree's scratch.
-constexpr int kMlpSplitMaxCtas = 192;
-constexpr size_t kMlpPartialBytes = static_cast<size_t>(kMlpSplitMaxCtas) * 128 * 64 * sizeof(float);
-constexpr size_t kMlpTicketBytes = 1024;      // kMlpSplitMaxCtas counters, rounded up
 size_t mlp_packed_bytes(int hidden);
 cudaError_t launch_mlp_pack(const uint16_t* W1, const uint16_t* W2, int hidden, void* packed, cudaStream_t s);
 cudaError_t launch_debug_trip(int32_t* status, cudaStream_t s);     // debug build: fails one index test on purpose (no access involved)
 cudaError_t launch_mlp(const float* latents, int64_t pool_elems, int64_t tree_stride, int64_t row_offset, int n_trees, int64_t tokens_per_tree,
-                       const void* packed, int hidden, float* v_out, float* split_partials, unsigned int* split_tickets,
-                       int32_t* status, cudaStream_t s);
+                       const void* packed, int hidden, float* v_out, int32_t* status, cudaStream_t s);
 
 }  // namespace bgrpo

@@ -31,9 +31,9 @@
 // address; the weights are reordered once into exactly that image (bgrpo_velocity_mlp_pack), so a chunk arrives with
 // one copy per matrix.  No cluster multicast is used anywhere.
 //
-// Small frontiers (fewer tiles than SMs) are cut along the hidden dimension as well: S = 2, 4 or 8 CTAs share a tile, each
-// takes 1/S of the chunks and writes its partial output tile to scratch; the CTA that draws the tile's last ticket adds the
-// S partials in part order and writes v, so the result does not depend on which CTA finishes first.
+// Small frontiers (fewer tiles than SMs) are cut along the hidden dimension as well: a cluster of S = 2 to 8 CTAs shares
+// a tile, each takes 1/S of the chunks and leaves its partial output tile in its shared memory; then each adds 1/S of the
+// rows over all S parts, in part order, and writes them to v.
 //
 // Every wait is bounded (about 2 s of SM clock): on a timeout the thread raises the abort flag, all roles drain, tensor memory is
 // released and bit 2 of the status word is set.
@@ -49,6 +49,7 @@ constexpr int kCh = 64;                   // channels = K of GEMM1 = N of GEMM2
 constexpr int kHc = 128;                  // hidden chunk = N of GEMM1 = K of GEMM2
 constexpr int kW1Stages = 3;               // W1 slot q is free again when the GEMM1 that read it has completed
 constexpr int kW2Stages = 4;               // W2 slot q is free again when the GEMM2 that read it has completed
+constexpr int kMaxSplit = 8;               // CTAs of a cluster that share a tile
 constexpr int kEpiWarps = 16;             // two groups of eight: two warps per TMEM lane quarter, 64 columns of a chunk each
 constexpr int kLoaderWarp = 2 + kEpiWarps;
 constexpr int kGemm2Warp = 3 + kEpiWarps;
@@ -65,11 +66,10 @@ struct MlpSmem {
     alignas(1024) unsigned char w1[kW1Stages][kTileBytes];  // W1_c tile [128 n = hidden][128 B = 64 channels]
     alignas(1024) unsigned char w2[kW2Stages][kTileBytes];  // W2_c as two [64 n = channel][128 B = 64 hidden] tiles
     alignas(1024) unsigned char a[2][kTileBytes];           // bf16(z) tile [128 tok][128 B], double-buffered over tiles
-    alignas(1024) float stage[kTok * kCh];                   // float32 latents of the next tile, as they are in global memory
+    alignas(1024) float stage[kTok * kCh];                   // float32 latents of the next tile, as they are in global memory; split
+                                                             // mode, at the end: this CTA's partial output tile
     unsigned long long w1_full[kW1Stages], w1_free[kW1Stages], w2_full[kW2Stages], w2_free[kW2Stages];
     unsigned long long stage_full, first_a, a_full[2], a_empty[2], d1_full[kBufs], h_full[kBufs], buf_free[kBufs], d2_full[2], d2_empty[2];
-    unsigned long long part_done, part_verdict;   // split mode: all epilogue warps have stored their partials / the ticket is drawn
-    int is_last_part;
     uint32_t tmem_base;
     int abort_flag;
 };
@@ -281,6 +281,22 @@ __device__ __forceinline__ void convert_rows(float* stage, unsigned char* atile,
     }
 }
 
+// Thread-block cluster: barrier over all threads of its CTAs (release / acquire), load from another CTA's shared memory.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ float4 cluster_load(uint32_t addr, uint32_t rank) {
+    uint32_t remote;
+    float4 v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(rank));
+    asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(remote) : "memory");
+    return v;
+}
+// 16-byte piece c4 of row r of a partial output tile; rows are staggered so that a warp's row-per-thread stores and its
+// row-by-row loads both spread over the banks
+__device__ __forceinline__ float4* part_piece(float* tile, uint32_t r, uint32_t c4) {
+    return reinterpret_cast<float4*>(tile) + r * (kCh / 4) + (c4 ^ (r & (kCh / 4 - 1)));
+}
+
 struct MlpArgs {
     const float* latents;     // pool base
     int64_t pool_elems;       // elements in the pool
@@ -292,9 +308,7 @@ struct MlpArgs {
     float* v_out;
     int32_t n_chunks;         // hidden / 128
     int32_t n_tiles;
-    int32_t split;            // CTAs per tile along the hidden dimension (1: none); > 1 only with one tile per CTA group
-    float* partials;          // split > 1: [n_tiles][split][128][64] partial output tiles
-    unsigned int* tickets;    // split > 1: one counter per tile, zero before and after the launch
+    int32_t split;            // CTAs per tile along the hidden dimension (1: none); > 1 only with one tile per cluster of that size
     int32_t* status;
 };
 
@@ -319,8 +333,6 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p) {
         }
         mbar_init(&sm.stage_full, 1);
         mbar_init(&sm.first_a, kEpiWarps);
-        mbar_init(&sm.part_done, kEpiWarps);
-        mbar_init(&sm.part_verdict, 1);
         for (int q = 0; q < 2; ++q) {
             mbar_init(&sm.a_full[q], 1);
             mbar_init(&sm.a_empty[q], 1);
@@ -544,59 +556,9 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p) {
                 val[j] = make_float4(0.25f * __uint_as_float(out[4 * j]), 0.25f * __uint_as_float(out[4 * j + 1]),
                                      0.25f * __uint_as_float(out[4 * j + 2]), 0.25f * __uint_as_float(out[4 * j + 3]));
             if (S > 1) {
-                // This CTA holds the sum over its share of the hidden dimension only.  Every part stores its tile; the
-                // part that draws the last ticket adds them up in part order (the host gives such a CTA one tile).
-                float4* mine = reinterpret_cast<float4*>(p.partials + ((tile * S + part) * kTok + row) * kCh + sub * 16u);
+                // This CTA holds the sum over its share of the hidden dimension only; the tail of the kernel adds the parts.
 #pragma unroll
-                for (int j = 0; j < 4; ++j) __stcg(mine + j, val[j]);
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&sm.part_done);      // release at CTA scope; the ticket thread's fence carries it further
-                if (ew == 0) {
-                    const bool all_in = __all_sync(0xffffffffu, mbar_wait(&sm.part_done, 0u, abort_flag) ? 1 : 0) != 0;
-                    if (lane == 0) {
-                        int last = 0;
-                        if (all_in) {
-                            __threadfence();           // every warp's partial stores (seen through part_done) before the ticket
-                            const unsigned int ticket = atomicAdd(&p.tickets[tile], 1u);
-                            last = ticket == static_cast<unsigned int>(S) - 1u;
-                            if (last) p.tickets[tile] = 0u;            // every part has arrived: ready for the next launch
-                        }
-                        sm.is_last_part = last;
-                        __threadfence();
-                        mbar_arrive(&sm.part_verdict);
-                    }
-                }
-                if (!__all_sync(0xffffffffu, mbar_wait(&sm.part_verdict, 0u, abort_flag) ? 1 : 0)) return false;
-                if (!*reinterpret_cast<volatile int*>(&sm.is_last_part)) return true;
-                // The tile as 2048 float4, each warp on consecutive addresses: S partial tiles in, one output tile out.
-                // (With the row-per-thread mapping of the accumulator every load touched 32 lines and the sum took 10 us.)
-                const float4* parts = reinterpret_cast<const float4*>(p.partials) + tile * S * (kTok * kCh / 4);
-                float4* vt = reinterpret_cast<float4*>(p.v_out) + tile * (kTok * kCh / 4);
-                const int64_t rows_left = p.n_tokens - tile * kTok;
-                constexpr int kPer = (kTok * kCh / 4) / (kEpiWarps * 32);      // float4 per thread: 4
-                constexpr int64_t kTile4 = kTok * kCh / 4;
-                float4 sum[kPer];
-#pragma unroll
-                for (int i = 0; i < kPer; ++i) sum[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-                const int idx0 = ew * 32 + lane;
-                for (int o = 0; o < S; o += 2) {       // S is even: parts added in order, eight loads in flight
-                    float4 x[2][kPer];
-#pragma unroll
-                    for (int i = 0; i < kPer; ++i) {
-                        x[0][i] = __ldcg(parts + static_cast<int64_t>(o) * kTile4 + idx0 + i * (kEpiWarps * 32));
-                        x[1][i] = __ldcg(parts + static_cast<int64_t>(o + 1) * kTile4 + idx0 + i * (kEpiWarps * 32));
-                    }
-#pragma unroll
-                    for (int i = 0; i < kPer; ++i) {
-                        sum[i].x += x[0][i].x; sum[i].y += x[0][i].y; sum[i].z += x[0][i].z; sum[i].w += x[0][i].w;
-                        sum[i].x += x[1][i].x; sum[i].y += x[1][i].y; sum[i].z += x[1][i].z; sum[i].w += x[1][i].w;
-                    }
-                }
-#pragma unroll
-                for (int i = 0; i < kPer; ++i) {
-                    const int idx = idx0 + i * (kEpiWarps * 32);
-                    if (idx / (kCh / 4) < rows_left) vt[idx] = sum[i];
-                }
+                for (int j = 0; j < 4; ++j) *part_piece(sm.stage, row, sub * 4u + j) = val[j];
                 return true;
             }
             if (q < p.n_tokens) {
@@ -665,7 +627,32 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p) {
     }
     // ---------------------------------------------------------------- teardown
     tc_fence_before();
-    __syncthreads();
+    __syncwarp();
+    if (S == 1) {
+        __syncthreads();
+    } else {
+        // The S parts of the tile are in the shared memory of the S CTAs of this cluster.  Each CTA adds every S-th row,
+        // the parts in order, and leaves only when the others have read its own.  (Every thread gets here: the waits above are
+        // bounded.)  With partial tiles through L2 and a ticket for the last CTA to add them all a launch took 2 to 3 us
+        // more (two tiles, hidden 3072: 10.4 -> 7.7 us; 64 tiles: 14.1 -> 12.2).
+        cluster_arrive();
+        cluster_wait();
+        const int64_t first = static_cast<int64_t>(cta) * kTok;
+        const uint32_t c4 = threadIdx.x % (kCh / 4);
+        for (uint32_t r = part + S * (threadIdx.x / (kCh / 4)); r < kTok; r += S * (kMlpThreads / (kCh / 4))) {
+            const uint32_t piece = smem_u32(part_piece(sm.stage, r, c4));
+            float4 x[kMaxSplit], sum = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int o = 0; o < kMaxSplit; ++o)
+                if (o < S) x[o] = cluster_load(piece, static_cast<uint32_t>(o));
+#pragma unroll
+            for (int o = 0; o < kMaxSplit; ++o)
+                if (o < S) { sum.x += x[o].x; sum.y += x[o].y; sum.z += x[o].z; sum.w += x[o].w; }
+            if (first + r < p.n_tokens) reinterpret_cast<float4*>(p.v_out)[(first + r) * (kCh / 4) + c4] = sum;
+        }
+        cluster_arrive();
+        cluster_wait();
+    }
     if (warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
@@ -705,19 +692,38 @@ cudaError_t launch_mlp_pack(const uint16_t* W1, const uint16_t* W2, int hidden, 
 }
 
 cudaError_t launch_mlp(const float* latents, int64_t pool_elems, int64_t tree_stride, int64_t row_offset, int n_trees, int64_t tokens_per_tree,
-                       const void* packed, int hidden, float* v_out, float* split_partials, unsigned int* split_tickets,
-                       int32_t* status, cudaStream_t s) {
-    static bool configured[64] = {false};
-    int dev = 0, sms = 0;
+                       const void* packed, int hidden, float* v_out, int32_t* status, cudaStream_t s) {
+    struct Device {
+        bool known = false;
+        int sms = 0, clusters[kMaxSplit + 1] = {0};       // clusters[S]: how many clusters of S CTAs run at a time
+    };
+    static Device devices[64];
+    constexpr size_t smem = sizeof(MlpSmem) + 1024;
+    int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64 || !configured[dev]) {
-        e = cudaFuncSetAttribute(mlp_velocity_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sizeof(MlpSmem) + 1024));
+    Device d;
+    if (dev >= 0 && dev < 64) d = devices[dev];
+    if (!d.known) {
+        e = cudaFuncSetAttribute(mlp_velocity_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev);
+        for (int cand = 2; e == cudaSuccess && cand <= kMaxSplit; ++cand) {
+            cudaLaunchConfig_t cfg = {};
+            cudaLaunchAttribute attr[1];
+            cfg.gridDim = cand;
+            cfg.blockDim = kMlpThreads;
+            cfg.dynamicSmemBytes = smem;
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = static_cast<unsigned int>(cand);
+            attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            e = cudaOccupancyMaxActiveClusters(&d.clusters[cand], mlp_velocity_kernel, &cfg);
+        }
         if (e != cudaSuccess) return e;
-        if (dev >= 0 && dev < 64) configured[dev] = true;
+        d.known = true;
+        if (dev >= 0 && dev < 64) devices[dev] = d;
     }
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
     MlpArgs a;
     a.latents = latents;
     a.pool_elems = pool_elems;
@@ -732,20 +738,14 @@ cudaError_t launch_mlp(const float* latents, int64_t pool_elems, int64_t tree_st
     if (tiles <= 0 || tiles > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     a.n_tiles = static_cast<int32_t>(tiles);
     a.status = status;
-    // A frontier of fewer tiles than SMs is cut along the hidden dimension too, as far as the SMs (and the scratch) go.
+    // A frontier of fewer tiles than SMs is cut along the hidden dimension too, as far as all its clusters run at once (on
+    // this chip 74 clusters of two, 45 of three, 33 of four, 22 of six, 15 of eight).  Any divisor of the chunk count will do:
+    // with powers of two alone 16 tiles took 9.4 us (8.9 with six), 40 tiles 12.1 (10.6 with three).
     a.split = 1;
-    a.partials = split_partials;
-    a.tickets = split_tickets;
-    if (split_partials && split_tickets) {
-        const int room = sms < kMlpSplitMaxCtas ? sms : kMlpSplitMaxCtas;
-        for (int cand = 8; cand > 1; cand >>= 1)
-            if (a.n_chunks % cand == 0 && static_cast<int64_t>(a.n_tiles) * cand <= room) {
-                a.split = cand;
-                break;
-            }
-    }
-    const int grid = a.split > 1 ? a.n_tiles * a.split : (a.n_tiles < sms ? a.n_tiles : sms);
-    return launch_overlapped(mlp_velocity_kernel, grid, kMlpThreads, sizeof(MlpSmem) + 1024, s, a);
+    for (int cand = kMaxSplit; cand > 1 && a.split == 1; --cand)
+        if (a.n_chunks % cand == 0 && a.n_tiles <= d.clusters[cand]) a.split = cand;
+    const int grid = a.split > 1 ? a.n_tiles * a.split : (a.n_tiles < d.sms ? a.n_tiles : d.sms);
+    return launch_overlapped_clusters(mlp_velocity_kernel, grid, kMlpThreads, smem, s, a.split, a);
 }
 
 }  // namespace bgrpo

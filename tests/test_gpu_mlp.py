@@ -204,3 +204,27 @@ def test_repeated_passes_are_bit_identical(B):
     for a, b, c in zip(first, second, third):
         assert torch.equal(a, b) and torch.equal(a, c)
     assert not torch.equal(first[0], other[0])
+
+
+@pytest.mark.parametrize("chunks", [2, 3, 4, 5, 6, 7, 8, 9, 11, 24])      # clusters of 2, 3, 4, 5, 6, 7, 8, 3, none, 8 CTAs a tile
+def test_every_cluster_size_agrees_with_the_unsplit_kernel(B, chunks):
+    """Two tiles, the second one of two tokens, cut along the hidden dimension into each size of cluster there is; the
+    reference is the same tree inside a batch of 82 tiles, which is not cut (float32 sums in another order)."""
+    from paper_2509_06040_b200.session import TreeSession
+    small = Workload(name="mlp_cluster", n_trees=1, tokens=130, channels=64, T=1, K=1, splits=(), sigma=0.3,
+                     velocity="mlp", reward="mixture", hidden=128 * chunks)
+    outs = []
+    for w in (small, small, small.scaled(n_trees=80)):
+        s = TreeSession(w)
+        s.upload_inputs(make_inputs(w))
+        s.init()
+        s.v.fill_(float("nan"))
+        B.velocity_mlp(s.tree, s.packed, w.hidden, s.v)
+        B.tree_sync_status(s.tree)
+        outs.append(s.v.view(-1)[:small.D].clone())
+    assert torch.equal(outs[0], outs[1])
+    # either side rounds a running float32 sum 8 times a chunk (one MMA per 16 hidden units), by at most 2^-23 of its value;
+    # a running sum does not get past twice the largest output
+    bound = 2 * (8 * chunks) * 2.0 ** -23 * 2 * outs[2].abs().max().item()
+    err = (outs[0] - outs[2]).abs().max().item()
+    assert err <= bound, (err, bound)
