@@ -47,7 +47,7 @@ size_t scratch_bytes_of(const bgrpo_tree_desc* d) {
     const int64_t rows = static_cast<int64_t>(d->n_trees) * d->nodes_cap;
     const int64_t D = static_cast<int64_t>(d->tokens) * d->channels;
     size_t b = kScratchHeader;
-    b += ((static_cast<size_t>(rows) * sizeof(unsigned int) + 255) / 256) * 256;
+    b += ((static_cast<size_t>(rows) * sizeof(unsigned long long) + 255) / 256) * 256;
     b += static_cast<size_t>(rows) * nchunks_of(D) * 3 * sizeof(double);
     b += static_cast<size_t>(rows) * 2 * sizeof(double);
     b += static_cast<size_t>(rows) * static_cast<size_t>(partials_per_row(D)) * sizeof(float);
@@ -104,8 +104,8 @@ void bind_buffers(bgrpo_tree* t, const bgrpo_buffers* b) {
     char* sc = static_cast<char*>(b->scratch);
     const size_t rows = static_cast<size_t>(desc->n_trees) * desc->nodes_cap;
     t->status = reinterpret_cast<int32_t*>(sc);
-    t->counters = reinterpret_cast<unsigned int*>(sc + kScratchHeader);
-    t->partials = reinterpret_cast<double*>(sc + kScratchHeader + ((rows * sizeof(unsigned int) + 255) / 256) * 256);
+    t->row_sums = reinterpret_cast<unsigned long long*>(sc + kScratchHeader);
+    t->partials = reinterpret_cast<double*>(sc + kScratchHeader + ((rows * sizeof(unsigned long long) + 255) / 256) * 256);
     t->node_scratch = t->partials + rows * static_cast<size_t>(t->nchunks) * 3;
     t->partials_logp = t->node_scratch + rows * 2;
     t->pending.logp_out = nullptr;
@@ -261,7 +261,8 @@ static void fill_step_launch(const bgrpo_tree* t, int step, const float* v_dev, 
     p->mix_innov = t->mix_innov;
 }
 
-bgrpo_status bgrpo_tree_step(bgrpo_tree* t, int32_t split_flag, const float* v_dev, void* stream) {
+// Checks the step and fills in its launch.
+static bgrpo_status prepare_step(bgrpo_tree* t, int32_t split_flag, const float* v_dev, StepLaunch* p) {
     if (!t) return fail(BGRPO_ERR_INVALID_ARG, "tree is NULL");
     if (t->depth >= t->desc.T) return fail(BGRPO_ERR_STATE, "tree already at depth T");
     if (!v_dev && !t->mu) return fail(BGRPO_ERR_STATE, "no velocity: pass v_dev or bind a linear velocity");
@@ -273,29 +274,44 @@ bgrpo_status bgrpo_tree_step(bgrpo_tree* t, int32_t split_flag, const float* v_d
     const int64_t W_out = static_cast<int64_t>(t->lv.width[i]) * fan;
     const int64_t off_out = t->lv.offset[i + 1];
     if (off_out + W_out > t->desc.nodes_cap) return fail(BGRPO_ERR_CAPACITY, "children exceed nodes_cap");
-    StepLaunch p;
-    fill_step_launch(t, i, v_dev, &p);
-    p.W_in = t->lv.width[i];
-    p.off_in = t->lv.offset[i];
-    p.off_out = static_cast<int32_t>(off_out);
-    p.fan = fan;
-    p.is_split = split_flag ? 1 : 0;
-    p.shared_noise = (split_flag && !t->independent && t->coef[i].g > 0.0f) ? 1 : 0;
-    cudaError_t e = launch_step(p, as_stream(stream));
-    if (e != cudaSuccess) return cuda_fail(e, "step kernel");
-    // this launch summed the previous level's log-probs in its prologue; its own are pending until the next
-    // launch, or until the flush below when the tree is complete
-    const int warps = step_threads(static_cast<int64_t>(p.n_trees) * p.W_in * p.nchunks) / 32;
-    t->pending = FinalizeDesc{t->buf.logp, static_cast<int32_t>(W_out), static_cast<int32_t>(off_out), p.nchunks * warps, t->coef[i].g, t->coef[i].logp_const};
+    fill_step_launch(t, i, v_dev, p);
+    p->W_in = t->lv.width[i];
+    p->off_in = t->lv.offset[i];
+    p->off_out = static_cast<int32_t>(off_out);
+    p->fan = fan;
+    p->is_split = split_flag ? 1 : 0;
+    p->shared_noise = (split_flag && !t->independent && t->coef[i].g > 0.0f) ? 1 : 0;
+    return BGRPO_OK;
+}
+
+// The step's kernel is on the stream.  It summed the previous level's log-probs; its own are pending until the next launch, or
+// until the flush below when the tree is complete.
+static bgrpo_status step_done(bgrpo_tree* t, const StepLaunch& p, const unsigned long long* sums, int per_row, int stride, void* stream) {
+    const int i = t->depth;
+    const int32_t W_out = p.W_in * p.fan;
+    t->pending = FinalizeDesc{t->buf.logp, W_out, p.off_out, per_row, t->coef[i].g, t->coef[i].logp_const, sums, stride};
     if (i + 1 == t->desc.T) {
-        e = flush_pending(t, as_stream(stream));
+        const cudaError_t e = flush_pending(t, as_stream(stream));
         if (e != cudaSuccess) return cuda_fail(e, "log-prob flush kernel");
     }
-    t->lv.fanout[i] = fan;
-    t->lv.width[i + 1] = static_cast<int32_t>(W_out);
-    t->lv.offset[i + 2] = static_cast<int32_t>(off_out + W_out);
+    t->lv.fanout[i] = p.fan;
+    t->lv.width[i + 1] = W_out;
+    t->lv.offset[i + 2] = p.off_out + W_out;
     t->depth = i + 1;
     return BGRPO_OK;
+}
+
+static bgrpo_status check_mlp(const bgrpo_tree* t, const void* packed_dev, int32_t hidden, const float* v_out_dev);
+static cudaError_t enqueue_mlp(bgrpo_tree* t, const void* packed_dev, int32_t hidden, float* v_out_dev, const StepLaunch* step, bool* stepped, void* stream);
+
+bgrpo_status bgrpo_tree_step(bgrpo_tree* t, int32_t split_flag, const float* v_dev, void* stream) {
+    StepLaunch p;
+    const bgrpo_status st = prepare_step(t, split_flag, v_dev, &p);
+    if (st != BGRPO_OK) return st;
+    const cudaError_t e = launch_step(p, as_stream(stream));
+    if (e != cudaSuccess) return cuda_fail(e, "step kernel");
+    const int warps = step_threads(static_cast<int64_t>(p.n_trees) * p.W_in * p.nchunks) / 32;
+    return step_done(t, p, t->partials_u64(), p.nchunks * warps, p.per_row >> 1, stream);
 }
 
 bgrpo_status bgrpo_tree_rollout(bgrpo_tree* t, const uint8_t* split_flags_host, const void* packed_dev, int32_t hidden,
@@ -322,8 +338,18 @@ bgrpo_status bgrpo_tree_rollout(bgrpo_tree* t, const uint8_t* split_flags_host, 
     }
     for (int i = t->depth; i < t->desc.T; ++i) {
         if (packed_dev) {
-            const bgrpo_status st = bgrpo_velocity_mlp(t, packed_dev, hidden, v_dev, stream);
+            bgrpo_status st = check_mlp(t, packed_dev, hidden, v_dev);
             if (st != BGRPO_OK) return st;
+            StepLaunch p;
+            st = prepare_step(t, split_flags_host[i] ? 1 : 0, v_dev, &p);
+            bool stepped = false;
+            const cudaError_t e = enqueue_mlp(t, packed_dev, hidden, v_dev, st == BGRPO_OK ? &p : nullptr, &stepped, stream);
+            if (e != cudaSuccess) return cuda_fail(e, "mlp kernel");
+            if (stepped) {
+                st = step_done(t, p, t->row_sums, 1, 1, stream);
+                if (st != BGRPO_OK) return st;
+                continue;
+            }
         }
         const bgrpo_status st = bgrpo_tree_step(t, split_flags_host[i] ? 1 : 0, packed_dev ? v_dev : nullptr, stream);
         if (st != BGRPO_OK) return st;
@@ -475,7 +501,6 @@ static bgrpo_status reward_common(bgrpo_tree* t, const float* target, float scal
     p.target = target;
     p.r = r;
     p.partials = t->partials;
-    p.counters = t->counters;
     p.status = t->status;
     p.nchunks_cap = t->nchunks;
     p.D = t->D;
@@ -695,16 +720,27 @@ bgrpo_status bgrpo_velocity_mlp_pack(const uint16_t* W1, const uint16_t* W2, int
     return e == cudaSuccess ? BGRPO_OK : cuda_fail(e, "mlp pack kernel");
 }
 
-bgrpo_status bgrpo_velocity_mlp(bgrpo_tree* t, const void* packed_dev, int32_t hidden, float* v_out_dev, void* stream) {
+static bgrpo_status check_mlp(const bgrpo_tree* t, const void* packed_dev, int32_t hidden, const float* v_out_dev) {
     if (!t || !packed_dev || !v_out_dev) return fail(BGRPO_ERR_INVALID_ARG, "NULL pointer");
     if (t->desc.channels != BGRPO_MLP_CHANNELS) return fail(BGRPO_ERR_UNSUPPORTED, "the MLP stage needs 64 channels");
     if (hidden < BGRPO_MLP_HIDDEN_MULTIPLE || hidden % BGRPO_MLP_HIDDEN_MULTIPLE != 0) return fail(BGRPO_ERR_INVALID_ARG, "hidden must be a positive multiple of 128");
     if (!aligned(packed_dev, 1024) || !aligned(v_out_dev, 16)) return fail(BGRPO_ERR_INVALID_ARG, "misaligned buffer");
     if (t->depth >= t->desc.T) return fail(BGRPO_ERR_STATE, "tree already at depth T");
+    return BGRPO_OK;
+}
+
+static cudaError_t enqueue_mlp(bgrpo_tree* t, const void* packed_dev, int32_t hidden, float* v_out_dev, const StepLaunch* step, bool* stepped, void* stream) {
     const int i = t->depth;
-    cudaError_t e = launch_mlp(t->buf.latents, static_cast<int64_t>(t->desc.n_trees) * t->desc.nodes_cap * t->D, static_cast<int64_t>(t->desc.nodes_cap) * t->D, static_cast<int64_t>(t->lv.offset[i]) * t->D,
-                               t->desc.n_trees, static_cast<int64_t>(t->lv.width[i]) * t->desc.tokens, packed_dev, hidden,
-                               v_out_dev, t->status, as_stream(stream));
+    const int64_t tree_stride = static_cast<int64_t>(t->desc.nodes_cap) * t->D;
+    return launch_mlp(t->buf.latents, t->desc.n_trees * tree_stride, tree_stride, static_cast<int64_t>(t->lv.offset[i]) * t->D, t->desc.n_trees,
+                      static_cast<int64_t>(t->lv.width[i]) * t->desc.tokens, packed_dev, hidden, v_out_dev, t->status, step, t->row_sums, stepped,
+                      as_stream(stream));
+}
+
+bgrpo_status bgrpo_velocity_mlp(bgrpo_tree* t, const void* packed_dev, int32_t hidden, float* v_out_dev, void* stream) {
+    const bgrpo_status st = check_mlp(t, packed_dev, hidden, v_out_dev);
+    if (st != BGRPO_OK) return st;
+    const cudaError_t e = enqueue_mlp(t, packed_dev, hidden, v_out_dev, nullptr, nullptr, stream);
     return e == cudaSuccess ? BGRPO_OK : cuda_fail(e, "mlp kernel");
 }
 
@@ -768,11 +804,12 @@ bgrpo_status bgrpo_tree_import(const void* blob_host, size_t blob_bytes, const b
     t->ode_bits = b.ode_bits;
     t->depth = b.depth;
     fill_coefficients(t);
-    // the status word lives in scratch, which may be a fresh allocation: it starts at zero
+    // the status word and the row sums live in scratch, which may be a fresh allocation: they start at zero
     cudaError_t e = cudaMemsetAsync(t->status, 0, sizeof(int32_t), as_stream(stream));
+    if (e == cudaSuccess) e = cudaMemsetAsync(t->row_sums, 0, static_cast<size_t>(t->desc.n_trees) * t->desc.nodes_cap * sizeof(unsigned long long), as_stream(stream));
     if (e != cudaSuccess) {
         delete t;
-        return cuda_fail(e, "clearing the status word");
+        return cuda_fail(e, "clearing the status word and the row sums");
     }
     *out = t;
     return BGRPO_OK;

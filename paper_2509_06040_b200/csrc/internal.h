@@ -84,8 +84,10 @@ struct StepCoef {
 struct FinalizeDesc {
     float* logp_out;       // nullptr: nothing pending
     int32_t W, off;        // rows off .. off+W-1 of every tree
-    int32_t per_row;       // partials per row
+    int32_t per_row;       // sums per row
     float g, logp_const;
+    const unsigned long long* sums;   // row r's start at sums + r * stride
+    int32_t stride;        // the same for every launch of a tree: a level is summed while the next one's sums are written
 };
 
 struct LevelInfo {                       // layout of the tree grown so far
@@ -144,7 +146,7 @@ struct bgrpo_tree {
     float s0;
     // scratch carving (device pointers inside buf.scratch)
     int32_t* status;
-    unsigned int* counters;              // one ticket counter per (tree, node row)
+    unsigned long long* row_sums;        // [n_trees*nodes_cap] squares of a row's noise, where the MLP stage takes the step; zero until then
     double* partials;                    // [n_trees*nodes_cap][nchunks][3]   (reward reductions)
     double* node_scratch;                // [n_trees][2][nodes_cap]: per-chain state of the tree reductions when a tree
                                          // is too large for one CTA's shared memory
@@ -214,7 +216,7 @@ struct StepLaunch {
     int32_t shared_noise;      // 1: finite s at a split step
     int32_t* status;           // the tree's status word
     int32_t per_row;           // 32-bit words reserved per node row in the partials
-    unsigned long long* partials;   // [rows][nchunks][warps of a CTA] sums of quantized squares (philox.cuh)
+    unsigned long long* partials;   // by row, per_row / 2 apart: [nchunks][warps of a CTA] sums of quantized squares (philox.cuh)
     FinalizeDesc prev;         // level to finalize in this launch's prologue (logp_out == nullptr: none)
 };
 cudaError_t launch_root(const bgrpo_tree* t, cudaStream_t s);
@@ -257,7 +259,7 @@ struct LogprobStepLaunch {
 cudaError_t launch_logprob_step(const LogprobStepLaunch& p, cudaStream_t s);
 
 struct RewardLaunch {
-    const float* latents; const float* target; float* r; double* partials; unsigned int* counters; int32_t* status;
+    const float* latents; const float* target; float* r; double* partials; int32_t* status;
     int64_t D; int32_t n_trees, nodes_cap, nchunks, nchunks_cap, leaves, off_leaf; float scale; double inv_D; int32_t mode;  // 0 mse, 1 cos; nchunks_cap: partial slots reserved per row
 };
 cudaError_t launch_reward(const RewardLaunch& p, cudaStream_t s);
@@ -327,7 +329,10 @@ cudaError_t launch_objective(const ObjectiveLaunch& p, cudaStream_t s);
 size_t mlp_packed_bytes(int hidden);
 cudaError_t launch_mlp_pack(const uint16_t* W1, const uint16_t* W2, int hidden, void* packed, cudaStream_t s);
 cudaError_t launch_debug_trip(int32_t* status, cudaStream_t s);     // debug build: fails one index test on purpose (no access involved)
+// `step`: the step that follows, or nullptr.  Where the launch can take it along (launch_mlp in mlp_velocity.cu), *stepped is
+// set, the squares of the noise go to row_sums, and no step kernel is needed.
 cudaError_t launch_mlp(const float* latents, int64_t pool_elems, int64_t tree_stride, int64_t row_offset, int n_trees, int64_t tokens_per_tree,
-                       const void* packed, int hidden, float* v_out, int32_t* status, cudaStream_t s);
+                       const void* packed, int hidden, float* v_out, int32_t* status, const StepLaunch* step, unsigned long long* row_sums,
+                       bool* stepped, cudaStream_t s);
 
 }  // namespace bgrpo

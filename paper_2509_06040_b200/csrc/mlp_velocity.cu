@@ -39,7 +39,10 @@
 // released and bit 2 of the status word is set.
 #include <cuda_bf16.h>
 
+#include <cstring>
+
 #include "internal.h"
+#include "philox.cuh"
 
 namespace bgrpo {
 namespace {
@@ -70,6 +73,7 @@ struct MlpSmem {
                                                              // mode, at the end: this CTA's partial output tile
     unsigned long long w1_full[kW1Stages], w1_free[kW1Stages], w2_full[kW2Stages], w2_free[kW2Stages];
     unsigned long long stage_full, first_a, a_full[2], a_empty[2], d1_full[kBufs], h_full[kBufs], buf_free[kBufs], d2_full[2], d2_empty[2];
+    uint32_t node_sums[kTok][BGRPO_MAX_K][2];    // the step taken along: squares of the noise by parent in the tile and child, low 16 bits and the rest
     uint32_t tmem_base;
     int abort_flag;
 };
@@ -310,10 +314,82 @@ struct MlpArgs {
     int32_t n_tiles;
     int32_t split;            // CTAs per tile along the hidden dimension (1: none); > 1 only with one tile per cluster of that size
     int32_t* status;
+    int32_t tokens;           // of a node
+    unsigned long long* row_sums;
 };
 
+// One float4 of a parent of the step taken along: where it is, and the noise of its children.
+struct StepPiece {
+    bool live;
+    int32_t row, node0;       // frontier row (tree * W + j) and first child's row in the pool
+    uint32_t e;               // float4 index in the row
+    float4 z, xi[BGRPO_MAX_K];
+    uint32_t squares[BGRPO_MAX_K];
+};
+__device__ __forceinline__ void step_piece(const StepLaunch& sp, const MlpArgs& p, int64_t first, uint32_t r, uint32_t c4, StepPiece& q) {
+    const uint32_t token = static_cast<uint32_t>(first) + r;          // fewer than 2^15: one tile per cluster
+    q.live = r < kTok && token < p.n_tokens;
+    if (!q.live) return;
+    q.row = static_cast<int32_t>(token / static_cast<uint32_t>(p.tokens));
+    q.e = (token - static_cast<uint32_t>(q.row) * p.tokens) * (kCh / 4) + c4;
+    const int tree = q.row / sp.W_in, j = q.row - tree * sp.W_in;
+    const int32_t parent = tree * sp.nodes_cap + sp.off_in + j;
+    q.node0 = tree * sp.nodes_cap + sp.off_out + j * sp.fan;
+    q.live = BGRPO_IN_BOUNDS(sp.status, tree < sp.n_trees && sp.off_in + j < sp.nodes_cap && sp.off_out + (j + 1) * sp.fan <= sp.nodes_cap && q.e < sp.D / 4);
+    if (!q.live) return;
+    q.z = __ldcs(reinterpret_cast<const float4*>(sp.latents + parent * sp.D) + q.e);
+    if (q.e == 0u) {          // node-table rows of the new children
+        const int64_t rows = static_cast<int64_t>(sp.n_trees) * sp.nodes_cap;
+        for (int b = 0; b < sp.fan; ++b) {
+            const int64_t r = q.node0 + b;
+            sp.table[r] = sp.off_in + j;
+            sp.table[rows + r] = sp.step + 1;
+            sp.table[2 * rows + r] = sp.is_split ? sp.step : sp.table[2 * rows + parent];
+            sp.table[3 * rows + r] = sp.is_split ? b : sp.table[3 * rows + parent];
+        }
+    }
+    if (sp.g == 0.0f) return;
+    float squares;
+    float4 xi0;
+    if (sp.shared_noise)
+        xi0 = mul4(sp.mix_shared, normal4(philox_from(noise_element(q.e, BGRPO_TAG_SHARED, sp.keys), noise_node(sp.node_id_base + parent, sp.step, sp.keys), sp.keys), squares));
+    const NoiseElement el = noise_element(q.e, BGRPO_TAG_INNOV, sp.keys);
+#pragma unroll
+    for (int b = 0; b < BGRPO_MAX_K; ++b)
+        if (b < sp.fan) {
+            q.xi[b] = normal4(philox_from(el, noise_node(sp.node_id_base + q.node0 + b, sp.step, sp.keys), sp.keys), squares);
+            if (sp.shared_noise) {
+                q.xi[b] = fma4(sp.mix_innov, q.xi[b], xi0);
+                squares = squares_of(q.xi[b]);
+            }
+            q.squares[b] = quantized_squares(squares);
+        }
+}
+// The children of one float4, given the velocity; adds the squares of a token (16 lanes) to the node's sums.
+__device__ __forceinline__ void step_children(const StepLaunch& sp, int row0, const StepPiece& q, const float4& v, uint32_t (*node_sums)[BGRPO_MAX_K][2]) {
+    const float4 m = fma4(sp.ca, q.z, mul4(sp.cb, v));
+    float4* child = reinterpret_cast<float4*>(sp.latents + q.node0 * sp.D) + q.e;
+    const uint32_t half = 0xffffu << (threadIdx.x & 16u);
+#pragma unroll
+    for (int b = 0; b < BGRPO_MAX_K; ++b)
+        if (b < sp.fan) {
+            child[b * (sp.D / 4)] = sp.g == 0.0f ? m : fma4(sp.g, q.xi[b], m);
+            if (sp.g != 0.0f) {
+                const uint32_t lo = __reduce_add_sync(half, q.squares[b] & 0xffffu), hi = __reduce_add_sync(half, q.squares[b] >> 16);
+                if ((threadIdx.x & 15u) == 0u) {        // 128 tokens of 16 lanes: 27 bits.  (A 64-bit add would be a loop.)
+                    atomicAdd(&node_sums[q.row - row0][b][0], lo);
+                    atomicAdd(&node_sums[q.row - row0][b][1], hi);
+                }
+            }
+        }
+}
+
+// STEP: the step that follows is taken along (split tiles): the tail has the velocity of its rows in registers, so it writes
+// the children next to it, and the launch and the reload of a step kernel are saved.  What does not need the velocity - the
+// parent, the noise, the table - is done while the cluster's barrier is on its way.
+template <bool STEP>
 __global__ void __launch_bounds__(kMlpThreads, 1)
-mlp_velocity_kernel(const __grid_constant__ MlpArgs p) {
+mlp_velocity_kernel(const __grid_constant__ MlpArgs p, const __grid_constant__ StepLaunch sp) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     // the swizzled operand tiles need 1024-byte alignment; the launch reserves 1 KiB of slack for this round-up
     MlpSmem& sm = *reinterpret_cast<MlpSmem*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
@@ -347,6 +423,8 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p) {
         sm.abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if (STEP)
+        for (int i = threadIdx.x; i < kTok * BGRPO_MAX_K * 2; i += kMlpThreads) (&sm.node_sums[0][0][0])[i] = 0u;
     if (warp == 1) {      // tensor memory: this warp allocates and, at the end, frees
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sm.tmem_base)), "r"(kTmemCols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -517,6 +595,9 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p) {
                 if (it + 1 < n_my_tiles) issue_tile_copy(it + 1);      // every lane has read the staging buffer
             }
         }
+        if (STEP && sp.prev.logp_out != nullptr)      // the previous level's log-probs, off the critical path
+            finalize_rows(sp.prev, sp.n_trees, sp.nodes_cap, sp.half_per, blockIdx.x, gridDim.x, sp.status, sp.per_row);
+        __syncwarp();
     } else {
         // ---------------------------------------------------------------- epilogue warps
         const int ew = warp - 2;                  // 0..15
@@ -555,7 +636,7 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p) {
             for (int j = 0; j < 4; ++j)
                 val[j] = make_float4(0.25f * __uint_as_float(out[4 * j]), 0.25f * __uint_as_float(out[4 * j + 1]),
                                      0.25f * __uint_as_float(out[4 * j + 2]), 0.25f * __uint_as_float(out[4 * j + 3]));
-            if (S > 1) {
+            if (STEP || S > 1) {
                 // This CTA holds the sum over its share of the hidden dimension only; the tail of the kernel adds the parts.
 #pragma unroll
                 for (int j = 0; j < 4; ++j) *part_piece(sm.stage, row, sub * 4u + j) = val[j];
@@ -628,29 +709,50 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p) {
     // ---------------------------------------------------------------- teardown
     tc_fence_before();
     __syncwarp();
-    if (S == 1) {
+    if (!STEP && S == 1) {
         __syncthreads();
     } else {
         // The S parts of the tile are in the shared memory of the S CTAs of this cluster.  Each CTA adds every S-th row,
         // the parts in order, and leaves only when the others have read its own.  (Every thread gets here: the waits above are
         // bounded.)  With partial tiles through L2 and a ticket for the last CTA to add them all a launch took 2 to 3 us
         // more (two tiles, hidden 3072: 10.4 -> 7.7 us; 64 tiles: 14.1 -> 12.2).
-        cluster_arrive();
-        cluster_wait();
         const int64_t first = static_cast<int64_t>(cta) * kTok;
         const uint32_t c4 = threadIdx.x % (kCh / 4);
-        for (uint32_t r = part + S * (threadIdx.x / (kCh / 4)); r < kTok; r += S * (kMlpThreads / (kCh / 4))) {
-            const uint32_t piece = smem_u32(part_piece(sm.stage, r, c4));
+        uint32_t r = part + S * (threadIdx.x / (kCh / 4));
+        StepPiece piece;
+        cluster_arrive();
+        if (STEP) step_piece(sp, p, first, r, c4, piece);        // the load and the noise travel with the barrier
+        __syncwarp();
+        cluster_wait();
+        const int row0 = STEP ? static_cast<int>(static_cast<uint32_t>(first) / static_cast<uint32_t>(p.tokens)) : 0;
+        while (r < kTok) {
+            const uint32_t addr = smem_u32(part_piece(sm.stage, r, c4));
             float4 x[kMaxSplit], sum = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
             for (int o = 0; o < kMaxSplit; ++o)
-                if (o < S) x[o] = cluster_load(piece, static_cast<uint32_t>(o));
+                if (o < S) x[o] = cluster_load(addr, static_cast<uint32_t>(o));
 #pragma unroll
             for (int o = 0; o < kMaxSplit; ++o)
                 if (o < S) { sum.x += x[o].x; sum.y += x[o].y; sum.z += x[o].z; sum.w += x[o].w; }
             if (first + r < p.n_tokens) reinterpret_cast<float4*>(p.v_out)[(first + r) * (kCh / 4) + c4] = sum;
+            if (STEP && piece.live) step_children(sp, row0, piece, sum, sm.node_sums);
+            r += S * (kMlpThreads / (kCh / 4));
+            if (STEP) step_piece(sp, p, first, r, c4, piece);
         }
+        __syncwarp();
         cluster_arrive();
+        if (STEP && sp.g != 0.0f) {          // the sums of this CTA's tokens, by child
+            __syncthreads();
+            for (int i = threadIdx.x; i < kTok * BGRPO_MAX_K; i += kMlpThreads) {
+                const int row = row0 + i / BGRPO_MAX_K, b = i % BGRPO_MAX_K;
+                const uint32_t* both = sm.node_sums[i / BGRPO_MAX_K][b];
+                const unsigned long long sum = (static_cast<unsigned long long>(both[1]) << 16) + both[0];
+                if (sum == 0ull) continue;
+                const int tree = row / sp.W_in, j = row - tree * sp.W_in;
+                atomicAdd(p.row_sums + static_cast<int64_t>(tree) * sp.nodes_cap + sp.off_out + j * sp.fan + b, sum);
+            }
+            __syncwarp();
+        }
         cluster_wait();
     }
     if (warp == 1) {
@@ -692,7 +794,8 @@ cudaError_t launch_mlp_pack(const uint16_t* W1, const uint16_t* W2, int hidden, 
 }
 
 cudaError_t launch_mlp(const float* latents, int64_t pool_elems, int64_t tree_stride, int64_t row_offset, int n_trees, int64_t tokens_per_tree,
-                       const void* packed, int hidden, float* v_out, int32_t* status, cudaStream_t s) {
+                       const void* packed, int hidden, float* v_out, int32_t* status, const StepLaunch* step, unsigned long long* row_sums,
+                       bool* stepped, cudaStream_t s) {
     struct Device {
         bool known = false;
         int sms = 0, clusters[kMaxSplit + 1] = {0};       // clusters[S]: how many clusters of S CTAs run at a time
@@ -705,7 +808,8 @@ cudaError_t launch_mlp(const float* latents, int64_t pool_elems, int64_t tree_st
     Device d;
     if (dev >= 0 && dev < 64) d = devices[dev];
     if (!d.known) {
-        e = cudaFuncSetAttribute(mlp_velocity_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+        e = cudaFuncSetAttribute(mlp_velocity_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(mlp_velocity_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev);
         for (int cand = 2; e == cudaSuccess && cand <= kMaxSplit; ++cand) {
             cudaLaunchConfig_t cfg = {};
@@ -718,7 +822,7 @@ cudaError_t launch_mlp(const float* latents, int64_t pool_elems, int64_t tree_st
             attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
             cfg.attrs = attr;
             cfg.numAttrs = 1;
-            e = cudaOccupancyMaxActiveClusters(&d.clusters[cand], mlp_velocity_kernel, &cfg);
+            e = cudaOccupancyMaxActiveClusters(&d.clusters[cand], mlp_velocity_kernel<true>, &cfg);
         }
         if (e != cudaSuccess) return e;
         d.known = true;
@@ -745,7 +849,21 @@ cudaError_t launch_mlp(const float* latents, int64_t pool_elems, int64_t tree_st
     for (int cand = kMaxSplit; cand > 1 && a.split == 1; --cand)
         if (a.n_chunks % cand == 0 && a.n_tiles <= d.clusters[cand]) a.split = cand;
     const int grid = a.split > 1 ? a.n_tiles * a.split : (a.n_tiles < d.sms ? a.n_tiles : d.sms);
-    return launch_overlapped_clusters(mlp_velocity_kernel, grid, kMlpThreads, smem, s, a.split, a);
+    a.tokens = 1;
+    a.row_sums = row_sums;
+    StepLaunch sp;
+    std::memset(&sp, 0, sizeof(sp));
+    // The step goes along where a tile is split: each CTA then has at most half a tile of children to make.  Whole passes, in
+    // us, with no step taken along / those of split tiles / also those of whole tiles: one tree of 256 tokens 198 / 170 / 170,
+    // of 2 025 tokens 380 / 368 / 381.
+    if (step && a.split > 1) {
+        sp = *step;
+        sp.half_per = logp_half_per(sp.D);
+        a.tokens = static_cast<int32_t>(tokens_per_tree / sp.W_in);
+        *stepped = true;
+        return launch_overlapped_clusters(mlp_velocity_kernel<true>, grid, kMlpThreads, smem, s, a.split, a, sp);
+    }
+    return launch_overlapped_clusters(mlp_velocity_kernel<false>, grid, kMlpThreads, smem, s, a.split, a, sp);
 }
 
 }  // namespace bgrpo

@@ -169,6 +169,25 @@ __device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long x)
     return x;
 }
 
+// Adds up the pending level's partial sums: one warp per row.
+__device__ __forceinline__ void finalize_rows(const FinalizeDesc& f, int32_t n_trees, int32_t nodes_cap,
+                                              double half_per, int warp_global, int warps_total, int32_t* status, int32_t per_row_cap) {
+    const int lane = threadIdx.x & 31;
+    const int n_rows = n_trees * f.W;
+    const int per_row = f.per_row;
+    for (int idx = warp_global; idx < n_rows; idx += warps_total) {
+        const int tree = idx / f.W;
+        const int64_t row = static_cast<int64_t>(tree) * nodes_cap + f.off + (idx - tree * f.W);
+        if (!BGRPO_IN_BOUNDS(status, f.off + f.W <= nodes_cap && 2 * per_row <= per_row_cap)) continue;
+        const unsigned long long* q = f.sums + row * f.stride;
+        unsigned long long s = 0;
+#pragma unroll 4
+        for (int c = lane; c < per_row; c += 32) s += __ldcg(q + c);
+        s = warp_sum_u64(s);
+        if (lane == 0) f.logp_out[row] = logp_from_squares(s, half_per, f.g, f.logp_const);
+    }
+}
+
 __device__ __forceinline__ float4 noise4(uint32_t block, uint32_t node, uint32_t step, uint32_t tag,
                                          const PhiloxKeys& keys) {
     float squares;

@@ -11,9 +11,9 @@ namespace {
 
 constexpr int kVecPerThread = kChunkVec / kStreamThreads;   // 4
 // ---------------------------------------------------------------------------------------------------------------
-// Root: z_0 ~ N(0, I) from the ROOT stream, node-table row of the root, and a clean scratch (counters, status).
+// Root: z_0 ~ N(0, I) from the ROOT stream, node-table row of the root, and a clean scratch (row sums, status).
 __global__ void __launch_bounds__(kStreamThreads)
-root_kernel(float* latents, int32_t* table, float* logp, unsigned int* counters, int32_t* status, int64_t D,
+root_kernel(float* latents, int32_t* table, float* logp, unsigned long long* row_sums, int32_t* status, int64_t D,
             int32_t n_trees, int32_t nodes_cap, int32_t nchunks, uint32_t node_id_base, const __grid_constant__ PhiloxKeys keys) {
     pdl_release();
     const int chunk = blockIdx.x % nchunks;
@@ -34,7 +34,7 @@ root_kernel(float* latents, int32_t* table, float* logp, unsigned int* counters,
     }
     const int64_t rows = static_cast<int64_t>(n_trees) * nodes_cap;
     if (chunk == 0) {
-        for (int n = threadIdx.x; n < nodes_cap; n += kStreamThreads) counters[static_cast<int64_t>(tree) * nodes_cap + n] = 0u;
+        for (int n = threadIdx.x; n < nodes_cap; n += kStreamThreads) row_sums[static_cast<int64_t>(tree) * nodes_cap + n] = 0ull;
         if (threadIdx.x == 0) {
             const int64_t r = static_cast<int64_t>(tree) * nodes_cap;
             table[r] = -1;
@@ -65,25 +65,6 @@ root_kernel(float* latents, int32_t* table, float* logp, unsigned int* counters,
 // FAN children per parent; SHARED: xi_b mixes a per-parent xi_0 (finite s at a split step); FULL: the tile holds
 // kStepChunkVec float4, so no element needs a bounds test; NOISY = false: a deterministic step (sigma = 0) of the
 // hybrid schedule, no noise is generated at all.
-
-// Adds up the pending level's partial sums: one warp per row.
-__device__ __forceinline__ void finalize_rows(const FinalizeDesc& f, const unsigned long long* partials, int32_t n_trees, int32_t nodes_cap,
-                                              double half_per, int warp_global, int warps_total, int32_t* status, int32_t per_row_cap) {
-    const int lane = threadIdx.x & 31;
-    const int n_rows = n_trees * f.W;
-    const int per_row = f.per_row;
-    for (int idx = warp_global; idx < n_rows; idx += warps_total) {
-        const int tree = idx / f.W;
-        const int64_t row = static_cast<int64_t>(tree) * nodes_cap + f.off + (idx - tree * f.W);
-        if (!BGRPO_IN_BOUNDS(status, f.off + f.W <= nodes_cap && 2 * per_row <= per_row_cap)) continue;
-        const unsigned long long* q = partials + row * per_row;
-        unsigned long long s = 0;
-#pragma unroll 4
-        for (int c = lane; c < per_row; c += 32) s += __ldcg(q + c);
-        s = warp_sum_u64(s);
-        if (lane == 0) f.logp_out[row] = logp_from_squares(s, half_per, f.g, f.logp_const);
-    }
-}
 
 template <int THREADS, bool FULL>
 __device__ __forceinline__ void load_tile(const float4* __restrict__ zp, const float4* __restrict__ xop, bool streamed,
@@ -158,7 +139,7 @@ step_kernel(const __grid_constant__ StepLaunch p) {
     // the previous level's log-probs (a handful of rows) are summed by this launch
     auto finalize_previous = [&] {
         if (p.prev.logp_out != nullptr)
-            finalize_rows(p.prev, p.partials, p.n_trees, p.nodes_cap, p.half_per, blockIdx.x * kWarps + warp, gridDim.x * kWarps, p.status, p.per_row);
+            finalize_rows(p.prev, p.n_trees, p.nodes_cap, p.half_per, blockIdx.x * kWarps + warp, gridDim.x * kWarps, p.status, p.per_row);
     };
     // The parents, the velocity and the pending partial sums come from earlier kernels.  A launch of many waves waits for
     // them here: its loads travel while the noise is generated.
@@ -222,7 +203,7 @@ step_kernel(const __grid_constant__ StepLaunch p) {
     for (int b = 0; b < FAN; ++b) {
         const uint32_t lo = __reduce_add_sync(0xffffffffu, acc[b] & 0xffffu), hi = __reduce_add_sync(0xffffffffu, acc[b] >> 16);
         if (lane == 0)
-            p.partials[((tree_row0 + child0 + b) * p.nchunks + chunk) * kWarps + warp] = (static_cast<unsigned long long>(hi) << 16) + lo;
+            p.partials[(tree_row0 + child0 + b) * (p.per_row >> 1) + chunk * kWarps + warp] = (static_cast<unsigned long long>(hi) << 16) + lo;
     }
     if (chunk == 0 && threadIdx.x < FAN) {      // node-table rows of the new children
         const int b = threadIdx.x;
@@ -237,11 +218,11 @@ step_kernel(const __grid_constant__ StepLaunch p) {
 
 // Flush: adds up a pending level outside a step launch (the tree is complete, or tree_logprob is done).
 __global__ void __launch_bounds__(kStreamThreads)
-finalize_kernel(const FinalizeDesc f, const unsigned long long* partials, int32_t n_trees, int32_t nodes_cap, double half_per,
+finalize_kernel(const FinalizeDesc f, int32_t n_trees, int32_t nodes_cap, double half_per,
                 int32_t* status, int32_t per_row_cap) {
     pdl_release();
     pdl_wait();
-    finalize_rows(f, partials, n_trees, nodes_cap, half_per, blockIdx.x * (kStreamThreads / 32) + (threadIdx.x >> 5),
+    finalize_rows(f, n_trees, nodes_cap, half_per, blockIdx.x * (kStreamThreads / 32) + (threadIdx.x >> 5),
                   gridDim.x * (kStreamThreads / 32), status, per_row_cap);
 }
 
@@ -284,7 +265,7 @@ cudaError_t launch_debug_trip(int32_t* status, cudaStream_t s) {
 
 cudaError_t launch_root(const bgrpo_tree* t, cudaStream_t s) {
     const unsigned int grid = static_cast<unsigned int>(t->desc.n_trees) * t->nchunks;
-    return launch_overlapped(root_kernel, grid, kStreamThreads, 0, s, t->buf.latents, t->buf.node_table, t->buf.logp, t->counters,
+    return launch_overlapped(root_kernel, grid, kStreamThreads, 0, s, t->buf.latents, t->buf.node_table, t->buf.logp, t->row_sums,
                              t->status, t->D, t->desc.n_trees, t->desc.nodes_cap, t->nchunks,
                              static_cast<uint32_t>(t->desc.tree_id_base * t->desc.nodes_cap), make_philox_keys(t->desc.seed));
 }
@@ -301,7 +282,7 @@ cudaError_t launch_step(const StepLaunch& p0, cudaStream_t s) {
 cudaError_t launch_finalize(const bgrpo_tree* t, const FinalizeDesc& f, cudaStream_t s) {
     const int rows = t->desc.n_trees * f.W;
     const int grid = (rows + (kStreamThreads / 32) - 1) / (kStreamThreads / 32);
-    return launch_overlapped(finalize_kernel, grid < 1 ? 1 : grid, kStreamThreads, 0, s, f, static_cast<const unsigned long long*>(t->partials_u64()),
+    return launch_overlapped(finalize_kernel, grid < 1 ? 1 : grid, kStreamThreads, 0, s, f,
                              t->desc.n_trees, t->desc.nodes_cap, logp_half_per(t->D), t->status,
                              static_cast<int32_t>(partials_per_row(t->D)));
 }

@@ -132,9 +132,16 @@ class TreeSession:
     def kernel_launches_per_pass(self) -> int:
         w = self.w
         if w.velocity == "linear" and len(w.splits) <= 6:
-            n = 1 + 2                                              # root + whole-tree rollout + its log-prob sums
+            n = 1 + (1 if w.D <= 2048 and w.nodes <= 1024 else 2)  # root + whole-tree rollout (+ its log-prob sums)
+        elif w.velocity == "mlp":
+            # root + mlp (+ step, where the mlp launch does not take it along: tiles that are not split) per depth + log-prob flush
+            sms = torch.cuda.get_device_properties(self.latents.device).multi_processor_count
+            tiles = [-(-self.n_trees * W * w.tokens // 128) for W in w.widths()[:w.T]]
+            split = [any(w.hidden // 128 % c == 0 and n * c <= sms for c in range(2, 9)) for n in tiles]
+            n = 1 + sum(1 if along else 2 for along in split) + 1
         else:
-            n = 1 + w.T * (2 if w.velocity == "mlp" else 1) + 1   # root + (mlp +) step per depth + log-prob flush
-        n += 2 if w.reward in ("neg_mse_mu", "neg_mse_target", "normal_plus_cos") else 0   # partial sums + their fixed-order total
+            n = 1 + w.T + 1                                        # root + step per depth + log-prob flush
+        if w.reward in ("neg_mse_mu", "neg_mse_target", "normal_plus_cos"):
+            n += 1 if w.D <= 16384 else 2                          # partial sums (+ their fixed-order total)
         n += 2                                                     # fuse+advantage, prune
         return n

@@ -228,3 +228,43 @@ def test_every_cluster_size_agrees_with_the_unsplit_kernel(B, chunks):
     bound = 2 * (8 * chunks) * 2.0 ** -23 * 2 * outs[2].abs().max().item()
     err = (outs[0] - outs[2]).abs().max().item()
     assert err <= bound, (err, bound)
+
+
+@pytest.mark.parametrize("tokens,n_trees,T,K,splits,s,hidden,sde", [
+    (1, 5, 3, 4, (0, 1), 2.0, 256, None),              # one token a node: up to 80 nodes in a tile, shared noise
+    (48, 3, 4, 3, (0, 2), math.inf, 384, None),        # nodes that straddle tiles, clusters of three
+    (130, 1, 4, 2, (1,), math.inf, 1024, (0, 1, 1, 0)),    # a tile of two tokens; ODE steps first and last
+    (256, 2, 3, 1, (), math.inf, 1408, None),          # eleven chunks: not cut
+    (4736, 2, 3, 2, (1,), math.inf, 256, None),        # 74 tiles in clusters of two, then 148: the step has its own launch
+    (4737, 2, 2, 2, (0,), 1.0, 256, None),             # 75 tiles: not cut
+])
+def test_rollout_that_takes_the_step_along_is_the_step_by_step_rollout(B, tokens, n_trees, T, K, splits, s, hidden, sde):
+    """Small frontiers: the velocity launch also makes the children.  Same noise, same float32 expressions, integer sums of
+    squares: latents, velocity, log-probs and table are bit-equal to velocity and step in launches of their own."""
+    from paper_2509_06040_b200.session import TreeSession
+    w = Workload(name="along", n_trees=n_trees, tokens=tokens, channels=64, T=T, K=K, splits=splits, sigma=0.3,
+                 velocity="mlp", reward="mixture", hidden=hidden, branch_corr_s=s)
+    inp = make_inputs(w)
+    flags = [1 if i in splits else 0 for i in range(T)]
+    runs = []
+    for along in (False, True, True):
+        r = TreeSession(w, nodes_cap=w.nodes + 2)
+        r.upload_inputs(inp)
+        r.logp.fill_(7.0)
+        r.init()
+        if sde:
+            B.tree_set_sde_steps(r.tree, list(sde))
+        if along:
+            B.tree_rollout(r.tree, flags, r.packed, hidden, r.v)
+        else:
+            for i in range(T):
+                B.velocity_mlp(r.tree, r.packed, hidden, r.v)
+                B.tree_step(r.tree, flags[i], r.v)
+        B.tree_sync_status(r.tree)
+        runs.append(r)
+    n = n_trees * w.widths()[T - 1] * w.D
+    for r in runs[1:]:
+        assert torch.equal(r.latents[:, :w.nodes], runs[0].latents[:, :w.nodes])
+        assert torch.equal(r.logp, runs[0].logp)
+        assert torch.equal(r.node_table.view(4, n_trees, -1)[:, :, :w.nodes], runs[0].node_table.view(4, n_trees, -1)[:, :, :w.nodes])
+        assert torch.equal(r.v.view(-1)[:n], runs[0].v.view(-1)[:n])
