@@ -145,8 +145,8 @@ bgrpo_status bgrpo_velocity_linear_bind(bgrpo_tree* tree, const float* mu_dev, f
 bgrpo_status bgrpo_tree_step(bgrpo_tree* tree, int32_t split_flag, const float* v_dev, void* stream);
 
 /* tree_rollout: the remaining steps of the tree, depth .. T-1, in one host call (Algorithm 1, "Build rollout tree": for
- * every step, the velocity of every live node, then the step that forks or advances it).  With packed_dev the same kernels
- * in the same order as calling bgrpo_velocity_mlp and bgrpo_tree_step step by step; a whole tree under the bound linear
+ * every step, the velocity of every live node, then the step that forks or advances it).  With packed_dev the kernels
+ * of bgrpo_velocity_mlp and bgrpo_tree_step in turn, one launch for both on a small frontier; a whole tree under the bound linear
  * velocity takes the one launch of bgrpo_tree_rollout_fused where that covers it.  Every output is identical bit for bit to
  * the step-by-step calls either way (log-probs because the sums of squares are added as integers).
  *   split_flags_host  host array of T flags (indexed by step), non-zero = fork every node into K children
@@ -263,7 +263,7 @@ bgrpo_status bgrpo_tree_sync_status(bgrpo_tree* tree, void* stream);
  * log-prob sums (so buffers.logp is final once `stream` has run), then writes the record to blob_host
  * (bgrpo_tree_export_bytes() bytes).  bgrpo_tree_import builds a new handle from such a record and a set of buffers that
  * hold what the exported tree's buffers held (the same allocations, or copies made after `stream` had run; scratch may be
- * fresh), without launching a kernel; it clears the status word and the MLP stage's tickets on `stream`.  A bound linear
+ * fresh), without launching a kernel; it clears the status word and the row sums on `stream`.  A bound linear
  * velocity is a device pointer and is not saved: call bgrpo_velocity_linear_bind again.  Continuing an imported tree gives
  * the bits an uninterrupted tree gives.  Errors: INVALID_ARG (NULL, foreign or inconsistent record, misaligned buffer),
  * CAPACITY (blob or scratch too small), CUDA. */

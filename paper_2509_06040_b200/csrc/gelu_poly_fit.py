@@ -5,7 +5,8 @@
 2 GELU(x) = x + x erf(x / sqrt 2) = x + s Q(s), s = x^2.  Q (degree 2 in s) is fitted to erf(x / sqrt 2) / x on
 |x| <= 1 so that the largest error of s Q(s) is smallest (weighted least squares with Lawson's reweighting); the
 kernel evaluates in bf16, so the coefficients are rounded to bf16 one after the other, each time refitting the ones
-not yet fixed.  Prints the coefficients, their bf16 bit patterns and the largest error of the rounded polynomial.
+not yet fixed.  (The kernel works on y = 2x and uses the coefficients divided by 2, 8 and 32: exact.)  Prints the
+coefficients, their bf16 bit patterns and the largest error of the rounded polynomial.
 """
 import numpy as np
 from scipy.special import erf
