@@ -436,6 +436,7 @@ def test_prune_masks_bit_exact(B, T, K, splits):
     rbar = rng.standard_normal((2, topo.nodes)).astype(np.float32)
     rbar[1] = np.round(rbar[1])                    # many exact ties
     s.rbar.copy_(torch.from_numpy(rbar))
+    s.adv.copy_(torch.from_numpy(rng.standard_normal(rbar.shape).astype(np.float32)))   # nothing has written it yet: a NaN left in that memory is not equal to itself
     before_adv, before_lat = s.adv.clone(), s.latents.clone()
     pruned = sorted(rng.choice(T, size=min(4, T), replace=False).tolist())
     cases = [(B.WIDTH_NONE, 0, (), False), (B.WIDTH_PER_SPLIT_TOPK, 1, (), False), (B.WIDTH_PER_SPLIT_TOPK, 2, pruned, False),
