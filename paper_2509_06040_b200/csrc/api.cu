@@ -286,10 +286,10 @@ static bgrpo_status prepare_step(bgrpo_tree* t, int32_t split_flag, const float*
 
 // The step's kernel is on the stream.  It summed the previous level's log-probs; its own are pending until the next launch, or
 // until the flush below when the tree is complete.
-static bgrpo_status step_done(bgrpo_tree* t, const StepLaunch& p, const unsigned long long* sums, int per_row, int stride, void* stream) {
+static bgrpo_status step_done(bgrpo_tree* t, const StepLaunch& p, unsigned long long* sums, int per_row, int stride, int clear, void* stream) {
     const int i = t->depth;
     const int32_t W_out = p.W_in * p.fan;
-    t->pending = FinalizeDesc{t->buf.logp, W_out, p.off_out, per_row, t->coef[i].g, t->coef[i].logp_const, sums, stride};
+    t->pending = FinalizeDesc{t->buf.logp, W_out, p.off_out, per_row, t->coef[i].g, t->coef[i].logp_const, sums, stride, clear};
     if (i + 1 == t->desc.T) {
         const cudaError_t e = flush_pending(t, as_stream(stream));
         if (e != cudaSuccess) return cuda_fail(e, "log-prob flush kernel");
@@ -311,7 +311,7 @@ bgrpo_status bgrpo_tree_step(bgrpo_tree* t, int32_t split_flag, const float* v_d
     const cudaError_t e = launch_step(p, as_stream(stream));
     if (e != cudaSuccess) return cuda_fail(e, "step kernel");
     const int warps = step_threads(static_cast<int64_t>(p.n_trees) * p.W_in * p.nchunks) / 32;
-    return step_done(t, p, t->partials_u64(), p.nchunks * warps, p.per_row >> 1, stream);
+    return step_done(t, p, t->partials_u64(), p.nchunks * warps, p.per_row >> 1, 0, stream);
 }
 
 bgrpo_status bgrpo_tree_rollout(bgrpo_tree* t, const uint8_t* split_flags_host, const void* packed_dev, int32_t hidden,
@@ -346,7 +346,7 @@ bgrpo_status bgrpo_tree_rollout(bgrpo_tree* t, const uint8_t* split_flags_host, 
             const cudaError_t e = enqueue_mlp(t, packed_dev, hidden, v_dev, st == BGRPO_OK ? &p : nullptr, &stepped, stream);
             if (e != cudaSuccess) return cuda_fail(e, "mlp kernel");
             if (stepped) {
-                st = step_done(t, p, t->row_sums, 1, 1, stream);
+                st = step_done(t, p, t->row_sums, 1, 1, 1, stream);
                 if (st != BGRPO_OK) return st;
                 continue;
             }

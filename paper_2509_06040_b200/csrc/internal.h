@@ -86,8 +86,10 @@ struct FinalizeDesc {
     int32_t W, off;        // rows off .. off+W-1 of every tree
     int32_t per_row;       // sums per row
     float g, logp_const;
-    const unsigned long long* sums;   // row r's start at sums + r * stride
+    unsigned long long* sums;   // row r's start at sums + r * stride
     int32_t stride;        // the same for every launch of a tree: a level is summed while the next one's sums are written
+    int32_t clear;         // 1: the sums were added up with atomics; whoever takes them leaves zeros for the next who adds (a
+                           // replayed graph that starts after the root kernel, say)
 };
 
 struct LevelInfo {                       // layout of the tree grown so far
@@ -146,7 +148,7 @@ struct bgrpo_tree {
     float s0;
     // scratch carving (device pointers inside buf.scratch)
     int32_t* status;
-    unsigned long long* row_sums;        // [n_trees*nodes_cap] squares of a row's noise, where the MLP stage takes the step; zero until then
+    unsigned long long* row_sums;        // [n_trees*nodes_cap] squares of a row's noise, where the MLP stage takes the step; zero before it and after they were taken
     double* partials;                    // [n_trees*nodes_cap][nchunks][3]   (reward reductions)
     double* node_scratch;                // [n_trees][2][nodes_cap]: per-chain state of the tree reductions when a tree
                                          // is too large for one CTA's shared memory

@@ -179,10 +179,12 @@ __device__ __forceinline__ void finalize_rows(const FinalizeDesc& f, int32_t n_t
         const int tree = idx / f.W;
         const int64_t row = static_cast<int64_t>(tree) * nodes_cap + f.off + (idx - tree * f.W);
         if (!BGRPO_IN_BOUNDS(status, f.off + f.W <= nodes_cap && 2 * per_row <= per_row_cap)) continue;
-        const unsigned long long* q = f.sums + row * f.stride;
+        unsigned long long* q = f.sums + row * f.stride;
         unsigned long long s = 0;
 #pragma unroll 4
         for (int c = lane; c < per_row; c += 32) s += __ldcg(q + c);
+        if (f.clear)
+            for (int c = lane; c < per_row; c += 32) q[c] = 0ull;
         s = warp_sum_u64(s);
         if (lane == 0) f.logp_out[row] = logp_from_squares(s, half_per, f.g, f.logp_const);
     }

@@ -268,3 +268,27 @@ def test_rollout_that_takes_the_step_along_is_the_step_by_step_rollout(B, tokens
         assert torch.equal(r.logp, runs[0].logp)
         assert torch.equal(r.node_table.view(4, n_trees, -1)[:, :, :w.nodes], runs[0].node_table.view(4, n_trees, -1)[:, :, :w.nodes])
         assert torch.equal(r.v.view(-1)[:n], runs[0].v.view(-1)[:n])
+
+
+def test_replayed_rollout_gives_the_same_log_probs_every_time(B):
+    """A rollout captured into a CUDA graph without the root kernel in front of it: every replay writes what the call writes
+    (two tiles a level in clusters of eight, so the step goes along and its sums of squares are added with atomics)."""
+    from paper_2509_06040_b200.session import TreeSession
+    w = Workload(name="replay", n_trees=1, tokens=200, channels=64, T=4, K=2, splits=(0, 2), sigma=0.3,
+                 velocity="mlp", reward="mixture", hidden=1024)
+    inp = make_inputs(w)
+    eager, s = TreeSession(w), TreeSession(w)
+    for r in (eager, s):
+        r.upload_inputs(inp)
+        r.init()
+    B.tree_rollout(eager.tree, eager._split_flags, eager.packed, w.hidden, eager.v)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        B.tree_rollout(s.tree, s._split_flags, s.packed, w.hidden, s.v)
+    for _ in range(3):
+        s.logp[:, 1:].fill_(7.0)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(s.logp, eager.logp) and torch.equal(s.latents, eager.latents)
+    B.tree_sync_status(s.tree)
