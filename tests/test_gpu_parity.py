@@ -429,6 +429,25 @@ def test_fuse_and_advantage_against_enumeration(B, T, K, splits):
     B.tree_sync_status(s.tree)
 
 
+@pytest.mark.parametrize("T,K,splits", [(8, 3, (0, 2, 3, 4, 6)), (7, 3, (0, 1, 2, 3, 4, 5)), (4, 3, (2,)), (6, 2, (0, 2, 5)), (5, 4, (1, 3))])
+def test_equal_rewards_have_no_advantage(B, T, K, splits):
+    """All leaves of a tree with the same reward: every fused value is that reward and every advantage exactly zero (a sum of
+    up to 729 equal float32 is exact in float64, and so is its correctly rounded quotient)."""
+    w, s, topo = _grown_session(B, T, K, splits)
+    for pair in ((0.1, 0.7), (1.0 / 3.0, -2.6), (1234.567, 1e-3), (0.0, 1.0)):
+        r = np.repeat(np.array(pair, dtype=np.float32)[:, None], topo.leaves, axis=1)
+        B.tree_fuse_advantage(s.tree, torch.from_numpy(np.ascontiguousarray(r)).cuda(), 0.0, 1.0, 1e-12, 0.0)
+        torch.cuda.synchronize()
+        assert np.array_equal(s.rbar.cpu().numpy(), np.repeat(r[:, :1], topo.nodes, axis=1)), pair
+        assert not s.adv.cpu().numpy().any(), pair
+    inf = torch.full((2, topo.leaves), float("inf"), device="cuda")      # an infinite reward stays what it was
+    B.tree_fuse_advantage(s.tree, inf, 0.0, 1.0, 1e-6, 0.0)
+    torch.cuda.synchronize()
+    assert bool(torch.isinf(s.rbar).all())
+    with pytest.raises(B.BgrpoError):
+        B.tree_sync_status(s.tree)
+
+
 @pytest.mark.parametrize("T,K,splits", [(16, 2, (0, 3, 6, 9)), (6, 4, (0, 2, 5)), (5, 3, (1, 2, 4)), (20, 2, (0, 5, 10))])
 def test_prune_masks_bit_exact(B, T, K, splits):
     w, s, topo = _grown_session(B, T, K, splits)
