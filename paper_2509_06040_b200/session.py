@@ -46,7 +46,6 @@ class TreeSession:
         self.tree = None
         self.mu = self.target = self.packed = self.v = self.reward_draws = None
         self.pruned_steps = ()
-        self._beta, self._eps, self._adv_clip = (float(np.float32(x)) for x in (w.beta, w.eps, w.adv_clip))
         self._split_flags = np.ascontiguousarray([1 if i in w.splits else 0 for i in range(w.T)], dtype=np.uint8)
 
     # -- inputs ---------------------------------------------------------------------------------------------------
@@ -116,7 +115,8 @@ class TreeSession:
             raise ValueError(w.reward)
 
     def fuse_advantage(self):
-        B.tree_fuse_advantage(self.tree, self.leaf_r, self._beta, 1.0, self._eps, self._adv_clip)
+        w = self.w                                                 # read at every call; the C call takes them as float32
+        B.tree_fuse_advantage(self.tree, self.leaf_r, w.beta, 1.0, w.eps, w.adv_clip)
 
     def prune(self):
         w = self.w
