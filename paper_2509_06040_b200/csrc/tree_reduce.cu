@@ -161,7 +161,8 @@ fuse_advantage_kernel(const __grid_constant__ FuseLaunch p) {
 // Effective sample size of the fusion weights (appendix "Reward Fusion"): ESS(n) = (sum_l w_l)^2 / sum_l w_l^2 over the
 // descendant leaves of n, w_l = exp(beta s_l).  Both sums factorise along the paths like S above:
 //   log S_n = logsumexp_c(a_c + log S_c),   log Q_n = logsumexp_c(2 a_c + log Q_c),   ESS = exp(2 log S - log Q),
-// and along a chain both numerator and denominator pick up the same factor.
+// and along a chain both numerator and denominator pick up the same factor - unless that factor is not finite: nodes of a
+// chain above such an edge have no value.
 __global__ void __launch_bounds__(kTreeThreads)
 fusion_ess_kernel(const __grid_constant__ EssLaunch p) {
     pdl_release();
@@ -179,9 +180,26 @@ fusion_ess_kernel(const __grid_constant__ EssLaunch p) {
     if (!BGRPO_IN_BOUNDS(p.status, chains <= p.nodes && p.nodes <= p.nodes_cap && tree < p.n_trees)) return;
     pdl_wait();
     chain_sums(ls, p.logp + row0, lay, p.runs, p.beta_scaled);
-    for (int m = threadIdx.x; m < chains; m += kTreeThreads) lq[m] = 2.0 * ls[m];      // written by this thread
+    bool odd = false;
+    for (int m = threadIdx.x; m < chains; m += kTreeThreads) {      // written by this thread
+        lq[m] = 2.0 * ls[m];
+        odd = odd || !isfinite(ls[m]);
+    }
     for (int n = lay.off[p.runs.first[R - 1]] + threadIdx.x; n < p.nodes; n += kTreeThreads) p.ess[row0 + n] = 1.0f;
-    __syncthreads();
+    odd = __syncthreads_or(odd) != 0;          // some edge's factor is not finite (no usual case)
+    // The value of chain j of run r at all of its depths; the sums of a chain with such an edge below its first node are lost.
+    auto write_chain = [&](int r, int j, float ess) {
+        for (int d = p.runs.first[r + 1] - 1; d >= p.runs.first[r]; --d) {
+            const int64_t n = row0 + lay.off[d] + j;
+            p.ess[n] = ess;
+            if (odd && d > p.runs.first[r] && !isfinite(p.beta_scaled * static_cast<double>(p.logp[n])))
+                ess = ls[lay.chain0[r] + j] = lq[lay.chain0[r] + j] = NAN;
+        }
+    };
+    if (odd) {
+        for (int j = threadIdx.x; j < chains - lay.chain0[R - 1]; j += kTreeThreads) write_chain(R - 1, j, 1.0f);
+        __syncthreads();
+    }
     for (int r = R - 2; r >= 0; --r) {
         const int fan = p.lv.fanout[p.runs.first[r + 1] - 1];
         const int W = lay.chain0[r + 1] - lay.chain0[r];
@@ -210,8 +228,7 @@ fusion_ess_kernel(const __grid_constant__ EssLaunch p) {
             const double lS = m1 + log(S), lQ = m2 + log(Q);
             ls[me] += lS;
             lq[me] += lQ;
-            const float ess = static_cast<float>(exp(2.0 * lS - lQ));
-            for (int d = p.runs.first[r]; d < p.runs.first[r + 1]; ++d) p.ess[row0 + lay.off[d] + j] = ess;
+            write_chain(r, j, static_cast<float>(exp(2.0 * lS - lQ)));
         }
         __syncthreads();
     }

@@ -713,6 +713,34 @@ def test_path_weighted_fusion_and_ess_on_wide_trees(B, T, K, splits):
     B.tree_sync_status(s.tree)
 
 
+@pytest.mark.parametrize("bad", [float("nan"), float("inf"), float("-inf")])
+def test_ess_has_no_value_above_an_edge_that_is_not_finite(B, bad):
+    """A log-prob that is not finite leaves the effective sample size of every node above its edge without a value, wherever on
+    a chain the edge lies, and all other nodes untouched.  Minus infinity below a fork is a weight of zero among others."""
+    w, s, topo = _grown_session(B, 12, 2, (1, 6), n_trees=1)
+    lp = np.full(topo.nodes, -0.9, dtype=np.float32)
+    ess, ref = torch.empty_like(s.logp), torch.empty_like(s.logp)
+    s.logp.copy_(torch.from_numpy(lp[None]))
+    B.tree_fusion_ess(s.tree, 1.0, 1.0, ref)
+    for n in [1] + [int(topo.level(d)[-1]) for d in (2, 4, 6, 7, 9, 12)]:      # edges into: the first chain, both forks' children, mid-chain, a leaf
+        lp_n = lp.copy()
+        lp_n[n] = bad
+        s.logp.copy_(torch.from_numpy(lp_n[None]))
+        B.tree_fusion_ess(s.tree, 1.0, 1.0, ess)
+        torch.cuda.synchronize()
+        above, q = set(), int(topo.parent[n])
+        while q >= 0:
+            above.add(q)
+            q = int(topo.parent[q])
+        no_weight = bad == float("-inf") and int(topo.depth[n]) - 1 in (1, 6)
+        for q in range(topo.nodes):
+            got = float(ess[0, q])
+            if q in above:
+                assert got < float(ref[0, q]) if no_weight else math.isnan(got), (n, q, got)
+            else:
+                assert got == float(ref[0, q]), (n, q, got)
+
+
 def test_reductions_on_a_tree_larger_than_shared_memory(B):
     """K = 4 with seven splits: 21 845 nodes, more than one CTA's shared memory holds as doubles; the reduction kernels
     keep their per-node state in the caller's scratch instead.  Fusion, advantages, ESS and masks against the oracle."""
