@@ -64,3 +64,54 @@ def test_sizes_beyond_the_built_in_array_are_refused(B):
     assert e.value.status == B.ERR_INVALID_ARG
     torch.cuda.synchronize()
     assert torch.all(out == 3.0)
+
+
+def test_calls_that_overlapped_spoil_no_later_call(B):
+    """Calls on two streams that start together, rows of 63 and of 64 chunks; afterwards ordered calls of either shape give
+    the float64 rewards.  (Only rows of more than 64 chunks share anything, so the overlapping calls come out right as well.)"""
+    g = torch.Generator(device="cuda").manual_seed(1)
+    sizes = (63 * 4096, 64 * 4096)
+    rows, target = [torch.randn(1, D, device="cuda", generator=g) for D in sizes], torch.randn(sizes[1], device="cuda", generator=g)
+    refs = [-((r.double() - target[:D].double()) ** 2).mean(1) for r, D in zip(rows, sizes)]
+    outs = [torch.full((1,), float("nan"), device="cuda") for _ in sizes]
+    streams = [torch.cuda.Stream() for _ in sizes]
+    gate = torch.cuda.Event()
+
+    def call(i):
+        B.reward_mse_static(rows[i], target[:sizes[i]], 1, sizes[i], outs[i])
+
+    def right(i):
+        return bool(((outs[i].double() - refs[i]).abs() <= 1e-6 * refs[i].abs()).all())
+
+    overlapped = True
+    for _ in range(20):
+        torch.cuda._sleep(100_000)
+        gate.record()
+        for i, stream in enumerate(streams):
+            stream.wait_event(gate)
+            with torch.cuda.stream(stream):
+                call(i)
+        torch.cuda.synchronize()
+        overlapped = overlapped and right(0) and right(1)
+        for i in (0, 1):
+            outs[i].fill_(float("nan"))
+            call(i)
+            torch.cuda.synchronize()
+            assert right(i), i
+    assert overlapped
+
+
+@pytest.mark.parametrize("n_rows,D", [(1, 4), (3, 4096), (2, 4100), (5, 8 * 4096), (4, 8 * 4096 + 4), (2, 63 * 4096 + 8), (3, 64 * 4096),
+                                      (3, 64 * 4096 + 4), (9, 100 * 4096 - 4), (1024, 64)])
+def test_rows_where_the_launch_changes(B, n_rows, D):
+    """One CTA, clusters of two to eight, one chunk a CTA and several, and the rows that are too long for a cluster; sums in
+    float64 above sixteen elements, one rounding to float32."""
+    g = torch.Generator(device="cuda").manual_seed(D)
+    rows, target = torch.randn(n_rows, D, device="cuda", generator=g), torch.randn(D, device="cuda", generator=g)
+    out = torch.full((n_rows + 2,), 3.0, device="cuda")
+    for _ in range(2):
+        B.reward_mse_static(rows, target, n_rows, D, out[1:n_rows + 1])
+        torch.cuda.synchronize()
+        ref = -((rows.double() - target.double()) ** 2).mean(1)
+        assert bool(((out[1:n_rows + 1].double() - ref).abs() <= 1e-6 * ref.abs()).all())
+        assert float(out[0]) == 3.0 and float(out[-1]) == 3.0
