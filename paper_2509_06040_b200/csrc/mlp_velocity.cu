@@ -40,6 +40,7 @@
 #include <cuda_bf16.h>
 
 #include <cstring>
+#include <mutex>
 
 #include "internal.h"
 #include "philox.cuh"
@@ -793,41 +794,63 @@ cudaError_t launch_mlp_pack(const uint16_t* W1, const uint16_t* W2, int hidden, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_mlp(const float* latents, int64_t pool_elems, int64_t tree_stride, int64_t row_offset, int n_trees, int64_t tokens_per_tree,
-                       const void* packed, int hidden, float* v_out, int32_t* status, const StepLaunch* step, unsigned long long* row_sums,
-                       bool* stepped, cudaStream_t s) {
-    struct Device {
-        bool known = false;
-        int sms = 0, clusters[kMaxSplit + 1] = {0};       // clusters[S]: how many clusters of S CTAs run at a time
-    };
-    static Device devices[64];
-    constexpr size_t smem = sizeof(MlpSmem) + 1024;
+namespace {
+// What a launch has to know of the current device.  Asked for once per device; host threads may get here together.
+struct MlpDevice {
+    int sms = 0, clusters[kMaxSplit + 1] = {0};       // clusters[S]: how many clusters of S CTAs run at a time
+};
+std::mutex g_mlp_device_mutex;
+struct {
+    bool known = false;
+    MlpDevice device;
+} g_mlp_devices[64];
+
+cudaError_t mlp_query_device(int dev, size_t smem, MlpDevice* d) {
+    cudaError_t e = cudaFuncSetAttribute(mlp_velocity_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(mlp_velocity_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&d->sms, cudaDevAttrMultiProcessorCount, dev);
+    for (int cand = 2; e == cudaSuccess && cand <= kMaxSplit; ++cand) {
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[1];
+        cfg.gridDim = cand;
+        cfg.blockDim = kMlpThreads;
+        cfg.dynamicSmemBytes = smem;
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = static_cast<unsigned int>(cand);
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        e = cudaOccupancyMaxActiveClusters(&d->clusters[cand], mlp_velocity_kernel<true>, &cfg);
+    }
+    return e;
+}
+
+cudaError_t mlp_device(size_t smem, MlpDevice* out) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    Device d;
-    if (dev >= 0 && dev < 64) d = devices[dev];
-    if (!d.known) {
-        e = cudaFuncSetAttribute(mlp_velocity_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(mlp_velocity_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev);
-        for (int cand = 2; e == cudaSuccess && cand <= kMaxSplit; ++cand) {
-            cudaLaunchConfig_t cfg = {};
-            cudaLaunchAttribute attr[1];
-            cfg.gridDim = cand;
-            cfg.blockDim = kMlpThreads;
-            cfg.dynamicSmemBytes = smem;
-            attr[0].id = cudaLaunchAttributeClusterDimension;
-            attr[0].val.clusterDim.x = static_cast<unsigned int>(cand);
-            attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-            cfg.attrs = attr;
-            cfg.numAttrs = 1;
-            e = cudaOccupancyMaxActiveClusters(&d.clusters[cand], mlp_velocity_kernel<true>, &cfg);
-        }
+    std::lock_guard<std::mutex> lock(g_mlp_device_mutex);
+    if (dev < 0 || dev >= 64) return mlp_query_device(dev, smem, out);
+    auto& slot = g_mlp_devices[dev];
+    if (!slot.known) {
+        MlpDevice d;
+        e = mlp_query_device(dev, smem, &d);
         if (e != cudaSuccess) return e;
-        d.known = true;
-        if (dev >= 0 && dev < 64) devices[dev] = d;
+        slot.device = d;
+        slot.known = true;
     }
+    *out = slot.device;
+    return cudaSuccess;
+}
+}  // namespace
+
+cudaError_t launch_mlp(const float* latents, int64_t pool_elems, int64_t tree_stride, int64_t row_offset, int n_trees, int64_t tokens_per_tree,
+                       const void* packed, int hidden, float* v_out, int32_t* status, const StepLaunch* step, unsigned long long* row_sums,
+                       bool* stepped, cudaStream_t s) {
+    constexpr size_t smem = sizeof(MlpSmem) + 1024;
+    MlpDevice d;
+    cudaError_t e = mlp_device(smem, &d);
+    if (e != cudaSuccess) return e;
     MlpArgs a;
     a.latents = latents;
     a.pool_elems = pool_elems;
