@@ -3,6 +3,7 @@
 #include <cstddef>
 #include <cstdint>
 #include <cuda_runtime.h>
+#include <mutex>
 #include <utility>
 
 #include "../../include/bgrpo.h"
@@ -198,6 +199,28 @@ cudaError_t launch_overlapped(void (*kernel)(Params...), dim3 grid, dim3 block, 
     return launch_overlapped_clusters(kernel, grid, block, smem, s, 1, std::forward<Args>(args)...);
 }
 #endif
+
+// The most dynamic shared memory any launch of a kernel takes, allowed once per device.  The limit belongs to the process: set
+// to each launch's own size, a thread could lower it between another thread's setting and its launch.
+struct SharedMemoryLimit {
+    const void* kernel;
+    int bytes;
+    std::mutex mutex;
+    uint64_t devices = 0;      // bit d: allowed on device d
+    SharedMemoryLimit(const void* k, int b) : kernel(k), bytes(b) {}
+    cudaError_t allow() {
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        std::lock_guard<std::mutex> lock(mutex);
+        const uint64_t bit = dev < 64 ? 1ull << dev : 0ull;
+        if (devices & bit) return cudaSuccess;
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        if (e == cudaSuccess) devices |= bit;
+        return e;
+    }
+};
+constexpr size_t kSharedWithoutAsking = 40 * 1024;      // of the 48 KB a launch may take as it is; the rest is for static arrays
 
 // ---- streaming kernels (tree_step.cu) -------------------------------------------------------------------------
 struct StepLaunch {

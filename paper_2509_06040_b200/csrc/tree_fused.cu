@@ -214,6 +214,13 @@ finalize_tree_kernel(const __grid_constant__ FusedLaunch p, int32_t nodes) {
     if (threadIdx.x % THREADS == 0) p.logp[row] = logp_from_squares(s, p.half_per, p.step[step].g, p.step[step].logp_const);
 }
 
+// six open forks with their shared noise, and the sums of a small tree
+constexpr int32_t kSumsInSharedNodes = 1024;
+constexpr int kMostShared = kFusedMaxSplits * kFusedChunkVec * static_cast<int>(sizeof(float4)) * 2 +
+                            kSumsInSharedNodes * (kFusedThreads / 32) * static_cast<int>(sizeof(uint32_t));
+SharedMemoryLimit g_limit_own(reinterpret_cast<const void*>(&rollout_fused_kernel<false>), kMostShared);
+SharedMemoryLimit g_limit_shared(reinterpret_cast<const void*>(&rollout_fused_kernel<true>), kMostShared);
+
 }  // namespace
 
 cudaError_t launch_rollout_fused(const FusedLaunch& p0, int32_t nodes, cudaStream_t s) {
@@ -259,14 +266,12 @@ cudaError_t launch_rollout_fused(const FusedLaunch& p0, int32_t nodes, cudaStrea
     // host time (toy pass, with the rewards' second launch gone as well: 27.8 -> 23.8 us).
     p.nodes = nodes;
     p.sums_at = 0;
-    if (p.nchunks == 1 && nodes <= 1024) {
+    if (p.nchunks == 1 && nodes <= kSumsInSharedNodes) {
         p.sums_at = static_cast<int32_t>(smem / sizeof(float4)) + 1;
         smem += static_cast<size_t>(nodes) * (kFusedThreads / 32) * sizeof(uint32_t);
     }
     cudaError_t e = cudaSuccess;
-    if (smem > 48 * 1024)
-        e = p.shared_noise ? cudaFuncSetAttribute(rollout_fused_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem))
-                           : cudaFuncSetAttribute(rollout_fused_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (smem > kSharedWithoutAsking) e = p.shared_noise ? g_limit_shared.allow() : g_limit_own.allow();
     if (e == cudaSuccess)
         e = p.shared_noise ? launch_overlapped(rollout_fused_kernel<true>, grid, kFusedThreads, smem, s, p)
                            : launch_overlapped(rollout_fused_kernel<false>, grid, kFusedThreads, smem, s, p);

@@ -462,6 +462,10 @@ objective_kernel(const __grid_constant__ ObjectiveLaunch p) {
     }
 }
 
+SharedMemoryLimit g_limit_ess(reinterpret_cast<const void*>(&fusion_ess_kernel), kTreeSmemLimit);
+SharedMemoryLimit g_limit_fuse(reinterpret_cast<const void*>(&fuse_advantage_kernel), kTreeSmemLimit);
+SharedMemoryLimit g_limit_prune(reinterpret_cast<const void*>(&prune_kernel), kTreeSmemLimit);
+
 }  // namespace
 
 cudaError_t launch_objective(const ObjectiveLaunch& p, cudaStream_t s) {
@@ -471,8 +475,8 @@ cudaError_t launch_objective(const ObjectiveLaunch& p, cudaStream_t s) {
 cudaError_t launch_fusion_ess(const EssLaunch& p, cudaStream_t s) {
     size_t smem = static_cast<size_t>(p.runs.chain0[p.runs.n]) * 2 * sizeof(double);
     if (smem > kTreeSmemLimit) smem = 0;          // per-chain state in the caller's scratch
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(fusion_ess_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (smem > kSharedWithoutAsking) {
+        const cudaError_t e = g_limit_ess.allow();
         if (e != cudaSuccess) return e;
     }
     return launch_overlapped(fusion_ess_kernel, p.n_trees, kTreeThreads, smem, s, p);
@@ -481,8 +485,8 @@ cudaError_t launch_fusion_ess(const EssLaunch& p, cudaStream_t s) {
 cudaError_t launch_fuse_advantage(const FuseLaunch& p, cudaStream_t s) {
     size_t smem = static_cast<size_t>(p.runs.chain0[p.runs.n]) * 2 * sizeof(double);
     if (smem > kTreeSmemLimit) smem = 0;          // per-chain state in the caller's scratch
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(fuse_advantage_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (smem > kSharedWithoutAsking) {
+        const cudaError_t e = g_limit_fuse.allow();
         if (e != cudaSuccess) return e;
     }
     return launch_overlapped(fuse_advantage_kernel, p.n_trees, kTreeThreads, smem, s, p);
@@ -491,8 +495,8 @@ cudaError_t launch_fuse_advantage(const FuseLaunch& p, cudaStream_t s) {
 cudaError_t launch_prune(const PruneLaunch& p, cudaStream_t s) {
     size_t smem = static_cast<size_t>(p.runs.chain0[p.runs.n]);
     if (smem > kTreeSmemLimit) smem = 0;          // the paths are walked node by node, Extreme-b flags live in the mask
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(prune_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (smem > kSharedWithoutAsking) {
+        const cudaError_t e = g_limit_prune.allow();
         if (e != cudaSuccess) return e;
     }
     return launch_overlapped(prune_kernel, p.n_trees, kTreeThreads, smem, s, p);

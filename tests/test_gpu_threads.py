@@ -2,11 +2,24 @@
 import os
 import subprocess
 import sys
+import threading
 
 import pytest
+import torch
+
+from workloads import Workload, make_inputs
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2509_06040_b200 import binding
+    return binding
+
 
 FIRST_CALLS = """
 import threading, sys
@@ -45,3 +58,39 @@ def test_first_velocity_calls_of_several_threads():
     """The stage asks its device once how many clusters fit; threads that get there together all launch the same split."""
     out = subprocess.run([sys.executable, "-c", FIRST_CALLS], cwd=ROOT, capture_output=True, text=True, timeout=300)
     assert out.returncode == 0 and "same bits" in out.stdout, out.stderr[-2000:]
+
+
+def test_whole_tree_rollouts_of_different_depth_in_two_threads(B):
+    """Trees whose open forks take 96 and 64 KB of shared memory, rolled out over and over by two threads: no launch is refused
+    and each tree comes out as on its own."""
+    from paper_2509_06040_b200.session import TreeSession
+    sessions = []
+    for splits in ((1, 2, 3, 4, 5, 6), (1, 2, 3, 4)):           # three trees an SM: no fork is dealt out to the grid
+        w = Workload(name="threads", n_trees=444, tokens=9, channels=4, T=splits[-1] + 1, K=2, splits=splits, sigma=0.3, velocity="linear",
+                     reward="neg_mse_mu", branch_corr_s=2.0)
+        s = TreeSession(w)
+        s.upload_inputs(make_inputs(w))
+        s.rollout()
+        sessions.append(s)
+    torch.cuda.synchronize()
+    alone = [s.latents.clone() for s in sessions]
+    together, errors = threading.Barrier(2), []
+
+    def work(s):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                together.wait()
+                for _ in range(1000):
+                    s.rollout()
+        except Exception as e:
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(s,)) for s in sessions]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not errors, errors
+    for s, ref in zip(sessions, alone):
+        assert torch.equal(s.latents, ref)
