@@ -34,14 +34,21 @@ constexpr int kFusedVec = 4;
 constexpr int kFusedCtasPerSm = 4;
 constexpr int kFusedChunkVec = kFusedThreads * kFusedVec;   // float4 of a row per CTA
 constexpr int kFusedMaxSplits = 6;
-// log-prob partials of the whole-tree kernel per node row: one 32-bit word per warp of every CTA that covers the row
-inline int64_t fused_partials_per_row(int64_t D) { return ((D / 4 + kFusedChunkVec - 1) / kFusedChunkVec) * (kFusedThreads / 32); }
+// log-prob partials of the whole-tree kernel per node row: one 32-bit word per warp of every CTA that covers the row, two with
+// shared noise (a half-warp's squares each: see the bound in tree_fused.cu)
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+constexpr int fused_words_per_cta(bool shared_noise) { return kFusedThreads / 32 * (shared_noise ? 2 : 1); }
+inline int64_t fused_partials_per_row(int64_t D, bool shared_noise) {
+    return ((D / 4 + kFusedChunkVec - 1) / kFusedChunkVec) * fused_words_per_cta(shared_noise);
+}
 // 32-bit words of log-prob partials reserved per node row: the larger of the rollout kernels' layouts (64 bits per chunk and
 // warp in the step kernel); an even number, so that every row starts on 8 bytes
 inline int64_t partials_per_row(int64_t D) {
     const int64_t D4 = D / 4;
     const int64_t step = ((D4 + kStepChunkVec - 1) / kStepChunkVec) * (kStepThreadsSmall / 32) * 2;
-    const int64_t fused = fused_partials_per_row(D);
+    const int64_t fused = fused_partials_per_row(D, true);
     return step > fused ? step : fused;
 }
 constexpr int kScratchHeader = 256;    // bytes reserved at the start of scratch for the status word
@@ -305,7 +312,7 @@ struct FusedLaunch {
     const float* mu;           // [n_trees][D]
     float* logp;
     int32_t* table;
-    uint32_t* partials;        // [rows][per_row]: one word per warp of the CTAs that cover a row
+    uint32_t* partials;        // [rows][per_row]: fused_words_per_cta() words per CTA that covers a row
     int32_t* status;           // the tree's status word
     int32_t per_row_cap;       // words reserved per node row
     int64_t D;

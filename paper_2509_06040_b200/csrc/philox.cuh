@@ -152,9 +152,11 @@ __device__ __forceinline__ uint4 philox_from(const NoiseElement& e, const NoiseN
 // Log-prob sums of the rollout kernels.  The squares of four normals (at most 2 * 33.3 with independent noise, twice that
 // with a shared part) are rounded to a multiple of 2^-18 - 2e-6 of their mean, the rounding of a float32 log-prob of four
 // elements - and added as integers: sums are exact from there on, so they do not depend on how a kernel cuts the row, and
-// the level-by-level and the whole-tree kernel agree bit for bit.  One thread may add up to eight (2^31), one warp's sum of
-// at most two per lane fits 32 bits.
+// the level-by-level and the whole-tree kernel agree bit for bit.  A thread may add up to 32 of them in 32 bits (2^30 for eight);
+// what a warp adds is bounded where it is added.
 constexpr float kSquareScale = 262144.0f;
+constexpr double kMostSquares = 66.6;          // of four normals: two r^2 = -2 ln u of u >= 2^-24; twice that with a shared part
+static_assert(8 * 2 * kMostSquares * kSquareScale < 2147483648.0, "a thread of the step kernel adds eight");
 __device__ __forceinline__ uint32_t quantized_squares(float squares) { return __float2uint_rn(squares * kSquareScale); }
 __device__ __forceinline__ float squares_of(const float4& x) { return fmaf(x.x, x.x, fmaf(x.y, x.y, fmaf(x.z, x.z, x.w * x.w))); }
 // the log-prob of an edge from its row's sum: -(1/D) sum (z' - mean)^2 / (2 g^2) + const with (z' - mean)^2 = g^2 xi^2

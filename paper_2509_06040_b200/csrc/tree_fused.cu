@@ -27,12 +27,14 @@
 namespace bgrpo {
 namespace {
 
-constexpr uint32_t kNotMine = 0xffffffffu;          // no warp's sum: that is at most 128 squares of 133 * 2^18
+constexpr uint32_t kNotMine = 0xffffffffu;          // no sum of a warp, or with shared noise of half a warp
+static_assert(32 * kFusedVec * kMostSquares * kSquareScale < 4294967295.0, "a warp's sum in 32 bits");
+static_assert(16 * kFusedVec * 2 * kMostSquares * kSquareScale < 4294967295.0, "a half-warp's sum with shared noise in 32 bits");
 
 template <bool SHARED>
 __global__ void __launch_bounds__(kFusedThreads, kFusedCtasPerSm)
 rollout_fused_kernel(const __grid_constant__ FusedLaunch p) {
-    constexpr int VEC = kFusedVec;
+    constexpr int VEC = kFusedVec, WORDS = fused_words_per_cta(SHARED);
     extern __shared__ float4 s_stack[];             // [open fork][VEC] means, SHARED: and as many xi_0; rows of one CTA: the sums of all nodes
     pdl_release();
     const int chunk = blockIdx.x % p.nchunks;
@@ -59,11 +61,11 @@ rollout_fused_kernel(const __grid_constant__ FusedLaunch p) {
         live[k] = e[k] < D4;
         el[k] = noise_element(e[k], BGRPO_TAG_INNOV, p.keys);
     }
-    if (!BGRPO_IN_BOUNDS(p.status, tree < p.n_trees && static_cast<uint32_t>(chunk) * VEC * kFusedThreads < D4 && (chunk + 1) * (kFusedThreads / 32) <= p.per_row &&
+    if (!BGRPO_IN_BOUNDS(p.status, tree < p.n_trees && static_cast<uint32_t>(chunk) * VEC * kFusedThreads < D4 && (chunk + 1) * WORDS <= p.per_row &&
                                        p.per_row <= p.per_row_cap)) return;
-    uint32_t* const partials = p.partials + row0 * p.per_row + chunk * (kFusedThreads / 32) + warp;
+    uint32_t* const partials = p.partials + row0 * p.per_row + chunk * WORDS + warp * (WORDS * 32 / kFusedThreads);
     // a row that is one CTA's alone: its sums stay here and the CTA writes the log-probs of the nodes it makes
-    uint32_t (*const s_sums)[kFusedThreads / 32] = p.sums_at > 0 ? reinterpret_cast<uint32_t (*)[kFusedThreads / 32]>(s_stack + p.sums_at - 1) : nullptr;
+    uint32_t (*const s_sums)[WORDS] = p.sums_at > 0 ? reinterpret_cast<uint32_t (*)[WORDS]>(s_stack + p.sums_at - 1) : nullptr;
     if (s_sums) {
         for (int n = threadIdx.x; n < p.nodes; n += kFusedThreads) s_sums[n][0] = kNotMine;
         __syncthreads();
@@ -135,10 +137,19 @@ rollout_fused_kernel(const __grid_constant__ FusedLaunch p) {
 #pragma unroll
             for (int k = 0; k < VEC; ++k)
                 if (live[k]) __stcs(row + e[k], z[k]);
-            acc = __reduce_add_sync(0xffffffffu, acc);
-            if (lane == 0) {
-                if (s_sums) s_sums[child][warp] = acc;
-                else partials[static_cast<uint64_t>(child) * static_cast<uint32_t>(p.per_row)] = acc;
+            if (SHARED) {
+                const uint32_t low = __reduce_add_sync(0xffffffffu, lane < 16 ? acc : 0u), high = __reduce_add_sync(0xffffffffu, lane < 16 ? 0u : acc);
+                if (lane == 0) {
+                    uint32_t* const out = s_sums ? s_sums[child] + 2 * warp : partials + static_cast<uint64_t>(child) * static_cast<uint32_t>(p.per_row);
+                    out[0] = low;
+                    out[1] = high;
+                }
+            } else {
+                acc = __reduce_add_sync(0xffffffffu, acc);
+                if (lane == 0) {
+                    if (s_sums) s_sums[child][warp] = acc;
+                    else partials[static_cast<uint64_t>(child) * static_cast<uint32_t>(p.per_row)] = acc;
+                }
             }
             if (writes_table) {
                 const int64_t rows = static_cast<int64_t>(p.n_trees) * p.nodes_cap, r = row0 + child;
@@ -176,7 +187,7 @@ rollout_fused_kernel(const __grid_constant__ FusedLaunch p) {
         if (n == 0 || s_sums[n][0] == kNotMine) continue;
         unsigned long long s = 0;
 #pragma unroll
-        for (int w = 0; w < kFusedThreads / 32; ++w) s += s_sums[n][w];
+        for (int w = 0; w < WORDS; ++w) s += s_sums[n][w];
         int step = 0;                                       // the node's depth is step + 1
         while (step + 1 < p.T && static_cast<uint32_t>(n) >= (p.step[step + 1].child0 & ~kForks)) ++step;
         p.logp[row0 + n] = logp_from_squares(s, p.half_per, p.step[step].g, p.step[step].logp_const);
@@ -217,7 +228,7 @@ finalize_tree_kernel(const __grid_constant__ FusedLaunch p, int32_t nodes) {
 // six open forks with their shared noise, and the sums of a small tree
 constexpr int32_t kSumsInSharedNodes = 1024;
 constexpr int kMostShared = kFusedMaxSplits * kFusedChunkVec * static_cast<int>(sizeof(float4)) * 2 +
-                            kSumsInSharedNodes * (kFusedThreads / 32) * static_cast<int>(sizeof(uint32_t));
+                            kSumsInSharedNodes * fused_words_per_cta(true) * static_cast<int>(sizeof(uint32_t));
 SharedMemoryLimit g_limit_own(reinterpret_cast<const void*>(&rollout_fused_kernel<false>), kMostShared);
 SharedMemoryLimit g_limit_shared(reinterpret_cast<const void*>(&rollout_fused_kernel<true>), kMostShared);
 
@@ -235,7 +246,7 @@ cudaError_t launch_rollout_fused(const FusedLaunch& p0, int32_t nodes, cudaStrea
     }
     const int64_t D4 = p.D / 4;
     p.nchunks = static_cast<int32_t>((D4 + kFusedChunkVec - 1) / kFusedChunkVec);
-    p.per_row = static_cast<int32_t>(fused_partials_per_row(p.D));
+    p.per_row = static_cast<int32_t>(fused_partials_per_row(p.D, p.shared_noise != 0));
     // Dealing out a fork more makes K times as many CTAs that walk a shorter subtree but compute the prefix again.  An SM works
     // at the same rate from about three CTAs on, so the time goes with the CTAs of the busiest SM (at least three) times the
     // nodes a CTA walks.  Measured, us a rollout, forks dealt out 0 / 1 / 2 / 3 (the rule's choice in brackets): four trees of
@@ -262,13 +273,13 @@ cudaError_t launch_rollout_fused(const FusedLaunch& p0, int32_t nodes, cudaStrea
     if (items <= 0 || items > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     const unsigned int grid = static_cast<unsigned int>(items);
     size_t smem = static_cast<size_t>(p.levels) * kFusedChunkVec * sizeof(float4) * (p.shared_noise ? 2 : 1);
-    // Rows of one CTA keep their sums in shared memory (up to 16 KB of them) and need no second launch, which costs about 4 us of
+    // Rows of one CTA keep their sums in shared memory (up to 16 KB of them, 32 with shared noise) and need no second launch, which costs about 4 us of
     // host time (toy pass, with the rewards' second launch gone as well: 27.8 -> 23.8 us).
     p.nodes = nodes;
     p.sums_at = 0;
     if (p.nchunks == 1 && nodes <= kSumsInSharedNodes) {
         p.sums_at = static_cast<int32_t>(smem / sizeof(float4)) + 1;
-        smem += static_cast<size_t>(nodes) * (kFusedThreads / 32) * sizeof(uint32_t);
+        smem += static_cast<size_t>(nodes) * fused_words_per_cta(p.shared_noise != 0) * sizeof(uint32_t);
     }
     cudaError_t e = cudaSuccess;
     if (smem > kSharedWithoutAsking) e = p.shared_noise ? g_limit_shared.allow() : g_limit_own.allow();

@@ -904,7 +904,9 @@ def test_logprob_families_at_their_edges(B, tokens, channels, n_trees, T, K, spl
     (1, 4, 3, 4, 3, (0, 2), 1.0),                 # one float4 a row; every fork dealt out to the grid
     (9, 4, 1, 20, 2, (0, 1, 2, 3, 4, 5), math.inf),   # 1023 nodes: the rows' sums stay in shared memory
     (9, 4, 1, 21, 2, (0, 1, 2, 3, 4, 5), math.inf),   # 1087 nodes: they do not
-    (9, 4, 450, 6, 2, (0, 1, 2, 3, 4, 5), 2.0),   # no fork dealt out: six open forks with their shared noise in shared memory
+    (9, 4, 450, 6, 2, (0, 1, 2, 3, 4, 5), 2.0),   # two forks dealt out, four open ones with their shared noise in shared memory
+    (9, 4, 444, 7, 2, (1, 2, 3, 4, 5, 6), 2.0),   # three trees an SM, no fork dealt out: six open forks
+    (513, 4, 444, 7, 2, (1, 2, 3, 4, 5, 6), 2.0),     # the same with rows of two CTAs
 ])
 def test_step_and_whole_tree_launches_agree_where_their_shapes_change(B, tokens, channels, n_trees, T, K, splits, s):
     """The two rollouts share the noise stream, the float32 expressions and the integer sums, and nothing of their launch
