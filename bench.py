@@ -623,12 +623,14 @@ def run_ours(args, w):
     ev = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(args.steps)]
     sampler = ClockSampler(local) if rank == 0 else None
     sync_all()
+    launches = -B.launch_count()
     for k in range(args.steps):
         if flush:
             flush_buf.fill_(float(k))
         ev[k][0].record()
         s.run_all(seed=w.seed + 1000 + k)
         ev[k][1].record()
+    launches += B.launch_count()
     sync_all()
     clocks = sampler.stop() if sampler else None
     total_ms = grp.max(sum(a.elapsed_time(b) for a, b in ev))
@@ -727,7 +729,6 @@ def run_ours(args, w):
     savings = None
     if rank == 0 and world == 1 and not args.no_also:
         savings = savings_line(w, s, f"cuda:{local}", max(3, min(10, args.steps)))
-    launches = s.kernel_launches_per_pass() * args.steps
     dtype = "f32" if w.velocity == "linear" else "f32 (step) + bf16/f32-accumulate (MLP velocity)"
     rollout_kind = "one launch" if s.fused_rollout else "one tree_step per depth"
     del s, stage, flush_buf

@@ -315,6 +315,9 @@ void        bgrpo_tree_destroy(bgrpo_tree* tree);
 const char* bgrpo_status_string(bgrpo_status status);
 /* Last CUDA error text seen by this thread's most recent failing call ("" if none). */
 const char* bgrpo_last_error(void);
+/* Kernels this host thread has enqueued through the library so far (no counterpart in the paper): what a program that
+ * counts its launches takes the difference of, whatever the library chose to launch. */
+int64_t     bgrpo_launch_count(void);
 
 #ifdef __cplusplus
 }

@@ -94,6 +94,7 @@ _SIGNATURES = {
     "bgrpo_tree_destroy": (None, [C.c_void_p]),
     "bgrpo_status_string": (C.c_char_p, [C.c_int]),
     "bgrpo_last_error": (C.c_char_p, []),
+    "bgrpo_launch_count": (C.c_int64, []),
 }
 for _name, (_res, _args) in _SIGNATURES.items():
     _fn = getattr(lib, _name)       # AttributeError here = the library does not export a declared symbol
@@ -138,6 +139,10 @@ class Tree:
         if getattr(self, "handle", None) and lib is not None:     # `lib` is gone at interpreter shutdown
             lib.bgrpo_tree_destroy(self.handle)
             self.handle = None
+
+
+def launch_count() -> int:
+    return lib.bgrpo_launch_count()
 
 
 def make_desc(n_trees, tokens, channels, T, K, nodes_cap, sigma, t_grid, seed, branch_corr_s=math.inf, tree_id_base=0):

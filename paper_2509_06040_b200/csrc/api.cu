@@ -140,6 +140,8 @@ const char* bgrpo_status_string(bgrpo_status s) {
 
 const char* bgrpo_last_error(void) { return g_last_error; }
 
+int64_t bgrpo_launch_count(void) { return launch_count(); }
+
 bgrpo_status bgrpo_tree_workspace(const bgrpo_tree_desc* desc, bgrpo_sizes* out) {
     if (!out) return fail(BGRPO_ERR_INVALID_ARG, "out is NULL");
     bgrpo_status st = check_desc(desc);

@@ -181,6 +181,16 @@ namespace bgrpo {
 // on the stream is still draining, so the gap between two dependent launches shrinks to the set-up the new kernel can do
 // on its own.  Such a kernel calls pdl_wait() before it touches anything an earlier kernel wrote or still reads, and
 // pdl_release() as early as it likes to let its own successor in.
+//
+// Kernels the calling host thread has enqueued so far (bgrpo_launch_count): every launch goes through count_launch().
+inline int64_t& launch_count() {
+    thread_local int64_t n = 0;
+    return n;
+}
+inline cudaError_t count_launch(cudaError_t e) {
+    if (e == cudaSuccess) ++launch_count();
+    return e;
+}
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
@@ -199,7 +209,7 @@ cudaError_t launch_overlapped_clusters(void (*kernel)(Params...), dim3 grid, dim
     attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = cluster > 1 ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+    return count_launch(cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...));
 }
 template <typename... Params, typename... Args>
 cudaError_t launch_overlapped(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args&&... args) {

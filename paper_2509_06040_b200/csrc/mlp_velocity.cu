@@ -791,7 +791,7 @@ size_t mlp_packed_bytes(int hidden) { return static_cast<size_t>(hidden / kHc) *
 cudaError_t launch_mlp_pack(const uint16_t* W1, const uint16_t* W2, int hidden, void* packed, cudaStream_t s) {
     const int n = hidden * kCh;
     mlp_pack_kernel<<<(n + 255) / 256, 256, 0, s>>>(W1, W2, hidden, static_cast<unsigned char*>(packed));
-    return cudaGetLastError();
+    return count_launch(cudaGetLastError());
 }
 
 namespace {

@@ -260,7 +260,7 @@ cudaError_t launch_step_threads(const StepLaunch& p, unsigned int grid, cudaStre
 
 cudaError_t launch_debug_trip(int32_t* status, cudaStream_t s) {
     debug_trip_kernel<<<1, 32, 0, s>>>(status);
-    return cudaGetLastError();
+    return count_launch(cudaGetLastError());
 }
 
 cudaError_t launch_root(const bgrpo_tree* t, cudaStream_t s) {
@@ -291,14 +291,14 @@ cudaError_t launch_philox_words(uint64_t seed, uint32_t node, uint32_t step, uin
     if (nblk <= 0) return cudaSuccess;
     philox_words_kernel<<<static_cast<unsigned int>((nblk + 255) / 256), 256, 0, s>>>(
         make_philox_keys(seed), node, step, tag, reinterpret_cast<uint4*>(out), nblk);
-    return cudaGetLastError();
+    return count_launch(cudaGetLastError());
 }
 cudaError_t launch_philox_normals(uint64_t seed, uint32_t node, uint32_t step, uint32_t tag, float* out, int64_t n, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
     const int64_t nblk = n / 4;
     philox_normals_kernel<<<static_cast<unsigned int>((nblk + 255) / 256), 256, 0, s>>>(
         make_philox_keys(seed), node, step, tag, reinterpret_cast<float4*>(out), nblk);
-    return cudaGetLastError();
+    return count_launch(cudaGetLastError());
 }
 
 }  // namespace bgrpo

@@ -46,6 +46,7 @@ class TreeSession:
         self.tree = None
         self.mu = self.target = self.packed = self.v = self.reward_draws = None
         self.pruned_steps = ()
+        self._pass_launches = None
         self._split_flags = np.ascontiguousarray([1 if i in w.splits else 0 for i in range(w.T)], dtype=np.uint8)
 
     # -- inputs ---------------------------------------------------------------------------------------------------
@@ -124,24 +125,15 @@ class TreeSession:
 
     def run_all(self, seed=None):
         """One pass of the whole path over this batch."""
+        before = B.launch_count()
         self.rollout(seed)
         self.rewards()
         self.fuse_advantage()
         self.prune()
+        self._pass_launches = B.launch_count() - before
 
     def kernel_launches_per_pass(self) -> int:
-        w = self.w
-        if w.velocity == "linear" and len(w.splits) <= 6:
-            n = 1 + (1 if w.D <= 2048 and w.nodes <= 1024 else 2)  # root + whole-tree rollout (+ its log-prob sums)
-        elif w.velocity == "mlp":
-            # root + mlp (+ step, where the mlp launch does not take it along: tiles that are not split) per depth + log-prob flush
-            sms = torch.cuda.get_device_properties(self.latents.device).multi_processor_count
-            tiles = [-(-self.n_trees * W * w.tokens // 128) for W in w.widths()[:w.T]]
-            split = [any(w.hidden // 128 % c == 0 and n * c <= sms for c in range(2, 9)) for n in tiles]
-            n = 1 + sum(1 if along else 2 for along in split) + 1
-        else:
-            n = 1 + w.T + 1                                        # root + step per depth + log-prob flush
-        if w.reward in ("neg_mse_mu", "neg_mse_target", "normal_plus_cos"):
-            n += 1 if w.D <= 16384 else 2                          # partial sums (+ their fixed-order total)
-        n += 2                                                     # fuse+advantage, prune
-        return n
+        """Kernels of the library that run_all() enqueues, as counted in the last pass (it takes one if there was none)."""
+        if self._pass_launches is None:
+            self.run_all()
+        return self._pass_launches

@@ -292,3 +292,31 @@ def test_replayed_rollout_gives_the_same_log_probs_every_time(B):
         torch.cuda.synchronize()
         assert torch.equal(s.logp, eager.logp) and torch.equal(s.latents, eager.latents)
     B.tree_sync_status(s.tree)
+
+
+@pytest.mark.parametrize("tokens,channels,n_trees,T,K,splits,velocity,hidden,reward", [
+    (16, 4, 1, 4, 2, (0, 2), "linear", 0, "neg_mse_target"),            # one-launch rollout and rewards
+    (513, 4, 2, 8, 2, (0, 1, 2, 3, 4, 5, 6), "linear", 0, "mixture"),   # seven splits: step by step
+    (300, 64, 2, 3, 2, (0,), "mlp", 1024, "normal_plus_cos"),           # the step goes along
+    (45 * 128, 64, 1, 2, 1, (), "mlp", 1152, "mixture"),                # nine chunks: 45 tiles fit as clusters of three,
+    (46 * 128, 64, 1, 2, 1, (), "mlp", 1152, "mixture"),                # 46 and 49 do not
+    (49 * 128, 64, 1, 2, 1, (), "mlp", 1152, "neg_mse_target"),
+])
+def test_launches_of_a_pass_are_counted(B, tokens, channels, n_trees, T, K, splits, velocity, hidden, reward):
+    """The session's count of a pass against the kernel nodes of the same pass captured into a graph."""
+    from cuda.bindings import runtime
+    from paper_2509_06040_b200.session import TreeSession
+    w = Workload(name="count", n_trees=n_trees, tokens=tokens, channels=channels, T=T, K=K, splits=splits, sigma=0.3,
+                 velocity=velocity, reward=reward, hidden=hidden or 3072)
+    s = TreeSession(w)
+    s.upload_inputs(make_inputs(w))
+    s.run_all()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        s.run_all()
+    raw = runtime.cudaGraph_t(graph.raw_cuda_graph())
+    _, _, n = runtime.cudaGraphGetNodes(raw)
+    _, nodes, n = runtime.cudaGraphGetNodes(raw, n)
+    kernels = sum(1 for q in nodes if runtime.cudaGraphNodeGetType(q)[1] == runtime.cudaGraphNodeType.cudaGraphNodeTypeKernel)
+    assert s.kernel_launches_per_pass() == kernels > 0
