@@ -16,7 +16,6 @@ from dataclasses import dataclass
 from typing import Optional, Sequence
 
 import numpy as np
-import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 # BGRPO_DEBUG_BOUNDS=1 selects the build whose kernels check every index they derive (python -m ...build --debug-bounds)
@@ -116,12 +115,26 @@ def _ptr(t) -> Optional[int]:
     return t.data_ptr()
 
 
+_shortcut = None      # (torch.cuda.is_initialized, current device, raw handle of its current stream); (): this torch has no such functions
+
+
+def _find_shortcut():
+    import torch
+    found = (torch.cuda.is_initialized, getattr(torch._C, "_cuda_getDevice", None), getattr(torch._C, "_cuda_getCurrentRawStream", None))
+    return () if None in found else found
+
+
 def _stream(stream) -> Optional[int]:
+    global _shortcut
     if stream is None:
         # The raw handle of the current stream, without the Stream object and the device probing around it (0.3 us instead
-        # of 4.3 us: as much as a kernel launch, on every call of a launch-bound program).
-        if torch.cuda.is_initialized():
-            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()) or None
+        # of 4.3 us: as much as a kernel launch, on every call of a launch-bound program).  torch offers it for generated code
+        # and not as an interface: without it, the Stream object.
+        if _shortcut is None:
+            _shortcut = _find_shortcut()
+        if _shortcut and _shortcut[0]():
+            return _shortcut[2](_shortcut[1]()) or None
+        import torch
         if not torch.cuda.is_available():
             return None
         return torch.cuda.current_stream().cuda_stream or None

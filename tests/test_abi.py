@@ -106,3 +106,24 @@ def test_binding_refuses_to_import_without_the_library(tmp_path):
                          env={k: v for k, v in os.environ.items() if k != "PYTHONPATH"})
     assert out.returncode != 0
     assert "libbgrpo.so is missing" in out.stderr and "no CPU or PyTorch fallback" in out.stderr
+
+
+def test_binding_needs_no_torch_to_load_and_no_private_torch_function(B, monkeypatch):
+    """A caller that passes its own streams loads the binding without torch; a torch without the raw-stream shortcut gives the
+    same stream through the Stream object."""
+    import subprocess
+    import sys
+    code = "import sys; import paper_2509_06040_b200.binding as B; assert 'torch' not in sys.modules; assert B._stream(7) == 7"
+    out = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
+    assert out.returncode == 0, out.stderr[-1000:]
+
+    import types
+    import torch
+    monkeypatch.setattr(torch.cuda, "is_initialized", lambda: True)
+    monkeypatch.setattr(torch.cuda, "is_available", lambda: True)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=11))
+    for shortcut, expected in ((None, 11), (lambda device: 5 if device == 2 else None, 5)):
+        monkeypatch.setattr(B, "_shortcut", None)
+        monkeypatch.setattr(torch._C, "_cuda_getDevice", lambda: 2, raising=False)
+        monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", shortcut, raising=False)
+        assert B._stream(None) == expected and B._stream(None) == expected
