@@ -14,16 +14,19 @@ constexpr int kStreamThreads = 256;    // threads per CTA of the root / reward k
 constexpr int kChunkVec = 1024;        // float4 per (row, chunk) work item of the root kernel
 constexpr int kRewardVec = 16;         // float4 of a row per thread of the leaf-reward kernel
 constexpr int kRewardChunkVec = kStreamThreads * kRewardVec;   // float4 per (row, chunk) work item of the leaf-reward kernel
-// Step kernel: 64-thread CTAs, 8 float4 per thread.  Measured on B200 against 128/256-thread CTAs, 2/4/6 float4 per
-// thread, persistent grids and a shared-memory ring fed by bulk asynchronous copies: the kernel is bound by
-// instruction issue (Philox + Box-Muller), and eight independent noise chains per thread with many small CTAs
-// per SM gave the best rate on both the 8 B/element and the 12 B/element workloads.
+// Step kernel: 128-thread CTAs, 4 float4 per thread, four CTAs per SM so that 128 registers hold a thread's loads and noise.
+// What bounds it is HBM, as far as loads are in flight while other warps draw noise.  16 steps of 32 image trees (12 B/element,
+// 4.2 GB) in 1 140 us; 64 threads of 8 float4, eight CTAs per SM - the same warps, in smaller CTAs - took 1 200 us, five CTAs of
+// 128 threads (96 registers) 1 170 us, eight (64 registers, spills) 1 160 us and on a video tree 622 us for 598.
 // A launch of less than four such CTAs per SM has no throughput to lose: it takes as long as one thread's work, so the same
 // chunk goes to 256 threads of 2 float4.
-constexpr int kStepThreads = 64, kStepThreadsSmall = 256;
-constexpr int kStepVec = 8;
+constexpr int kStepThreads = 128, kStepThreadsSmall = 256;
+constexpr int kStepVec = 4;
 constexpr int kStepChunkVec = kStepThreads * kStepVec;   // 512 float4 = 8 KiB per operand tile
-constexpr int kStepCtasPerSm = 8, kStepCtasPerSmSmall = 4;
+// Three or four children with noise of their own store more than they load: a fifth CTA is worth more there than the registers
+// (16 image trees, forks of three and of four: 1 168 -> 1 149 us, 2 621 -> 2 598 us).
+constexpr int step_ctas_per_sm(int fan, bool shared_noise) { return fan >= 3 && !shared_noise ? 5 : 4; }
+constexpr int kStepCtasPerSmSmall = 4;
 constexpr int64_t kStepSmallGrid = 148 * 4;
 inline int step_threads(int64_t items) { return items < kStepSmallGrid ? kStepThreadsSmall : kStepThreads; }
 // Whole-tree rollout kernel: 128-thread CTAs, 4 float4 per thread (1 and 2 measured 37 and 16 % slower on the video tree), four

@@ -152,11 +152,10 @@ __device__ __forceinline__ uint4 philox_from(const NoiseElement& e, const NoiseN
 // Log-prob sums of the rollout kernels.  The squares of four normals (at most 2 * 33.3 with independent noise, twice that
 // with a shared part) are rounded to a multiple of 2^-18 - 2e-6 of their mean, the rounding of a float32 log-prob of four
 // elements - and added as integers: sums are exact from there on, so they do not depend on how a kernel cuts the row, and
-// the level-by-level and the whole-tree kernel agree bit for bit.  A thread may add up to 32 of them in 32 bits (2^30 for eight);
-// what a warp adds is bounded where it is added.
+// the level-by-level and the whole-tree kernel agree bit for bit.  A thread may add up to 30 of them in 32 bits; what a
+// warp adds is bounded where it is added.
 constexpr float kSquareScale = 262144.0f;
 constexpr double kMostSquares = 66.6;          // of four normals: two r^2 = -2 ln u of u >= 2^-24; twice that with a shared part
-static_assert(8 * 2 * kMostSquares * kSquareScale < 2147483648.0, "a thread of the step kernel adds eight");
 __device__ __forceinline__ uint32_t quantized_squares(float squares) { return __float2uint_rn(squares * kSquareScale); }
 __device__ __forceinline__ float squares_of(const float4& x) { return fmaf(x.x, x.x, fmaf(x.y, x.y, fmaf(x.z, x.z, x.w * x.w))); }
 // the log-prob of an edge from its row's sum: -(1/D) sum (z' - mean)^2 / (2 g^2) + const with (z' - mean)^2 = g^2 xi^2
@@ -171,24 +170,35 @@ __device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long x)
     return x;
 }
 
-// Adds up the pending level's partial sums: one warp per row.
+// Adds up a row of the pending level: THREADS threads of a CTA, `t` the thread's number among them; thread 0 writes.
+// s_sum: the CTA's, when more than a warp works on the row (all of the CTA then gets here).
+template <int THREADS>
+__device__ __forceinline__ void finalize_row(const FinalizeDesc& f, int64_t row, double half_per, int t, unsigned long long* s_sum) {
+    unsigned long long* q = f.sums + row * f.stride;
+    unsigned long long s = 0;
+#pragma unroll 8
+    for (int c = t; c < f.per_row; c += THREADS) s += __ldcg(q + c);
+    if (f.clear)
+        for (int c = t; c < f.per_row; c += THREADS) q[c] = 0ull;
+    s = warp_sum_u64(s);
+    if (THREADS > 32) {
+        if ((t & 31) == 0) s_sum[t >> 5] = s;
+        __syncthreads();
+        if (t == 0)
+            for (int w = 1; w < THREADS / 32; ++w) s += s_sum[w];
+    }
+    if (t == 0) f.logp_out[row] = logp_from_squares(s, half_per, f.g, f.logp_const);
+}
+
+// All rows of the pending level, one warp per row.
 __device__ __forceinline__ void finalize_rows(const FinalizeDesc& f, int32_t n_trees, int32_t nodes_cap,
                                               double half_per, int warp_global, int warps_total, int32_t* status, int32_t per_row_cap) {
-    const int lane = threadIdx.x & 31;
     const int n_rows = n_trees * f.W;
-    const int per_row = f.per_row;
     for (int idx = warp_global; idx < n_rows; idx += warps_total) {
         const int tree = idx / f.W;
         const int64_t row = static_cast<int64_t>(tree) * nodes_cap + f.off + (idx - tree * f.W);
-        if (!BGRPO_IN_BOUNDS(status, f.off + f.W <= nodes_cap && 2 * per_row <= per_row_cap)) continue;
-        unsigned long long* q = f.sums + row * f.stride;
-        unsigned long long s = 0;
-#pragma unroll 4
-        for (int c = lane; c < per_row; c += 32) s += __ldcg(q + c);
-        if (f.clear)
-            for (int c = lane; c < per_row; c += 32) q[c] = 0ull;
-        s = warp_sum_u64(s);
-        if (lane == 0) f.logp_out[row] = logp_from_squares(s, half_per, f.g, f.logp_const);
+        if (!BGRPO_IN_BOUNDS(status, f.off + f.W <= nodes_cap && 2 * f.per_row <= per_row_cap)) continue;
+        finalize_row<32>(f, row, half_per, threadIdx.x & 31, nullptr);
     }
 }
 

@@ -49,7 +49,7 @@ root_kernel(float* latents, int32_t* table, float* logp, unsigned long long* row
 
 // ---------------------------------------------------------------------------------------------------------------
 // Fused step.  One CTA per work item (tree, parent, chunk of kStepChunkVec float4): kStepThreads threads of kStepVec float4,
-// or kStepThreadsSmall threads of a quarter of that where the launch is less than one wave (step_threads()).
+// or kStepThreadsSmall threads of half of that where the launch is less than one wave (step_threads()).
 //
 // A thread issues the 128-bit loads of its kStepVec float4 of the parent tile and of the operand tile (velocity or
 // target mean) first, then generates the noise of all its elements - Philox and Box-Muller depend on indices only,
@@ -58,9 +58,11 @@ root_kernel(float* latents, int32_t* table, float* logp, unsigned long long* row
 // squares of the noise.  The parent is read once however many children it has.
 //
 // Log-prob: a warp adds its squares per child as integers (philox.cuh) and stores one number per (child row, chunk, warp).
-// Nothing waits for those stores: the sums over chunks and warps are taken by the prologue of the NEXT launch on the
-// stream (FinalizeDesc), or by the small flush kernel when the tree is complete, so the kernel has no fence, no atomic
-// and no CTA-wide barrier.
+// Nothing waits for those stores: the sums over chunks and warps are taken by the NEXT launch on the stream (FinalizeDesc), or
+// by the flush kernel when the tree is complete, so the kernel has no fence and no atomic.  One of the launch's first CTAs adds
+// a row up, behind its own loads.  (One warp per row, 16 steps of a video tree: 589 us for 574, and 605 ahead of the loads, as
+// launches of one wave wait for it; the CTA of the row's own first chunk, four image trees: 161 us for 149, as the last rows'
+// come in the last wave; one number per CTA, which takes a barrier at its end, 32 image trees: 1 157 us for 1 120.)
 //
 // FAN children per parent; SHARED: xi_b mixes a per-parent xi_0 (finite s at a split step); FULL: the tile holds
 // kStepChunkVec float4, so no element needs a bounds test; NOISY = false: a deterministic step (sigma = 0) of the
@@ -131,22 +133,14 @@ __device__ __forceinline__ void compute_tile(const StepLaunch& p, const float4 (
 }
 
 template <int FAN, bool SHARED, bool NOISY, int THREADS>
-__global__ void __launch_bounds__(THREADS, THREADS == kStepThreads ? kStepCtasPerSm : kStepCtasPerSmSmall)
+__global__ void __launch_bounds__(THREADS, THREADS == kStepThreads ? step_ctas_per_sm(FAN, SHARED) : kStepCtasPerSmSmall)
 step_kernel(const __grid_constant__ StepLaunch p) {
     constexpr int kWarps = THREADS / 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     pdl_release();
-    // the previous level's log-probs (a handful of rows) are summed by this launch
-    auto finalize_previous = [&] {
-        if (p.prev.logp_out != nullptr)
-            finalize_rows(p.prev, p.n_trees, p.nodes_cap, p.half_per, blockIdx.x * kWarps + warp, gridDim.x * kWarps, p.status, p.per_row);
-    };
     // The parents, the velocity and the pending partial sums come from earlier kernels.  A launch of many waves waits for
     // them here: its loads travel while the noise is generated.
-    if (THREADS == kStepThreads) {
-        pdl_wait();
-        finalize_previous();
-    }
+    if (THREADS == kStepThreads) pdl_wait();
 
     const int chunk = blockIdx.x % p.nchunks;
     const int row = blockIdx.x / p.nchunks;             // tree * W_in + j
@@ -168,6 +162,14 @@ step_kernel(const __grid_constant__ StepLaunch p) {
     const uint32_t gid_parent = p.node_id_base + static_cast<uint32_t>(tree_row0 + parent);
     const uint32_t gid_child0 = p.node_id_base + static_cast<uint32_t>(tree_row0 + child0);
 
+    // the parents' own log-probs, from the sums the launch before left: a row for each of the first CTAs
+    __shared__ unsigned long long s_sum[kWarps];
+    auto finalize_previous = [&] {
+        if (p.prev.logp_out == nullptr || blockIdx.x >= p.n_trees * p.prev.W) return;
+        const int t = blockIdx.x / p.prev.W;
+        if (BGRPO_IN_BOUNDS(p.status, p.prev.W == p.W_in && p.prev.off == p.off_in && 2 * p.prev.per_row <= p.per_row))
+            finalize_row<THREADS>(p.prev, static_cast<int64_t>(t) * p.nodes_cap + p.prev.off + (blockIdx.x - t * p.prev.W), p.half_per, threadIdx.x, s_sum);
+    };
     uint32_t acc[FAN];
 #pragma unroll
     for (int b = 0; b < FAN; ++b) acc[b] = 0u;
@@ -193,12 +195,14 @@ step_kernel(const __grid_constant__ StepLaunch p) {
         }
     } else if (vecs == kStepChunkVec) {
         load_tile<THREADS, true>(zp, xop, streamed, vecs, z, x);
+        finalize_previous();
         compute_tile<FAN, SHARED, THREADS, true, NOISY>(p, z, x, vecs, e_base, D4, zc, noise, acc);
     } else {
         load_tile<THREADS, false>(zp, xop, streamed, vecs, z, x);
+        finalize_previous();
         compute_tile<FAN, SHARED, THREADS, false, NOISY>(p, z, x, vecs, e_base, D4, zc, noise, acc);
     }
-    // one number per (child row, chunk, warp): a lane's sum takes up to 31 bits, so its halves are added apart
+    // one number per (child row, chunk, warp): a lane's sum takes up to 30 bits, so its halves are added apart
 #pragma unroll
     for (int b = 0; b < FAN; ++b) {
         const uint32_t lo = __reduce_add_sync(0xffffffffu, acc[b] & 0xffffu), hi = __reduce_add_sync(0xffffffffu, acc[b] >> 16);
@@ -216,14 +220,18 @@ step_kernel(const __grid_constant__ StepLaunch p) {
     }
 }
 
-// Flush: adds up a pending level outside a step launch (the tree is complete, or tree_logprob is done).
+// Flush: adds up a pending level outside a step launch (the tree is complete, or its record is saved): THREADS threads per row.
+template <int THREADS>
 __global__ void __launch_bounds__(kStreamThreads)
-finalize_kernel(const FinalizeDesc f, int32_t n_trees, int32_t nodes_cap, double half_per,
-                int32_t* status, int32_t per_row_cap) {
+finalize_kernel(const FinalizeDesc f, int32_t n_trees, int32_t nodes_cap, double half_per, int32_t* status, int32_t per_row_cap) {
+    __shared__ unsigned long long s_sum[kStreamThreads / 32];
     pdl_release();
     pdl_wait();
-    finalize_rows(f, n_trees, nodes_cap, half_per, blockIdx.x * (kStreamThreads / 32) + (threadIdx.x >> 5),
-                  gridDim.x * (kStreamThreads / 32), status, per_row_cap);
+    const int idx = blockIdx.x * (kStreamThreads / THREADS) + threadIdx.x / THREADS;
+    if (idx >= n_trees * f.W) return;
+    const int tree = idx / f.W;
+    if (!BGRPO_IN_BOUNDS(status, f.off + f.W <= nodes_cap && 2 * f.per_row <= per_row_cap)) return;
+    finalize_row<THREADS>(f, static_cast<int64_t>(tree) * nodes_cap + f.off + (idx - tree * f.W), half_per, threadIdx.x % THREADS, s_sum);
 }
 
 __global__ void philox_words_kernel(const __grid_constant__ PhiloxKeys keys, uint32_t node, uint32_t step, uint32_t tag, uint4* out, int64_t nblk) {
@@ -280,11 +288,10 @@ cudaError_t launch_step(const StepLaunch& p0, cudaStream_t s) {
 }
 
 cudaError_t launch_finalize(const bgrpo_tree* t, const FinalizeDesc& f, cudaStream_t s) {
-    const int rows = t->desc.n_trees * f.W;
-    const int grid = (rows + (kStreamThreads / 32) - 1) / (kStreamThreads / 32);
-    return launch_overlapped(finalize_kernel, grid < 1 ? 1 : grid, kStreamThreads, 0, s, f,
-                             t->desc.n_trees, t->desc.nodes_cap, logp_half_per(t->D), t->status,
-                             static_cast<int32_t>(partials_per_row(t->D)));
+    const int rows = t->desc.n_trees * f.W, row_threads = f.per_row >= 512 ? kStreamThreads : 32;
+    const int grid = (rows + kStreamThreads / row_threads - 1) / (kStreamThreads / row_threads);
+    return launch_overlapped(row_threads == 32 ? finalize_kernel<32> : finalize_kernel<kStreamThreads>, grid < 1 ? 1 : grid, kStreamThreads, 0, s, f,
+                             t->desc.n_trees, t->desc.nodes_cap, logp_half_per(t->D), t->status, static_cast<int32_t>(partials_per_row(t->D)));
 }
 
 cudaError_t launch_philox_words(uint64_t seed, uint32_t node, uint32_t step, uint32_t tag, uint32_t* out, int64_t nblk, cudaStream_t s) {

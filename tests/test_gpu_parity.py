@@ -894,7 +894,7 @@ def test_logprob_families_at_their_edges(B, tokens, channels, n_trees, T, K, spl
 
 
 @pytest.mark.parametrize("tokens,channels,n_trees,T,K,splits,s", [
-    (9, 4, 591, 2, 1, (), math.inf),              # step launches of 591, 592, 593 CTAs: the wide ones and the narrow ones
+    (9, 4, 591, 2, 1, (), math.inf),              # step launches of 591, 592, 593 CTAs: the small ones and the large ones
     (9, 4, 592, 2, 1, (), math.inf),
     (9, 4, 593, 2, 1, (), math.inf),
     (513, 4, 295, 2, 1, (), math.inf),            # the same with a second chunk of one float4 (two-CTA rows in the whole-tree launch)
@@ -907,6 +907,10 @@ def test_logprob_families_at_their_edges(B, tokens, channels, n_trees, T, K, spl
     (9, 4, 450, 6, 2, (0, 1, 2, 3, 4, 5), 2.0),   # two forks dealt out, four open ones with their shared noise in shared memory
     (9, 4, 444, 7, 2, (1, 2, 3, 4, 5, 6), 2.0),   # three trees an SM, no fork dealt out: six open forks
     (513, 4, 444, 7, 2, (1, 2, 3, 4, 5, 6), 2.0),     # the same with rows of two CTAs
+    (63 * 512, 4, 1, 3, 2, (1,), math.inf),       # sums of 504 and 520 numbers a row: the last launch takes a warp or a CTA per row
+    (64 * 512 + 1, 4, 1, 3, 2, (1,), math.inf),
+    (127 * 512, 4, 5, 3, 2, (1,), math.inf),      # 508 and 512 of the wide launches
+    (128 * 512, 4, 5, 3, 2, (1,), 2.0),
 ])
 def test_step_and_whole_tree_launches_agree_where_their_shapes_change(B, tokens, channels, n_trees, T, K, splits, s):
     """The two rollouts share the noise stream, the float32 expressions and the integer sums, and nothing of their launch
