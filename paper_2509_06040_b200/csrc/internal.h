@@ -29,31 +29,27 @@ constexpr int step_ctas_per_sm(int fan, bool shared_noise) { return fan >= 3 && 
 constexpr int kStepCtasPerSmSmall = 4;
 constexpr int64_t kStepSmallGrid = 148 * 4;
 inline int step_threads(int64_t items) { return items < kStepSmallGrid ? kStepThreadsSmall : kStepThreads; }
-// Whole-tree rollout kernel: 128-thread CTAs, 4 float4 per thread (1 and 2 measured 37 and 16 % slower on the video tree), four
-// CTAs per SM (5 and 6: equal and 6 % slower there, 16 and 40 % slower on a single image tree), one log-prob partial per
-// node row and warp; at most kFusedMaxSplits split steps (the means of the open forks wait in shared memory).
+// Whole-tree rollout kernel: 128-thread CTAs of up to 4 float4 per thread (launch_rollout_fused chooses), four CTAs per SM (5 and
+// 6: equal and 6 % slower on the video tree, 16 and 40 % slower on a single image tree), one log-prob partial per node row and
+// warp; at most kFusedMaxSplits split steps (the means of the open forks wait in shared memory).
 constexpr int kFusedThreads = 128;
-constexpr int kFusedVec = 4;
+constexpr int kFusedMostVec = 4;
 constexpr int kFusedCtasPerSm = 4;
-constexpr int kFusedChunkVec = kFusedThreads * kFusedVec;   // float4 of a row per CTA
 constexpr int kFusedMaxSplits = 6;
-// log-prob partials of the whole-tree kernel per node row: one 32-bit word per warp of every CTA that covers the row, two with
-// shared noise (a half-warp's squares each: see the bound in tree_fused.cu)
+// log-prob partials of the whole-tree kernel per CTA that covers a node row: one 32-bit word per warp, two with shared noise and
+// four float4 a thread (a half-warp's squares each: see the bound in tree_fused.cu)
 #ifdef __CUDACC__
 __host__ __device__
 #endif
-constexpr int fused_words_per_cta(bool shared_noise) { return kFusedThreads / 32 * (shared_noise ? 2 : 1); }
-inline int64_t fused_partials_per_row(int64_t D, bool shared_noise) {
-    return ((D / 4 + kFusedChunkVec - 1) / kFusedChunkVec) * fused_words_per_cta(shared_noise);
-}
-// 32-bit words of log-prob partials reserved per node row: the larger of the rollout kernels' layouts (64 bits per chunk and
-// warp in the step kernel); an even number, so that every row starts on 8 bytes
+constexpr int fused_words_per_cta(bool shared_noise, int vec) { return kFusedThreads / 32 * (shared_noise && vec == 4 ? 2 : 1); }
+// 32-bit words of log-prob partials reserved per node row: those of the step kernel, 64 bits per chunk and warp.  The whole-tree
+// kernel's fit as well: per step chunk of 512 float4 at most four CTAs of one float4 a thread, four words each.  An even number,
+// so that every row starts on 8 bytes.
 inline int64_t partials_per_row(int64_t D) {
-    const int64_t D4 = D / 4;
-    const int64_t step = ((D4 + kStepChunkVec - 1) / kStepChunkVec) * (kStepThreadsSmall / 32) * 2;
-    const int64_t fused = fused_partials_per_row(D, true);
-    return step > fused ? step : fused;
+    return ((D / 4 + kStepChunkVec - 1) / kStepChunkVec) * (kStepThreadsSmall / 32) * 2;
 }
+static_assert(kStepChunkVec / kFusedThreads * (kFusedThreads / 32) <= kStepThreadsSmall / 32 * 2 && kStepChunkVec == kFusedThreads * kFusedMostVec,
+              "the whole-tree kernel's partials fit the step kernel's");
 constexpr int kScratchHeader = 256;    // bytes reserved at the start of scratch for the status word
 
 constexpr uint32_t kPhiloxM0 = 0xD2511F53u;   // Philox4x32 multipliers and Weyl key increments (Salmon et al., SC'11)
@@ -330,7 +326,7 @@ struct FusedLaunch {
     int32_t per_row_cap;       // words reserved per node row
     int64_t D;
     int32_t n_trees, nodes_cap, T, K, shared_noise;
-    int32_t nchunks, per_row;  // CTAs that cover a row; set by launch_rollout_fused, like the next six
+    int32_t nchunks, per_row;  // CTAs that cover a row, words of partials they leave; set by launch_rollout_fused, like the next six
     int32_t par, subtrees, levels, nodes;              // forks dealt out to the grid, K^par, forks walked, nodes of a tree
     int32_t sums_at;           // 0, or 1 + where in shared memory (float4) the sums of a row of one CTA are
     int32_t split_step[kFusedMaxSplits];

@@ -13,8 +13,8 @@
 // float32 operations one each, and they do not overlap; a register-only loop draws 1.18 T normals a second.  So everything
 // around the noise is kept small.  The walk is one loop with one copy of the noise code, not a recursion over split levels
 // (which took 113-168 registers, spilled, and did not fit the instruction cache): a node's local index, written in base K,
-// is the path that leads to it, and the means of the open forks wait in shared memory.  A thread takes four float4 (one: 42
-// instructions per element instead of 24, nearly twice the time), the first two Philox rounds are split into a part per element
+// is the path that leads to it, and the means of the open forks wait in shared memory.  A thread takes four float4 of long rows
+// (24 instructions per element, one: 42), the first two Philox rounds are split into a part per element
 // and a part per node.  Video tree (110 edges x 2.1 M elements): 379 -> 249 us, 0.93 T normals/s; four trees of 129 600
 // elements: 162 -> 102 us; one: 103 -> 40 us.
 //
@@ -28,13 +28,15 @@ namespace bgrpo {
 namespace {
 
 constexpr uint32_t kNotMine = 0xffffffffu;          // no sum of a warp, or with shared noise of half a warp
-static_assert(32 * kFusedVec * kMostSquares * kSquareScale < 4294967295.0, "a warp's sum in 32 bits");
-static_assert(16 * kFusedVec * 2 * kMostSquares * kSquareScale < 4294967295.0, "a half-warp's sum with shared noise in 32 bits");
+static_assert(32 * 4 * kMostSquares * kSquareScale < 4294967295.0, "a warp's sum in 32 bits");
+static_assert(32 * 2 * 2 * kMostSquares * kSquareScale < 4294967295.0, "with shared noise a warp's at two float4 a thread,");
+static_assert(16 * 4 * 2 * kMostSquares * kSquareScale < 4294967295.0, "and a half-warp's at four");
 
-template <bool SHARED>
+// VEC: float4 per thread.
+template <bool SHARED, int VEC>
 __global__ void __launch_bounds__(kFusedThreads, kFusedCtasPerSm)
 rollout_fused_kernel(const __grid_constant__ FusedLaunch p) {
-    constexpr int VEC = kFusedVec, WORDS = fused_words_per_cta(SHARED);
+    constexpr int WORDS = fused_words_per_cta(SHARED, VEC);
     extern __shared__ float4 s_stack[];             // [open fork][VEC] means, SHARED: and as many xi_0; rows of one CTA: the sums of all nodes
     pdl_release();
     const int chunk = blockIdx.x % p.nchunks;
@@ -137,7 +139,7 @@ rollout_fused_kernel(const __grid_constant__ FusedLaunch p) {
 #pragma unroll
             for (int k = 0; k < VEC; ++k)
                 if (live[k]) __stcs(row + e[k], z[k]);
-            if (SHARED) {
+            if (WORDS > kFusedThreads / 32) {
                 const uint32_t low = __reduce_add_sync(0xffffffffu, lane < 16 ? acc : 0u), high = __reduce_add_sync(0xffffffffu, lane < 16 ? 0u : acc);
                 if (lane == 0) {
                     uint32_t* const out = s_sums ? s_sums[child] + 2 * warp : partials + static_cast<uint64_t>(child) * static_cast<uint32_t>(p.per_row);
@@ -225,12 +227,27 @@ finalize_tree_kernel(const __grid_constant__ FusedLaunch p, int32_t nodes) {
     if (threadIdx.x % THREADS == 0) p.logp[row] = logp_from_squares(s, p.half_per, p.step[step].g, p.step[step].logp_const);
 }
 
-// six open forks with their shared noise, and the sums of a small tree
 constexpr int32_t kSumsInSharedNodes = 1024;
-constexpr int kMostShared = kFusedMaxSplits * kFusedChunkVec * static_cast<int>(sizeof(float4)) * 2 +
-                            kSumsInSharedNodes * fused_words_per_cta(true) * static_cast<int>(sizeof(uint32_t));
-SharedMemoryLimit g_limit_own(reinterpret_cast<const void*>(&rollout_fused_kernel<false>), kMostShared);
-SharedMemoryLimit g_limit_shared(reinterpret_cast<const void*>(&rollout_fused_kernel<true>), kMostShared);
+
+// What a launch of VEC float4 per thread needs of shared memory: the means of `levels` open forks (and their shared noise), and
+// where a row is one CTA's the sums of `nodes` nodes.
+constexpr size_t stack_bytes(bool shared_noise, int vec, int levels) {
+    return static_cast<size_t>(levels) * kFusedThreads * vec * sizeof(float4) * (shared_noise ? 2 : 1);
+}
+constexpr size_t sums_bytes(bool shared_noise, int vec, int nodes) {
+    return static_cast<size_t>(nodes) * fused_words_per_cta(shared_noise, vec) * sizeof(uint32_t);
+}
+
+template <bool SHARED, int VEC>
+cudaError_t launch_as(const FusedLaunch& p, unsigned int grid, size_t smem, cudaStream_t s) {
+    static SharedMemoryLimit limit(reinterpret_cast<const void*>(&rollout_fused_kernel<SHARED, VEC>),
+                                   static_cast<int>(stack_bytes(SHARED, VEC, kFusedMaxSplits) + sums_bytes(SHARED, VEC, kSumsInSharedNodes)));
+    if (smem > kSharedWithoutAsking) {
+        const cudaError_t e = limit.allow();
+        if (e != cudaSuccess) return e;
+    }
+    return launch_overlapped(rollout_fused_kernel<SHARED, VEC>, grid, kFusedThreads, smem, s, p);
+}
 
 }  // namespace
 
@@ -238,15 +255,26 @@ cudaError_t launch_rollout_fused(const FusedLaunch& p0, int32_t nodes, cudaStrea
     FusedLaunch p = p0;
     p.half_per = logp_half_per(p.D);
     int n_splits = 0;
+    int64_t leaves = 1;
     for (int i = 0; i < p.T; ++i) {
         noise_step(static_cast<uint32_t>(i), p.keys, p.step[i].px, p.step[i].ph);
         if (!(p.step[i].child0 & kForks)) continue;
         if (n_splits == kFusedMaxSplits) return cudaErrorInvalidValue;
         p.split_step[n_splits++] = i;
+        leaves *= p.K;
     }
     const int64_t D4 = p.D / 4;
-    p.nchunks = static_cast<int32_t>((D4 + kFusedChunkVec - 1) / kFusedChunkVec);
-    p.per_row = static_cast<int32_t>(fused_partials_per_row(p.D, p.shared_noise != 0));
+    const bool shared_noise = p.shared_noise != 0;
+    // Four float4 a thread are the fewest instructions per element (video tree: 355 us; two 375, one 462).  But a row that does
+    // not fill a CTA of four draws noise for nothing - K = 4, six splits, 64 elements a row: 189 us with four, 98 with one, 162
+    // level by level; 1 024 elements: 122 with two, 223 level by level - and a tree without forks has none to deal out: 64 steps
+    // of one tree of 16 384 elements 51 us with four, 32 with one, 32 trees 98 and 79, 128 trees 160 and 197, so up to two CTAs of
+    // four an SM take one (16 steps of eight image trees, 512 CTAs: equal).
+    int vec = D4 <= kFusedThreads ? 1 : D4 <= 2 * kFusedThreads ? 2 : 4;
+    if (leaves == 1 && p.n_trees * ((D4 + kFusedThreads * 4 - 1) / (kFusedThreads * 4)) <= 2 * 148) vec = 1;
+    p.nchunks = static_cast<int32_t>((D4 + kFusedThreads * vec - 1) / (kFusedThreads * vec));
+    p.per_row = p.nchunks * fused_words_per_cta(shared_noise, vec);
+    if (p.per_row > p.per_row_cap) return cudaErrorInvalidValue;
     // Dealing out a fork more makes K times as many CTAs that walk a shorter subtree but compute the prefix again.  An SM works
     // at the same rate from about three CTAs on, so the time goes with the CTAs of the busiest SM (at least three) times the
     // nodes a CTA walks.  Measured, us a rollout, forks dealt out 0 / 1 / 2 / 3 (the rule's choice in brackets): four trees of
@@ -272,20 +300,17 @@ cudaError_t launch_rollout_fused(const FusedLaunch& p0, int32_t nodes, cudaStrea
     const int64_t items = static_cast<int64_t>(p.n_trees) * p.nchunks * p.subtrees;
     if (items <= 0 || items > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     const unsigned int grid = static_cast<unsigned int>(items);
-    size_t smem = static_cast<size_t>(p.levels) * kFusedChunkVec * sizeof(float4) * (p.shared_noise ? 2 : 1);
-    // Rows of one CTA keep their sums in shared memory (up to 16 KB of them, 32 with shared noise) and need no second launch, which costs about 4 us of
-    // host time (toy pass, with the rewards' second launch gone as well: 27.8 -> 23.8 us).
+    size_t smem = stack_bytes(shared_noise, vec, p.levels);
+    // Rows of one CTA keep their sums in shared memory (up to 16 KB of them, 32 with shared noise) and need no second launch,
+    // which costs about 4 us of host time (toy pass, with the rewards' second launch gone as well: 27.8 -> 23.8 us).
     p.nodes = nodes;
     p.sums_at = 0;
     if (p.nchunks == 1 && nodes <= kSumsInSharedNodes) {
         p.sums_at = static_cast<int32_t>(smem / sizeof(float4)) + 1;
-        smem += static_cast<size_t>(nodes) * fused_words_per_cta(p.shared_noise != 0) * sizeof(uint32_t);
+        smem += sums_bytes(shared_noise, vec, nodes);
     }
-    cudaError_t e = cudaSuccess;
-    if (smem > kSharedWithoutAsking) e = p.shared_noise ? g_limit_shared.allow() : g_limit_own.allow();
-    if (e == cudaSuccess)
-        e = p.shared_noise ? launch_overlapped(rollout_fused_kernel<true>, grid, kFusedThreads, smem, s, p)
-                           : launch_overlapped(rollout_fused_kernel<false>, grid, kFusedThreads, smem, s, p);
+    const cudaError_t e = shared_noise ? (vec == 1 ? launch_as<true, 1>(p, grid, smem, s) : vec == 2 ? launch_as<true, 2>(p, grid, smem, s) : launch_as<true, 4>(p, grid, smem, s))
+                                       : (vec == 1 ? launch_as<false, 1>(p, grid, smem, s) : vec == 2 ? launch_as<false, 2>(p, grid, smem, s) : launch_as<false, 4>(p, grid, smem, s));
     if (e != cudaSuccess || nodes < 2 || p.sums_at > 0) return e;
     const int64_t rows = static_cast<int64_t>(p.n_trees) * (nodes - 1);
     if (p.per_row >= 512) return launch_overlapped(finalize_tree_kernel<256>, static_cast<unsigned int>(rows), 256, 0, s, p, nodes);

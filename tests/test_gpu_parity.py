@@ -907,6 +907,12 @@ def test_logprob_families_at_their_edges(B, tokens, channels, n_trees, T, K, spl
     (9, 4, 450, 6, 2, (0, 1, 2, 3, 4, 5), 2.0),   # two forks dealt out, four open ones with their shared noise in shared memory
     (9, 4, 444, 7, 2, (1, 2, 3, 4, 5, 6), 2.0),   # three trees an SM, no fork dealt out: six open forks
     (513, 4, 444, 7, 2, (1, 2, 3, 4, 5, 6), 2.0),     # the same with rows of two CTAs
+    (128, 4, 3, 4, 3, (0, 2), 1.0),               # the whole-tree launch takes one float4 a thread, two, two, four
+    (129, 4, 3, 4, 4, (0, 2), 2.0),
+    (256, 4, 2, 5, 2, (0, 3), math.inf),
+    (257, 4, 2, 5, 2, (0, 3), 2.0),
+    (513, 4, 148, 3, 2, (), 2.0),                 # no fork: one float4 a thread, and four with one tree more
+    (513, 4, 149, 3, 2, (), 2.0),
     (63 * 512, 4, 1, 3, 2, (1,), math.inf),       # sums of 504 and 520 numbers a row: the last launch takes a warp or a CTA per row
     (64 * 512 + 1, 4, 1, 3, 2, (1,), math.inf),
     (127 * 512, 4, 5, 3, 2, (1,), math.inf),      # 508 and 512 of the wide launches
