@@ -357,6 +357,7 @@ cudaError_t launch_fusion_ess(const EssLaunch& p, cudaStream_t s);
 struct PruneLaunch {
     const float* rbar; uint8_t* mask; int32_t* status;
     LevelInfo lv; RunInfo runs; int32_t n_trees, nodes_cap, T, nodes, mode, k, last_split, ignore_last; uint64_t pruned_bits;
+    int32_t wide_run, narrow_nodes;      // first run written chain by chain and the nodes before it; set by launch_prune
 };
 cudaError_t launch_prune(const PruneLaunch& p, cudaStream_t s);
 

@@ -812,10 +812,11 @@ def test_prune_has_no_node_limit(B):
 
 
 @pytest.mark.parametrize("T,K,splits", [(1, 2, ()), (1, 3, (0,)), (9, 2, tuple(range(9))), (12, 2, (0, 1, 2, 3, 4, 5, 6, 8, 9, 10)), (8, 1, (2, 5)),
-                                        (7, 4, (0, 1, 3, 4, 5))])
+                                        (7, 4, (0, 1, 3, 4, 5)), (9, 4, (0, 1, 4, 6)), (11, 3, (0, 2, 3, 5, 7)), (10, 2, tuple(range(8)))])
 def test_reductions_where_their_branches_change(B, T, K, splits):
     """Trees at the edges of the reductions' branches: one run only, forks at every step, long chains, K = 1 "forks", and
-    Extreme-b on 512 leaves (ranked by counting) and 1024 (radix selection), with exact ties.  Masks are whole numbers;
+    Extreme-b on 512 leaves (ranked by counting) and 1024 (radix selection), with exact ties; runs of 243, 256 and more chains
+    (masks written node by node, chain by chain).  Masks are whole numbers;
     fused values, advantages and effective sample sizes within the bounds of the tests above."""
     w, s, topo = _grown_session(B, T, K, splits)
     rng = np.random.default_rng(100 * T + K)
