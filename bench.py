@@ -358,9 +358,26 @@ def run_reference(args, w):
 
 
 # ------------------------------------------------------------------------------------------------ per-kernel timing
-def kernel_rooflines(s, w, peaks, flush_buf, reps):
-    """Times every launch group of `reps` passes with in-stream events and returns (roofline of the dominant kernel,
-    roofline of the step kernel, ms per pass by kernel).  An interval between two events holds one launch and the gap
+def rollout_kind(w, launches):
+    """What the library made of a rollout, from the kernels it enqueued for it (the root's included): level by level that
+    is the root, T steps (and T velocity launches) and the last level's log-prob sums."""
+    if w.velocity == "mlp":
+        along = 2 * w.T + 2 - launches
+        return "velocity and step per depth" + (f", {along} of {w.T} depths in one launch" if along > 0 else "")
+    return "one launch" if launches < w.T + 2 else "one tree_step per depth"
+
+
+def count_rollout_launches(s, seed):
+    from paper_2509_06040_b200 import binding as B
+    before = B.launch_count()
+    s.rollout(seed=seed)
+    return B.launch_count() - before
+
+
+def kernel_rooflines(s, w, peaks, flush_buf, reps, one_launch_ms=None):
+    """Times every launch group of `reps` passes, level by level, with in-stream events and returns (roofline of the
+    dominant kernel, roofline of the step kernel, ms per pass by kernel).  one_launch_ms: the rollout of the timed pass is one
+    kernel of that many ms; the step kernel's figures are then those of tree_step called depth by depth, not a part of it.  An interval between two events holds one launch and the gap
     the event itself inserts (it also keeps the next launch's ramp from overlapping this launch's tail), so on
     workloads made of launches of a few microseconds the intervals add up to more than the un-instrumented pass."""
     import torch
@@ -442,8 +459,10 @@ def kernel_rooflines(s, w, peaks, flush_buf, reps):
         roof_step["algorithmic_gbs_l2_assisted"] = {"gbs": r4(sb[:-1].sum() / (ms_group * 1e-3) / 1e9), "ms": r4(ms_group),
                                                     "launches": w.T - 1}
     reward_bytes = 0.0 if w.reward == "mixture" else float(w.n_trees * (w.leaves + 1) * 4 * w.D)   # leaf rows once, target once per tree
-    parts = {"mlp": t_mlp.sum(), "step": t_step.sum(), "root": t_root, "leaf_reward": t_tail[0], "fuse_advantage": t_tail[1],
-             "prune": t_tail[2]}
+    parts = {"mlp": t_mlp.sum(), "step": t_step.sum()} if one_launch_ms is None else {"rollout": one_launch_ms}
+    parts.update({"root": t_root, "leaf_reward": t_tail[0], "fuse_advantage": t_tail[1], "prune": t_tail[2]})
+    if one_launch_ms is not None:
+        roof_step["basis"] += "; tree_step depth by depth, not in the timed pass"
     breakdown = {k: r4(v) for k, v in parts.items()}
     breakdown["sum"] = r4(sum(parts.values()))
     breakdown["leaf_reward_gbs"] = r4(reward_bytes / (t_tail[0] * 1e-3) / 1e9) if reward_bytes and t_tail[0] > 0 else None
@@ -467,7 +486,7 @@ def kernel_rooflines(s, w, peaks, flush_buf, reps):
 
 
 def fused_rollout_line(w, device, peaks, reps):
-    """The same pass with all T steps in one launch (closed-form velocity): whole-pass throughput, and the rollout
+    """The pass with all T steps in one launch (closed-form velocity): whole-pass throughput, and the rollout
     kernel alone against the bytes it must move (every node written once, root and target mean read once)."""
     import torch
     from paper_2509_06040_b200.session import TreeSession
@@ -562,7 +581,10 @@ def brief_workload(name, device, peaks):
         torch.cuda.synchronize()
         tot += a0.elapsed_time(a1)
     ms = tot / n2
-    r2, rs2, bd2 = kernel_rooflines(s2, w2, peaks, flush_buf, 3)
+    kind = rollout_kind(w2, count_rollout_launches(s2, w2.seed))
+    fused = fused_rollout_line(w2, device, peaks, n2)["roofline"] if kind == "one launch" else None
+    r2, rs2, bd2 = kernel_rooflines(s2, w2, peaks, flush_buf, 3, fused and fused["ms_per_launch"])
+    r2 = fused or r2
 
     def compact(r):
         keep = ("kernel", "achieved", "peak", "unit", "frac", "frac_of_nominal_8TBs", "peak_kind", "basis")
@@ -573,16 +595,12 @@ def brief_workload(name, device, peaks):
             out["algorithmic_gbs_l2_assisted"] = r["algorithmic_gbs_l2_assisted"]["gbs"]
         return out
 
-    out = {"value": r4(w2.n_trees * w2.node_steps / (ms * 1e-3)), "ms_per_step": r4(ms), "roofline": compact(r2),
+    out = {"value": r4(w2.n_trees * w2.node_steps / (ms * 1e-3)), "ms_per_step": r4(ms), "rollout": kind, "roofline": compact(r2),
            "kernel_ms_sum": bd2["sum"]}
     if r2 is not rs2:
         out["roofline_step"] = compact(rs2)
     del s2, flush_buf
     torch.cuda.empty_cache()
-    if w2.velocity == "linear":
-        fr = fused_rollout_line(w2, device, peaks, n2)
-        out["one_launch_rollout"] = {"value": fr["value"], "ms_per_step": fr["ms_per_step"],
-                                     "gbs": fr["roofline"]["achieved"], "frac": fr["roofline"]["frac"]}
     return out
 
 
@@ -715,22 +733,22 @@ def run_ours(args, w):
     roof = roof_step = None
     breakdown = {}
     peaks = load_peaks()
+    kind = rollout_kind(w, count_rollout_launches(s, w.seed))
     if rank == 0:
-        if s.fused_rollout:
-            roof = roof_step = fused_rollout_line(w, f"cuda:{local}", peaks, max(3, min(10, args.steps)))["roofline"]
-        else:
-            roof, roof_step, breakdown = kernel_rooflines(s, w, peaks, flush_buf, max(3, min(10, args.steps)))
-            breakdown["pass"] = r4(total_ms / args.steps)
-            breakdown["note"] = ("one event interval per launch; each holds the event's own gap, so the sum exceeds the pass "
-                                 "where launches take microseconds" if breakdown["sum"] > 1.1 * breakdown["pass"]
-                                 else "one event interval per launch")
+        reps = max(3, min(10, args.steps))
+        fused = fused_rollout_line(w, f"cuda:{local}", peaks, reps)["roofline"] if kind == "one launch" else None
+        roof, roof_step, breakdown = kernel_rooflines(s, w, peaks, flush_buf, reps, fused and fused["ms_per_launch"])
+        roof = fused or roof
+        breakdown["pass"] = r4(total_ms / args.steps)
+        breakdown["note"] = ("one event interval per launch; each holds the event's own gap, so the sum exceeds the pass "
+                             "where launches take microseconds" if breakdown["sum"] > 1.1 * breakdown["pass"]
+                             else "one event interval per launch")
 
     # ---- the tree against independent sequential rollouts with as many final samples (rank 0, single GPU)
     savings = None
     if rank == 0 and world == 1 and not args.no_also:
         savings = savings_line(w, s, f"cuda:{local}", max(3, min(10, args.steps)))
     dtype = "f32" if w.velocity == "linear" else "f32 (step) + bf16/f32-accumulate (MLP velocity)"
-    rollout_kind = "one launch" if s.fused_rollout else "one tree_step per depth"
     del s, stage, flush_buf
     torch.cuda.empty_cache()
 
@@ -755,7 +773,7 @@ def run_ours(args, w):
                        "splits": list(w.splits), "velocity": w.velocity, "node_steps_per_tree": w.node_steps,
                        "model_evals_per_tree": w.model_evals, "latent_pool_bytes": pool_bytes,
                        "l2": "flushed between steps" if flush else "pool larger than L2",
-                       "rollout": rollout_kind, "parallelism": f"dp{world} over trees, no collective"},
+                       "rollout": kind, "parallelism": f"dp{world} over trees, no collective"},
             "roofline": roof, "cpu_baseline": cpu,
             "e2e": {"value": r4(e2e_value), "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                     "mode": "next pass's inputs copied under this pass", "one_pass_at_a_time": r4(e2e_serial)},
@@ -776,7 +794,8 @@ def main():
     ap.add_argument("--workload", default="group", choices=list(CONFIGS),
                     help="default: group, the largest single-GPU configuration (8 trees x 765 nodes x 4096 x 64, MLP velocity)")
     ap.add_argument("--fused-rollout", action="store_true",
-                    help="closed-form-velocity workloads: all T steps in one launch (tree_rollout_fused)")
+                    help="closed-form-velocity workloads: all T steps in one launch asked for by name (tree_rollout_fused); "
+                         "tree_rollout takes it by itself where it covers the tree")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-also", action="store_true", help="skip the brief runs of the other workloads and the savings run")
     args = ap.parse_args()

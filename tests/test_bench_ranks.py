@@ -47,3 +47,15 @@ def test_rank_group_without_a_launcher_is_a_single_rank():
         for k, v in saved.items():
             if v is not None:
                 os.environ[k] = v
+
+
+def test_the_line_names_the_rollout_that_was_launched():
+    """Kernels of a rollout (the root's, the last log-prob sums' included) -> what the printed line calls it."""
+    sys.path.insert(0, ROOT)
+    import bench
+    from workloads import CONFIGS
+    video, image = CONFIGS["video"], CONFIGS["image"]
+    assert bench.rollout_kind(video, 3) == "one launch" and bench.rollout_kind(video, 2) == "one launch"
+    assert bench.rollout_kind(video, video.T + 2) == "one tree_step per depth"
+    assert bench.rollout_kind(image, 2 * image.T + 2) == "velocity and step per depth"
+    assert bench.rollout_kind(image, 2 * image.T + 2 - 9) == f"velocity and step per depth, 9 of {image.T} depths in one launch"

@@ -186,9 +186,9 @@ def test_sharded_batch_draws_the_same_noise(B):
 
 
 def test_one_call_rollout_is_the_step_by_step_rollout(B):
-    """bgrpo_tree_rollout enqueues the same kernels as T x [velocity, tree_step] (Algorithm 1, "Build rollout tree"):
-    every output is identical bit for bit, for the closed-form and the MLP velocity, and it continues a tree that has
-    already taken some steps."""
+    """bgrpo_tree_rollout makes what T x [velocity, tree_step] makes (Algorithm 1, "Build rollout tree"), a fresh closed-form
+    tree in one launch: every output is identical bit for bit, for the closed-form and the MLP velocity, and it continues a
+    tree that has already taken some steps."""
     for velocity, channels, hidden in (("linear", 4, 0), ("mlp", 64, 256)):
         w = Workload(name="one_call", n_trees=2, tokens=150, channels=channels, T=5, K=3, splits=(0, 3), sigma=0.3,
                      velocity=velocity, reward="mixture", hidden=hidden or 3072, branch_corr_s=2.0)
