@@ -34,7 +34,13 @@ for w in cases:
         s = TreeSession(w, nodes_cap=w.nodes + 3, fused_rollout=fused)
         s.upload_inputs(make_inputs(w))
         for seed in (1, 2):
-            s.run_all(seed=seed)
+            if fused or w.velocity == "mlp":
+                s.run_all(seed=seed)
+            else:                                            # depth by depth (run_all would take the one-launch rollout)
+                s.init(seed)
+                for i in range(w.T):
+                    s.step(i)
+                s.rewards(); s.fuse_advantage(); s.prune()
         out = torch.zeros_like(s.logp)
         if w.velocity == "linear":
             B.tree_logprob(s.tree, -1, None, out)

@@ -39,6 +39,14 @@ def test_video_config_whole_workload(B):
     r = np.array([rewards.neg_mse(lat[0][l], inp.target[0]) for l in topo.leaf_ids()])
     got_r = s.leaf_r.cpu().numpy()[0]
     assert np.abs(got_r - r).max() <= 1e-6 * np.abs(r).max()
+    # depth by depth, in the step kernel's launches of this size, the same bits
+    first_lat, first_logp = s.latents.clone(), s.logp.clone()
+    s.latents.fill_(float("nan"))
+    s.init()
+    for i in range(w.T):
+        s.step(i)
+    torch.cuda.synchronize()
+    assert torch.equal(s.latents, first_lat) and torch.equal(s.logp, first_logp)
     # reductions, teacher-forced on the oracle's float32 rewards and log-probs
     s.logp.copy_(torch.from_numpy(logp.astype(np.float32)))
     s.leaf_r.copy_(torch.from_numpy(r.astype(np.float32)[None]))

@@ -62,6 +62,11 @@ def test_guard_bands_survive_whole_ragged_passes(B, velocity):
     s, g = _guarded_session(w, nodes_cap=w.nodes + 5)
     for seed in (3, 4):
         s.run_all(seed=seed)
+    if velocity == "linear":                                 # depth by depth (run_all takes the one-launch rollout)
+        s.init(seed=5)
+        for i in range(w.T):
+            s.step(i)
+        s.rewards(); s.fuse_advantage(); s.prune()
     extra = g.make("logp_new", s.logp)
     ess = g.make("ess", s.logp)
     terms = g.make("terms", s.logp)
@@ -69,7 +74,7 @@ def test_guard_bands_survive_whole_ragged_passes(B, velocity):
     fused_guards = None
     if velocity == "linear":
         B.tree_logprob(s.tree, -1, None, extra)
-        fused, fused_guards = _guarded_session(w, nodes_cap=w.nodes + 5)      # the one-launch rollout on the same shapes
+        fused, fused_guards = _guarded_session(w, nodes_cap=w.nodes + 5)      # the one-launch rollout asked for by name
         fused.fused_rollout = True
         fused.run_all(seed=5)
     else:

@@ -135,8 +135,18 @@ RAGGED = [
 ]
 
 
+def _grow(s, by_steps, seed=None):
+    """A rollout of a closed-form session: tree_rollout, which takes one launch where it can, or tree_step depth by depth."""
+    if not by_steps:
+        return s.rollout(seed)
+    s.init(seed)
+    for i in range(s.w.T):
+        s.step(i)
+
+
+@pytest.mark.parametrize("by_steps", [False, True], ids=["one_call", "by_steps"])
 @pytest.mark.parametrize("case", RAGGED, ids=[c[0] for c in RAGGED])
-def test_rollout_parity_over_tiles_and_tails(B, case):
+def test_rollout_parity_over_tiles_and_tails(B, case, by_steps):
     name, n_trees, tokens, channels, T, K, splits, sigma, s_corr, base, extra = case
     w = Workload(name=name, n_trees=n_trees, tokens=tokens, channels=channels, T=T, K=K, splits=splits, sigma=sigma,
                  velocity="linear", reward="neg_mse_mu", branch_corr_s=s_corr, seed=991 + T)
@@ -145,7 +155,8 @@ def test_rollout_parity_over_tiles_and_tails(B, case):
     s = _session(w, tree_id_base=base, nodes_cap=cap)
     s.upload_inputs(inp)
     s.latents.fill_(float("nan"))
-    s.run_all()
+    _grow(s, by_steps)
+    s.rewards()
     torch.cuda.synchronize()
     topo, lat, logp = oracle_rollout(w, inp, n_trees, tree_id_base=base, nodes_cap=cap)
     assert_table(s, topo, n_trees)
@@ -159,12 +170,12 @@ def test_rollout_parity_over_tiles_and_tails(B, case):
         assert np.abs(s.leaf_r.cpu().numpy()[t] - r).max() <= 1e-5 * max(1.0, np.abs(r).max())
     # running the same handle again with the same seed reproduces every bit (fixed reduction order)
     first_lat, first_logp = s.latents.clone(), s.logp.clone()
-    s.rollout()
+    _grow(s, by_steps)
     torch.cuda.synchronize()
     assert torch.equal(first_logp[:, :topo.nodes], s.logp[:, :topo.nodes])
     assert torch.equal(first_lat[:, :topo.nodes], s.latents[:, :topo.nodes])
     # and another seed gives another tree
-    s.rollout(seed=12345)
+    _grow(s, by_steps, seed=12345)
     torch.cuda.synchronize()
     if sigma > 0:
         assert not torch.equal(first_lat[:, :topo.nodes], s.latents[:, :topo.nodes])
@@ -612,7 +623,7 @@ def test_fused_rollout_matches_oracle_and_stepwise(B, tokens, channels, n_trees,
     fused.rollout()
     step = _session(w)
     step.upload_inputs(inp)
-    step.rollout()
+    _grow(step, by_steps=True)
     torch.cuda.synchronize()
     B.tree_sync_status(fused.tree)
     assert_table(fused, topo, n_trees)
