@@ -47,14 +47,14 @@ NOMINAL_HBM_GBS = 8000.0
 # proportion to the units).  It is reported only while the kernel's sources still hash to what was captured.
 NCU_TRAFFIC = {
     # step kernel: one capture per operand layout (8 B/element with the closed-form velocity, 12 B/element with a velocity buffer)
-    "step_kernel_linear": {"bytes": 75.596544e6 + 13.034496e6, "units": 8 * 2096640,             # profiles/step_kernel_video.md
-                           "sources": ("tree_step.cu", "philox.cuh"), "shape": "kStep", "source_hash": "d569995ada83"},
-    "step_kernel_mlp": {"bytes": 531.169024e6 + 215.974400e6, "units": 32 * 16 * 129600,         # profiles/step_kernel_image_batch.md
-                        "sources": ("tree_step.cu", "philox.cuh"), "shape": "kStep", "source_hash": "d569995ada83"},
-    "mlp_velocity_kernel": {"bytes": 266.295296e6 + 213.379328e6, "units": 1036800,       # profiles/mlp_velocity_kernel_image_batch.md
-                            "sources": ("mlp_velocity.cu",), "shape": "kMlp", "source_hash": "74593cdd150d"},
-    "rollout_fused_kernel": {"bytes": 16.816640e6 + 866.172416e6, "units": 110 * 2096640,  # profiles/rollout_fused_kernel_video.md
-                             "sources": ("tree_fused.cu", "philox.cuh"), "shape": "kFused", "source_hash": "d4f0707c5632"},
+    "step_kernel_linear": {"bytes": 75.786752e6 + 13.725440e6, "units": 8 * 2096640,             # profiles/step_kernel_video.md
+                           "sources": ("tree_step.cu", "philox.cuh"), "shape": "kStep", "source_hash": "7f2c0e55c310"},
+    "step_kernel_mlp": {"bytes": 531.953408e6 + 218.003968e6, "units": 32 * 16 * 129600,         # profiles/step_kernel_image_batch.md
+                        "sources": ("tree_step.cu", "philox.cuh"), "shape": "kStep", "source_hash": "7f2c0e55c310"},
+    "mlp_velocity_kernel": {"bytes": 266.727680e6 + 215.012096e6, "units": 1036800,       # profiles/mlp_velocity_kernel_image_batch.md
+                            "sources": ("mlp_velocity.cu",), "shape": "kMlp", "source_hash": "cccfd06d2864"},
+    "rollout_fused_kernel": {"bytes": 25.279488e6 + 864.974592e6, "units": 110 * 2096640,  # profiles/rollout_fused_kernel_video.md
+                             "sources": ("tree_fused.cu", "philox.cuh"), "shape": "kFused", "source_hash": "1330d07d262f"},
 }
 
 

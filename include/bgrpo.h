@@ -138,8 +138,8 @@ bgrpo_status bgrpo_velocity_linear_bind(bgrpo_tree* tree, const float* mu_dev, f
  * 1e-7 * D in the exponent - fine for D up to a few thousand, meaningless at D ~ 1e5 (use a scale of order 1 there, as the
  * workloads do).  At step time the squared residual is taken as g^2 xi^2 from the drawn noise, tree_logprob takes it
  * from the stored child; the two agree to the rounding of the child (test: rho = 1 within 1e-5).
- * The sums are completed, in a fixed order, by the next call for this tree that is enqueued on the stream (the next
- * tree_step's kernel does it in its prologue) and at the latest by the step that completes the tree, which enqueues a
+ * The sums are completed by the next call for this tree that is enqueued on the stream (the next tree_step's kernel
+ * does it beside its own work) and at the latest by the step that completes the tree, which enqueues a
  * small flush kernel: buffers.logp of a level is final once one of those has run.  Use one stream per tree handle.
  * Errors: STATE (already at depth T; NULL v_dev without a bound velocity), CAPACITY (children exceed nodes_cap), CUDA. */
 bgrpo_status bgrpo_tree_step(bgrpo_tree* tree, int32_t split_flag, const float* v_dev, void* stream);
@@ -181,8 +181,8 @@ bgrpo_status bgrpo_tree_logprob(bgrpo_tree* tree, int32_t step, const float* v_d
  * streams (packed_dev: device, bgrpo_velocity_mlp_packed_bytes(hidden) bytes, 1024-byte aligned).
  * W1_bf16_dev: device [64][hidden] bf16 bits; W2_bf16_dev: device [hidden][64] bf16 bits.
  * v_out_dev: device [n_trees][W_i][D] float32.  Frontiers of fewer 128-token tiles than SMs are cut along the hidden
- * dimension as well; the partial sums of that split live in the tree's scratch (the workspace query accounts for them)
- * and are added in a fixed order, so repeated calls give identical bits. */
+ * dimension as well; the partial sums of that split stay in the shared memory of a thread-block cluster and are added in
+ * a fixed order, so repeated calls give identical bits. */
 size_t       bgrpo_velocity_mlp_packed_bytes(int32_t hidden);
 bgrpo_status bgrpo_velocity_mlp_pack(const uint16_t* W1_bf16_dev, const uint16_t* W2_bf16_dev, int32_t hidden,
                                      void* packed_dev, void* stream);

@@ -87,7 +87,7 @@ struct StepCoef {
 };
 
 // Log-probs of a level whose per-(row, chunk, warp) partial sums are in scratch but not yet added up.  The sum is
-// taken by the next kernel the library enqueues on the stream (the next step's prologue, or a small flush kernel).
+// taken by the next kernel the library enqueues on the stream (the next step, beside its own work, or a small flush kernel).
 struct FinalizeDesc {
     float* logp_out;       // nullptr: nothing pending
     int32_t W, off;        // rows off .. off+W-1 of every tree
@@ -258,7 +258,7 @@ struct StepLaunch {
     int32_t* status;           // the tree's status word
     int32_t per_row;           // 32-bit words reserved per node row in the partials
     unsigned long long* partials;   // by row, per_row / 2 apart: [nchunks][warps of a CTA] sums of quantized squares (philox.cuh)
-    FinalizeDesc prev;         // level to finalize in this launch's prologue (logp_out == nullptr: none)
+    FinalizeDesc prev;         // level whose sums this launch takes (logp_out == nullptr: none)
 };
 cudaError_t launch_root(const bgrpo_tree* t, cudaStream_t s);
 cudaError_t launch_step(const StepLaunch& p, cudaStream_t s);
