@@ -48,13 +48,13 @@ NOMINAL_HBM_GBS = 8000.0
 NCU_TRAFFIC = {
     # step kernel: one capture per operand layout (8 B/element with the closed-form velocity, 12 B/element with a velocity buffer)
     "step_kernel_linear": {"bytes": 75.786752e6 + 13.725440e6, "units": 8 * 2096640,             # profiles/step_kernel_video.md
-                           "sources": ("tree_step.cu", "philox.cuh"), "shape": "kStep", "source_hash": "7f2c0e55c310"},
+                           "sources": ("tree_step.cu", "philox.cuh"), "shape": "kStep", "source_hash": "c4501886b74e"},
     "step_kernel_mlp": {"bytes": 531.953408e6 + 218.003968e6, "units": 32 * 16 * 129600,         # profiles/step_kernel_image_batch.md
-                        "sources": ("tree_step.cu", "philox.cuh"), "shape": "kStep", "source_hash": "7f2c0e55c310"},
+                        "sources": ("tree_step.cu", "philox.cuh"), "shape": "kStep", "source_hash": "c4501886b74e"},
     "mlp_velocity_kernel": {"bytes": 266.727680e6 + 215.012096e6, "units": 1036800,       # profiles/mlp_velocity_kernel_image_batch.md
                             "sources": ("mlp_velocity.cu",), "shape": "kMlp", "source_hash": "cccfd06d2864"},
     "rollout_fused_kernel": {"bytes": 25.279488e6 + 864.974592e6, "units": 110 * 2096640,  # profiles/rollout_fused_kernel_video.md
-                             "sources": ("tree_fused.cu", "philox.cuh"), "shape": "kFused", "source_hash": "1330d07d262f"},
+                             "sources": ("tree_fused.cu", "philox.cuh"), "shape": "kFused", "source_hash": "2ce9e3414b6a"},
 }
 
 

@@ -190,10 +190,21 @@ __device__ __forceinline__ void finalize_row(const FinalizeDesc& f, int64_t row,
     if (t == 0) f.logp_out[row] = logp_from_squares(s, half_per, f.g, f.logp_const);
 }
 
-// All rows of the pending level, one warp per row.
+// All rows of the pending level: one warp per row, or one lane where a row's sum is one number (added with atomics, and cleared
+// for the next who adds).
 __device__ __forceinline__ void finalize_rows(const FinalizeDesc& f, int32_t n_trees, int32_t nodes_cap,
                                               double half_per, int warp_global, int warps_total, int32_t* status, int32_t per_row_cap) {
     const int n_rows = n_trees * f.W;
+    if (f.clear) {
+        for (int idx = warp_global + (threadIdx.x & 31) * warps_total; idx < n_rows; idx += 32 * warps_total) {      // spread over the warps first
+            const int tree = idx / f.W;
+            const int64_t row = static_cast<int64_t>(tree) * nodes_cap + f.off + (idx - tree * f.W);
+            if (!BGRPO_IN_BOUNDS(status, f.off + f.W <= nodes_cap && f.per_row == 1 && f.stride == 1)) continue;
+            f.logp_out[row] = logp_from_squares(__ldcg(f.sums + row), half_per, f.g, f.logp_const);
+            f.sums[row] = 0ull;
+        }
+        return;
+    }
     for (int idx = warp_global; idx < n_rows; idx += warps_total) {
         const int tree = idx / f.W;
         const int64_t row = static_cast<int64_t>(tree) * nodes_cap + f.off + (idx - tree * f.W);
