@@ -146,13 +146,13 @@ bgrpo_status bgrpo_tree_step(bgrpo_tree* tree, int32_t split_flag, const float* 
 
 /* tree_rollout: the remaining steps of the tree, depth .. T-1, in one host call (Algorithm 1, "Build rollout tree": for
  * every step, the velocity of every live node, then the step that forks or advances it).  With packed_dev the kernels
- * of bgrpo_velocity_mlp and bgrpo_tree_step in turn, one launch for both on a small frontier; a whole tree under the bound linear
+ * of bgrpo_velocity_mlp and bgrpo_tree_step in turn, or one launch for both; a whole tree under the bound linear
  * velocity takes the one launch of bgrpo_tree_rollout_fused where that covers it.  Every output is identical bit for bit to
  * the step-by-step calls either way (log-probs because the sums of squares are added as integers).
  *   split_flags_host  host array of T flags (indexed by step), non-zero = fork every node into K children
  *   packed_dev        device, packed MLP weights (bgrpo_velocity_mlp_pack), or NULL for the bound linear velocity
- *   v_dev             device [n_trees][W_max][D] float32 scratch for the velocities of the widest frontier (NULL allowed
- *                     with packed_dev == NULL)
+ *   v_dev             device [n_trees][W_max][D] float32 scratch for the velocities of the widest frontier, holds the last
+ *                     step's afterwards (NULL allowed with packed_dev == NULL)
  * Errors: those of the two calls (the tree keeps the depth it reached); INVALID_ARG, STATE as stated for them. */
 bgrpo_status bgrpo_tree_rollout(bgrpo_tree* tree, const uint8_t* split_flags_host, const void* packed_dev, int32_t hidden,
                                 float* v_dev, void* stream);
@@ -175,8 +175,9 @@ bgrpo_status bgrpo_tree_rollout_fused(bgrpo_tree* tree, const uint8_t* split_fla
  * logp_out_dev: device [n_trees][nodes_cap], indexed like buffers.logp; only the addressed edges are written. */
 bgrpo_status bgrpo_tree_logprob(bgrpo_tree* tree, int32_t step, const float* v_dev, float* logp_out_dev, void* stream);
 
-/* Per-token MLP stand-in for the denoiser: v = bf16(GELU(bf16(z) W1)) W2, bf16 operands, float32 accumulation, float32
- * output, evaluated for every node of the CURRENT frontier on tcgen05 tensor cores.  channels must be 64 and hidden a
+/* Per-token MLP stand-in for the denoiser: v = GELU(bf16(z) W1) W2 with bf16 operands, float32 accumulation and float32 output.
+ * Of an activation only the even half GELU(x) - x/2 is rounded to bf16; the linear half is a product with W1 W2 / 2, which the
+ * packing forms in 64 bits and keeps to 16.  Evaluated for every node of the CURRENT frontier on tcgen05 tensor cores.  channels must be 64 and hidden a
  * multiple of 128.  bgrpo_velocity_mlp_pack reorders the weights once into the tiled shared-memory image the kernel
  * streams (packed_dev: device, bgrpo_velocity_mlp_packed_bytes(hidden) bytes, 1024-byte aligned).
  * W1_bf16_dev: device [64][hidden] bf16 bits; W2_bf16_dev: device [hidden][64] bf16 bits.

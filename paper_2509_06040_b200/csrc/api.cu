@@ -261,6 +261,7 @@ static void fill_step_launch(const bgrpo_tree* t, int step, const float* v_dev, 
     p->g = k.g;
     p->mix_shared = t->mix_shared;
     p->mix_innov = t->mix_innov;
+    p->keep_v = 0;
 }
 
 // Checks the step and fills in its launch.
@@ -344,6 +345,7 @@ bgrpo_status bgrpo_tree_rollout(bgrpo_tree* t, const uint8_t* split_flags_host, 
             if (st != BGRPO_OK) return st;
             StepLaunch p;
             st = prepare_step(t, split_flags_host[i] ? 1 : 0, v_dev, &p);
+            p.keep_v = i + 1 == t->desc.T ? 1 : 0;      // what the buffer holds in the end are the last step's
             bool stepped = false;
             const cudaError_t e = enqueue_mlp(t, packed_dev, hidden, v_dev, st == BGRPO_OK ? &p : nullptr, &stepped, stream);
             if (e != cudaSuccess) return cuda_fail(e, "mlp kernel");

@@ -1,17 +1,17 @@
-"""Derives the bf16 coefficients of the packed GELU polynomial in mlp_velocity.cu.
+"""Derives the constants of the even part of GELU in mlp_velocity.cu.
 
     python paper_2509_06040_b200/csrc/gelu_poly_fit.py
 
-2 GELU(x) = x + x erf(x / sqrt 2) = x + s Q(s), s = x^2.  Q (degree 2 in s) is fitted to erf(x / sqrt 2) / x on
-|x| <= 1 so that the largest error of s Q(s) is smallest (weighted least squares with Lawson's reweighting); the
-kernel evaluates in bf16, so the coefficients are rounded to bf16 one after the other, each time refitting the ones
-not yet fixed.  (The kernel works on y = 2x and uses the coefficients divided by 2, 8 and 32: exact.)  Prints the
-coefficients, their bf16 bit patterns and the largest error of the rounded polynomial.
+GELU(x) = x / 2 + E(x), E(x) = x erf(x / sqrt 2) / 2, which is even.  On |x| <= 1 the kernel evaluates, with y = 2x and
+t = y^2,  kappa E(x) = t (R0 + R1 t)  in packed bf16.  The factor kappa is free (it is taken back on the outputs), so of the
+two coefficients only the ratio has to suit bf16: for every bf16 R0 in [1, 2) the ratio of the unrounded fit gives R1, and the
+pair is kept whose largest error is smallest (weighted least squares with Lawson's reweighting for the fit and for kappa).  Prints the
+coefficients, their bf16 bit patterns, kappa and the largest error in exact arithmetic.
 """
 import numpy as np
 from scipy.special import erf
 
-RANGE, DEGREE = 1.0, 2
+RANGE = 1.0
 
 
 def to_bf16(x):
@@ -21,30 +21,30 @@ def to_bf16(x):
 
 
 def fit():
-    x = RANGE * np.cos(np.linspace(0.0, np.pi / 2, 4000))
-    s = x * x
-    target = np.where(x > 1e-9, erf(x / np.sqrt(2.0)) / np.maximum(x, 1e-9), np.sqrt(2.0 / np.pi))
-    fixed = {}
-    for _ in range(DEGREE + 1):
-        free = [j for j in range(DEGREE + 1) if j not in fixed]
-        basis = np.stack([s ** j for j in free], axis=1)
-        rest = target - sum(fixed[j] * s ** j for j in fixed)
-        weight = np.ones_like(x)
-        for _ in range(60):
-            coef, *_ = np.linalg.lstsq(basis * (s * weight)[:, None], rest * s * weight, rcond=None)
-            err = np.abs((basis @ coef - rest) * s)
-            weight *= 0.5 + err / err.max()
-            weight /= weight.max()
-        fixed[free[0]] = to_bf16(coef[0])
-    return [fixed[j] for j in range(DEGREE + 1)]
+    x = np.linspace(1e-3, RANGE, 4000)
+    t = 4.0 * x * x
+    target = 0.5 * x * erf(x / np.sqrt(2.0))
+    basis = np.stack([t, t * t], axis=1)
+    weight = np.ones_like(x)
+    for _ in range(200):
+        coef, *_ = np.linalg.lstsq(basis * weight[:, None], target * weight, rcond=None)
+        err = np.abs(basis @ coef - target)
+        weight *= 0.5 + err / err.max()
+        weight /= weight.max()
+    best = None
+    for m in range(128, 256):
+        r0 = m / 128.0
+        r1 = to_bf16(r0 * coef[1] / coef[0])
+        poly = t * (r0 + r1 * t)
+        kappa = float(np.float32(np.dot(weight * target, weight * poly) / np.dot(weight * target, weight * target)))
+        err = np.abs(poly / kappa - target).max()
+        if best is None or err < best[0]:
+            best = (err, r0, r1, kappa)
+    return best
 
 
 if __name__ == "__main__":
-    q = fit()
-    x = np.linspace(-RANGE, RANGE, 400001)
-    s = x * x
-    approx = x + s * sum(q[k] * s ** k for k in range(DEGREE + 1))
-    exact = x * (1.0 + erf(x / np.sqrt(2.0)))
-    for k, c in enumerate(q):
-        print(f"Q{k} = {c!r}  bf16 bits 0x{int(np.float32(c).view(np.uint32)) >> 16:04x}")
-    print("largest |x + s Q(s) - 2 GELU(x)| on |x| <= %.2f: %.3g" % (RANGE, np.abs(approx - exact).max()))
+    err, r0, r1, kappa = fit()
+    for name, v in (("R0", r0), ("R1", r1)):
+        print(f"{name} = {v!r}  bf16 bits 0x{int(np.float32(v).view(np.uint32)) >> 16:04x}")
+    print(f"kappa = {kappa!r}; largest |E| error on |x| <= {RANGE:.2f}: {err:.3g}")

@@ -255,6 +255,7 @@ struct StepLaunch {
     float g;
     float mix_shared, mix_innov;
     int32_t shared_noise;      // 1: finite s at a split step
+    int32_t keep_v;            // step taken along by the MLP stage: 1 if the velocities are to be left in its buffer
     int32_t* status;           // the tree's status word
     int32_t per_row;           // 32-bit words reserved per node row in the partials
     unsigned long long* partials;   // by row, per_row / 2 apart: [nchunks][warps of a CTA] sums of quantized squares (philox.cuh)

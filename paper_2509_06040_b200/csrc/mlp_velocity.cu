@@ -1,14 +1,16 @@
 // Per-token MLP velocity stage on the 5th-generation tensor cores (tcgen05 + tensor memory):
-//     v = bf16(GELU(bf16(z) W1)) W2,   z: [tokens][64] fp32,  W1: [64][H],  W2: [H][64],  fp32 accumulation, fp32 output.
+//     v = GELU(bf16(z) W1) W2,   z: [tokens][64] fp32,  W1: [64][H],  W2: [H][64] bf16,  fp32 accumulation, fp32 output.
 // It stands in for the denoiser mu_theta of Eq. 2 and is evaluated once per PARENT node of the frontier; the
 // K children of a parent share the result (the saving the rollout tree exists for).
 //
 // One persistent CTA per SM walks 128-token tiles.  For each tile the hidden dimension is cut into chunks of 128:
 //     GEMM1(c): D1[128 tok][128 hid]  = A[128 tok][64]      * 2 W1_c      (4 MMAs of K = 16, accumulator in TMEM)
-//     GELU     : H_c = bf16(4 GELU(D1 / 2))  TMEM -> registers -> TMEM: the hidden activation never leaves tensor memory
+//     GELU     : H_c = bf16(kappa E(D1 / 2)), E(x) = GELU(x) - x / 2, TMEM -> registers -> TMEM: it never leaves tensor memory
 //     GEMM2(c): D2[128 tok][64]      += H_c[128 tok][128]   * W2_c        (8 MMAs of K = 16, A operand read from TMEM)
-// and the output tile is v = D2 / 4 (the factors are powers of two: taking them out of the 3072 activations of a token and
-// applying them to the 64 outputs changes no rounding).
+// where D2 starts as A * (kappa W1 W2 / 2), the linear half of GELU (a 64 x 64 matrix held as the sum of two bf16 ones, 8 MMAs a
+// tile), and the output tile is v = D2 / kappa.  Only the even half E goes through bf16, and as |E| is a fraction of |x| / 2 its
+// roundings weigh less than those of the whole activation: rms error against 64 bits 1.6e-3 of rms(v), where 2.5e-3 was reached with
+// bf16(GELU), and a polynomial with one coefficient less (1 036 800 tokens, hidden 3072: 712 -> 705 us, 16 200 tokens 17.3 -> 16.5).
 // Tensor memory (512 columns): three chunk buffers of 128 columns and two output accumulators of 64.  A chunk buffer
 // holds D1 of its chunk and then, in place, the packed activations: a warp reads its 64 accumulator columns into
 // registers and later writes its 32 packed columns over the first half of exactly those columns, so no warp ever writes
@@ -23,6 +25,7 @@
 //     warps 2..17  GELU epilogue in two groups of eight: group p takes the chunks of parity p, two warps per TMEM lane
 //                  quarter with 64 columns each.  All sixteen warps write the output tile (D2 is double-buffered, and a
 //                  tile is written out two chunks after its last GEMM2 was issued, when it has long completed);
+//     warps 20..27 (where the step is taken along with whole tiles) make the children of the tile before;
 //     warp 18      brings the NEXT tile's latents in with bulk asynchronous copies (one per tree the tile touches) into
 //                  a float32 staging buffer and converts them to the bf16 A tile while the current tile computes.  (Plain
 //                  loads from one warp kept only 4 KiB in flight and took longer per tile than the arithmetic.)  The
@@ -57,7 +60,11 @@ constexpr int kMaxSplit = 8;               // CTAs of a cluster that share a til
 constexpr int kEpiWarps = 16;             // two groups of eight: two warps per TMEM lane quarter, 64 columns of a chunk each
 constexpr int kLoaderWarp = 2 + kEpiWarps;
 constexpr int kGemm2Warp = 3 + kEpiWarps;
-constexpr int kMlpThreads = (4 + kEpiWarps) * 32;
+constexpr int kStepWarps = 8;              // make the children of whole tiles; four: 880 us where eight take 842 (see launch_mlp), twelve 909
+// What a launch does besides the velocity: nothing, or the step that follows, where tiles are split over a cluster or whole.
+enum { kNoStep = 0, kStepOfSplit = 1, kStepOfWhole = 2 };
+template <int MODE>
+constexpr int kMlpThreads = (4 + kEpiWarps + (MODE == kStepOfWhole ? kStepWarps : 0)) * 32;
 constexpr uint32_t kTileBytes = kTok * 128;              // one [128 rows][128 B] operand tile = 16 KiB
 constexpr uint32_t kChunkBytes = 2 * kTileBytes;         // packed weights of a chunk: W1_c (16 KiB) then W2_c (16 KiB)
 constexpr uint32_t kTmemCols = 512;       // three chunk buffers of 128 columns (index = chunk mod 3), then D2: 2 x 64 (index = tile parity)
@@ -66,15 +73,18 @@ constexpr uint32_t kD2Col = kBufs * kHc;
 constexpr int kGroupWarps = kEpiWarps / 2; // epilogue warps that work on one chunk
 constexpr long long kWaitCycles = 4000000000ll;      // about two seconds of SM clock
 
+template <int MODE>
 struct MlpSmem {
     alignas(1024) unsigned char w1[kW1Stages][kTileBytes];  // W1_c tile [128 n = hidden][128 B = 64 channels]
     alignas(1024) unsigned char w2[kW2Stages][kTileBytes];  // W2_c as two [64 n = channel][128 B = 64 hidden] tiles
     alignas(1024) unsigned char a[2][kTileBytes];           // bf16(z) tile [128 tok][128 B], double-buffered over tiles
     alignas(1024) float stage[kTok * kCh];                   // float32 latents of the next tile, as they are in global memory; split
                                                              // mode, at the end: this CTA's partial output tile
+    alignas(1024) float vtile[MODE == kStepOfWhole ? kTok * kCh : 4];     // velocities of the tile whose children are being made
+    unsigned long long v_full, v_free;
     unsigned long long w1_full[kW1Stages], w1_free[kW1Stages], w2_full[kW2Stages], w2_free[kW2Stages];
     unsigned long long stage_full, first_a, a_full[2], a_empty[2], d1_full[kBufs], h_full[kBufs], buf_free[kBufs], d2_full[2], d2_empty[2];
-    uint32_t node_sums[kTok][BGRPO_MAX_K][2];    // the step taken along: squares of the noise by parent in the tile and child, low 16 bits and the rest
+    uint32_t node_sums[MODE == kStepOfSplit ? kTok : 1][BGRPO_MAX_K][2];    // the step taken along: squares of the noise by parent in the tile and child, low 16 bits and the rest
     uint32_t tmem_base;
     int abort_flag;
 };
@@ -216,19 +226,20 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
     return r;
 }
-// The packed W1 is 2 W1, so the accumulator of GEMM1 is y = 2x, and the activation handed to GEMM2 is 4 GELU(x); the
-// output tile takes the factor back.  All of it is powers of two: no rounding changes.
+// GELU(x) = x / 2 + E(x) with E(x) = x erf(x / sqrt 2) / 2 even.  The packed W1 is 2 W1, so the accumulator of GEMM1 is y = 2x,
+// and what GEMM2 gets for an activation is kappa E(x); the linear part is a product with kappa W1 W2 / 2.
 //
-// 4 GELU(y / 2) in the tanh form on the hardware tanh: 2x (1 + tanh(sqrt(2/pi) (x + 0.044715 x^3))).  The tanh form
+// kappa E in the tanh form on the hardware tanh: kappa x / 2 tanh(sqrt(2/pi) (x + 0.044715 x^3)).  The tanh form
 // differs from the erf form by < 5e-4 absolute, below the bf16 rounding of the activation that follows.  One
 // special-function instruction per activation: this is the slow, range-free form, used only where the packed polynomial
 // below does not apply.
-__device__ __forceinline__ float gelu_x4(float y) {
+constexpr float kKappa = 11.144685745239258f, kInvKappa = static_cast<float>(1.0 / 11.144685745239258);
+__device__ __forceinline__ float even_tanh(float y) {
     const float x = 0.5f * y, x2 = x * x;
     const float u = x * fmaf(x2, 0.0356774081f, 0.7978845608f);
     float th;
     asm("tanh.approx.f32 %0, %1;" : "=f"(th) : "f"(u));
-    return fmaf(y, th, y);
+    return 0.25f * kKappa * (y * th);
 }
 // Packed bf16 arithmetic on two activations at a time (one FMA-pipe instruction for both halves).
 __device__ __forceinline__ uint32_t bf2_mul(uint32_t a, uint32_t b) {
@@ -241,28 +252,20 @@ __device__ __forceinline__ uint32_t bf2_fma(uint32_t a, uint32_t b, uint32_t c) 
     asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
     return d;
 }
-// The erf-form GELU for |x| < 1 without a special-function instruction:
-//     2 GELU(x) = x + x erf(x / sqrt 2) = x + s Q(s),   s = x^2,
-// with Q a quadratic in s fitted to erf(x / sqrt 2) / x on [0, 1] (minimax in s Q(s), the coefficients rounded to bf16
-// one after the other and the rest refitted by csrc/gelu_poly_fit.py; the polynomial is within 8e-5 of the function).
-// In y = 2x it is 4 GELU(x) = y + t R(t) with t = y^2 and R's coefficients Q0 / 2, Q1 / 8, Q2 / 32, exact in bf16 too.
-// Evaluated on a packed pair in bf16: one multiply and three fused multiply-adds on the FMA pipe, where one hardware
-// tanh per activation (sixteen per clock and SM) bounds the whole stage at twice the tensor-core time.  The last
-// operation adds the small even part to y and rounds once, so for the usual |x| << 1 the result differs from the
-// correctly rounded activation by the rounding of x to bf16 and little else.
-constexpr uint32_t kGeluR0 = 0x3ecc3eccu;   //  0.796875 / 2
-constexpr uint32_t kGeluR1 = 0xbc84bc84u;   // -0.12890625 / 8
-constexpr uint32_t kGeluR2 = 0x39f239f2u;   //  0.0147705078125 / 32
+// kappa E(x) for |x| < 1 without a special-function instruction: t (R0 + R1 t), t = y^2 (csrc/gelu_poly_fit.py; within 3.1e-4 of
+// E, and E is rounded to bf16 at once).  kappa is what gives both coefficients short bf16 forms.  Two multiplies and one fused
+// multiply-add on a packed pair, where one hardware tanh per activation (sixteen per clock and SM) bounds the whole stage at twice
+// the tensor-core time.  (In float32 on pairs, fma.f32x2, three of them for a cubic: 747 us for 1 036 800 tokens.)
+constexpr uint32_t kEvenR0 = 0x3f8d3f8du;   //  1.1015625
+constexpr uint32_t kEvenR1 = 0xbd1bbd1bu;   // -0.037841796875
+__device__ __forceinline__ uint32_t even_poly(uint32_t y) {
+    const uint32_t t = bf2_mul(y, y);
+    return bf2_mul(t, bf2_fma(kEvenR1, t, kEvenR0));
+}
 // The polynomial's range |x| < 1 is |y| < 2: the top exponent bit of both bf16 halves clear.  One bit to look at is why y
 // is doubled: the check of 32 packed pairs is 16 three-operand ORs where a running maximum of magnitudes took 32
 // operations (1 036 800 tokens, hidden 3072: 733 -> 719 us).  NaN and infinity have the bit set.
-constexpr uint32_t kGeluOutside = 0x40004000u;
-__device__ __forceinline__ uint32_t gelu_x4_poly(uint32_t y) {
-    const uint32_t s = bf2_mul(y, y);
-    uint32_t t = bf2_fma(kGeluR2, s, kGeluR1);
-    t = bf2_fma(t, s, kGeluR0);
-    return bf2_fma(t, s, y);
-}
+constexpr uint32_t kEvenOutside = 0x40004000u;
 // byte offset of the 16-byte piece `c16` of row r inside a 128-byte-swizzled tile of 128-byte rows
 __device__ __forceinline__ uint32_t sw128(uint32_t r, uint32_t c16) { return r * 128u + ((c16 ^ (r & 7u)) << 4); }
 
@@ -310,7 +313,7 @@ struct MlpArgs {
     int64_t tokens_per_tree;  // frontier tokens of one tree (W_i * tokens)
     int64_t n_tokens;         // all frontier tokens
     const unsigned char* packed;
-    float* v_out;
+    float* v_out;             // nullptr: the step is taken along and the velocities are not kept
     int32_t n_chunks;         // hidden / 128
     int32_t n_tiles;
     int32_t split;            // CTAs per tile along the hidden dimension (1: none); > 1 only with one tile per cluster of that size
@@ -385,15 +388,144 @@ __device__ __forceinline__ void step_children(const StepLaunch& sp, int row0, co
         }
 }
 
-// STEP: the step that follows is taken along (split tiles): the tail has the velocity of its rows in registers, so it writes
+// A whole tile of the step taken along, of nodes of at least kTok tokens: it touches two nodes at most, A up to row `edge` and
+// B behind it.  Addresses and element numbers are those of row 0, so that a row is one multiply-add away from its own.
+struct StepTile {
+    int32_t rows, edge;
+    const float4 *z_a, *z_b;
+    float4 *child_a, *child_b;        // first child
+    uint32_t e_a, e_b;
+    int32_t parent_a, parent_b, child0_a, child0_b;       // rows of the pool
+};
+__device__ __forceinline__ StepTile make_step_tile(const StepLaunch& sp, const MlpArgs& p, int64_t first_token, int rows) {
+    StepTile q;
+    const uint32_t tokens = static_cast<uint32_t>(p.tokens), first = static_cast<uint32_t>(first_token);      // a pool of 2^32 tokens is 1 TB
+    const uint32_t row = first / tokens, tok = first - row * tokens;
+    q.rows = rows;
+    q.edge = tokens - tok < static_cast<uint32_t>(kTok) ? static_cast<int32_t>(tokens - tok) : kTok;
+    auto node = [&](int32_t n, int32_t tok0, const float4*& z, float4*& child, uint32_t& e, int32_t& parent, int32_t& child0) {
+        const int32_t tree = n / sp.W_in, j = n - tree * sp.W_in;
+        parent = tree * sp.nodes_cap + sp.off_in + j;
+        child0 = tree * sp.nodes_cap + sp.off_out + j * sp.fan;
+        if (tok0 < rows && !BGRPO_IN_BOUNDS(sp.status, tree < sp.n_trees && sp.off_in + j < sp.nodes_cap && sp.off_out + (j + 1) * sp.fan <= sp.nodes_cap)) q.rows = 0;
+        e = static_cast<uint32_t>(-tok0) * (kCh / 4);
+        z = reinterpret_cast<const float4*>(sp.latents + parent * sp.D) - static_cast<int64_t>(tok0) * (kCh / 4);
+        child = reinterpret_cast<float4*>(sp.latents + child0 * sp.D) - static_cast<int64_t>(tok0) * (kCh / 4);
+    };
+    node(static_cast<int32_t>(row), -static_cast<int32_t>(tok), q.z_a, q.child_a, q.e_a, q.parent_a, q.child0_a);
+    node(static_cast<int32_t>(row) + 1, q.edge, q.z_b, q.child_b, q.e_b, q.parent_b, q.child0_b);
+    return q;
+}
+// Node-table row of a child: one thread per child.
+__device__ __forceinline__ void step_table(const StepLaunch& sp, int32_t parent, int32_t child0, int b) {
+    const int64_t rows = static_cast<int64_t>(sp.n_trees) * sp.nodes_cap, n = child0 + b;
+    sp.table[n] = parent % sp.nodes_cap;
+    sp.table[rows + n] = sp.step + 1;
+    sp.table[2 * rows + n] = sp.is_split ? sp.step : sp.table[2 * rows + parent];
+    sp.table[3 * rows + n] = sp.is_split ? b : sp.table[3 * rows + parent];
+}
+template <int N>
+__device__ __forceinline__ void step_load(const StepTile& q, int32_t r0, int32_t stride, uint32_t c4, float4 (&z)[N]) {
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        const int32_t r = r0 + k * stride;
+        if (r < q.rows) z[k] = __ldcg((r < q.edge ? q.z_a : q.z_b) + r * (kCh / 4) + c4);
+    }
+}
+// The children of one float4 of N rows, given their velocities in shared memory: N chains of noise in flight.  `z` has the
+// parents; once they are used `then` may ask for the next ones.  Whole warps.
+template <int N, class Then>
+__device__ __forceinline__ void step_rows(const StepLaunch& sp, const MlpArgs& p, const StepTile& q, int64_t first, int32_t r0, int32_t stride, uint32_t c4,
+                                          float* vtile, float4 (&z)[N], Then then) {
+    float4 m[N];
+    NoiseElement el[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        const int32_t r = r0 + k * stride;
+        if (r < q.rows) {
+            const float4 v = *part_piece(vtile, static_cast<uint32_t>(r), c4);
+            if (p.v_out) reinterpret_cast<float4*>(p.v_out)[(first + r) * (kCh / 4) + c4] = v;
+            m[k] = fma4(sp.ca, z[k], mul4(sp.cb, v));
+        }
+    }
+    then();
+    if (sp.g != 0.0f)
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            const int32_t r = r0 + k * stride;
+            const uint32_t e = (r < q.edge ? q.e_a : q.e_b) + static_cast<uint32_t>(r) * (kCh / 4) + c4;
+            el[k] = noise_element(e, BGRPO_TAG_INNOV, sp.keys);
+        }
+#pragma unroll 1
+    for (int b = 0; b < sp.fan; ++b) {
+        float4* const child_a = q.child_a + b * (sp.D / 4);
+        float4* const child_b = q.child_b + b * (sp.D / 4);
+        if (sp.g == 0.0f) {
+#pragma unroll
+            for (int k = 0; k < N; ++k) {
+                const int32_t r = r0 + k * stride;
+                if (r < q.rows) (r < q.edge ? child_a : child_b)[r * (kCh / 4) + c4] = m[k];
+            }
+            continue;
+        }
+        const NoiseNode node_a = noise_node(sp.node_id_base + q.child0_a + b, sp.step, sp.keys), node_b = noise_node(sp.node_id_base + q.child0_b + b, sp.step, sp.keys);
+        uint32_t sum_a = 0u, sum_b = 0u;          // N numbers at most of 25 bits
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            const int32_t r = r0 + k * stride;
+            const bool in_a = r < q.edge;
+            float squares;
+            const float4 xi = normal4(philox_from(el[k], {node_a.x, in_a ? node_a.z : node_b.z, in_a ? node_a.w : node_b.w}, sp.keys), squares);
+            if (r < q.rows) {
+                const uint32_t n = quantized_squares(squares);
+                if (in_a) sum_a += n;
+                else sum_b += n;
+                (in_a ? child_a : child_b)[r * (kCh / 4) + c4] = fma4(sp.g, xi, m[k]);
+            }
+        }
+        // the warp's 32 numbers, their 16-bit halves by themselves
+        uint32_t lo = __reduce_add_sync(0xffffffffu, sum_a & 0xffffu), hi = __reduce_add_sync(0xffffffffu, sum_a >> 16);
+        if ((threadIdx.x & 31u) == 0u && (lo | hi) != 0u) atomicAdd(p.row_sums + q.child0_a + b, (static_cast<unsigned long long>(hi) << 16) + lo);
+        if (q.edge < kTok) {
+            lo = __reduce_add_sync(0xffffffffu, sum_b & 0xffffu);
+            hi = __reduce_add_sync(0xffffffffu, sum_b >> 16);
+            if ((threadIdx.x & 31u) == 0u && (lo | hi) != 0u) atomicAdd(p.row_sums + q.child0_b + b, (static_cast<unsigned long long>(hi) << 16) + lo);
+        }
+    }
+}
+// All rows of a tile by THREADS threads, 16 to a row, N rows of a thread at a time.  `v_ready` waits for the velocities; the
+// first parents are asked for before it.  (One row at a time: 849 us for 842; four rows of four warps, which spills, 893.)
+constexpr int kStepRows = 2;
+template <int THREADS, int N, class Wait>
+__device__ __forceinline__ bool step_tile(const StepLaunch& sp, const MlpArgs& p, const StepTile& q, int64_t first, uint32_t t, float* vtile, Wait v_ready) {
+    constexpr int kStride = THREADS / (kCh / 4);
+    const uint32_t c4 = t % (kCh / 4);
+    int32_t r = static_cast<int32_t>(t / (kCh / 4));
+    float4 z[N];
+    step_load<N>(q, r, kStride, c4, z);
+    if (t < static_cast<uint32_t>(sp.fan) && q.e_a == 0u && q.rows > 0) step_table(sp, q.parent_a, q.child0_a, t);
+    if (t >= 32u && t - 32u < static_cast<uint32_t>(sp.fan) && q.edge < q.rows) step_table(sp, q.parent_b, q.child0_b, t - 32);
+    if (!v_ready()) return false;
+#pragma unroll 1
+    for (int32_t done = 0; done < kTok; done += N * kStride, r += N * kStride)
+        step_rows<N>(sp, p, q, first, r, kStride, c4, vtile, z, [&] {
+            if (done + N * kStride < kTok) step_load<N>(q, r + N * kStride, kStride, c4, z);
+        });
+    return true;
+}
+
+// kStepOfWhole: see step_tile().  kStepOfSplit: the tail has the velocity of its rows in registers, so it writes
 // the children next to it, and the launch and the reload of a step kernel are saved.  What does not need the velocity - the
 // parent, the noise, the table - is done while the cluster's barrier is on its way.
-template <bool STEP>
-__global__ void __launch_bounds__(kMlpThreads, 1)
+template <int MODE>
+__global__ void __launch_bounds__(kMlpThreads<MODE>, 1)
 mlp_velocity_kernel(const __grid_constant__ MlpArgs p, const __grid_constant__ StepLaunch sp) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     // the swizzled operand tiles need 1024-byte alignment; the launch reserves 1 KiB of slack for this round-up
-    MlpSmem& sm = *reinterpret_cast<MlpSmem*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
+    using Smem = MlpSmem<MODE>;
+    constexpr int kThreads = kMlpThreads<MODE>;
+    constexpr bool STEP = MODE == kStepOfSplit, WHOLE = MODE == kStepOfWhole;
+    Smem& sm = *reinterpret_cast<Smem*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
     // The shuffle tells the compiler that the warp index is the same in all lanes: roles, ring positions and tensor-memory
     // addresses then live in uniform registers (1 036 800 tokens, hidden 3072: 775 -> 744 us; 7 200 tokens: 30.9 -> 29.3 us).
     const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
@@ -410,9 +542,11 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p, const __grid_constant__ S
         }
         mbar_init(&sm.stage_full, 1);
         mbar_init(&sm.first_a, kEpiWarps);
+        mbar_init(&sm.v_full, kEpiWarps);
+        mbar_init(&sm.v_free, kStepWarps);
         for (int q = 0; q < 2; ++q) {
             mbar_init(&sm.a_full[q], 1);
-            mbar_init(&sm.a_empty[q], 1);
+            mbar_init(&sm.a_empty[q], blockIdx.x % p.split == 0 ? 2 : 1);      // GEMM1 and, where this CTA has it, the linear part
             mbar_init(&sm.d2_full[q], 1);
             mbar_init(&sm.d2_empty[q], kEpiWarps);
         }
@@ -425,7 +559,7 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p, const __grid_constant__ S
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (STEP)
-        for (int i = threadIdx.x; i < kTok * BGRPO_MAX_K * 2; i += kMlpThreads) (&sm.node_sums[0][0][0])[i] = 0u;
+        for (int i = threadIdx.x; i < kTok * BGRPO_MAX_K * 2; i += kThreads) (&sm.node_sums[0][0][0])[i] = 0u;
     if (warp == 1) {      // tensor memory: this warp allocates and, at the end, frees
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sm.tmem_base)), "r"(kTmemCols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -444,6 +578,7 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p, const __grid_constant__ S
     const int n_my_tiles = (p.n_tiles > cta) ? (p.n_tiles - 1 - cta) / n_ctas + 1 : 0;
     const int NC = p.n_chunks / S;            // chunks this CTA adds up per tile: part * NC .. part * NC + NC - 1
     const int n_my_chunks = n_my_tiles * NC;
+    const int lin = part == 0 ? 1 : 0;        // the first of a tile's CTAs adds the linear part
 
     auto tile_rows = [&](int it) -> int {     // tokens of this CTA's tile number `it`
         const int64_t left = p.n_tokens - (static_cast<int64_t>(cta) + static_cast<int64_t>(it) * n_ctas) * kTok;
@@ -468,13 +603,15 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p, const __grid_constant__ S
             }
         } else if (lane == 1) {
             Ring<kW2Stages> r;
-            int cc = 0;
-            for (int g = 0; g < n_my_chunks; ++g) {
+            int cc = -lin;        // -1: the linear part
+            const int64_t n = static_cast<int64_t>(n_my_tiles) * (NC + lin);
+            for (int64_t g = 0; g < n; ++g) {
                 if (r.wrapped && !mbar_wait(&sm.w2_free[r.slot], r.phase ^ 1u, abort_flag)) break;    // GEMM2 that read this slot is done
                 mbar_expect_tx(&sm.w2_full[r.slot], kTileBytes);
-                bulk_load(sm.w2[r.slot], p.packed + static_cast<size_t>(part * NC + cc) * kChunkBytes + kTileBytes, kTileBytes, &sm.w2_full[r.slot]);
+                bulk_load(sm.w2[r.slot], p.packed + (cc < 0 ? static_cast<size_t>(p.n_chunks) * kChunkBytes : static_cast<size_t>(part * NC + cc) * kChunkBytes + kTileBytes),
+                          kTileBytes, &sm.w2_full[r.slot]);
                 r.advance();
-                if (++cc == NC) cc = 0;
+                if (++cc == NC) cc = -lin;
             }
         }
     } else if (warp == 1) {
@@ -519,16 +656,34 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p, const __grid_constant__ S
         // ---------------------------------------------------------------- GEMM2 issuer
         constexpr uint32_t idesc2 = umma_idesc(kTok, kCh);
         constexpr uint32_t kTileUnits = kTileBytes >> 4;
-        const uint32_t w2_lo = desc_lo(sm.w2[0]);
+        const uint32_t w2_lo = desc_lo(sm.w2[0]), a_lo = desc_lo(sm.a[0]);
         bool ok = true;
         Ring<kW2Stages> rw;       // weights of the next GEMM2
         Ring<kBufs> cb;           // chunk buffer of the next GEMM2
         for (int it = 0; it < n_my_tiles && ok; ++it) {
+            const uint32_t d2 = tmem + kD2Col + static_cast<uint32_t>(it & 1) * kCh;
+            if (it >= 2)      // the tile that used this D2 buffer two tiles ago has been written out
+                ok = __all_sync(0xffffffffu, mbar_wait(&sm.d2_empty[it & 1], static_cast<uint32_t>((it >> 1) - 1) & 1u, abort_flag) ? 1 : 0) != 0;
+            if (ok && lin) {          // D2 = A * (kappa W1 W2 / 2), the matrix as the sum of two bf16 ones
+                ok = mbar_wait(&sm.w2_full[rw.slot], rw.phase, abort_flag) && mbar_wait(&sm.a_full[it & 1], static_cast<uint32_t>(it >> 1) & 1u, abort_flag);
+                ok = __all_sync(0xffffffffu, ok ? 1 : 0) != 0;
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t a_cur = a_lo + static_cast<uint32_t>(it & 1) * kTileUnits;
+                const uint32_t wb_lo = w2_lo + static_cast<uint32_t>(rw.slot) * kTileUnits;
+                if (elect_one()) {
+#pragma unroll
+                    for (int k = 0; k < 2 * kCh / 16; ++k)
+                        umma_bf16(d2, desc64(a_cur + 2u * (k % 4)), desc64(wb_lo + (k / 4) * ((kCh * 128) >> 4) + 2u * (k % 4)), idesc2, k > 0 ? 1u : 0u);
+                    umma_commit(&sm.w2_free[rw.slot]);
+                    umma_commit(&sm.a_empty[it & 1]);
+                }
+                __syncwarp();
+                rw.advance();
+            }
             for (int c = 0; c < NC && ok; ++c) {            // D2 += H[cb] * W2[rw]
                 ok = mbar_wait(&sm.w2_full[rw.slot], rw.phase, abort_flag);
                 if (ok) ok = mbar_wait(&sm.h_full[cb.slot], cb.phase, abort_flag);
-                if (ok && c == 0 && it >= 2)      // the tile that used this D2 buffer two tiles ago has been written out
-                    ok = mbar_wait(&sm.d2_empty[it & 1], static_cast<uint32_t>((it >> 1) - 1) & 1u, abort_flag);
                 ok = __all_sync(0xffffffffu, ok ? 1 : 0) != 0;
                 if (!ok) break;
                 tc_fence_after();
@@ -538,8 +693,8 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p, const __grid_constant__ S
 #pragma unroll
                     for (int k = 0; k < kHc / 16; ++k)      // hidden 16k .. 16k+15 of the chunk: 8 packed columns, the chunk's
                                                             // first 64 hidden units at columns 0..31 of the buffer, the rest at 64..95
-                        umma_bf16_ts(tmem + kD2Col + static_cast<uint32_t>(it & 1) * kCh, h_col + (k / 4) * 64u + 8u * (k % 4),
-                                     desc64(wb_lo + (k / 4) * ((kCh * 128) >> 4) + 2u * (k % 4)), idesc2, (c > 0 || k > 0) ? 1u : 0u);
+                        umma_bf16_ts(d2, h_col + (k / 4) * 64u + 8u * (k % 4),
+                                     desc64(wb_lo + (k / 4) * ((kCh * 128) >> 4) + 2u * (k % 4)), idesc2, (lin || c > 0 || k > 0) ? 1u : 0u);
                     umma_commit(&sm.buf_free[cb.slot]);
                     umma_commit(&sm.w2_free[rw.slot]);
                     if (c == NC - 1) umma_commit(&sm.d2_full[it & 1]);
@@ -596,9 +751,22 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p, const __grid_constant__ S
                 if (it + 1 < n_my_tiles) issue_tile_copy(it + 1);      // every lane has read the staging buffer
             }
         }
-        if (STEP && sp.prev.logp_out != nullptr)      // the previous level's log-probs, off the critical path
+        if (MODE != kNoStep && sp.prev.logp_out != nullptr)      // the previous level's log-probs, off the critical path
             finalize_rows(sp.prev, sp.n_trees, sp.nodes_cap, sp.half_per, blockIdx.x, gridDim.x, sp.status, sp.per_row);
         __syncwarp();
+    } else if (WHOLE && warp > kGemm2Warp) {
+        // ---------------------------------------------------------------- step warps: children of whole tiles
+        // Tile t's children are made while tile t + 1 is computed, in the issue slots the other warps leave; those of the last
+        // tile by all warps, at the end.
+        const uint32_t t = threadIdx.x - (kGemm2Warp + 1) * 32;
+        for (int it = 0; it + 1 < n_my_tiles; ++it) {
+            const int64_t first = (static_cast<int64_t>(cta) + static_cast<int64_t>(it) * n_ctas) * kTok;
+            const StepTile q = make_step_tile(sp, p, first, kTok);
+            auto v_ready = [&] { return __all_sync(0xffffffffu, mbar_wait(&sm.v_full, static_cast<uint32_t>(it) & 1u, abort_flag) ? 1 : 0) != 0; };
+            if (!step_tile<kStepWarps * 32, kStepRows>(sp, p, q, first, t, sm.vtile, v_ready)) break;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sm.v_free);
+        }
     } else {
         // ---------------------------------------------------------------- epilogue warps
         const int ew = warp - 2;                  // 0..15
@@ -619,7 +787,7 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p, const __grid_constant__ S
             }
         }
 
-        // v = D2 / 4 of tile t (this warp's 32 rows x 16 channels)
+        // v = D2 / kappa of tile t (this warp's 32 rows x 16 channels)
         auto output_tile = [&](int t) -> bool {
             const int b = t & 1;
             if (!__all_sync(0xffffffffu, mbar_wait(&sm.d2_full[b], static_cast<uint32_t>(t >> 1) & 1u, abort_flag) ? 1 : 0)) return false;
@@ -635,12 +803,21 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p, const __grid_constant__ S
             float4 val[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j)
-                val[j] = make_float4(0.25f * __uint_as_float(out[4 * j]), 0.25f * __uint_as_float(out[4 * j + 1]),
-                                     0.25f * __uint_as_float(out[4 * j + 2]), 0.25f * __uint_as_float(out[4 * j + 3]));
-            if (STEP || S > 1) {
-                // This CTA holds the sum over its share of the hidden dimension only; the tail of the kernel adds the parts.
+                val[j] = make_float4(kInvKappa * __uint_as_float(out[4 * j]), kInvKappa * __uint_as_float(out[4 * j + 1]),
+                                     kInvKappa * __uint_as_float(out[4 * j + 2]), kInvKappa * __uint_as_float(out[4 * j + 3]));
+            if (STEP || S > 1 || (WHOLE && t == n_my_tiles - 1)) {
+                // The sum over a share of the hidden dimension only, and the tail of the kernel adds the parts; or the last tile,
+                // and all warps make its children there.
 #pragma unroll
                 for (int j = 0; j < 4; ++j) *part_piece(sm.stage, row, sub * 4u + j) = val[j];
+                return true;
+            }
+            if (WHOLE) {          // to the step warps, once they are done with the tile before
+                if (t > 0 && !__all_sync(0xffffffffu, mbar_wait(&sm.v_free, static_cast<uint32_t>(t - 1) & 1u, abort_flag) ? 1 : 0)) return false;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) *part_piece(sm.vtile, row, sub * 4u + j) = val[j];
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&sm.v_full);
                 return true;
             }
             if (q < p.n_tokens) {
@@ -650,32 +827,28 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p, const __grid_constant__ S
             }
             return true;
         };
-        // 32 accumulator columns -> 16 registers of packed bf16 activation pairs
-        // One chunk of this warp: 64 accumulator columns arrive as float32, are rounded to packed bf16 pairs at once (32
-        // registers) and D1 is handed back before any arithmetic, so GEMM1 of chunk g + 2 runs under the activation of
-        // chunk g.  The packed polynomial covers |x| < 1; one bit of the packed pairs shows whether any of this thread's
-        // 64 values lies outside (or is not finite), and only then the thread takes the hardware-tanh form for its values.  With weights and latents of the usual scale (pre-activations of standard deviation ~0.2) that
-        // never happens.
-        auto pack16 = [&](const uint32_t (&acc)[32], uint32_t* xb) {
-#pragma unroll
-            for (int m = 0; m < 16; ++m) xb[m] = pack_bf16(__uint_as_float(acc[2 * m]), __uint_as_float(acc[2 * m + 1]));
-        };
-        auto activate = [&](uint32_t (&xb)[32]) {
+        // 32 accumulator columns of this thread's token, rounded to 16 registers of packed bf16 pairs, then the activations in
+        // their place.  The packed polynomial covers |x| < 1; one bit of the pairs shows whether any of the 32 values lies outside
+        // (or is not finite), and only then the thread takes the hardware-tanh form for them.  With weights and latents of the
+        // usual scale (pre-activations of standard deviation ~0.2) that never happens.
+        auto activate = [&](const uint32_t (&acc)[32], uint32_t (&xb)[16]) {
             uint32_t bits = 0u;
 #pragma unroll
-            for (int m = 0; m < 32; m += 2) bits |= xb[m] | xb[m + 1];
-            if ((bits & kGeluOutside) == 0u) {
+            for (int m = 0; m < 16; ++m) xb[m] = pack_bf16(__uint_as_float(acc[2 * m]), __uint_as_float(acc[2 * m + 1]));
 #pragma unroll
-                for (int m = 0; m < 32; ++m) xb[m] = gelu_x4_poly(xb[m]);
+            for (int m = 0; m < 16; m += 2) bits |= xb[m] | xb[m + 1];
+            if ((bits & kEvenOutside) == 0u) {
+#pragma unroll
+                for (int m = 0; m < 16; ++m) xb[m] = even_poly(xb[m]);
             } else {
 #pragma unroll
-                for (int m = 0; m < 32; ++m)
-                    xb[m] = pack_bf16(gelu_x4(__uint_as_float(xb[m] << 16)), gelu_x4(__uint_as_float(xb[m] & 0xffff0000u)));
+                for (int m = 0; m < 16; ++m)
+                    xb[m] = pack_bf16(even_tanh(__uint_as_float(xb[m] << 16)), even_tanh(__uint_as_float(xb[m] & 0xffff0000u)));
             }
         };
         const uint32_t my_cols = tmem + lane_addr + (sub & 1u) * 64u;     // this warp's 64 columns inside a chunk buffer
 
-        uint32_t acc[32], xb[32];
+        uint32_t acc[32], xb[16];
         // chunk index within this CTA's sequence of tiles x chunks; its buffer is g mod 3, the buffer's use number g / 3
         int buf = group, use = 0;
         for (int g = group; g < n_my_chunks && ok; g += 2) {
@@ -686,16 +859,15 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p, const __grid_constant__ S
             if (!ok) break;
             const uint32_t slice = my_cols + static_cast<uint32_t>(buf) * kHc;
             tc_fence_after();
-            tmem_ld32(slice, acc);
-            tmem_ld_wait32(acc);
-            pack16(acc, xb);
-            tmem_ld32(slice + 32u, acc);
-            tmem_ld_wait32(acc);
-            pack16(acc, xb + 16);
-            activate(xb);
-            // the packed activations go over the first 32 of the 64 columns this warp has just read
-            tmem_st16(slice, reinterpret_cast<const uint32_t (&)[16]>(xb[0]));
-            tmem_st16(slice + 16u, reinterpret_cast<const uint32_t (&)[16]>(xb[16]));
+            // Half by half: the packed activations go over the first 32 of this warp's 64 columns, each half over columns already
+            // read.  (The second half's load ahead of the first half's arithmetic: 725 us for 720.)
+#pragma unroll
+            for (uint32_t h = 0; h < 2; ++h) {
+                tmem_ld32(slice + 32u * h, acc);
+                tmem_ld_wait32(acc);
+                activate(acc, xb);
+                tmem_st16(slice + 16u * h, xb);
+            }
             tmem_st_wait();
             tc_fence_before();
             __syncwarp();
@@ -710,8 +882,12 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p, const __grid_constant__ S
     // ---------------------------------------------------------------- teardown
     tc_fence_before();
     __syncwarp();
-    if (!STEP && S == 1) {
+    if (MODE == kNoStep && S == 1) {
         __syncthreads();
+    } else if (WHOLE) {
+        const int64_t first = (static_cast<int64_t>(cta) + static_cast<int64_t>(n_my_tiles - 1) * n_ctas) * kTok;
+        const StepTile q = make_step_tile(sp, p, first, tile_rows(n_my_tiles - 1));
+        step_tile<kThreads, 1>(sp, p, q, first, threadIdx.x, sm.stage, [&] { __syncthreads(); return true; });
     } else {
         // The S parts of the tile are in the shared memory of the S CTAs of this cluster.  Each CTA adds every S-th row,
         // the parts in order, and leaves only when the others have read its own.  (Every thread gets here: the waits above are
@@ -735,16 +911,16 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p, const __grid_constant__ S
 #pragma unroll
             for (int o = 0; o < kMaxSplit; ++o)
                 if (o < S) { sum.x += x[o].x; sum.y += x[o].y; sum.z += x[o].z; sum.w += x[o].w; }
-            if (first + r < p.n_tokens) reinterpret_cast<float4*>(p.v_out)[(first + r) * (kCh / 4) + c4] = sum;
+            if (first + r < p.n_tokens && (!STEP || p.v_out)) reinterpret_cast<float4*>(p.v_out)[(first + r) * (kCh / 4) + c4] = sum;
             if (STEP && piece.live) step_children(sp, row0, piece, sum, sm.node_sums);
-            r += S * (kMlpThreads / (kCh / 4));
+            r += S * (kThreads / (kCh / 4));
             if (STEP) step_piece(sp, p, first, r, c4, piece);
         }
         __syncwarp();
         cluster_arrive();
         if (STEP && sp.g != 0.0f) {          // the sums of this CTA's tokens, by child
             __syncthreads();
-            for (int i = threadIdx.x; i < kTok * BGRPO_MAX_K; i += kMlpThreads) {
+            for (int i = threadIdx.x; i < kTok * BGRPO_MAX_K; i += kThreads) {
                 const int row = row0 + i / BGRPO_MAX_K, b = i % BGRPO_MAX_K;
                 const uint32_t* both = sm.node_sums[i / BGRPO_MAX_K][b];
                 const unsigned long long sum = (static_cast<unsigned long long>(both[1]) << 16) + both[0];
@@ -784,17 +960,46 @@ __global__ void mlp_pack_kernel(const uint16_t* __restrict__ W1, const uint16_t*
     }
 }
 
+// kappa W1 W2 / 2 as the sum of two bf16 matrices (16 bits of each element), behind the chunks and laid out like a chunk of W2:
+// two tiles [64 n = output channel][64 k = input channel].  One CTA per row k, sums in double.
+constexpr int kLinParts = 16;
+__global__ void __launch_bounds__(kCh * kLinParts) mlp_pack_linear_kernel(const uint16_t* __restrict__ W1, const uint16_t* __restrict__ W2, int hidden, unsigned char* __restrict__ packed) {
+    __shared__ double parts[kLinParts][kCh];
+    const int k = blockIdx.x, n = threadIdx.x % kCh, q = threadIdx.x / kCh;
+    double sum = 0.0;
+#pragma unroll 8
+    for (int j = q; j < hidden; j += kLinParts)
+        sum = fma(static_cast<double>(__bfloat162float(__ushort_as_bfloat16(W1[static_cast<size_t>(k) * hidden + j]))),
+                  static_cast<double>(__bfloat162float(__ushort_as_bfloat16(W2[static_cast<size_t>(j) * kCh + n]))), sum);
+    parts[q][n] = sum;
+    __syncthreads();
+    if (q != 0) return;
+    for (int o = 1; o < kLinParts; ++o) sum += parts[o][n];
+    const float m = static_cast<float>(0.5 * static_cast<double>(kKappa) * sum);
+    const __nv_bfloat16 hi = __float2bfloat16(m), lo = __float2bfloat16(m - __bfloat162float(hi));
+    const uint32_t off = sw128(static_cast<uint32_t>(n), static_cast<uint32_t>(k) >> 3) + (static_cast<uint32_t>(k) & 7u) * 2u;
+    unsigned char* tile = packed + static_cast<size_t>(hidden / kHc) * kChunkBytes;
+    *reinterpret_cast<uint16_t*>(tile + off) = __bfloat16_as_ushort(hi);
+    *reinterpret_cast<uint16_t*>(tile + kCh * 128 + off) = __bfloat16_as_ushort(lo);
+}
+
 }  // namespace
 
-size_t mlp_packed_bytes(int hidden) { return static_cast<size_t>(hidden / kHc) * kChunkBytes; }
+size_t mlp_packed_bytes(int hidden) { return static_cast<size_t>(hidden / kHc) * kChunkBytes + kTileBytes; }
 
 cudaError_t launch_mlp_pack(const uint16_t* W1, const uint16_t* W2, int hidden, void* packed, cudaStream_t s) {
     const int n = hidden * kCh;
     mlp_pack_kernel<<<(n + 255) / 256, 256, 0, s>>>(W1, W2, hidden, static_cast<unsigned char*>(packed));
+    const cudaError_t e = count_launch(cudaGetLastError());
+    if (e != cudaSuccess) return e;
+    mlp_pack_linear_kernel<<<kCh, kCh * kLinParts, 0, s>>>(W1, W2, hidden, static_cast<unsigned char*>(packed));
     return count_launch(cudaGetLastError());
 }
 
 namespace {
+template <int MODE>
+constexpr size_t kMlpSmemBytes = sizeof(MlpSmem<MODE>) + 1024;
+static_assert(kMlpSmemBytes<kStepOfWhole> <= 227 * 1024, "shared memory of an SM");
 // What a launch has to know of the current device.  Asked for once per device; host threads may get here together.
 struct MlpDevice {
     int sms = 0, clusters[kMaxSplit + 1] = {0};       // clusters[S]: how many clusters of S CTAs run at a time
@@ -805,36 +1010,37 @@ struct {
     MlpDevice device;
 } g_mlp_devices[64];
 
-cudaError_t mlp_query_device(int dev, size_t smem, MlpDevice* d) {
-    cudaError_t e = cudaFuncSetAttribute(mlp_velocity_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(mlp_velocity_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+cudaError_t mlp_query_device(int dev, MlpDevice* d) {
+    cudaError_t e = cudaFuncSetAttribute(mlp_velocity_kernel<kNoStep>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kMlpSmemBytes<kNoStep>));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(mlp_velocity_kernel<kStepOfSplit>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kMlpSmemBytes<kStepOfSplit>));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(mlp_velocity_kernel<kStepOfWhole>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kMlpSmemBytes<kStepOfWhole>));
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&d->sms, cudaDevAttrMultiProcessorCount, dev);
     for (int cand = 2; e == cudaSuccess && cand <= kMaxSplit; ++cand) {
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute attr[1];
         cfg.gridDim = cand;
-        cfg.blockDim = kMlpThreads;
-        cfg.dynamicSmemBytes = smem;
+        cfg.blockDim = kMlpThreads<kStepOfSplit>;
+        cfg.dynamicSmemBytes = kMlpSmemBytes<kStepOfSplit>;
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = static_cast<unsigned int>(cand);
         attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        e = cudaOccupancyMaxActiveClusters(&d->clusters[cand], mlp_velocity_kernel<true>, &cfg);
+        e = cudaOccupancyMaxActiveClusters(&d->clusters[cand], mlp_velocity_kernel<kStepOfSplit>, &cfg);
     }
     return e;
 }
 
-cudaError_t mlp_device(size_t smem, MlpDevice* out) {
+cudaError_t mlp_device(MlpDevice* out) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     std::lock_guard<std::mutex> lock(g_mlp_device_mutex);
-    if (dev < 0 || dev >= 64) return mlp_query_device(dev, smem, out);
+    if (dev < 0 || dev >= 64) return mlp_query_device(dev, out);
     auto& slot = g_mlp_devices[dev];
     if (!slot.known) {
         MlpDevice d;
-        e = mlp_query_device(dev, smem, &d);
+        e = mlp_query_device(dev, &d);
         if (e != cudaSuccess) return e;
         slot.device = d;
         slot.known = true;
@@ -847,9 +1053,8 @@ cudaError_t mlp_device(size_t smem, MlpDevice* out) {
 cudaError_t launch_mlp(const float* latents, int64_t pool_elems, int64_t tree_stride, int64_t row_offset, int n_trees, int64_t tokens_per_tree,
                        const void* packed, int hidden, float* v_out, int32_t* status, const StepLaunch* step, unsigned long long* row_sums,
                        bool* stepped, cudaStream_t s) {
-    constexpr size_t smem = sizeof(MlpSmem) + 1024;
     MlpDevice d;
-    cudaError_t e = mlp_device(smem, &d);
+    cudaError_t e = mlp_device(&d);
     if (e != cudaSuccess) return e;
     MlpArgs a;
     a.latents = latents;
@@ -876,17 +1081,29 @@ cudaError_t launch_mlp(const float* latents, int64_t pool_elems, int64_t tree_st
     a.row_sums = row_sums;
     StepLaunch sp;
     std::memset(&sp, 0, sizeof(sp));
-    // The step goes along where a tile is split: each CTA then has at most half a tile of children to make.  Whole passes, in
-    // us, with no step taken along / those of split tiles / also those of whole tiles: one tree of 256 tokens 198 / 170 / 170,
-    // of 2 025 tokens 380 / 368 / 381.
-    if (step && a.split > 1) {
+    const int64_t tokens = step ? tokens_per_tree / step->W_in : 0;
+    // The step goes along where a tile is split: each CTA then has at most half a tile of children to make, and a launch is saved.
+    // One tree of 256 tokens 198 us a pass without, 170 with.
+    // In large launches it goes along tile by tile, on warps of its own: the noise fills issue slots the activation leaves, and
+    // the velocities never leave the chip (8 B an element of 20).  One launch of 1 036 800 tokens and its step (with the root
+    // kernel, about 50 us), one child: 895 -> 842 us, at the power cap 1 006 -> 948; hidden 1536, 512, 256: 579 -> 543,
+    // 454 -> 401, 433 -> 385.  The children of a CTA's last tile come after it, so a few tiles an SM gain nothing: 1.7 (254 tiles, hidden
+    // 3072 and 1024) 41.5 -> 41.3 and 27.1 -> 28.2, 3.4 (507 tiles) 70.6 -> 67.9.  Two children are as much noise as a tile has
+    // room for (1 013 tiles 130 - 146 -> 128 - 148, 4 050 tiles 480 - 520 -> 459 - 471), three or a shared part more (323 tiles
+    // 42 -> 53).  Nodes of less than a tile of tokens would be more than two to a tile.
+    const bool whole = step && a.split == 1 && tokens >= kTok && !step->shared_noise && step->fan <= 2 &&
+                       a.n_tiles > (step->fan == 1 ? 2 : 16) * d.sms;
+    if (step && (a.split > 1 || whole)) {
         sp = *step;
         sp.half_per = logp_half_per(sp.D);
-        a.tokens = static_cast<int32_t>(tokens_per_tree / sp.W_in);
+        a.tokens = static_cast<int32_t>(tokens);
+        if (!sp.keep_v) a.v_out = nullptr;
         *stepped = true;
-        return launch_overlapped_clusters(mlp_velocity_kernel<true>, grid, kMlpThreads, smem, s, a.split, a, sp);
+        if (a.split > 1)
+            return launch_overlapped_clusters(mlp_velocity_kernel<kStepOfSplit>, grid, kMlpThreads<kStepOfSplit>, kMlpSmemBytes<kStepOfSplit>, s, a.split, a, sp);
+        return launch_overlapped(mlp_velocity_kernel<kStepOfWhole>, grid, kMlpThreads<kStepOfWhole>, kMlpSmemBytes<kStepOfWhole>, s, a, sp);
     }
-    return launch_overlapped_clusters(mlp_velocity_kernel<false>, grid, kMlpThreads, smem, s, a.split, a, sp);
+    return launch_overlapped_clusters(mlp_velocity_kernel<kNoStep>, grid, kMlpThreads<kNoStep>, kMlpSmemBytes<kNoStep>, s, a.split, a, sp);
 }
 
 }  // namespace bgrpo

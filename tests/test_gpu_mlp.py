@@ -2,7 +2,7 @@
 oracle's frontier latents are written into the device pool (so both sides see the same z), the CUDA stage runs
 through the C ABI, and its output is compared under  |d| <= 2e-2 |v| + 2e-2 rms(v)  and, on outputs of at least rms size,
 under the plain relative bound 2e-2 (bf16 operands, fp32 accumulation; the CUDA side evaluates the erf-form GELU by a
-polynomial in packed bf16 on |x| < 1 and by the tanh form on the hardware tanh outside).  The tree is then advanced with the oracle's velocity, so
+polynomial for its even half in packed bf16 on |x| < 1 and by the tanh form on the hardware tanh outside).  The tree is then advanced with the oracle's velocity, so
 later depths exercise frontiers of several nodes, several trees and ragged 128-token tiles."""
 import math
 
@@ -268,6 +268,50 @@ def test_rollout_that_takes_the_step_along_is_the_step_by_step_rollout(B, tokens
         assert torch.equal(r.logp, runs[0].logp)
         assert torch.equal(r.node_table.view(4, n_trees, -1)[:, :, :w.nodes], runs[0].node_table.view(4, n_trees, -1)[:, :, :w.nodes])
         assert torch.equal(r.v.view(-1)[:n], runs[0].v.view(-1)[:n])
+
+
+@pytest.mark.parametrize("tokens,n_trees,T,K,splits,hidden,sde", [
+    (128, 300, 2, 1, (), 128, None),                   # a node is a tile; a third tile for four CTAs only
+    (127, 400, 2, 1, (), 128, None),                   # less than a tile: the step has its own launch
+    (1011, 38, 3, 2, (2,), 256, None),                 # 301 tiles, nodes end inside them, a last tile of 18 rows; then a fork, on its own
+    (37889, 1, 4, 1, (), 128, (1, 0, 1, 0)),           # 297 tiles, one row in the last; ODE steps, the last one too
+    (199, 1900, 2, 2, (0,), 128, None),                # 2 954 tiles: two children each, then 5 908
+    (4096, 20, 3, 1, (), 1408, None),                  # eleven chunks, 640 tiles
+])
+def test_children_of_whole_tiles_are_the_step_by_step_rollouts(B, tokens, n_trees, T, K, splits, hidden, sde):
+    """Large frontiers: warps of the velocity launch make the children tile by tile.  The same bits as velocity and step in
+    launches of their own, the velocities of the last step included."""
+    test_rollout_that_takes_the_step_along_is_the_step_by_step_rollout(B, tokens, n_trees, T, K, splits, math.inf, hidden, sde)
+
+
+@pytest.mark.parametrize("w1_std", [0.003, 0.02, 0.06, 0.12, 0.5])
+def test_mlp_stage_against_64_bits(B, w1_std):
+    """Against the unrounded GELU MLP of the bf16 latents in 64 bits.  Only the even half of an activation is rounded to bf16
+    (2^-9 relative at most, as is its argument, which counts twice; 3.1e-4 the polynomial, 5e-4 the tanh form), and the roundings
+    of the hidden units add up like independent ones: rms error <= sqrt(sum_j W2_j^2 e_j^2) with e_j the largest of each."""
+    from paper_2509_06040_b200.session import TreeSession
+    from workloads import Inputs, _to_bf16_values
+    w = Workload(name="mlp_64", n_trees=1, tokens=600, channels=64, T=1, K=1, splits=(), sigma=0.3,
+                 velocity="mlp", reward="mixture", hidden=1024)
+    g = np.random.default_rng([5, int(w1_std * 1000)])
+    W1 = _to_bf16_values(w1_std * g.standard_normal((64, 1024), dtype=np.float32))
+    W2 = _to_bf16_values(0.02 * g.standard_normal((1024, 64), dtype=np.float32))
+    s = TreeSession(w)
+    s.upload_inputs(Inputs(W1=W1, W2=W2))
+    s.init()
+    B.velocity_mlp(s.tree, s.packed, w.hidden, s.v)
+    B.tree_sync_status(s.tree)
+    z = s.latents[0, 0].view(600, 64).to(torch.bfloat16).double()
+    x = z @ torch.from_numpy(W1).cuda().double()
+    W2d = torch.from_numpy(W2).cuda().double()
+    ref = torch.nn.functional.gelu(x) @ W2d
+    d = s.v.view(-1)[:ref.numel()].view_as(ref).double() - ref
+    E = (x * torch.special.erf(x / 2 ** 0.5) / 2).abs()
+    e = 2.0 ** -9 * 3 * E + 5e-4 * x.abs().clamp(max=1.0)
+    bound = ((e ** 2) @ (W2d ** 2)).mean().sqrt().item() + 2.0 ** -16 * ref.pow(2).mean().sqrt().item()
+    err = d.pow(2).mean().sqrt().item()
+    print(f"w1_std {w1_std}: rms error {err / ref.pow(2).mean().sqrt().item():.2e} of rms(v), bound {bound:.2e}, is {err:.2e}")
+    assert err <= bound
 
 
 def test_replayed_rollout_gives_the_same_log_probs_every_time(B):
