@@ -29,7 +29,7 @@
 //     warp 18      brings the NEXT tile's latents in with bulk asynchronous copies (one per tree the tile touches) into
 //                  a float32 staging buffer and converts them to the bf16 A tile while the current tile computes.  (Plain
 //                  loads from one warp kept only 4 KiB in flight and took longer per tile than the arithmetic.)  The
-//                  first tile of a launch is converted by the sixteen epilogue warps, idle until then.
+//                  first tile of a launch is loaded and converted by the sixteen epilogue warps, idle until then.
 // Shared-memory operands are K-major tiles of 128-byte rows in the 128-byte-swizzle layout the MMA descriptors
 // address; the weights are reordered once into exactly that image (bgrpo_velocity_mlp_pack), so a chunk arrives with
 // one copy per matrix.  No cluster multicast is used anywhere.
@@ -269,17 +269,17 @@ constexpr uint32_t kEvenOutside = 0x40004000u;
 // byte offset of the 16-byte piece `c16` of row r inside a 128-byte-swizzled tile of 128-byte rows
 __device__ __forceinline__ uint32_t sw128(uint32_t r, uint32_t c16) { return r * 128u + ((c16 ^ (r & 7u)) << 4); }
 
-// Converts rows [r_begin, r_end) of the float32 staging tile to the bf16 K-major swizzled A tile; one warp, two rows per
+// Converts the float32 staging tile to the bf16 K-major swizzled A tile; one warp, two rows per
 // step (16 lanes x 16 bytes cover a row).  Rows from `valid` on lie past the last token and are made zero first: left to
 // what the staging buffer held before, a few NaNs sent the rows of a ragged last tile through the slow activation, and
 // with one tile per CTA that CTA took twice as long as all others (16 200 tokens, hidden 3072: 31 us in place of 16).
-__device__ __forceinline__ void convert_rows(float* stage, unsigned char* atile, int r_begin, int r_end, int valid, int lane) {
+__device__ __forceinline__ void convert_tile(float* stage, unsigned char* atile, int valid, int lane) {
     const uint32_t c4 = static_cast<uint32_t>(lane & 15);
-    if (valid < r_end)        // at most once in a launch
-        for (int r = r_begin + (lane >> 4); r < r_end; r += 2)
+    if (valid < kTok)         // at most once in a launch
+        for (int r = lane >> 4; r < kTok; r += 2)
             if (r >= valid) *reinterpret_cast<float4*>(stage + r * kCh + c4 * 4u) = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 8
-    for (int r0 = r_begin; r0 < r_end; r0 += 2) {
+    for (int r0 = 0; r0 < kTok; r0 += 2) {
         const uint32_t r = static_cast<uint32_t>(r0 + (lane >> 4));
         const float4 zv = *reinterpret_cast<const float4*>(stage + r * kCh + c4 * 4u);
         uint2 packed2;
@@ -572,7 +572,7 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p, const __grid_constant__ S
     pdl_release();
     pdl_wait();
     const uint32_t tmem = sm.tmem_base;
-    const int S = p.split;
+    const int S = WHOLE ? 1 : p.split;
     const int cta = static_cast<int>(blockIdx.x) / S, part = static_cast<int>(blockIdx.x) - cta * S;   // tile walker, share of the hidden dimension
     const int n_ctas = static_cast<int>(gridDim.x) / S;
     const int n_my_tiles = (p.n_tiles > cta) ? (p.n_tiles - 1 - cta) / n_ctas + 1 : 0;
@@ -583,6 +583,10 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p, const __grid_constant__ S
     auto tile_rows = [&](int it) -> int {     // tokens of this CTA's tile number `it`
         const int64_t left = p.n_tokens - (static_cast<int64_t>(cta) + static_cast<int64_t>(it) * n_ctas) * kTok;
         return left < kTok ? static_cast<int>(left) : kTok;
+    };
+
+    auto a_ready = [&](int it) -> bool {      // the bf16 latents of tile number `it`: the first has a barrier of its own
+        return it == 0 ? mbar_wait(&sm.first_a, 0u, abort_flag) : mbar_wait(&sm.a_full[it & 1], static_cast<uint32_t>((it - 1) >> 1) & 1u, abort_flag);
     };
 
     if (warp == 0) {
@@ -627,7 +631,7 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p, const __grid_constant__ S
         Ring<kBufs> cb;           // chunk buffer of the next GEMM1: slot = chunk mod 3, phase = parity of its use number
         for (int it = 0; it < n_my_tiles && ok; ++it) {
             const int ab = it & 1;
-            ok = __all_sync(0xffffffffu, mbar_wait(&sm.a_full[ab], static_cast<uint32_t>(it >> 1) & 1u, abort_flag) ? 1 : 0) != 0;
+            ok = __all_sync(0xffffffffu, a_ready(it) ? 1 : 0) != 0;
             const uint32_t a_cur = a_lo + static_cast<uint32_t>(ab) * kTileUnits;
             for (int c = 0; c < NC && ok; ++c) {            // D1[cb] = A * W1[r]
                 ok = mbar_wait(&sm.w1_full[r.slot], r.phase, abort_flag);
@@ -665,7 +669,7 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p, const __grid_constant__ S
             if (it >= 2)      // the tile that used this D2 buffer two tiles ago has been written out
                 ok = __all_sync(0xffffffffu, mbar_wait(&sm.d2_empty[it & 1], static_cast<uint32_t>((it >> 1) - 1) & 1u, abort_flag) ? 1 : 0) != 0;
             if (ok && lin) {          // D2 = A * (kappa W1 W2 / 2), the matrix as the sum of two bf16 ones
-                ok = mbar_wait(&sm.w2_full[rw.slot], rw.phase, abort_flag) && mbar_wait(&sm.a_full[it & 1], static_cast<uint32_t>(it >> 1) & 1u, abort_flag);
+                ok = mbar_wait(&sm.w2_full[rw.slot], rw.phase, abort_flag) && a_ready(it);
                 ok = __all_sync(0xffffffffu, ok ? 1 : 0) != 0;
                 if (!ok) break;
                 tc_fence_after();
@@ -728,23 +732,20 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p, const __grid_constant__ S
                 remaining -= seg;
             }
         };
+        // The first tile is on the critical path of the launch and the sixteen epilogue warps have nothing to do yet: they load
+        // and convert it, eight rows each, and report on a barrier of its own.  (Through the
+        // staging buffer like the others, converted by the same warps: 1.8 us from the wait to the first GEMM, 1.6 so; a pass of one
+        // tree of 256 tokens 170 -> 163 us, of 2 025 tokens 367 -> 360, the 1 531-token trees of 27 leaves 802 -> 773.)
         bool ok = true;
-        if (n_my_tiles > 0 && lane == 0) issue_tile_copy(0);
-        for (int it = 0; it < n_my_tiles && ok; ++it) {
+        if (n_my_tiles > 1 && lane == 0) issue_tile_copy(1);
+        for (int it = 1; it < n_my_tiles && ok; ++it) {
             const int ab = it & 1;
-            if (it == 0) {
-                // The first tile is on the critical path of the launch and the sixteen epilogue warps have nothing to do
-                // yet: they convert it, eight rows each (one warp needs about 2 us for a tile), and report here.
-                ok = __all_sync(0xffffffffu, mbar_wait(&sm.first_a, 0u, abort_flag) ? 1 : 0) != 0;
-                if (!ok) break;
-            } else {
-                ok = mbar_wait(&sm.stage_full, static_cast<uint32_t>(it) & 1u, abort_flag);
-                if (ok && it >= 2) ok = mbar_wait(&sm.a_empty[ab], static_cast<uint32_t>((it >> 1) - 1) & 1u, abort_flag);
-                ok = __all_sync(0xffffffffu, ok ? 1 : 0) != 0;
-                if (!ok) break;
-                convert_rows(sm.stage, sm.a[ab], 0, kTok, tile_rows(it), lane);
-                proxy_fence();
-            }
+            ok = mbar_wait(&sm.stage_full, static_cast<uint32_t>(it - 1) & 1u, abort_flag);
+            if (ok && it >= 2) ok = mbar_wait(&sm.a_empty[ab], static_cast<uint32_t>((it >> 1) - 1) & 1u, abort_flag);
+            ok = __all_sync(0xffffffffu, ok ? 1 : 0) != 0;
+            if (!ok) break;
+            convert_tile(sm.stage, sm.a[ab], tile_rows(it), lane);
+            proxy_fence();
             __syncwarp();
             if (lane == 0) {
                 mbar_arrive(&sm.a_full[ab]);
@@ -778,13 +779,25 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p, const __grid_constant__ S
         bool ok = true;
         int next_out = 0;             // first tile this warp has not written out yet
         if (n_my_tiles > 0) {         // this warp's eight rows of the first A tile (see the loader warp)
-            ok = __all_sync(0xffffffffu, mbar_wait(&sm.stage_full, 0u, abort_flag) ? 1 : 0) != 0;
-            if (ok) {
-                convert_rows(sm.stage, sm.a[0], ew * (kTok / kEpiWarps), (ew + 1) * (kTok / kEpiWarps), tile_rows(0), lane);
-                proxy_fence();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&sm.first_a);
+            float4 z[kTok / kEpiWarps / 2];
+            const int64_t tok0 = static_cast<int64_t>(cta) * kTok;
+            const uint32_t c4 = static_cast<uint32_t>(lane & 15), per_tree = static_cast<uint32_t>(p.tokens_per_tree);
+            const uint32_t r0 = static_cast<uint32_t>(ew * (kTok / kEpiWarps) + (lane >> 4));
+#pragma unroll
+            for (uint32_t k = 0; k < kTok / kEpiWarps / 2; ++k) {      // rows past the last token are zero (see convert_tile)
+                const uint32_t token = static_cast<uint32_t>(tok0) + r0 + 2u * k, tree = token / per_tree;
+                const int64_t at = tree * p.tree_stride + p.row_offset + static_cast<int64_t>(token - tree * per_tree) * kCh;
+                z[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (token < p.n_tokens && BGRPO_IN_BOUNDS(p.status, at >= 0 && at + kCh <= p.pool_elems)) z[k] = __ldcg(reinterpret_cast<const float4*>(p.latents + at) + c4);
             }
+#pragma unroll
+            for (uint32_t k = 0; k < kTok / kEpiWarps / 2; ++k) {
+                const uint32_t r = r0 + 2u * k;
+                *reinterpret_cast<uint2*>(sm.a[0] + sw128(r, c4 >> 1) + (c4 & 1u) * 8u) = make_uint2(pack_bf16(z[k].x, z[k].y), pack_bf16(z[k].z, z[k].w));
+            }
+            proxy_fence();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sm.first_a);
         }
 
         // v = D2 / kappa of tile t (this warp's 32 rows x 16 channels)
