@@ -432,6 +432,21 @@ __device__ __forceinline__ void step_load(const StepTile& q, int32_t r0, int32_t
         if (r < q.rows) z[k] = __ldcg((r < q.edge ? q.z_a : q.z_b) + r * (kCh / 4) + c4);
     }
 }
+// Adds a warp's squares of child b to the nodes' sums: 32 numbers, their 16-bit halves by themselves.
+__device__ __forceinline__ void add_squares(const MlpArgs& p, const StepTile& q, int b, uint32_t sum_a, uint32_t sum_b) {
+    uint32_t lo = __reduce_add_sync(0xffffffffu, sum_a & 0xffffu), hi = __reduce_add_sync(0xffffffffu, sum_a >> 16);
+    if ((threadIdx.x & 31u) == 0u && (lo | hi) != 0u) atomicAdd(p.row_sums + q.child0_a + b, (static_cast<unsigned long long>(hi) << 16) + lo);
+    if (q.edge < kTok) {
+        lo = __reduce_add_sync(0xffffffffu, sum_b & 0xffffu);
+        hi = __reduce_add_sync(0xffffffffu, sum_b >> 16);
+        if ((threadIdx.x & 31u) == 0u && (lo | hi) != 0u) atomicAdd(p.row_sums + q.child0_b + b, (static_cast<unsigned long long>(hi) << 16) + lo);
+    }
+}
+// Node-table rows of the children whose nodes start in the tile.
+__device__ __forceinline__ void step_tables(const StepLaunch& sp, const StepTile& q, uint32_t t) {
+    if (t < static_cast<uint32_t>(sp.fan) && q.e_a == 0u && q.rows > 0) step_table(sp, q.parent_a, q.child0_a, t);
+    if (t >= 32u && t - 32u < static_cast<uint32_t>(sp.fan) && q.edge < q.rows) step_table(sp, q.parent_b, q.child0_b, t - 32);
+}
 // The children of one float4 of N rows, given their velocities in shared memory: N chains of noise in flight.  `z` has the
 // parents; once they are used `then` may ask for the next ones.  Whole warps.
 template <int N, class Then>
@@ -483,13 +498,52 @@ __device__ __forceinline__ void step_rows(const StepLaunch& sp, const MlpArgs& p
                 (in_a ? child_a : child_b)[r * (kCh / 4) + c4] = fma4(sp.g, xi, m[k]);
             }
         }
-        // the warp's 32 numbers, their 16-bit halves by themselves
-        uint32_t lo = __reduce_add_sync(0xffffffffu, sum_a & 0xffffu), hi = __reduce_add_sync(0xffffffffu, sum_a >> 16);
-        if ((threadIdx.x & 31u) == 0u && (lo | hi) != 0u) atomicAdd(p.row_sums + q.child0_a + b, (static_cast<unsigned long long>(hi) << 16) + lo);
-        if (q.edge < kTok) {
-            lo = __reduce_add_sync(0xffffffffu, sum_b & 0xffffu);
-            hi = __reduce_add_sync(0xffffffffu, sum_b >> 16);
-            if ((threadIdx.x & 31u) == 0u && (lo | hi) != 0u) atomicAdd(p.row_sums + q.child0_b + b, (static_cast<unsigned long long>(hi) << 16) + lo);
+        add_squares(p, q, b, sum_a, sum_b);
+    }
+}
+// The noise of a tile's only children ahead of its velocities, to shared memory (whole warps, 128 rows by THREADS threads); then,
+// with the velocities there, the children by all threads of the CTA, up to N rows each.
+template <int THREADS, int N>
+__device__ __forceinline__ void step_tile_noise(const StepLaunch& sp, const MlpArgs& p, const StepTile& q, uint32_t t, float* xi_tile) {
+    constexpr int kStride = THREADS / (kCh / 4);
+    const uint32_t c4 = t % (kCh / 4);
+    const NoiseNode node_a = noise_node(sp.node_id_base + q.child0_a, sp.step, sp.keys), node_b = noise_node(sp.node_id_base + q.child0_b, sp.step, sp.keys);
+    uint32_t sum_a = 0u, sum_b = 0u;          // eight numbers at most of 25 bits
+    static_assert(kTok / kStride <= 8, "the sums of a thread");
+#pragma unroll 1
+    for (int32_t r0 = static_cast<int32_t>(t / (kCh / 4)); r0 < kTok; r0 += N * kStride) {
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            const int32_t r = r0 + k * kStride;
+            const bool in_a = r < q.edge;
+            const NoiseElement el = noise_element((in_a ? q.e_a : q.e_b) + static_cast<uint32_t>(r) * (kCh / 4) + c4, BGRPO_TAG_INNOV, sp.keys);
+            float squares;
+            *part_piece(xi_tile, static_cast<uint32_t>(r), c4) = normal4(philox_from(el, {node_a.x, in_a ? node_a.z : node_b.z, in_a ? node_a.w : node_b.w}, sp.keys), squares);
+            if (r < q.rows) {
+                const uint32_t n = quantized_squares(squares);
+                if (in_a) sum_a += n;
+                else sum_b += n;
+            }
+        }
+    }
+    add_squares(p, q, 0, sum_a, sum_b);
+}
+template <int THREADS>
+__device__ __forceinline__ void step_tile_children(const StepLaunch& sp, const MlpArgs& p, const StepTile& q, int64_t first, uint32_t t, float* vtile, float* xi_tile) {
+    constexpr int kStride = THREADS / (kCh / 4), N = (kTok + kStride - 1) / kStride;
+    const uint32_t c4 = t % (kCh / 4);
+    const int32_t r0 = static_cast<int32_t>(t / (kCh / 4));
+    float4 z[N];
+    step_load<N>(q, r0, kStride, c4, z);
+    step_tables(sp, q, t);
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        const int32_t r = r0 + k * kStride;
+        if (r < q.rows) {
+            const float4 v = *part_piece(vtile, static_cast<uint32_t>(r), c4);
+            if (p.v_out) reinterpret_cast<float4*>(p.v_out)[(first + r) * (kCh / 4) + c4] = v;
+            (r < q.edge ? q.child_a : q.child_b)[r * (kCh / 4) + c4] = fma4(sp.g, *part_piece(xi_tile, static_cast<uint32_t>(r), c4), fma4(sp.ca, z[k], mul4(sp.cb, v)));
         }
     }
 }
@@ -503,8 +557,7 @@ __device__ __forceinline__ bool step_tile(const StepLaunch& sp, const MlpArgs& p
     int32_t r = static_cast<int32_t>(t / (kCh / 4));
     float4 z[N];
     step_load<N>(q, r, kStride, c4, z);
-    if (t < static_cast<uint32_t>(sp.fan) && q.e_a == 0u && q.rows > 0) step_table(sp, q.parent_a, q.child0_a, t);
-    if (t >= 32u && t - 32u < static_cast<uint32_t>(sp.fan) && q.edge < q.rows) step_table(sp, q.parent_b, q.child0_b, t - 32);
+    step_tables(sp, q, t);
     if (!v_ready()) return false;
 #pragma unroll 1
     for (int32_t done = 0; done < kTok; done += N * kStride, r += N * kStride)
@@ -585,6 +638,11 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p, const __grid_constant__ S
         return left < kTok ? static_cast<int>(left) : kTok;
     };
 
+    // The step of whole tiles: where a node has one child the noise of a CTA's last tile is drawn before its velocities are there.
+    const bool ahead = WHOLE && sp.fan == 1 && sp.g != 0.0f;
+    auto last_tile = [&]() -> StepTile {
+        return make_step_tile(sp, p, (static_cast<int64_t>(cta) + static_cast<int64_t>(n_my_tiles - 1) * n_ctas) * kTok, tile_rows(n_my_tiles - 1));
+    };
     auto a_ready = [&](int it) -> bool {      // the bf16 latents of tile number `it`: the first has a barrier of its own
         return it == 0 ? mbar_wait(&sm.first_a, 0u, abort_flag) : mbar_wait(&sm.a_full[it & 1], static_cast<uint32_t>((it - 1) >> 1) & 1u, abort_flag);
     };
@@ -768,6 +826,10 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p, const __grid_constant__ S
             __syncwarp();
             if (lane == 0) mbar_arrive(&sm.v_free);
         }
+        if (ahead) {      // the last tile's velocities go elsewhere, so this buffer can take its noise meanwhile
+            __syncwarp();
+            step_tile_noise<kStepWarps * 32, kStepRows>(sp, p, last_tile(), t, sm.vtile);
+        }
     } else {
         // ---------------------------------------------------------------- epilogue warps
         const int ew = warp - 2;                  // 0..15
@@ -899,8 +961,8 @@ mlp_velocity_kernel(const __grid_constant__ MlpArgs p, const __grid_constant__ S
         __syncthreads();
     } else if (WHOLE) {
         const int64_t first = (static_cast<int64_t>(cta) + static_cast<int64_t>(n_my_tiles - 1) * n_ctas) * kTok;
-        const StepTile q = make_step_tile(sp, p, first, tile_rows(n_my_tiles - 1));
-        step_tile<kThreads, 1>(sp, p, q, first, threadIdx.x, sm.stage, [&] { __syncthreads(); return true; });
+        if (ahead) step_tile_children<kThreads>(sp, p, last_tile(), first, threadIdx.x, sm.stage, sm.vtile);
+        else step_tile<kThreads, 1>(sp, p, last_tile(), first, threadIdx.x, sm.stage, [&] { __syncthreads(); return true; });
     } else {
         // The S parts of the tile are in the shared memory of the S CTAs of this cluster.  Each CTA adds every S-th row,
         // the parts in order, and leaves only when the others have read its own.  (Every thread gets here: the waits above are
@@ -1097,15 +1159,16 @@ cudaError_t launch_mlp(const float* latents, int64_t pool_elems, int64_t tree_st
     const int64_t tokens = step ? tokens_per_tree / step->W_in : 0;
     // The step goes along where a tile is split: each CTA then has at most half a tile of children to make, and a launch is saved.
     // One tree of 256 tokens 198 us a pass without, 170 with.
-    // In large launches it goes along tile by tile, on warps of its own: the noise fills issue slots the activation leaves, and
-    // the velocities never leave the chip (8 B an element of 20).  One launch of 1 036 800 tokens and its step (with the root
-    // kernel, about 50 us), one child: 895 -> 842 us, at the power cap 1 006 -> 948; hidden 1536, 512, 256: 579 -> 543,
-    // 454 -> 401, 433 -> 385.  The children of a CTA's last tile come after it, so a few tiles an SM gain nothing: 1.7 (254 tiles, hidden
-    // 3072 and 1024) 41.5 -> 41.3 and 27.1 -> 28.2, 3.4 (507 tiles) 70.6 -> 67.9.  Two children are as much noise as a tile has
-    // room for (1 013 tiles 130 - 146 -> 128 - 148, 4 050 tiles 480 - 520 -> 459 - 471), three or a shared part more (323 tiles
-    // 42 -> 53).  Nodes of less than a tile of tokens would be more than two to a tile.
-    const bool whole = step && a.split == 1 && tokens >= kTok && !step->shared_noise && step->fan <= 2 &&
-                       a.n_tiles > (step->fan == 1 ? 2 : 16) * d.sms;
+    // Elsewhere it goes along tile by tile, on warps of its own: the noise fills issue slots the activation leaves, and the
+    // velocities never leave the chip (8 B an element of 20).  Launch and step of one child (with the root kernel, about 50 us of
+    // the first line), us: 1 036 800 tokens of hidden 3072 891 -> 839 (at the power cap 1 006 -> 948), of 1536, 512, 256 577 -> 520,
+    // 456 -> 373, 433 -> 347; 254 tiles of 3072, 1408, 1024 41.7 -> 39.3, 29.9 -> 28.6, 27.2 -> 26.4; 79 tiles of 3072, 1024
+    // 25.4 -> 22.3, 19.8 -> 16.5.  With less than four chunks there is no time to draw the last tile's noise in: 79 and 254 tiles of
+    // 256 14.2 -> 15.5 and 22.0 -> 23.0, which only more than two tiles an SM outweigh.
+    // Two children are as much noise as a tile has room for (1 013 tiles 130 - 146 -> 128 - 148, 4 050 tiles 480 - 520 -> 459 -
+    // 471), three or a shared part more (323 tiles 42 -> 53).  Nodes of less than a tile of tokens would be more than two to a tile.
+    const bool whole = step && a.split == 1 && tokens >= kTok && !step->shared_noise &&
+                       ((step->fan == 1 && (a.n_chunks >= 4 || a.n_tiles > 2 * d.sms)) || (step->fan == 2 && a.n_tiles > 16 * d.sms));
     if (step && (a.split > 1 || whole)) {
         sp = *step;
         sp.half_per = logp_half_per(sp.D);

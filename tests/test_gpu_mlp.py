@@ -277,6 +277,9 @@ def test_rollout_that_takes_the_step_along_is_the_step_by_step_rollout(B, tokens
     (37889, 1, 4, 1, (), 128, (1, 0, 1, 0)),           # 297 tiles, one row in the last; ODE steps, the last one too
     (199, 1900, 2, 2, (0,), 128, None),                # 2 954 tiles: two children each, then 5 908
     (4096, 20, 3, 1, (), 1408, None),                  # eleven chunks, 640 tiles
+    (5777, 2, 3, 2, (1,), 640, None),                  # 91 tiles, at most one to a CTA; a fork, on its own; 181 tiles
+    (9600, 1, 3, 1, (), 512, (0, 1, 0)),               # four chunks; ODE steps first and last
+    (9601, 1, 2, 1, (), 384, None),                    # three chunks: on its own
 ])
 def test_children_of_whole_tiles_are_the_step_by_step_rollouts(B, tokens, n_trees, T, K, splits, hidden, sde):
     """Large frontiers: warps of the velocity launch make the children tile by tile.  The same bits as velocity and step in
