@@ -379,7 +379,9 @@ def kernel_rooflines(s, w, peaks, flush_buf, reps, one_launch_ms=None):
     dominant kernel, roofline of the step kernel, ms per pass by kernel).  one_launch_ms: the rollout of the timed pass is one
     kernel of that many ms; the step kernel's figures are then those of tree_step called depth by depth, not a part of it.  An interval between two events holds one launch and the gap
     the event itself inserts (it also keeps the next launch's ramp from overlapping this launch's tail), so on
-    workloads made of launches of a few microseconds the intervals add up to more than the un-instrumented pass."""
+    workloads made of launches of a few microseconds the intervals add up to more than the un-instrumented pass.  Velocity and step
+    are timed in launches of their own here; a pass through tree_rollout has one launch for both where that is faster, so its
+    time is below the sum."""
     import torch
     from paper_2509_06040_b200 import binding as B
     t_step, t_mlp = np.zeros(w.T), np.zeros(w.T)
