@@ -51,8 +51,8 @@ NCU_TRAFFIC = {
                            "sources": ("tree_step.cu", "philox.cuh"), "shape": "kStep", "source_hash": "c4501886b74e"},
     "step_kernel_mlp": {"bytes": 531.953408e6 + 218.003968e6, "units": 32 * 16 * 129600,         # profiles/step_kernel_image_batch.md
                         "sources": ("tree_step.cu", "philox.cuh"), "shape": "kStep", "source_hash": "c4501886b74e"},
-    "mlp_velocity_kernel": {"bytes": 266.727680e6 + 215.012096e6, "units": 1036800,       # profiles/mlp_velocity_kernel_image_batch.md
-                            "sources": ("mlp_velocity.cu",), "shape": "kMlp", "source_hash": "cccfd06d2864"},
+    "mlp_velocity_kernel": {"bytes": 266.453760e6 + 214.518016e6, "units": 1036800,       # profiles/mlp_velocity_kernel_image_batch.md
+                            "sources": ("mlp_velocity.cu",), "shape": "kMlp", "source_hash": "9496c5f7790e"},
     "rollout_fused_kernel": {"bytes": 25.279488e6 + 864.974592e6, "units": 110 * 2096640,  # profiles/rollout_fused_kernel_video.md
                              "sources": ("tree_fused.cu", "philox.cuh"), "shape": "kFused", "source_hash": "2ce9e3414b6a"},
 }
