@@ -743,7 +743,7 @@ def run_ours(args, w):
         roof = fused or roof
         breakdown["pass"] = r4(total_ms / args.steps)
         breakdown["note"] = ("one event interval per launch; each holds the event's own gap, so the sum exceeds the pass "
-                             "where launches take microseconds" if breakdown["sum"] > 1.1 * breakdown["pass"]
+                             "where launches take microseconds, or where the pass has one launch for velocity and step" if breakdown["sum"] > 1.1 * breakdown["pass"]
                              else "one event interval per launch")
 
     # ---- the tree against independent sequential rollouts with as many final samples (rank 0, single GPU)
